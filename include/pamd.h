@@ -384,7 +384,7 @@ int pamd_device_status(void* stream);
 /* Launch-shape override for the Lennard-Jones kernels (0 or a negative skin
  * keeps the automatic choice): steps per CTA tile, threads per particle
  * (1, 2 or 4), neighbour-list capacity per particle, Verlet skin (sigma
- * units; double precision), steps per neighbour-list window (single
+ * units; Euler-Maruyama paths and the one-step form), steps per neighbour-list window (single
  * precision; >= 2).  Affects plans built afterwards.  Results do not depend
  * on the tile, capacity, skin or window (candidate order is fixed); the
  * number of threads per particle changes how a particle's force and
@@ -472,8 +472,8 @@ int pamd_fp64_fma_probe(int blocks, int threads, int iters, double* out, double*
  *   *checked : 1 in the debug build, 0 in the normal library (no checks);
  *   *count   : out-of-bounds accesses recorded since the last call;
  *   *site, *index, *bound : the first of them: file * 100000 + source line
- *              (files 1..5: ho_kernels, lj_kernels, lj_paired, update_kernels,
- *              fragment_kernels), the index and the array's extent,
+ *              (files 1..6: ho_kernels, lj_kernels, lj_paired, update_kernels,
+ *              fragment_kernels, lj_double), the index and the array's extent,
  * and clears the records.  Any pointer may be NULL. */
 int pamd_debug_status(int* checked, int* count, int* site, long long* index, long long* bound);
 

@@ -15,7 +15,8 @@ LIB = os.path.join(HERE, "libpamd.so")
 # bounds-checked variant (-DPAMD_DEBUG): every kernel array index is checked
 BUILD_DEBUG = os.path.join(HERE, "_build_debug")
 LIB_DEBUG = os.path.join(HERE, "libpamd_debug.so")
-SOURCES = ["pamd_api.cu", "ho_kernels.cu", "lj_kernels.cu", "lj_paired.cu", "update_kernels.cu", "noalloc.cu",
+SOURCES = ["pamd_api.cu", "ho_kernels.cu", "lj_kernels.cu", "lj_paired.cu", "lj_double.cu",
+           "update_kernels.cu", "noalloc.cu",
            "fragment_kernels.cu", "probe.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",

@@ -1,5 +1,6 @@
-// lj_kernels.cu -- Lennard-Jones path action and adjoint gradient, Euler-Maruyama
-// reference paths, and the single-precision pair-count diagnostic.
+// lj_kernels.cu -- Lennard-Jones path action and adjoint gradient one step at a time
+// (single precision, PAMD_LJ_ONE_STEP=1), Euler-Maruyama reference paths, and the
+// single-precision pair-count diagnostic.
 //
 // Pair potential (paper Eq. (11)), cut and force shifted:
 //   U(r) = u(r) - u(rc) - (r - rc) u'(rc)  (r <= rc),  u = 4 eps[(s/r)^12 - (s/r)^6].
@@ -410,14 +411,9 @@ cudaError_t launch_lj_items(const LJItem* items, int n_items, const void* sys_ta
 }
 
 template int lj_blocks_per_sm<float>(int, size_t, bool);
-template int lj_blocks_per_sm<double>(int, size_t, bool);
 template cudaError_t launch_lj_items<float>(const LJItem*, int, const void*, int, const float*,
                                             float*, double*, int*, int, size_t, int, bool,
                                             cudaStream_t, const float*, int*);
-template cudaError_t launch_lj_items<double>(const LJItem*, int, const void*, int, const double*,
-                                             double*, double*, int*, int, size_t, int, bool,
-                                             cudaStream_t, const double*, int*);
-
 // ------------------------------------------------------------------ hard-sphere path bias
 // Squared hard-sphere radii in the path's precision (a radius <= 0: no bias at
 // that slice, -1).

@@ -84,6 +84,7 @@ struct LJClass {
     bool pipe = false;           // gradient pass pipelined over step pairs
     size_t smem = 0;
     long long outer_words = 0;   // 32-bit words of each CTA's outer-list region
+    LJDoubleShape dbl;           // double precision: capacities of lj_double.cu
     int item_off = 0, n_items = 0;  // its items in d_lj_items (cost-sorted)
     int grp_off = 0;             // its items in d_lj_items_grp (grouped by chain)
     std::vector<int> grp_first;  // per global chain c: [grp_first[c], grp_first[c + 1]), relative
@@ -159,6 +160,11 @@ struct Plan {
     // (the classes of a lane run one after another and share its set)
     uint32_t* d_outer = nullptr;
     long long outer_lane_words = 0;  // 32-bit words of one lane's set
+    // double precision: one set of pair scratch (a region per CTA) per compute lane, and
+    // the edge records of every S slot
+    unsigned char* d_dbl_scratch = nullptr;
+    size_t dbl_lane_bytes = 0;
+    double* d_dbl_edge = nullptr;
     int n_lanes = 1;            // compute lanes of the host-buffer pipeline
     // hard-sphere path bias (pamd_action_grad_hs): radii of every LJ slice, per-chain flags
     long long hs_slices = 0;
@@ -391,6 +397,7 @@ void fill_lj_sys(Plan* P, const pamd_problem* p)
         // results are bitwise the same, which a test checks)
         d.shared_shift = std::getenv("PAMD_LJ_PER_STEP_SHIFT") == nullptr;
         d.write_nose = !si.halo_hi;
+        d.halo_lo = si.halo_lo;
         d.chain0 = si.chain0;
         d.hs_off = si.hs_off = P->hs_slices;  // this system's slices in the hard-sphere radii
         P->hs_slices += si.T + 1;
@@ -554,23 +561,44 @@ int build_plan(const pamd_problem* p, Plan** out)
                     si.NT = NT;
                     cap_used = std::max(cap_used, si.tune.maxnb);
                 }
+                if (P->fp64) {
+                    double pairs = 0.0;
+                    for (auto& si : P->sys) {
+                        if (si.kind != PAMD_LJ || si.lj_class != k) continue;
+                        const double L = si.pot.box, f = 4.18879020478639 * si.pot.rc * si.pot.rc * si.pot.rc / (L * L * L);
+                        pairs = std::max(pairs, 0.5 * si.N * si.N * f);
+                    }
+                    C.dbl = lj_double_shape(nmax, pairs, max_dynamic_smem() - 1024);
+                }
                 C.smem = P->lj_paired ? lj_paired_smem_bytes(NT, cap_used, C.pipe)
-                                      : lj_smem_bytes(nmax, NT, cap_used, P->fp64);
+                         : P->fp64    ? C.dbl.smem
+                                      : lj_smem_bytes(nmax, NT, cap_used, false);
                 const int bg = P->lj_paired ? lj_paired_blocks_per_sm(NT, C.smem, true, C.pipe)
-                               : P->fp64    ? lj_blocks_per_sm<double>(NT, C.smem, true)
+                               : P->fp64    ? lj_double_blocks_per_sm(C.smem, true)
                                             : lj_blocks_per_sm<float>(NT, C.smem, true);
                 const int bn = P->lj_paired ? lj_paired_blocks_per_sm(NT, C.smem, false, C.pipe)
-                               : P->fp64    ? lj_blocks_per_sm<double>(NT, C.smem, false)
+                               : P->fp64    ? lj_double_blocks_per_sm(C.smem, false)
                                             : lj_blocks_per_sm<float>(NT, C.smem, false);
                 if (bg <= 0 || bn <= 0) return PAMD_ERR_UNSUPPORTED;
                 bg_cls[k] = bg;
                 C.grid_grad = bg * sms;  // trimmed to the item count below
                 C.grid_nograd = bn * sms;
             }
+            // Double precision: a step costs tens of microseconds and an item nothing more
+            // than one deferred slice, so items are short, about eight per CTA, up to 32 steps.
+            if (P->fp64 && g_tune_override.tile_steps <= 0) {
+                long long steps = 0;
+                for (auto& si : P->sys)
+                    if (si.kind == PAMD_LJ) steps += (long long)si.chains * si.T;
+                const long long ctas = (long long)bg_cls[0] * sms;
+                for (auto& si : P->sys)
+                    if (si.kind == PAMD_LJ)
+                        si.tune.tile_steps = (int)std::max(1LL, std::min(32LL, steps / std::max(1LL, 8 * ctas)));
+            }
             // One LJ system of equal items: pick the tile near the chosen one whose item
             // count fills whole rounds of the persistent grid (no part-empty last round),
             // keeping at least 16 steps per item.
-            if (nlj == 1 && !one) {
+            if (nlj == 1 && !one && !P->fp64) {
                 for (auto& si : P->sys) {
                     if (si.kind != PAMD_LJ) continue;
                     const long long G = (long long)bg_cls[si.lj_class] * sms;
@@ -668,6 +696,17 @@ int build_plan(const pamd_problem* p, Plan** out)
                 }
                 if ((rc0 = P->alloc(&P->d_outer, sizeof(uint32_t) * P->n_lanes * P->outer_lane_words)))
                     return rc0;
+            }
+            if (P->fp64) {
+                P->n_lanes = pipeline_lanes();
+                int edge = 0;
+                for (auto& C : P->lj_cls) {
+                    P->dbl_lane_bytes = std::max(P->dbl_lane_bytes,
+                                                 C.dbl.scratch * (size_t)std::max(C.grid_grad, C.grid_nograd));
+                    edge = std::max(edge, C.dbl.edge_doubles);
+                }
+                if ((rc0 = P->alloc(&P->d_dbl_scratch, P->n_lanes * P->dbl_lane_bytes))) return rc0;
+                if ((rc0 = P->alloc(&P->d_dbl_edge, sizeof(double) * (size_t)edge * slot))) return rc0;
             }
             if (P->fp64)
                 fill_lj_sys<double>(P.get(), p);
@@ -800,14 +839,19 @@ int run_action(const pamd_problem* p, Plan* P, const R* pos, R* grad, double* S_
         const LJClass& C = P->lj_cls[k];
         if (C.n_items <= 0) continue;
         const int grid = with_grad ? C.grid_grad : C.grid_nograd;
-        auto launch = [&](const LJItem* items, int n, int g) {
+        auto launch = [&](const LJItem* items, int n, int g) -> cudaError_t {
             if (std::is_same<R, float>::value && P->lj_paired)
                 return launch_lj_paired(items, n, P->d_lj_sys, (const float*)pos, (float*)grad,
                                         P->d_part_S, counter, C.NT, C.smem, g, with_grad, C.pipe,
                                         P->d_outer + (long long)lane * P->outer_lane_words,
                                         C.outer_words, st, (const float*)hs2, overlap);
-            return launch_lj_items<R>(items, n, P->d_lj_sys, C.nmax, pos, grad, P->d_part_S, counter,
-                                      C.NT, C.smem, g, with_grad, st, hs2, overlap);
+            if constexpr (std::is_same<R, double>::value)
+                return launch_lj_double(items, n, P->d_lj_sys, C.nmax, C.dbl, pos, grad, P->d_part_S, counter,
+                                        g, with_grad, P->d_dbl_scratch + lane * P->dbl_lane_bytes, P->d_dbl_edge,
+                                        st, hs2, overlap);
+            else
+                return launch_lj_items(items, n, P->d_lj_sys, C.nmax, pos, grad, P->d_part_S, counter, C.NT,
+                                       C.smem, g, with_grad, st, hs2, overlap);
         };
         if (one) {
             for (int c = c0; c < c1; ++c) {
@@ -1014,10 +1058,11 @@ int pamd_debug_status(int* checked, int* count, int* site, long long* index, lon
     const int compiled = 0;
 #endif
     int (*const fetch[])(DebugRecord*) = {debug_fetch_ho, debug_fetch_lj, debug_fetch_lj_paired,
-                                          debug_fetch_update, debug_fetch_fragment};
+                                          debug_fetch_update, debug_fetch_fragment,
+                                          debug_fetch_lj_double};
     int total = 0, first_site = 0;
     long long first_index = 0, first_bound = 0;
-    for (int f = 0; f < 5; ++f) {
+    for (int f = 0; f < 6; ++f) {
         DebugRecord r;
         if (fetch[f](&r)) return PAMD_ERR_CUDA;
         if (r.count && !total) {

@@ -82,6 +82,7 @@ static inline int debug_fetch_record(DebugRecord* out)
 int debug_fetch_ho(DebugRecord* out);
 int debug_fetch_lj(DebugRecord* out);
 int debug_fetch_lj_paired(DebugRecord* out);
+int debug_fetch_lj_double(DebugRecord* out);
 int debug_fetch_update(DebugRecord* out);
 int debug_fetch_fragment(DebugRecord* out);
 
@@ -356,6 +357,7 @@ struct LJSysDev {
     int outer_cap;        // outer-list capacity per thread (paired kernel, global memory)
     int shared_shift;     // paired kernel: windows may use one image shift per list entry
     int write_nose;       // the last slice is owned (not a time-slab halo): write its gradient
+    int halo_lo;          // 1: local slice 0 is a time-slab halo (steps count from slice 1)
     int chain0;           // global index of chain 0
     long long hs_off;     // hard-sphere path bias: this system's slices in the radii array
     LJK<R> k;
@@ -406,6 +408,22 @@ cudaError_t launch_lj_paired(const LJItem* items, int n_items, const void* sys_t
                              size_t smem, int grid, bool with_grad, bool pipe, uint32_t* outer,
                              long long outer_words, cudaStream_t st, const float* hs2 = nullptr,
                              int* overlap = nullptr);
+
+// Double-precision action (+ adjoint), lj_double.cu: each unordered pair's coefficients
+// once per slice, in a scratch of `scratch` bytes per CTA (`cap` pairs; more are
+// evaluated again).  edge: edge_doubles doubles per S slot (with the gradient).
+struct LJDoubleShape {
+    int cap = 0;
+    bool pre_global = false;  // row prefixes in the scratch (shared memory too small)
+    size_t smem = 0, scratch = 0;
+    int edge_doubles = 0;
+};
+LJDoubleShape lj_double_shape(int nmax, double pairs_expected, int max_smem);
+int lj_double_blocks_per_sm(size_t smem, bool with_grad);
+cudaError_t launch_lj_double(const LJItem* items, int n_items, const void* sys_table, int nmax,
+                             const LJDoubleShape& h, const double* pos, double* grad, double* partials,
+                             int* counter, int grid, bool with_grad, unsigned char* scratch, double* edge,
+                             cudaStream_t st, const double* hs2, int* overlap);
 
 cudaError_t launch_lj_pair_counts(const float* pos, long long* counts, int N, int T, int n_chains,
                                   long long sys_offset, double L, double rc, cudaStream_t st);

@@ -1,0 +1,80 @@
+"""Double-precision Lennard-Jones action and gradient (lj_double.cu) where it can go
+wrong: row words of 32 particles and their remainders, one to eight threads per
+particle, the largest N, particles in other periodic images, pairs beyond the record
+capacity, items of one step, and cutoffs at half the box."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+import oracle  # noqa: E402
+import pamd_inputs as inputs  # noqa: E402
+from _common import rel  # noqa: E402
+
+
+@pytest.fixture(scope="module")
+def pamd():
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    import paper_1907_09529_gb300 as m
+    m.tune()
+    return m
+
+
+def _check(pamd, N, T, B, L, rc, x0, tile=0, jitter=0.01, seed=1, tol=1e-12):
+    """S and gradient of B paths jittering around x0 [3][N] against the oracle; the
+    tolerance is the double-precision one of the parity tests."""
+    D, beta, dt = 0.9, 1.1, 1e-4
+    rng = inputs.rng(seed)
+    walk = np.cumsum(jitter * rng.standard_normal((B, T + 1, 3, N)), axis=1)
+    paths = x0[None, None] + walk
+    prob = pamd.Problem([pamd.System("lj", N, 3, T, B, box=L, rc=rc)], D, beta, dt, "fp64")
+    buf = prob.empty("cuda")
+    prob.view(buf, 0).copy_(torch.from_numpy(paths))
+    try:
+        pamd.tune(tile)
+        S, g = pamd.action_grad(prob, buf)
+        S1 = pamd.action(prob, buf)
+        torch.cuda.synchronize()
+    finally:
+        pamd.tune()
+    assert torch.equal(S, S1)
+    pot = oracle.lennard_jones(L, rc)
+    for b in range(B):
+        So, go = oracle.action_grad(pot, paths[b], D, beta, dt, nthreads=8)
+        gb = prob.view(g, 0)[b].cpu().numpy()
+        assert abs(S[b].item() - So) <= tol * abs(So)
+        assert rel(gb, go) <= tol
+        assert np.abs(gb - go).max() <= tol * np.abs(go).max()
+    return g
+
+
+@pytest.mark.parametrize("N", [2, 3, 31, 32, 33, 63, 65, 127, 129, 257, 511, 513, 863, 1023, 1024])
+def test_sizes(pamd, N):
+    L = max(inputs.box_side(N, 0.85), 3.2)
+    _check(pamd, N, 3, 2, L, min(2.5, L / 2), inputs.fcc_lattice(N, L), seed=N)
+
+
+@pytest.mark.parametrize("T,tile", [(1, 0), (5, 1), (9, 4), (9, 0)])
+def test_items(pamd, T, tile):
+    L = inputs.box_side(64, 0.85)
+    g = _check(pamd, 64, T, 3, L, L / 2, inputs.fcc_lattice(64, L), tile=tile, seed=4)
+    assert torch.equal(g, _check(pamd, 64, T, 3, L, L / 2, inputs.fcc_lattice(64, L), tile=32, seed=4))
+
+
+def test_other_images(pamd):
+    """Particles stored up to 1000 boxes away: same forces as in the first box to the
+    rounding of the stored coordinates (eps * 1000 L on distances, steep pair forces)."""
+    N = 108
+    L = inputs.box_side(N, 0.85)
+    shift = inputs.rng(9).integers(-1000, 1001, size=(3, N)) * L
+    _check(pamd, N, 4, 1, L, 2.5, inputs.fcc_lattice(N, L) + shift, seed=5)
+
+
+def test_clustered_pairs_exceed_the_capacity(pamd):
+    """A droplet in a large box holds far more pairs than the uniform density that the
+    records are sized for."""
+    N = 256
+    x0 = inputs.fcc_lattice(N, inputs.box_side(N, 0.85))
+    _check(pamd, N, 4, 2, 60.0, 2.5, x0, seed=6)
