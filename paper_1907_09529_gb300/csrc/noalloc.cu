@@ -58,7 +58,7 @@ __global__ void __launch_bounds__(pamd::kElemThreads)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     R* xs = reinterpret_cast<R*>(smem_raw);
-    __shared__ double red[pamd::kElemThreads / 32];
+    __shared__ double red[pamd::kElemThreads];
     const long long base = sys_off + (long long)blockIdx.y * chain_len;
     const int e0 = blockIdx.x * pamd::kElemChunk;
     const int n = min(pamd::kElemChunk, chain_len - e0);
@@ -81,8 +81,9 @@ __global__ void __launch_bounds__(pamd::kElemThreads)
         grad[base + e] = pamd::fma_r(ak, r, rp - r) * ginv;
         acc = pamd::fma_r(r, r, acc);
     }
-    const double tot = pamd::block_sum((double)acc, red);
-    if (threadIdx.x == 0) partials[slot0 + blockIdx.y * gridDim.x + blockIdx.x] = tot;
+    double tot[1] = {pamd::to_double(acc)};
+    pamd::block_sums_256<1>(tot, red);
+    if (threadIdx.x == 0) partials[slot0 + blockIdx.y * gridDim.x + blockIdx.x] = tot[0];
 }
 
 // One warp per chain sums its chunks' partials in a fixed order.

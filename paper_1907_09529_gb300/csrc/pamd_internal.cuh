@@ -222,6 +222,68 @@ __device__ __forceinline__ double block_sum(double v, double* scratch)
     return s;
 }
 
+// Block sums of NV values in blocks of 256 threads, bitwise those of block_sum (the same
+// tree: lanes l and l ^ 16, ^ 8, ..., ^ 1 of a warp, then the eight warps), results in
+// thread 0.  block_sum issues 46 FP64 warp instructions per value however few lanes have
+// distinct sums, and GB300 takes 16 clocks for each; here one warp per value adds the
+// distinct pairs of each level densely, 12 instructions (in the 4096-element blocks of the
+// oscillator kernel the sums took half of a block's time at the copy rate).  `sm`: 256 NV
+// doubles.  Called by every thread.
+template <int NV>
+__device__ __forceinline__ void block_sums_256(double (&v)[NV], double* sm)
+{
+    static_assert(NV <= 8, "one warp per value");
+#pragma unroll
+    for (int n = 0; n < NV; ++n) sm[256 * n + threadIdx.x] = v[n];
+    __syncthreads();
+    const int lane = threadIdx.x & 31, n = threadIdx.x >> 5;
+    double r = 0.0;
+    if (n < NV) {
+        double* a = sm + 256 * n;
+        double b[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {  // (warp, l < 16): v_l + v_{l+16}
+            const int q = lane + 32 * k, o = 32 * (q >> 4) + (q & 15);
+            b[k] = a[o] + a[o + 16];
+        }
+        __syncwarp();
+#pragma unroll
+        for (int k = 0; k < 4; ++k) a[lane + 32 * k] = b[k];
+        __syncwarp();
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {  // (warp, l < 8)
+            const int q = lane + 32 * k, o = 16 * (q >> 3) + (q & 7);
+            b[k] = a[o] + a[o + 8];
+        }
+        __syncwarp();
+        a[lane] = b[0];
+        a[lane + 32] = b[1];
+        __syncwarp();
+        const int o = 8 * (lane >> 2) + (lane & 3);  // (warp, l < 4)
+        r = a[o] + a[o + 4];
+        r += __shfl_xor_sync(0xffffffffu, r, 2);
+        r += __shfl_xor_sync(0xffffffffu, r, 1);
+        // warp w's sum sits in lanes 4w..4w+3
+        r += __shfl_xor_sync(0xffffffffu, r, 16);
+        r += __shfl_xor_sync(0xffffffffu, r, 8);
+        r += __shfl_xor_sync(0xffffffffu, r, 4);
+        if (NV > 1 && lane == 0) a[0] = r;
+    }
+    if (NV > 1) __syncthreads();
+#pragma unroll
+    for (int q = 0; q < NV; ++q) v[q] = NV > 1 ? sm[256 * q] : r;
+}
+
+// The double of a float; ordinary values by bit moves, which keep the conversion off the
+// FP64 pipe.
+__device__ __forceinline__ double to_double(double v) { return v; }
+__device__ __forceinline__ double to_double(float v)
+{
+    const unsigned b = __float_as_uint(v), e = (b >> 23) & 0xFFu;
+    if (e - 1u >= 254u) return (double)v;  // zero, subnormal, infinite, NaN
+    return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7FFFFFFFu) >> 3) + 0x38000000u)), (int)(b << 29));
+}
+
 // A device buffer whose address is not 16-byte aligned: the element kernels read
 // and write whole 16-byte units, so such a buffer is refused (PAMD_ERR_ARG) before
 // anything is launched.  Host buffers are staged into the library's own aligned
