@@ -142,8 +142,6 @@ struct Plan {
     void* d_prop = nullptr;
     void* d_gprop = nullptr;
     double* d_Sprop = nullptr;
-    double* d_qf = nullptr;
-    double* d_qr = nullptr;
     int* d_flag = nullptr;
     MalaDev* d_md = nullptr;
     // host-pointer staging (allocated on first use)
@@ -773,8 +771,6 @@ int ensure_update_ws(Plan* P)
     if ((rc = P->alloc(&P->d_prop, P->esz * (size_t)P->span))) return rc;
     if ((rc = P->alloc(&P->d_gprop, P->esz * (size_t)P->span))) return rc;
     if ((rc = P->alloc(&P->d_Sprop, sizeof(double) * P->n_chains))) return rc;
-    if ((rc = P->alloc(&P->d_qf, sizeof(double) * P->n_chains))) return rc;
-    if ((rc = P->alloc(&P->d_qr, sizeof(double) * P->n_chains))) return rc;
     if ((rc = P->alloc(&P->d_flag, sizeof(int) * P->n_chains))) return rc;
     if (!P->d_md && (rc = P->alloc(&P->d_md, sizeof(MalaDev)))) return rc;
     PAMD_CUDA_TRY(cudaMemset(P->d_prop, 0, P->esz * (size_t)P->span));
@@ -795,11 +791,12 @@ bool is_host_ptr(const void* ptr)
 
 // S (and grad) of chains [c0, c1) into S_out (indexed by global chain), from
 // device pointers; c1 < 0 means every chain.  The results of a chain do not
-// depend on the range it is computed in.
+// depend on the range it is computed in.  finalize = false: the block sums of S stay in
+// d_part_S for the caller.
 template <typename R>
 int run_action(const pamd_problem* p, Plan* P, const R* pos, R* grad, double* S_out, bool with_grad,
                cudaStream_t st, int c0 = 0, int c1 = -1, int* counter = nullptr, int lane = 0,
-               const R* hs2 = nullptr, int* overlap = nullptr)
+               const R* hs2 = nullptr, int* overlap = nullptr, bool finalize = true)
 {
     if (c1 < 0) c1 = P->n_chains;
     if (!counter) counter = P->d_counter;  // LJ work-queue counter of this launch sequence
@@ -867,8 +864,9 @@ int run_action(const pamd_problem* p, Plan* P, const R* pos, R* grad, double* S_
             if (n > 0) PAMD_CUDA_TRY(launch(P->d_lj_items_grp + C.grp_off + f, n, std::min(grid, n)));
         }
     }
-    PAMD_CUDA_TRY(launch_finalize(P->d_part_S, P->d_S_slots + c0, c1 - c0, 1.0 / (4.0 * p->D * p->dt),
-                                  S_out + c0, st, P->d_err));
+    if (finalize)
+        PAMD_CUDA_TRY(launch_finalize(P->d_part_S, P->d_S_slots + c0, c1 - c0, 1.0 / (4.0 * p->D * p->dt),
+                                      S_out + c0, st, P->d_err));
     if (fault_injected("nonfinite")) PAMD_CUDA_TRY(launch_set_status(P->d_err, PAMD_ERR_NONFINITE, st));
     return PAMD_OK;
 }
@@ -886,14 +884,14 @@ int run_one_update(const pamd_problem* p, Plan* P, R* pos, R* grad, double* S, c
     R* gprop = reinterpret_cast<R*>(P->d_gprop);
     PAMD_CUDA_TRY(launch_mala_propose<R>(P->d_all + eb0, eb1 - eb0, pos, grad, noise, prop,
                                          P->d_part_qf + eb0, P->d_md, u, st, P->any_slab));
-    int rc = run_action<R>(p, P, prop, gprop, P->d_Sprop, true, st, c0, c1, counter, lane);
+    int rc = run_action<R>(p, P, prop, gprop, P->d_Sprop, true, st, c0, c1, counter, lane, (const R*)nullptr,
+                           nullptr, false);
     if (rc) return rc;
     PAMD_CUDA_TRY(launch_mala_reverse<R>(P->d_all + eb0, eb1 - eb0, pos, prop, gprop,
                                          P->d_part_qr + eb0, P->d_md, st, P->any_slab));
-    PAMD_CUDA_TRY(launch_finalize(P->d_part_qf, P->d_E_slots + c0, c1 - c0, 1.0, P->d_qf + c0, st));
-    PAMD_CUDA_TRY(launch_finalize(P->d_part_qr, P->d_E_slots + c0, c1 - c0, 1.0, P->d_qr + c0, st));
-    PAMD_CUDA_TRY(launch_mala_accept(c0, c1 - c0, S, P->d_Sprop, P->d_qf, P->d_qr, log_u, P->d_md, u,
-                                     P->d_flag, n_acc, la, st));
+    PAMD_CUDA_TRY(launch_mala_sums_accept(c0, c1 - c0, P->d_S_slots, P->d_E_slots, P->d_part_S, P->d_part_qf,
+                                          P->d_part_qr, 1.0 / (4.0 * p->D * p->dt), S, P->d_Sprop, log_u, P->d_md,
+                                          u, P->d_flag, n_acc, la, P->d_err, st));
     PAMD_CUDA_TRY(launch_mala_commit<R>(P->d_all + eb0, eb1 - eb0, pos, grad, prop, gprop, P->d_flag,
                                         S, P->d_Sprop, st));
     return PAMD_OK;

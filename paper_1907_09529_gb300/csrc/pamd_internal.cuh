@@ -513,6 +513,7 @@ struct MalaDev {
     uint64_t seed;
     uint64_t counter;
     double h;
+    double s2h;  // sqrt(2 h), taken once: a double square root in every thread kept the FP64 pipe busy
 };
 // slab: some block belongs to a time slab (halo elements copied / skipped, noise
 // indexed from the whole path's slice 0); false for whole paths.
@@ -529,6 +530,13 @@ cudaError_t launch_mala_accept(int chain0, int n_chains, const double* S, const 
                                const double* qf, const double* qr, const double* log_u,
                                const MalaDev* md, int update_index, int* accept_flag,
                                int* n_accepted, double* log_alpha, cudaStream_t st);
+// The sums of S', q_fwd, q_rev over the blocks of chains [chain0, chain0 + n_chains) and
+// their accept tests in one launch (bitwise launch_finalize x 3 and launch_mala_accept).
+cudaError_t launch_mala_sums_accept(int chain0, int n_chains, const ChainSlots* S_slots,
+                                    const ChainSlots* E_slots, const double* part_S, const double* part_qf,
+                                    const double* part_qr, double S_scale, const double* S, double* S_prop,
+                                    const double* log_u, const MalaDev* md, int update_index, int* accept_flag,
+                                    int* n_accepted, double* log_alpha, int* err, cudaStream_t st);
 template <typename R>
 cudaError_t launch_mala_commit(const ElemBlock* blocks, int n_blocks, R* pos, R* grad, const R* prop,
                                const R* grad_prop, const int* accept_flag, double* S,
