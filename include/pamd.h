@@ -212,7 +212,8 @@ int pamd_action_grad_hs(const pamd_problem* prob, const void* pos, const double*
  *   n_accepted   : int[n_chains_total], incremented by accepted updates (may be NULL).
  *   log_alpha    : double[n_chains_total], log alpha of the last update (may be NULL).
  * With device pointers and n_updates > 1 the updates are captured once into
- * a CUDA graph (cached per shape) and replayed.  With host buffers, no noise
+ * a CUDA graph (cached per shape) and replayed; batches of harmonic chains of up
+ * to 4096 elements run all updates in one launch per system instead.  With host buffers, no noise
  * and no log_u, and at least two chains, the call is pipelined over up to 8
  * chunks of chains: one chunk's buffers are copied in while earlier chunks
  * are updated (on up to three compute streams, so that several chunks' kernels
@@ -472,8 +473,8 @@ int pamd_fp64_fma_probe(int blocks, int threads, int iters, double* out, double*
  *   *checked : 1 in the debug build, 0 in the normal library (no checks);
  *   *count   : out-of-bounds accesses recorded since the last call;
  *   *site, *index, *bound : the first of them: file * 100000 + source line
- *              (files 1..6: ho_kernels, lj_kernels, lj_paired, update_kernels,
- *              fragment_kernels, lj_double), the index and the array's extent,
+ *              (files 1..7: ho_kernels, lj_kernels, lj_paired, update_kernels,
+ *              fragment_kernels, lj_double, ho_update), the index and the array's extent,
  * and clears the records.  Any pointer may be NULL. */
 int pamd_debug_status(int* checked, int* count, int* site, long long* index, long long* bound);
 

@@ -16,7 +16,7 @@ LIB = os.path.join(HERE, "libpamd.so")
 BUILD_DEBUG = os.path.join(HERE, "_build_debug")
 LIB_DEBUG = os.path.join(HERE, "libpamd_debug.so")
 SOURCES = ["pamd_api.cu", "ho_kernels.cu", "lj_kernels.cu", "lj_paired.cu", "lj_double.cu",
-           "update_kernels.cu", "noalloc.cu",
+           "update_kernels.cu", "ho_update.cu", "noalloc.cu",
            "fragment_kernels.cu", "probe.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",

@@ -168,6 +168,10 @@ struct Plan {
     long long hs_slices = 0;
     void* d_hs2 = nullptr;
     bool any_slab = false;      // some system is a time slab
+    // harmonic systems only: updates run the fused kernels of ho_update.cu, those of chains
+    // of one element block (at most ho_max_n elements) in one launch for all updates
+    bool ho_fused = false, ho_loop = false;
+    int ho_max_n = 0;
     int* d_overlap = nullptr;
     // host-buffer pipeline: copy streams, the extra compute streams (lanes 1..), events
     // and one LJ work counter per chunk (created on first use)
@@ -504,6 +508,12 @@ int build_plan(const pamd_problem* p, Plan** out)
             }
         }
     }
+    P->ho_fused = !P->any_slab && !(p->flags & PAMD_FLAG_ONE_CHAIN_PER_LAUNCH);
+    for (auto& si : P->sys) {
+        P->ho_fused = P->ho_fused && si.kind == PAMD_HARMONIC && ho_update_fusable(si.d * si.N);
+        P->ho_max_n = (int)std::max<long long>(P->ho_max_n, si.chain_len);
+    }
+    P->ho_loop = P->ho_fused && P->ho_max_n <= kElemChunk;
     int slot = (int)P->h_ho.size();
     // LJ: block-size classes, shared-memory budgets, per-system shapes, items.
     std::vector<LJItem> items, grouped;
@@ -871,6 +881,39 @@ int run_action(const pamd_problem* p, Plan* P, const R* pos, R* grad, double* S_
     return PAMD_OK;
 }
 
+// Updates u .. u + n - 1 of chains [c0, c1) of a batch of harmonic systems (Plan::ho_fused):
+// one launch for all of them (chains of one block), else n == 1 in three passes.
+template <typename R>
+int run_ho_updates(const pamd_problem* p, Plan* P, R* pos, R* grad, double* S, const double* log_u, int* n_acc,
+                   double* la, int u, int n, cudaStream_t st, int c0, int c1)
+{
+    const double a = p->beta * p->D * p->dt, ginv = 1.0 / (2.0 * p->D * p->dt), scale = 1.0 / (4.0 * p->D * p->dt);
+    R* prop = reinterpret_cast<R*>(P->d_prop);
+    for (int pass = 0; pass < 2; ++pass) {
+        for (const auto& si : P->sys) {
+            const int lo = std::max(c0, si.chain0), hi = std::min(c1, si.chain0 + si.chains);
+            if (lo >= hi) continue;
+            const int b0 = P->h_E_slots[lo].begin, nb = P->h_E_slots[hi - 1].end - b0, s = si.d * si.N;
+            if (P->ho_loop)
+                PAMD_CUDA_TRY(launch_ho_loop<R>(P->d_all + b0, nb, s, (int)si.chain_len, pos, grad, S, P->d_md, u, n,
+                                                a, ginv, scale, log_u, n_acc, la, P->d_err, st));
+            else if (pass == 0)
+                PAMD_CUDA_TRY(launch_ho_trial<R>(P->d_all + b0, nb, s, pos, grad, prop, P->d_part_S + b0,
+                                                 P->d_part_qf + b0, P->d_part_qr + b0, P->d_md, u, a, ginv, st));
+            else
+                PAMD_CUDA_TRY(launch_ho_commit<R>(P->d_all + b0, nb, s, pos, grad, prop, P->d_flag, S, P->d_Sprop,
+                                                  a, ginv, st));
+        }
+        if (P->ho_loop) break;
+        if (pass == 0)
+            PAMD_CUDA_TRY(launch_mala_sums_accept(c0, c1 - c0, P->d_S_slots, P->d_E_slots, P->d_part_S, P->d_part_qf,
+                                                  P->d_part_qr, scale, S, P->d_Sprop, log_u, P->d_md, u, P->d_flag,
+                                                  n_acc, la, P->d_err, st));
+    }
+    if (fault_injected("nonfinite")) PAMD_CUDA_TRY(launch_set_status(P->d_err, PAMD_ERR_NONFINITE, st));
+    return PAMD_OK;
+}
+
 // One path update of chains [c0, c1) (c1 < 0: every chain); arrays indexed by
 // global chain.
 template <typename R>
@@ -879,6 +922,7 @@ int run_one_update(const pamd_problem* p, Plan* P, R* pos, R* grad, double* S, c
                    int c1 = -1, int* counter = nullptr, int lane = 0)
 {
     if (c1 < 0) c1 = P->n_chains;
+    if (P->ho_fused && !noise) return run_ho_updates<R>(p, P, pos, grad, S, log_u, n_acc, la, u, 1, st, c0, c1);
     const int eb0 = P->h_E_slots[c0].begin, eb1 = P->h_E_slots[c1 - 1].end;
     R* prop = reinterpret_cast<R*>(P->d_prop);
     R* gprop = reinterpret_cast<R*>(P->d_gprop);
@@ -1057,10 +1101,10 @@ int pamd_debug_status(int* checked, int* count, int* site, long long* index, lon
 #endif
     int (*const fetch[])(DebugRecord*) = {debug_fetch_ho, debug_fetch_lj, debug_fetch_lj_paired,
                                           debug_fetch_update, debug_fetch_fragment,
-                                          debug_fetch_lj_double};
+                                          debug_fetch_lj_double, debug_fetch_ho_update};
     int total = 0, first_site = 0;
     long long first_index = 0, first_bound = 0;
-    for (int f = 0; f < 6; ++f) {
+    for (int f = 0; f < 7; ++f) {
         DebugRecord r;
         if (fetch[f](&r)) return PAMD_ERR_CUDA;
         if (r.count && !total) {
@@ -1308,8 +1352,14 @@ int pamd_path_update(const pamd_problem* prob, void* pos, void* grad, double* S,
         if (log_alpha && is_host_ptr(log_alpha)) dla = P->d_stage_dbl;
     }
     PAMD_CUDA_TRY(launch_set_mala_params(P->d_md, seed, counter, h, st));
-    const bool use_graph = !host && n_updates > 1;
-    if (!use_graph) {
+    const bool use_graph = !host && n_updates > 1 && !P->ho_loop;
+    if (P->ho_loop && !dnoise) {
+        rc = P->fp64 ? run_ho_updates<double>(prob, P, (double*)dpos, (double*)dgrad, dS, dlogu, dnacc, dla, 0,
+                                              n_updates, st, 0, P->n_chains)
+                     : run_ho_updates<float>(prob, P, (float*)dpos, (float*)dgrad, dS, dlogu, dnacc, dla, 0,
+                                             n_updates, st, 0, P->n_chains);
+        if (rc) return rc;
+    } else if (!use_graph) {
         for (int u = 0; u < n_updates; ++u) {
             rc = P->fp64 ? run_one_update<double>(prob, P, (double*)dpos, (double*)dgrad, dS,
                                                   (const double*)dnoise, dlogu, dnacc, dla, u, st)

@@ -85,6 +85,7 @@ int debug_fetch_lj_paired(DebugRecord* out);
 int debug_fetch_lj_double(DebugRecord* out);
 int debug_fetch_update(DebugRecord* out);
 int debug_fetch_fragment(DebugRecord* out);
+int debug_fetch_ho_update(DebugRecord* out);
 
 // ------------------------------------------------------------------ vector types
 struct alignas(32) double4a {
@@ -541,6 +542,26 @@ template <typename R>
 cudaError_t launch_mala_commit(const ElemBlock* blocks, int n_blocks, R* pos, R* grad, const R* prop,
                                const R* grad_prop, const int* accept_flag, double* S,
                                const double* S_prop, cudaStream_t st);
+
+// Updates of one harmonic system (whole paths, Philox noise), ho_update.cu.  Slices of up to
+// the s that ho_update_fusable accepts; s: elements per slice; blocks: element blocks of the
+// chains, part_* indexed like them.
+bool ho_update_fusable(int s);
+// Proposal into prop, block sums of S', q_fwd, q_rev (before launch_mala_sums_accept).
+template <typename R>
+cudaError_t launch_ho_trial(const ElemBlock* blocks, int n_blocks, int s, const R* pos, const R* grad, R* prop,
+                            double* part_S, double* part_qf, double* part_qr, const MalaDev* md,
+                            int update_index, double a, double ginv, cudaStream_t st);
+// Accepted chains take the proposal, its gradient (formed again) and S_prop.
+template <typename R>
+cudaError_t launch_ho_commit(const ElemBlock* blocks, int n_blocks, int s, R* pos, R* grad, const R* prop,
+                             const int* accept_flag, double* S, const double* S_prop, double a, double ginv,
+                             cudaStream_t st);
+// Updates update0 .. update0 + n_updates - 1 of chains of one block each (max_n elements).
+template <typename R>
+cudaError_t launch_ho_loop(const ElemBlock* blocks, int n_chains, int s, int max_n, R* pos, R* grad, double* S,
+                           const MalaDev* md, int update0, int n_updates, double a, double ginv, double S_scale,
+                           const double* log_u, int* n_accepted, double* log_alpha, int* err, cudaStream_t st);
 cudaError_t launch_set_mala_params(MalaDev* md, uint64_t seed, uint64_t counter, double h,
                                    cudaStream_t st);
 
