@@ -473,8 +473,8 @@ int pamd_fp64_fma_probe(int blocks, int threads, int iters, double* out, double*
  *   *checked : 1 in the debug build, 0 in the normal library (no checks);
  *   *count   : out-of-bounds accesses recorded since the last call;
  *   *site, *index, *bound : the first of them: file * 100000 + source line
- *              (files 1..7: ho_kernels, lj_kernels, lj_paired, update_kernels,
- *              fragment_kernels, lj_double, ho_update), the index and the array's extent,
+ *              (files 1..8: ho_kernels, lj_kernels, lj_paired, update_kernels,
+ *              fragment_kernels, lj_double, ho_update, lj_euler), the index and the array's extent,
  * and clears the records.  Any pointer may be NULL. */
 int pamd_debug_status(int* checked, int* count, int* site, long long* index, long long* bound);
 

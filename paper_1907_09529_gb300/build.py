@@ -15,7 +15,7 @@ LIB = os.path.join(HERE, "libpamd.so")
 # bounds-checked variant (-DPAMD_DEBUG): every kernel array index is checked
 BUILD_DEBUG = os.path.join(HERE, "_build_debug")
 LIB_DEBUG = os.path.join(HERE, "libpamd_debug.so")
-SOURCES = ["pamd_api.cu", "ho_kernels.cu", "lj_kernels.cu", "lj_paired.cu", "lj_double.cu",
+SOURCES = ["pamd_api.cu", "ho_kernels.cu", "lj_kernels.cu", "lj_paired.cu", "lj_double.cu", "lj_euler.cu",
            "update_kernels.cu", "ho_update.cu", "noalloc.cu",
            "fragment_kernels.cu", "probe.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

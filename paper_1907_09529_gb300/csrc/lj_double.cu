@@ -25,9 +25,7 @@
 // Formulas: the file lj_paired.cu states them; with ir2 = 1/r^2,
 //   fs  = ir8 (c12 ir6 - c1) + u'(rc)/r,   nb = [ir8 (8 c1 - c23 ir6) - u'(rc)/r] ir2
 //   (H v)_i = sum_j [fs w + nb (d . w) d],  w = v_j - v_i,  d = x_i - x_j.
-// 1/r: a single-precision seed (relative error e0 < 2^-21) and one third-order
-// Householder iteration for the inverse square root,
-//   e = 1 - r^2 y^2,  y <- y + y e (1/2 + 3/8 e)     (remaining error 5/16 e^3).
+// 1/r: inv_sqrt of lj_math.cuh (five FP64 instructions).
 //
 // Slices are independent up to r_{t-1} of the same particle, so a work item is a
 // short run of slices of one chain (an atomic queue feeds a persistent grid); the
@@ -37,7 +35,7 @@
 // where it is needed, by the same instructions).
 #include <algorithm>
 
-#include "pamd_internal.cuh"
+#include "lj_math.cuh"
 
 namespace pamd {
 
@@ -84,36 +82,11 @@ struct DblSmem {
     }
 };
 
-// Float of a positive double by truncation (relative error below 2^-23), and the
-// exact double of a float, by bit moves: conversion instructions run on the FP64 side.
-__device__ __forceinline__ float trunc_to_float(double v)
-{
-    const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
-    return __uint_as_float(__funnelshift_l(lo, hi, 3) - 0xC0000000u);
-}
-__device__ __forceinline__ double widen(float f)  // normal f
-{
-    const unsigned b = __float_as_uint(f);
-    return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7FFFFFFFu) >> 3) + 0x38000000u)),
-                            (int)(b << 29));
-}
+// Exact double of a small integer (any integer, but those by the conversion instruction).
 __device__ __forceinline__ double widen_int(int k)
 {
     if (k > -(1 << 24) && k < (1 << 24)) return k == 0 ? 0.0 : widen((float)k);
     return (double)k;
-}
-
-// 1/sqrt(v): see the head of the file.  Outside the range where the seed's exponent
-// fits a float (no physical distance) the library function is called.
-__device__ __forceinline__ double inv_sqrt(double v)
-{
-    const unsigned hi = (unsigned)__double2hiint(v);
-    if (hi - 0x39000000u >= 0x46000000u - 0x39000000u) return rsqrt(v);
-    float s;
-    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(s) : "f"(trunc_to_float(v)));
-    const double y = widen(s);
-    const double e = fma(-(v * y), y, 1.0);
-    return fma(y * e, fma(0.375, e, 0.5), y);
 }
 
 // Everything the device functions need of one item's system.

@@ -1,0 +1,370 @@
+// lj_euler.cu -- Euler-Maruyama paths of Lennard-Jones systems (Eq. (2)):
+//   x_{t+1} = x_t + a F(x_t) + sqrt(2 D dt) xi_t,  each new slice stored in the
+// path's precision and used as stored.
+//
+// What bounds it: the serial chain of steps.  A step's forces need every position of
+// the step before, so only the work inside one step can be spread, and what counts is the
+// latency of a step.
+//   * The normals do not depend on the path: a kernel over all elements first writes them
+//     into the slices that the steps will overwrite (slice t + 1 holds xi_t), and a step
+//     loads its own two steps ahead.  Drawing them inside the step put ten Philox rounds
+//     and Box-Muller on the chain.
+//   * A chain is stepped by a cluster of CTAs (up to 8).  Each CTA holds all positions
+//     and moves N / CS particles, up to 32 lanes to a particle; the new coordinates go to
+//     every CTA's shared memory, and one cluster barrier ends the step.
+//   * Small systems (N <= kEulerDense) evaluate every pair: no list, no displacement check,
+//     two candidates per packed f32x2 operation.  Larger ones walk Verlet lists of radius
+//     rc + skin, rebuilt when some particle has moved skin / 2 (a list that overflows scans
+//     all candidates).
+// N = 108, four chains of 1024 steps: 4.89 ms (4.8 us a step) with one CTA of four threads
+// per particle and the normals in the step, 1.69 ms (1.65 us) now; a step of N = 500, eight
+// chains, 17.5 -> 3.8 us, of N = 108 in double precision 101 -> 23 us.
+#include <algorithm>
+#include <cmath>
+#include <type_traits>
+
+#include "lj_math.cuh"
+
+namespace pamd {
+
+namespace {
+
+constexpr int kEulerDense = 192;   // largest N without lists
+
+__device__ __forceinline__ unsigned cluster_rank()
+{
+    unsigned r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void cluster_barrier()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void step_barrier(int cs)
+{
+    if (cs > 1)
+        cluster_barrier();
+    else
+        __syncthreads();
+}
+// Store to the same shared-memory address in CTA `rank` of the cluster.
+__device__ __forceinline__ void store_remote(float* p, unsigned rank, float v)
+{
+    unsigned a = (unsigned)__cvta_generic_to_shared(p), r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(r), "f"(v) : "memory");
+}
+__device__ __forceinline__ void store_remote(double* p, unsigned rank, double v)
+{
+    unsigned a = (unsigned)__cvta_generic_to_shared(p), r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(r), "d"(v) : "memory");
+}
+
+// The normals of every element of slices 1..T of a system's chains, into the path.
+template <typename R>
+__global__ void euler_normals_kernel(R* __restrict__ pos, long long off, long long chain_len, int s,
+                                     int chain0, uint64_t seed, uint64_t counter)
+{
+    const int b = blockIdx.x;
+    R* X = pos + off + (long long)b * chain_len;
+    const long long ng = (chain_len + 3) >> 2, g0 = s >> 2;
+    for (long long g = g0 + (long long)blockIdx.y * blockDim.x + threadIdx.x; g < ng;
+         g += (long long)gridDim.y * blockDim.x) {
+        const float4 z = philox_normals4(seed, counter, kStreamEuler, (uint32_t)(chain0 + b), (uint32_t)g);
+        const float v[4] = {z.x, z.y, z.z, z.w};
+#pragma unroll
+        for (int l = 0; l < 4; ++l) {
+            const long long e = 4 * g + l;
+            if (e >= s && e < chain_len && PAMD_OK_IDX(e, chain_len)) X[e] = (R)v[l];
+        }
+    }
+}
+
+// Positions of one slice in shared memory.  Single precision, no list: candidates 2k and
+// 2k + 1 of lane q (j = q + tpp m) form one float2 per component.  Otherwise three arrays.
+template <typename R, bool LIST>
+struct EulerPos {
+    R* p;
+    int n, lg;  // padded particles; log2 of the lanes per particle
+    __device__ __forceinline__ R* at(int j, int c) const
+    {
+        if (sizeof(R) == 4 && !LIST) {
+            const int m = j >> lg, q = j & ((1 << lg) - 1);
+            return p + c * n + (((m >> 1) << lg) + q) * 2 + (m & 1);
+        }
+        return p + c * n + j;
+    }
+};
+
+// Force on particle i from this lane's candidates, every pair, two per packed operation.
+__device__ __forceinline__ void force_dense(const float* p, int npad, int N, int lg, int q, int i, const float (&xi)[3],
+                                            const LJK<float>& k, float (&f)[3])
+{
+    const float2 nL = pk(-k.L), iL = pk(k.iL), mag = pk(12582912.0f), nmag = pk(-12582912.0f);
+    const float2 c1 = pk(k.c1), c2 = pk(k.c2), m1 = pk(-1.0f), duc = pk(k.duc);
+    const float2 x = pk(xi[0]), y = pk(xi[1]), z = pk(xi[2]);
+    const float inf = __int_as_float(0x7f800000);
+    float2 fx = pk(0.0f), fy = pk(0.0f), fz = pk(0.0f);
+    auto two = [&](int m, bool check) {  // candidates j and j + tpp
+        const float2* a = reinterpret_cast<const float2*>(p) + (m << lg) + q;
+        const int j = q + (m << (lg + 1)), j2 = j + (1 << lg);
+        float2 dx = sub2(x, a[0]), dy = sub2(y, a[npad / 2]), dz = sub2(z, a[npad]);
+        dx = fma2(nL, add2(fma2(dx, iL, mag), nmag), dx);
+        dy = fma2(nL, add2(fma2(dy, iL, mag), nmag), dy);
+        dz = fma2(nL, add2(fma2(dz, iL, mag), nmag), dz);
+        float2 r2 = fma2(dz, dz, fma2(dy, dy, mul2(dx, dx)));
+        // r^2 = +inf: exact zeros (outside the cutoff, itself, padding)
+        r2.x = (r2.x <= k.rc2 && j != i && (!check || j < N)) ? r2.x : inf;
+        r2.y = (r2.y <= k.rc2 && j2 != i && (!check || j2 < N)) ? r2.y : inf;
+        const float2 ri = pk(inv_sqrt(r2.x), inv_sqrt(r2.y)), ir2 = mul2(ri, ri);
+        const float2 ir6 = mul2(mul2(ir2, ir2), ir2), u = mul2(c1, ir6), t = fma2(c2, ir6, m1);
+        const float2 fs = fma2(mul2(u, t), ir2, mul2(duc, ri));
+        fx = fma2(fs, dx, fx);
+        fy = fma2(fs, dy, fy);
+        fz = fma2(fs, dz, fz);
+    };
+    const int full = N >> (lg + 1), all = npad >> (lg + 1);
+#pragma unroll 4
+    for (int m = 0; m < full; ++m) two(m, false);
+    if (full < all) two(full, true);
+    f[0] = fx.x + fx.y;
+    f[1] = fy.x + fy.y;
+    f[2] = fz.x + fz.y;
+}
+
+struct EulerShape {
+    int cs, nloc, lg, nt, cap, npad;
+    size_t smem;
+};
+
+template <typename R, bool LIST>
+__global__ void __launch_bounds__(1024)
+    lj_euler_kernel(R* __restrict__ pos, const R* __restrict__ noise, const LJSysDev<R> S, const EulerShape H)
+{
+    extern __shared__ __align__(32) unsigned char smem_raw[];
+    const int N = S.N, T = S.T, s = 3 * N, tid = threadIdx.x, NT = blockDim.x;
+    const int lg = H.lg, tpp = 1 << lg, q = tid & (tpp - 1), cs = H.cs, npad = H.npad;
+    const unsigned rank = cs > 1 ? cluster_rank() : 0u;
+    const int chain = blockIdx.x / cs;
+    const int i = (int)rank * H.nloc + (tid >> lg);
+    const bool active = (tid >> lg) < H.nloc && i < N;
+    const LJK<R>& k = S.k;
+    R* X = pos + S.off + (long long)chain * S.chain_len;
+    const R* Z = noise ? noise + S.off + (long long)chain * S.chain_len : X;
+    R* buf = reinterpret_cast<R*>(smem_raw);  // two slices, then (lists) the positions at the last build
+    R* ref = buf + 6 * npad;
+    uint16_t* nbr = reinterpret_cast<uint16_t*>(ref + (LIST ? 3 * npad : 0));
+    EulerPos<R, LIST> P{buf, npad, lg};
+    for (int j = tid; j < npad; j += NT)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            *P.at(j, c) = j < N ? X[c * N + j] : R(0);
+            P.at(j, c)[3 * npad] = R(0);  // (padding of the other buffer)
+        }
+    int cnt = 0;
+    bool ovf = false;
+    // candidates of this lane
+    auto build = [&](const EulerPos<R, LIST>& A) {
+        for (int j = tid; j < N; j += NT)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) ref[c * npad + j] = *A.at(j, c);
+        cnt = 0;
+        if (active) {
+            const R xi = *A.at(i, 0), yi = *A.at(i, 1), zi = *A.at(i, 2);
+            for (int j = q; j < N; j += tpp) {
+                R dx, dy, dz;
+                const R r2 = pair_r2<R>(xi, yi, zi, *A.at(j, 0), *A.at(j, 1), *A.at(j, 2), k, dx, dy, dz);
+                if (r2 <= k.rl2 && j != i) {
+                    if (cnt < H.cap && PAMD_OK_IDX(cnt * NT + tid, H.cap * NT)) nbr[cnt * NT + tid] = (uint16_t)j;
+                    ++cnt;
+                }
+            }
+        }
+        ovf = cnt > H.cap;
+    };
+    // Lanes 0..2 of a particle (one lane when it has fewer) take its components x, y, z; lane
+    // q writes component q mod 3 of the new position to CTAs q / 3, q / 3 + tpp / 3, ...
+    const int comp = tpp >= 3 ? q % 3 : 0, lanes3 = tpp / 3, first = tpp >= 3 ? q / 3 : 0, stride = tpp >= 3 ? lanes3 : 1;
+    const bool mover = active && (tpp >= 3 ? q < 3 * lanes3 : q == 0), owner = mover && q < 3;
+    constexpr int NC = 3;
+    const int nc = tpp >= 3 ? 1 : NC;  // components of a mover lane
+    const int oi = (int)(P.at(active ? i : 0, 0) - buf);
+    R* const W = buf + oi + comp * npad;                       // own component, buffer 0
+    const R* zp = Z + (long long)s + comp * N + (active ? i : 0);  // its normal of the step to load next
+    R* xp = X + (long long)comp * N + (active ? i : 0);            // its place in slice t
+    // (a ring indexed by the unrolled step: copying a register would wait for its load)
+    R z[4][NC], last[NC] = {R(0), R(0), R(0)};
+    auto load_zs = [&](bool in, R (&v)[NC]) {
+#pragma unroll
+        for (int c = 0; c < NC; ++c)
+            if (c < nc) v[c] = (in && mover) ? zp[c * N] : R(0);
+        zp += s;
+    };
+    load_zs(true, z[0]);
+    load_zs(T > 1, z[1]);
+    step_barrier(cs);  // (also: every lane holds its first normals before slice 1 is written)
+    // Step t from buffer PAR to the other; zt: its normals.  The slice that the step before
+    // made is stored here: a store directly before the barrier would hold it up (the
+    // barrier's release waits for it).
+    auto step = [&](int t, auto par, const R (&zt)[NC], R (&z2)[NC]) {
+        constexpr int PAR = decltype(par)::value;
+        const EulerPos<R, LIST> A{buf + PAR * 3 * npad, npad, lg};
+        if (t > 0 && owner) {
+#pragma unroll
+            for (int c = 0; c < NC; ++c)
+                if (c < nc) xp[c * N] = last[c];
+        }
+        xp += s;
+        load_zs(t + 2 < T, z2);
+        if (LIST) {
+            bool moved = t == 0;
+            for (int j = tid; j < N; j += NT) {
+                const R dx = *A.at(j, 0) - ref[j], dy = *A.at(j, 1) - ref[npad + j], dz = *A.at(j, 2) - ref[2 * npad + j];
+                moved |= !(dx * dx + dy * dy + dz * dz <= k.hs2);
+            }
+            if (__syncthreads_or(moved)) {
+                build(A);
+                __syncthreads();
+            }
+        }
+        R f[3] = {R(0), R(0), R(0)}, xi[3] = {R(0), R(0), R(0)};
+        if (active) {
+#pragma unroll
+            for (int c = 0; c < 3; ++c) xi[c] = A.p[oi + c * npad];
+            if constexpr (sizeof(R) == 4 && !LIST) {
+                force_dense(A.p, npad, N, lg, q, i, xi, k, f);
+            } else if (LIST && !ovf) {
+#pragma unroll 2
+                for (int m = 0; m < cnt; ++m) {
+                    const int j = nbr[m * NT + tid];
+                    pair_force<R>(xi[0], xi[1], xi[2], *A.at(j, 0), *A.at(j, 1), *A.at(j, 2), k, f);
+                }
+            } else {
+                for (int j = q; j < N; j += tpp)
+                    if (j != i) pair_force<R>(xi[0], xi[1], xi[2], *A.at(j, 0), *A.at(j, 1), *A.at(j, 2), k, f);
+            }
+        }
+        for (int o = tpp >> 1; o > 0; o >>= 1)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) f[c] += __shfl_xor_sync(0xffffffffu, f[c], o);
+        auto move = [&](int c, R x, R fc, R zc) {
+            const R xn = x + fma_r(k.a, fc, k.sig_em * zc);
+            last[c] = xn;
+            R* w = W + (1 - PAR) * 3 * npad + c * npad;
+            if (cs == 1) {
+                if (owner) *w = xn;
+            } else {
+                for (int d = first; d < cs; d += stride) store_remote(w, (unsigned)d, xn);
+            }
+        };
+        if (mover) {
+            if (tpp >= 3) {
+                move(0, comp == 0 ? xi[0] : comp == 1 ? xi[1] : xi[2], comp == 0 ? f[0] : comp == 1 ? f[1] : f[2], zt[0]);
+            } else {
+#pragma unroll
+                for (int c = 0; c < 3; ++c) move(c, xi[c], f[c], zt[c]);
+            }
+        }
+        step_barrier(cs);
+    };
+    using P0 = std::integral_constant<int, 0>;
+    using P1 = std::integral_constant<int, 1>;
+    for (int t = 0; t < T; t += 4) {
+        step(t, P0{}, z[0], z[2]);
+        if (t + 1 < T) step(t + 1, P1{}, z[1], z[3]);
+        if (t + 2 < T) step(t + 2, P0{}, z[2], z[0]);
+        if (t + 3 < T) step(t + 3, P1{}, z[3], z[1]);
+    }
+    if (owner) {
+#pragma unroll
+        for (int c = 0; c < NC; ++c)
+            if (c < nc) xp[c * N] = last[c];
+    }
+}
+
+// Cluster size, lanes per particle and block size.
+// A cluster barrier costs about 0.55 us (its release waits for the remote stores), so single
+// precision takes clusters where a step's pairs cost more than that (N = 32: 0.82 us a step
+// with one CTA, 1.38 with two; N = 108: 2.7, 2.1, 1.8 with one, two, four), down to
+// kEulerMinLocal particles per CTA; double precision, bound by the FP64 pipe, almost always
+// (N = 108: 110, 63, 31 us with one, two, four).  Chains beyond the SMs get no cluster.
+// Lanes per particle: about 512 threads (more lanes add shuffles and overhead: N = 108 on four
+// CTAs 1.92 us with 864 threads, 1.78 with 432), up to 1024 where that keeps four lanes.
+constexpr int kEulerClusterN = 80;
+constexpr int kEulerMinLocal = 13;
+constexpr int kEulerMinLocalDouble = 4;
+
+template <typename R>
+EulerShape euler_shape(int N, int n_chains, double list_volume, int sms, int max_smem)
+{
+    constexpr bool F32 = sizeof(R) == 4;
+    const int local = F32 ? kEulerMinLocal : kEulerMinLocalDouble;
+    EulerShape h;
+    h.cs = 1;
+    while (h.cs < 8 && (!F32 || N >= kEulerClusterN) && N >= 2 * h.cs * local && 2LL * h.cs * n_chains <= sms) h.cs *= 2;
+    h.nloc = (N + h.cs - 1) / h.cs;
+    h.lg = 0;
+    while (h.lg < 5 && (h.nloc << (h.lg + 1)) <= (h.lg < 2 ? 1024 : 512)) ++h.lg;
+    h.nt = std::max(64, ((h.nloc << h.lg) + 31) / 32 * 32);
+    const int tpp = 1 << h.lg;
+    const bool list = N > kEulerDense;
+    h.npad = (N + 2 * tpp - 1) / (2 * tpp) * (2 * tpp);
+    h.smem = sizeof(R) * (size_t)(list ? 9 : 6) * h.npad;
+    h.cap = 0;
+    if (list) {  // expected list length plus a margin, every candidate at most, what fits
+        const int fit = (int)((max_smem - (long long)h.smem) / (2 * h.nt));
+        h.cap = std::max(1, std::min(std::min((N + tpp - 1) / tpp, fit), (int)(1.5 * list_volume / tpp) + 12));
+    }
+    h.smem += sizeof(uint16_t) * (size_t)h.cap * h.nt;
+    return h;
+}
+
+}  // namespace
+
+template <typename R>
+cudaError_t launch_lj_euler(R* pos, const R* noise, const void* sys_entry_host, int n_chains, int chain0,
+                            uint64_t seed, uint64_t counter, cudaStream_t st)
+{
+    const LJSysDev<R> S = *static_cast<const LJSysDev<R>*>(sys_entry_host);
+    if (n_chains <= 0 || S.T <= 0) return cudaSuccess;
+    int dev = 0, sms = 0, max_smem = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e != cudaSuccess) return e;
+    if (!noise) {
+        const long long ng = S.chain_len / 4 + 1;
+        const dim3 grid((unsigned)n_chains, (unsigned)std::min<long long>(1024, (ng + 255) / 256));
+        euler_normals_kernel<R><<<grid, 256, 0, st>>>(pos, S.off, S.chain_len, 3 * S.N, chain0, seed, counter);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
+    const double rl2 = (double)S.k.rl2, L = (double)S.k.L;
+    const EulerShape h = euler_shape<R>(S.N, n_chains, 4.18879020478639 * rl2 * std::sqrt(rl2) * S.N / (L * L * L), sms,
+                                        max_smem - 1024);
+    auto kern = S.N > kEulerDense ? lj_euler_kernel<R, true> : lj_euler_kernel<R, false>;
+    if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)h.smem)) != cudaSuccess)
+        return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(n_chains * h.cs));
+    cfg.blockDim = dim3((unsigned)h.nt);
+    cfg.dynamicSmemBytes = h.smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)h.cs;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = h.cs > 1 ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kern, pos, noise, S, h);
+}
+
+template cudaError_t launch_lj_euler<float>(float*, const float*, const void*, int, int, uint64_t, uint64_t,
+                                            cudaStream_t);
+template cudaError_t launch_lj_euler<double>(double*, const double*, const void*, int, int, uint64_t, uint64_t,
+                                             cudaStream_t);
+
+PAMD_DEBUG_FETCHER(lj_euler)
+
+}  // namespace pamd

@@ -1,5 +1,5 @@
 // lj_kernels.cu -- Lennard-Jones path action and adjoint gradient one step at a time
-// (single precision, PAMD_LJ_ONE_STEP=1), Euler-Maruyama reference paths, and the
+// (single precision, PAMD_LJ_ONE_STEP=1), the hard-sphere path bias, and the
 // single-precision pair-count diagnostic.
 //
 // Pair potential (paper Eq. (11)), cut and force shifted:
@@ -28,60 +28,9 @@
 // visited in increasing j in either case, so every sum has the same order no
 // matter when the list was (re)built: results do not depend on the tiling.
 // The residual of the step before the tile (r_{t0-1}) is recomputed locally.
-#include "pamd_internal.cuh"
+#include "lj_math.cuh"
 
 namespace pamd {
-
-// Round-to-nearest-even of the exact product a*b (|a*b| < 2^22), by adding and
-// removing 1.5*2^23 (float) or 1.5*2^52 (double): one FMA and one add.
-__device__ __forceinline__ float round_prod(float a, float b)
-{
-    return __fsub_rn(__fmaf_rn(a, b, 12582912.0f), 12582912.0f);
-}
-__device__ __forceinline__ double round_prod(double a, double b)
-{
-    return __dsub_rn(__fma_rn(a, b, 6755399441055744.0), 6755399441055744.0);
-}
-
-// Minimum-image pair vector and |r_ij|^2 by the documented rule:
-//   dx = xi - xj;  dx = fma(-L, round(dx * (1/L)), dx);  r2 = fma(dz,dz,fma(dy,dy,dx*dx)).
-template <typename R>
-__device__ __forceinline__ R pair_r2(R xi, R yi, R zi, const vec4_t<R>& pj, const LJK<R>& k, R& dx,
-                                     R& dy, R& dz)
-{
-    dx = xi - pj.x;
-    dy = yi - pj.y;
-    dz = zi - pj.z;
-    dx = fma_r(-k.L, round_prod(dx, k.iL), dx);
-    dy = fma_r(-k.L, round_prod(dy, k.iL), dy);
-    dz = fma_r(-k.L, round_prod(dz, k.iL), dz);
-    return fma_r(dz, dz, fma_r(dy, dy, mul_r(dx, dx)));
-}
-
-// Reciprocal square root: the hardware approximation in single precision
-// (relative error below 2^-22), the library function in double.
-__device__ __forceinline__ float rsqrt_fast(float v)
-{
-    float r;
-    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
-    return r;
-}
-__device__ __forceinline__ double rsqrt_fast(double v) { return rsqrt(v); }
-
-// Pair scalars from r^2 (inside the cutoff):
-//   fs  = -U'(r)/r = ir2 * u * t + u'(rc)/r,  u = c1 ir6, t = c2 ir6 - 1
-//   upp = U''(r)   = ir2 * u * (c3 ir6 - 7)
-template <typename R>
-__device__ __forceinline__ R pair_fs(R r2, const LJK<R>& k, R& ir2, R& u, R& ir6)
-{
-    const R ri = rsqrt_fast(r2);
-    ir2 = ri * ri;
-    ir6 = ir2 * ir2 * ir2;
-    u = k.c1 * ir6;
-    const R t = fma_r(k.c2, ir6, R(-1));
-    return fma_r(u * t, ir2, k.duc * ri);
-}
-
 
 template <typename R>
 struct LJBlock {
@@ -497,78 +446,6 @@ template cudaError_t launch_lj_hs_slice<float>(const float*, const void*, int, i
                                                int*, cudaStream_t);
 template cudaError_t launch_lj_hs_slice<double>(const double*, const void*, int, int, const double*,
                                                 int*, cudaStream_t);
-
-// ------------------------------------------------------------------ Euler-Maruyama (Eq. (2))
-// One CTA per chain, sequential in time; forces as in the action kernel.
-template <typename R>
-__global__ void __launch_bounds__(1024)
-    lj_euler_kernel(R* __restrict__ pos, const R* __restrict__ noise, const LJSysDev<R> S,
-                    int chain0, uint64_t seed, uint64_t counter)
-{
-    using V4 = vec4_t<R>;
-    extern __shared__ __align__(32) unsigned char smem_raw[];
-    const int N = S.N, T = S.T;
-    V4* xa = reinterpret_cast<V4*>(smem_raw);
-    V4* xb = xa + N;
-    LJBlock<R> L;
-    L.init(N, S.tpp, S.lg_tpp, S.cap, reinterpret_cast<uint16_t*>(xb + 2 * N));
-    const LJK<R>& k = S.k;
-    const int chain = blockIdx.x, s = 3 * N, i = L.i;
-    R* X = pos + S.off + chain * S.chain_len;
-    const R* Z = noise ? noise + S.off + chain * S.chain_len : nullptr;
-    load_slice<R>(xa, X, N);
-    __syncthreads();
-    L.build(xa, k);
-    for (int t = 0; t < T; ++t) {
-        if (__syncthreads_or(L.moved(xa, k))) L.build(xa, k);
-        R f[3];
-        L.force(xa, k, f[0], f[1], f[2]);
-        if (L.active && L.q == 0) {
-            const V4 p = xa[i];
-            const R xo[3] = {p.x, p.y, p.z};
-            R xn[3];
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                const long long e = (long long)(t + 1) * s + c * N + i;
-                R z;
-                if (Z) {
-                    z = Z[e];
-                } else {
-                    const float4 w = philox_normals4(seed, counter, kStreamEuler,
-                                                     (uint32_t)(chain0 + chain), (uint32_t)(e >> 2));
-                    z = (R)pick4(w, (int)(e & 3));
-                }
-                xn[c] = xo[c] + fma_r(k.a, f[c], k.sig_em * z);
-                X[e] = xn[c];
-            }
-            xb[i] = make4<R>(xn[0], xn[1], xn[2]);
-        }
-        __syncthreads();
-        V4* tmp = xa;
-        xa = xb;
-        xb = tmp;
-    }
-}
-
-template <typename R>
-cudaError_t launch_lj_euler(R* pos, const R* noise, const void* sys_entry_host, int NT, size_t smem,
-                            int n_chains, int chain0, uint64_t seed, uint64_t counter,
-                            cudaStream_t st)
-{
-    if (n_chains <= 0) return cudaSuccess;
-    const LJSysDev<R> S = *static_cast<const LJSysDev<R>*>(sys_entry_host);
-    if (S.T <= 0) return cudaSuccess;
-    auto kern = lj_euler_kernel<R>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    kern<<<n_chains, NT, smem, st>>>(pos, noise, S, chain0, seed, counter);
-    return cudaGetLastError();
-}
-
-template cudaError_t launch_lj_euler<float>(float*, const float*, const void*, int, size_t, int, int,
-                                            uint64_t, uint64_t, cudaStream_t);
-template cudaError_t launch_lj_euler<double>(double*, const double*, const void*, int, size_t, int,
-                                             int, uint64_t, uint64_t, cudaStream_t);
 
 // ------------------------------------------------------------------ pair-count diagnostic
 // Ordered in-cutoff pairs per slice, single-precision rule, all pairs.

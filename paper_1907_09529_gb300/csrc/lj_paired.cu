@@ -50,27 +50,11 @@
 // 16-byte bank groups, and they drift apart only as their classes run out.
 #include <type_traits>
 
-#include "pamd_internal.cuh"
+#include "lj_math.cuh"
 
 namespace pamd {
 
 namespace {
-
-// ------------------------------------------------------------------ packed f32x2 arithmetic
-__device__ __forceinline__ float2 pk(float a, float b) { return make_float2(a, b); }
-__device__ __forceinline__ float2 pk(float a) { return make_float2(a, a); }
-__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-// a - b with one rounding: b * (-1) + a is exact before rounding.
-__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, pk(-1.0f), a); }
-
-__device__ __forceinline__ float rsqrt_approx(float v)
-{
-    float r;
-    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
-    return r;
-}
 
 // Slot o8 = 8 j of a per-particle shared-memory array; a PAMD_DEBUG build checks
 // j < NMAX and sends a bad access to the sink.
@@ -239,7 +223,7 @@ __device__ __forceinline__ float2 pair_r2(float2 dx, float2 dy, float2 dz, const
 __device__ __forceinline__ float2 pair_fs(float2 r2, const K2& k, float2& ri, float2& ir2,
                                           float2& ir6, float2& ir8)
 {
-    ri = pk(rsqrt_approx(r2.x), rsqrt_approx(r2.y));
+    ri = pk(inv_sqrt(r2.x), inv_sqrt(r2.y));
     ir2 = mul2(ri, ri);
     const float2 ir4 = mul2(ir2, ir2);
     ir6 = mul2(ir4, ir2);

@@ -1101,10 +1101,10 @@ int pamd_debug_status(int* checked, int* count, int* site, long long* index, lon
 #endif
     int (*const fetch[])(DebugRecord*) = {debug_fetch_ho, debug_fetch_lj, debug_fetch_lj_paired,
                                           debug_fetch_update, debug_fetch_fragment,
-                                          debug_fetch_lj_double, debug_fetch_ho_update};
+                                          debug_fetch_lj_double, debug_fetch_ho_update, debug_fetch_lj_euler};
     int total = 0, first_site = 0;
     long long first_index = 0, first_bound = 0;
-    for (int f = 0; f < 7; ++f) {
+    for (int f = 0; f < 8; ++f) {
         DebugRecord r;
         if (fetch[f](&r)) return PAMD_ERR_CUDA;
         if (r.count && !total) {
@@ -1560,15 +1560,12 @@ int pamd_euler_reference(const pamd_problem* prob, void* pos, uint64_t seed, uin
                                                      sig, seed, counter, st));
         } else {
             const void* row = &P->h_lj_sys[P->lj_sys_stride * si.lj_index];
-            const size_t smem = lj_smem_bytes(si.N, si.NT, si.tune.maxnb, P->fp64);
             if (P->fp64)
-                PAMD_CUDA_TRY(launch_lj_euler<double>((double*)dpos, (const double*)dnoise, row,
-                                                      si.NT, smem, si.chains, si.chain0, seed,
-                                                      counter, st));
+                PAMD_CUDA_TRY(launch_lj_euler<double>((double*)dpos, (const double*)dnoise, row, si.chains,
+                                                      si.chain0, seed, counter, st));
             else
-                PAMD_CUDA_TRY(launch_lj_euler<float>((float*)dpos, (const float*)dnoise, row,
-                                                     si.NT, smem, si.chains, si.chain0, seed,
-                                                     counter, st));
+                PAMD_CUDA_TRY(launch_lj_euler<float>((float*)dpos, (const float*)dnoise, row, si.chains, si.chain0,
+                                                     seed, counter, st));
         }
     }
     if (host) {

@@ -83,6 +83,7 @@ int debug_fetch_ho(DebugRecord* out);
 int debug_fetch_lj(DebugRecord* out);
 int debug_fetch_lj_paired(DebugRecord* out);
 int debug_fetch_lj_double(DebugRecord* out);
+int debug_fetch_lj_euler(DebugRecord* out);
 int debug_fetch_update(DebugRecord* out);
 int debug_fetch_fragment(DebugRecord* out);
 int debug_fetch_ho_update(DebugRecord* out);
@@ -497,9 +498,8 @@ cudaError_t launch_ho_euler(R* pos, const R* noise, int s, int T, int n_chains, 
                             int chain0, double k, double a, double sig, uint64_t seed,
                             uint64_t counter, cudaStream_t st);
 template <typename R>
-cudaError_t launch_lj_euler(R* pos, const R* noise, const void* sys_entry_host, int NT, size_t smem,
-                            int n_chains, int chain0, uint64_t seed, uint64_t counter,
-                            cudaStream_t st);
+cudaError_t launch_lj_euler(R* pos, const R* noise, const void* sys_entry_host, int n_chains, int chain0,
+                            uint64_t seed, uint64_t counter, cudaStream_t st);
 
 // Deterministic per-chain sums of partials: out[c] = scale * sum(partials[slots[c]]);
 // a non-finite sum sets *err (if given) to PAMD_ERR_NONFINITE.
