@@ -416,6 +416,30 @@ struct PairList {
         }
     }
 
+    // Calls f({8 j1, 8 j2}, 2) over the candidates in the same order, two at a time, and
+    // f({8 j, -}, 1) for an odd last one.
+    template <typename F>
+    __device__ __forceinline__ void for_each_word(F&& f) const
+    {
+        using One = std::integral_constant<int, 1>;
+        using Two = std::integral_constant<int, 2>;
+        if (!active) return;
+        if (!ovf) {
+            const uint32_t* w = nbr + tid;
+            int m = 0;
+            for (; m + 1 < cnt; m += 2, w += NT) {
+                const uint32_t v = PAMD_OK_IDX((m >> 1) * NT + tid, (cap >> 1) * NT) ? *w : 0u;
+                f({(int)(v & 0xFFFFu), (int)(v >> 16)}, Two{});
+            }
+            if (m < cnt) f({(int)((PAMD_OK_IDX((m >> 1) * NT + tid, (cap >> 1) * NT) ? *w : 0u) & 0xFFFFu), 0}, One{});
+        } else {
+            const int st = cls_stride();
+            for (int c = 0; c < 8; c += cstep())
+                for (int j = cls_first(c); j < N; j += st)
+                    if (j != i) f({8 * j, 0}, One{});
+        }
+    }
+
     __device__ __forceinline__ void group_sum(float2& x, float2& y, float2& z) const
     {
         for (int o = tpp >> 1; o > 0; o >>= 1) {
@@ -495,41 +519,63 @@ struct PairList {
             const float2 hxi = pk(hxy.x, hxy.y), hyi = pk(hxy.z, hxy.w), hzi = P.z(HB, 8 * i);
             const float4 fxy = P.xy(FB, 8 * i);
             const float2 fxi = pk(fxy.x, fxy.y), fyi = pk(fxy.z, fxy.w), fzi = P.z(FB, 8 * i);
-            for_each_candidate([&](int o8) {
-                float sx = 0.0f, sy = 0.0f, sz = 0.0f;
-                float2 hzj, fzj;  // z of particle j in the two buffers
-                if (DO_H && DO_F && HB != FB) {
-                    const float4 zz = P.zz(o8);
-                    hzj = HB ? pk(zz.z, zz.w) : pk(zz.x, zz.y);
-                    fzj = FB ? pk(zz.z, zz.w) : pk(zz.x, zz.y);
-                } else {
-                    if (DO_H) hzj = P.z(HB, o8);
-                    if (DO_F) fzj = P.z(FB, o8);
+            for_each_word([&](const int (&o8)[2], auto n_c) {
+                // both entries of a list word stage by stage: their chains of arithmetic overlap
+                constexpr int NE = decltype(n_c)::value;
+                float sx[NE], sy[NE], sz[NE];
+                float2 dx[NE], dy[NE], dz[NE], r2[NE], ri[NE], ir2[NE], ir6[NE], ir8[NE], fs[NE];
+                float2 gx[NE], gy[NE], gz[NE], q2[NE], qi[NE], j2[NE], j6[NE], j8[NE], gs[NE], hzj[NE], fzj[NE];
+#pragma unroll
+                for (int e = 0; e < NE; ++e) {
+                    if (DO_H && DO_F && HB != FB) {
+                        const float4 zz = P.zz(o8[e]);
+                        hzj[e] = HB ? pk(zz.z, zz.w) : pk(zz.x, zz.y);
+                        fzj[e] = FB ? pk(zz.z, zz.w) : pk(zz.x, zz.y);
+                    } else {
+                        if (DO_H) hzj[e] = P.z(HB, o8[e]);
+                        if (DO_F) fzj[e] = P.z(FB, o8[e]);
+                    }
+                    if (DO_H) {
+                        if (SK)
+                            pair_vec_shift(hxi, hyi, hzi, P.xy(HB, o8[e]), hzj[e], k, dx[e], dy[e], dz[e], sx[e], sy[e],
+                                           sz[e]);
+                        else
+                            pair_vec(hxi, hyi, hzi, P.xy(HB, o8[e]), hzj[e], k, dx[e], dy[e], dz[e]);
+                    }
+                    if (DO_F) {
+                        if (SK && DO_H)
+                            pair_vec_given(fxi, fyi, fzi, P.xy(FB, o8[e]), fzj[e], k, sx[e], sy[e], sz[e], gx[e], gy[e],
+                                           gz[e]);
+                        else if (SK)
+                            pair_vec_shift(fxi, fyi, fzi, P.xy(FB, o8[e]), fzj[e], k, gx[e], gy[e], gz[e], sx[e], sy[e],
+                                           sz[e]);
+                        else
+                            pair_vec(fxi, fyi, fzi, P.xy(FB, o8[e]), fzj[e], k, gx[e], gy[e], gz[e]);
+                    }
                 }
-                if (DO_H) {
-                    float2 dx, dy, dz, ri, ir2, ir6, ir8;
-                    if (SK)
-                        pair_vec_shift(hxi, hyi, hzi, P.xy(HB, o8), hzj, k, dx, dy, dz, sx, sy, sz);
-                    else
-                        pair_vec(hxi, hyi, hzi, P.xy(HB, o8), hzj, k, dx, dy, dz);
-                    const float2 fs = pair_fs(pair_r2(dx, dy, dz, k), k, ri, ir2, ir6, ir8);
-                    hvp_term(dx, dy, dz, fs, pair_nbc(ri, ir2, ir6, ir8, k), P.rxy(o8), P.rz(o8),
-                             vix, viy, viz, hx, hy, hz);
+#pragma unroll
+                for (int e = 0; e < NE; ++e) {
+                    if (DO_H) r2[e] = pair_r2(dx[e], dy[e], dz[e], k);
+                    if (DO_F) {
+                        q2[e] = pair_r2(gx[e], gy[e], gz[e], k);
+                        if (HS) o |= (q2[e].x <= hs2.x) | (q2[e].y <= hs2.y);
+                    }
                 }
-                if (DO_F) {
-                    float2 dx, dy, dz, ri, ir2, ir6, ir8;
-                    if (SK && DO_H)
-                        pair_vec_given(fxi, fyi, fzi, P.xy(FB, o8), fzj, k, sx, sy, sz, dx, dy, dz);
-                    else if (SK)
-                        pair_vec_shift(fxi, fyi, fzi, P.xy(FB, o8), fzj, k, dx, dy, dz, sx, sy, sz);
-                    else
-                        pair_vec(fxi, fyi, fzi, P.xy(FB, o8), fzj, k, dx, dy, dz);
-                    const float2 r2 = pair_r2(dx, dy, dz, k);
-                    if (HS) o |= (r2.x <= hs2.x) | (r2.y <= hs2.y);
-                    const float2 fs = pair_fs(r2, k, ri, ir2, ir6, ir8);
-                    fx = fma2(fs, dx, fx);
-                    fy = fma2(fs, dy, fy);
-                    fz = fma2(fs, dz, fz);
+#pragma unroll
+                for (int e = 0; e < NE; ++e) {
+                    if (DO_H) fs[e] = pair_fs(r2[e], k, ri[e], ir2[e], ir6[e], ir8[e]);
+                    if (DO_F) gs[e] = pair_fs(q2[e], k, qi[e], j2[e], j6[e], j8[e]);
+                }
+#pragma unroll
+                for (int e = 0; e < NE; ++e) {
+                    if (DO_H)
+                        hvp_term(dx[e], dy[e], dz[e], fs[e], pair_nbc(ri[e], ir2[e], ir6[e], ir8[e], k), P.rxy(o8[e]),
+                                 P.rz(o8[e]), vix, viy, viz, hx, hy, hz);
+                    if (DO_F) {
+                        fx = fma2(gs[e], gx[e], fx);
+                        fy = fma2(gs[e], gy[e], fy);
+                        fz = fma2(gs[e], gz[e], fz);
+                    }
                 }
             });
             if (HS && DO_F) *ov |= o;

@@ -56,6 +56,7 @@ struct LJTune {
 };
 
 LJTune g_tune_override;  // 0 / negative fields mean "automatic"
+constexpr double kItemOverhead = 4.2;   // cost of an item beyond its steps, in steps (paired LJ kernel)
 constexpr int kMaxListPerThread = 1024;  // list entries per thread (uint16 indices)
 std::mutex g_mutex;
 
@@ -328,6 +329,22 @@ int choose_lj_block(int nmax)
     return std::max(128, std::min(1024, ((nmax * tpp + 31) / 32) * 32));
 }
 
+// Outer-list capacity per thread.  The lists reach rc + Delta_i + Delta_j with item-wide
+// margins; sized for about 2.5 times the spread of a 3D displacement over half an item (a
+// particle beyond that builds its window lists from every candidate).
+int lj_outer_cap(int N, const pamd_potential& pot, double sig_step, int tile_steps, int tpp)
+{
+    const double dmax = 2.5 * sig_step * std::sqrt(3.0 * 0.5 * (tile_steps + 1));
+    const double ro = pot.rc + 2.0 * dmax, rho = N / (pot.box * pot.box * pot.box);
+    int ow = (int)std::min(1.0e6, 1.2 * 4.18879020478639 * ro * ro * ro * rho) + 16;
+    ow = std::min(ow, N - 1 + 2 * tpp);
+    return std::max(2, std::min((ow + tpp - 1) / tpp, kMaxListPerThread)) & ~1;
+}
+
+// Relative time of one step: list entries, and a constant for what does not shrink with
+// the system (barriers, staging and the latency of a short list; fitted to N = 108 and 500).
+double lj_step_cost(int N, const LJTune& t) { return (double)N * t.maxnb * t.tpp + 10000.0; }
+
 // Per-system LJ launch shape: threads per particle (largest power of two <= 8
 // with N * tpp <= NT), Verlet skin (one-step kernel) or window length (paired
 // kernel), list capacity per thread, tile length.  sig_step = sqrt(2 D dt), the
@@ -356,16 +373,7 @@ LJTune choose_lj_tune(const pamd_system& s, int NT, int cap_lane_max, bool paire
         rl = s.pot.rc + 2.0 * dmax;
     }
     const double L = s.pot.box, rho = N / (L * L * L);
-    if (paired) {
-        // Outer lists reach rc + Delta_i + Delta_j with item-wide margins; size them
-        // for about 2.5 times the spread of a 3D displacement over half a tile (a
-        // particle beyond that builds its window lists from every candidate).
-        const double dmax = 2.5 * sig_step * std::sqrt(3.0 * 0.5 * (t.tile_steps + 1));
-        const double ro = s.pot.rc + 2.0 * dmax;
-        int ow = (int)(1.2 * 4.18879020478639 * ro * ro * ro * rho) + 16;
-        ow = std::min(ow, N - 1 + 2 * tpp);
-        t.outer_cap = std::max(2, std::min((ow + tpp - 1) / tpp, kMaxListPerThread)) & ~1;
-    }
+    if (paired) t.outer_cap = lj_outer_cap(N, s.pot, sig_step, t.tile_steps, tpp);
     const double expect = 4.18879020478639 * rl * rl * rl * rho;  // 4/3 pi rl^3 rho
     int want = (int)(1.2 * expect) + 8;
     if (want > N - 1 + tpp) want = N - 1 + tpp;
@@ -603,20 +611,54 @@ int build_plan(const pamd_problem* p, Plan** out)
                     if (si.kind == PAMD_LJ)
                         si.tune.tile_steps = (int)std::max(1LL, std::min(32LL, steps / std::max(1LL, 8 * ctas)));
             }
-            // One LJ system of equal items: pick the tile near the chosen one whose item
-            // count fills whole rounds of the persistent grid (no part-empty last round),
-            // keeping at least 16 steps per item.
-            if (nlj == 1 && !one && !P->fp64) {
-                for (auto& si : P->sys) {
-                    if (si.kind != PAMD_LJ) continue;
-                    const long long G = (long long)bg_cls[si.lj_class] * sms;
-                    const int Tow = si.T - si.halo_lo;  // owned steps
-                    const long long items0 = (long long)si.chains * ((Tow + si.tune.tile_steps - 1) / si.tune.tile_steps);
-                    const long long rounds = (items0 + G - 1) / G;
-                    const long long per_chain = (rounds * G) / si.chains;
-                    if (per_chain >= 1) {
-                        const int tile = (int)((Tow + per_chain - 1) / per_chain);
-                        if (tile >= std::min(16, si.tune.tile_steps)) si.tune.tile_steps = tile;
+            // Single precision: items of equal cost that fill whole rounds of the persistent grid.
+            // An item costs its steps plus about kItemOverhead step-equivalents (the pair before
+            // it, staging and the outer list: 500 particles, 8 x 16384 steps, take 13.1 ms in
+            // items of 32 steps, 11.6 ms in items of 216), so items are as long as the step
+            // limit allows: the fewest rounds r for which cutting every chain into equal items
+            // of at most `limit` steps needs no more than r times the grid.  (Longer items also
+            // have longer outer lists; past 256 steps that costs more than it saves.)  Unlike
+            // systems get two rounds at least: the cost of a step is only estimated, and the
+            // second round evens it out (12 systems of N = 64..864: 1.90 ms, 1.97 with one).
+            if (P->lj_paired && !one) {
+                const int limit = g_tune_override.tile_steps > 0 ? g_tune_override.tile_steps : 256;
+                for (int k = 0; k < (int)P->lj_cls.size(); ++k) {
+                    const long long G = (long long)bg_cls[k] * sms;
+                    std::vector<SysInfo*> in;
+                    std::vector<double> cost;  // of one step
+                    double cmax = 0.0;
+                    for (auto& si : P->sys)
+                        if (si.kind == PAMD_LJ && si.lj_class == k) {
+                            in.push_back(&si);
+                            cost.push_back(lj_step_cost(si.N, si.tune));
+                            cmax = std::max(cmax, cost.back() * (si.T + kItemOverhead));
+                        }
+                    // steps per item of system q at cost c, and the items all chains then need
+                    auto tile = [&](size_t q, double c) {
+                        const int own = in[q]->T - in[q]->halo_lo;
+                        const int most = std::max(1, std::min(limit, (int)std::min(2.0e9, c / cost[q] - kItemOverhead)));
+                        const int n = (own + most - 1) / most;  // equal parts
+                        return (own + n - 1) / n;
+                    };
+                    auto items_at = [&](double c) {
+                        long long n = 0;
+                        for (size_t q = 0; q < in.size(); ++q) {
+                            const int own = in[q]->T - in[q]->halo_lo, t = tile(q, c);
+                            n += (long long)in[q]->chains * ((own + t - 1) / t);
+                        }
+                        return n;
+                    };
+                    const long long rounds = std::max<long long>(in.size() > 1 ? 2 : 1, (items_at(cmax) + G - 1) / G);
+                    double lo = 0.0, hi = cmax;  // smallest item cost that needs no more rounds
+                    for (int it = 0; it < 60; ++it) {
+                        const double mid = 0.5 * (lo + hi);
+                        (items_at(mid) <= rounds * G ? hi : lo) = mid;
+                    }
+                    for (size_t q = 0; q < in.size(); ++q) {
+                        in[q]->tune.tile_steps = tile(q, hi);
+                        const SysInfo& si = *in[q];
+                        in[q]->tune.outer_cap = lj_outer_cap(si.N, si.pot, std::sqrt(2.0 * p->D * p->dt),
+                                                             si.tune.tile_steps, si.tune.tpp);
                     }
                 }
             }
@@ -642,7 +684,7 @@ int build_plan(const pamd_problem* p, Plan** out)
                         it.t1 = std::min(si.T, it.t0 + si.tune.tile_steps);
                         it.slot = slot + b * si.n_tiles + tl;
                         sys_items[q].push_back(it);
-                        sys_cost[q].push_back((double)si.N * si.tune.maxnb * si.tune.tpp * (it.t1 - it.t0 + 1));
+                        sys_cost[q].push_back(lj_step_cost(si.N, si.tune) * (it.t1 - it.t0 + 1));
                     }
                 }
                 slot += si.chains * si.n_tiles;
@@ -993,7 +1035,11 @@ int path_update_pipelined(const pamd_problem* prob, Plan* P, void* pos, void* gr
         const ElemBlock& B = P->h_all[P->h_E_slots[c].begin];
         return B.chain_base + B.chain_len;
     };
-    const int K = std::min(nc, kMaxChunks);
+    // no more chunks than leave the compute lanes together enough Lennard-Jones items for the GPU
+    int K = std::min(nc, kMaxChunks);
+    for (const auto& C : P->lj_cls)
+        if (P->lj_paired)
+            K = std::max(1, std::min(K, (int)((long long)P->n_lanes * C.n_items / std::max(1, C.grid_grad))));
     long long total = 0;
     for (int c = 0; c < nc; ++c) total += e_end(c) - e_begin(c);
     std::vector<int> cut(K + 1, nc);
