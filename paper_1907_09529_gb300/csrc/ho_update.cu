@@ -336,6 +336,186 @@ __global__ void __launch_bounds__(kElemThreads)
     }
 }
 
+// ------------------------------------------------------------------ double precision, few chains
+// All updates of double-precision chains of one block, a cluster of CS = 2, 4 or 8 CTAs per
+// chain.  One SM issues the 14 FP64 instructions of an element at two lanes a clock, and the
+// update is a chain of dependent steps, so the elements are spread over the cluster, one per
+// thread.  The sums keep ho_loop_kernel's order: its thread v adds elements v, v + 256, ..., so
+// CTA `rank` takes the runs [256 k + 32 VW rank, + 32 VW) of every k (VW = 8 / CS of the eight
+// warps), forms their terms, adds them per v in increasing k and over each warp, and sends the
+// warp sums to every CTA; each then takes the accept test itself.  The s elements on either
+// side of a run are proposed again here; their gradients come from the CTA that owns them.
+// One cluster barrier per update, during which the next normals and log u are drawn.
+// 100 updates of one path of 1024 steps: 918 us with ho_loop_kernel, 360 us (3.6 us an update,
+// about a third of it the barrier's round trip, the rest FP64 latency).
+struct HoCluster {
+    int cs, vw, K, s;  // CTAs, warps of the sum order per CTA, runs per CTA, elements per slice
+    __host__ __device__ int run() const { return 32 * vw; }
+    __host__ __device__ int own() const { return 32 * vw * K; }
+    __host__ __device__ int halo() const { return 2 * s * K; }
+    __host__ __device__ int threads() const { return own() + (halo() + 31) / 32 * 32; }
+    __host__ __device__ size_t doubles() const  // x', terms, halo gradients (2), warp sums (2)
+    {
+        return (size_t)K * (run() + 2 * s) + 3 * (size_t)own() + 2 * (size_t)halo() + 2 * 24;
+    }
+};
+
+__device__ __forceinline__ void send(double* p, unsigned rank, double v)
+{
+    unsigned a = (unsigned)__cvta_generic_to_shared(p), r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(r), "d"(v) : "memory");
+}
+
+__global__ void __launch_bounds__(1024)
+    ho_cluster_kernel(const ElemBlock* __restrict__ blocks, double* __restrict__ pos, double* __restrict__ grad,
+                      double* __restrict__ Sv, const MalaDev* __restrict__ md, int update0, int n_updates, double a,
+                      double ginv, double S_scale, const double* __restrict__ log_u, int* __restrict__ n_accepted,
+                      double* __restrict__ log_alpha, int* __restrict__ err, const HoCluster H)
+{
+    extern __shared__ __align__(16) double smem_d[];
+    __shared__ int s_acc;
+    __shared__ double s_lu[2];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, NW = blockDim.x >> 5;
+    const int cs = H.cs, s = H.s, RL = H.run(), K = H.K, own_n = H.own(), pitch = RL + 2 * s;
+    unsigned rank;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+    const ElemBlock B = blocks[blockIdx.x / cs];
+    const MalaDev M = *md;
+    PAMD_ARR(double, XP, smem_d, K * pitch);
+    PAMD_ARR(double, V, smem_d + K * pitch, 3 * own_n);
+    double* HG = smem_d + K * pitch + 3 * own_n;  // [2][halo]
+    double* VS = HG + 2 * H.halo();               // [2][3][8]
+    // this thread's element: one of the CTA's runs, or a neighbour of one
+    const bool own = tid < own_n;
+    const int h = tid - own_n;
+    const bool halo = h >= 0 && h < H.halo();
+    const int k = own ? tid / RL : halo ? h / (2 * s) : 0;
+    const int p = own ? tid - k * RL : halo ? ((h / s) & 1 ? RL + h % s : h % s - s) : 0;  // place in the run
+    const int e = 256 * k + RL * (int)rank + p;
+    const bool in = (own || halo) && e >= 0 && e < B.n;
+    const bool moves = in && e >= s;  // not the fixed tail x_0
+    const int xi = k * pitch + s + p;
+    const double ak = a * B.k, hh = M.h, s2h = M.s2h;
+    const int rend = B.chain_len - s;
+    double* gx = pos + B.chain_base + e;
+    double* gg = grad + B.chain_base + e;
+    double x = in ? *gx : 0.0, g = in ? *gg : 0.0, S_cur = Sv[B.chain];
+    int n_acc = 0;
+    auto normal = [&](int u) -> double {
+        if (!moves) return 0.0;
+        const float4 q = philox_normals4(M.seed, M.counter + (uint64_t)u, kStreamMala, (uint32_t)B.chain, (uint32_t)(e >> 2));
+        return to_double(pick4(q, e & 3));
+    };
+    auto draw_lu = [&](int u) {  // the last warp, one lane
+        if (tid == 32 * (NW - 1))
+            s_lu[u & 1] = log_u ? log_u[B.chain]
+                                : log(philox_uniform53(M.seed, M.counter + (uint64_t)u, kStreamAccept, (uint32_t)B.chain));
+    };
+    double z = normal(update0);
+    draw_lu(update0);
+    if (own || halo) XP[xi] = 0.0;
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    for (int u = update0; u < update0 + n_updates; ++u) {
+        const int par = u & 1;
+        const double xp = moves ? x + fma_r(-hh, g, s2h * z) : x;
+        if (in) XP[xi] = xp;
+        __syncthreads();
+        double gp = 0.0;
+        if (own) {
+            double r = 0.0, f = 0.0, b = 0.0;
+            if (in) {
+                const double xm = XP[xi - s], xn = XP[xi + s];
+                const double rp = e >= s ? fma_r(ak, xm, xp - xm) : 0.0;
+                r = e < rend ? fma_r(ak, xp, xn - xp) : 0.0;
+                gp = fma_r(ak, r, rp - r) * ginv;
+                if (moves) {
+                    const double d = xp - x;
+                    f = fma_r(hh, g, d);
+                    b = fma_r(hh, gp, -d);
+                }
+                // the neighbours' copies of this gradient
+                if (p < s && (rank > 0 || k > 0)) {
+                    const int kk = rank > 0 ? k : k - 1;
+                    send(HG + par * H.halo() + kk * 2 * s + s + p, rank > 0 ? rank - 1 : cs - 1, gp);
+                }
+                if (p >= RL - s && ((int)rank < cs - 1 || k < K - 1)) {
+                    const int kk = (int)rank < cs - 1 ? k : k + 1;
+                    send(HG + par * H.halo() + kk * 2 * s + p - (RL - s), (int)rank < cs - 1 ? rank + 1 : 0u, gp);
+                }
+            }
+            V[tid] = r;
+            V[own_n + tid] = f;
+            V[2 * own_n + tid] = b;
+        }
+        __syncthreads();
+        for (int q = warp; q < 3 * H.vw; q += NW) {
+            const int w = q % H.vw, t = q / H.vw;
+            double acc = 0.0;
+            for (int kk = 0; kk < K; ++kk) {
+                const double v = V[t * own_n + kk * RL + 32 * w + lane];
+                acc = fma_r(v, v, acc);
+            }
+            acc = warp_sum(acc);
+            if (lane < cs) send(VS + 24 * par + 8 * t + (int)rank * H.vw + w, (unsigned)lane, acc);
+        }
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+        if (u + 1 < update0 + n_updates) {
+            z = normal(u + 1);
+            draw_lu(u + 1);
+        }
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        if (warp == 0) {
+            // lanes 8 t + w: sum t of warp w
+            double v = lane < 24 ? VS[24 * par + lane] : 0.0;
+            v += __shfl_xor_sync(0xffffffffu, v, 4);
+            v += __shfl_xor_sync(0xffffffffu, v, 2);
+            v += __shfl_xor_sync(0xffffffffu, v, 1);
+            const double S_new = v * S_scale, part = v / (4.0 * hh);  // lanes 0; 8 and 16
+            const double qf4 = __shfl_sync(0xffffffffu, part, 8), qr4 = __shfl_sync(0xffffffffu, part, 16);
+            if (lane == 0) {
+                if (rank == 0 && !isfinite(v)) atomicExch(err, PAMD_ERR_NONFINITE);
+                const double la = (S_cur - S_new) - qr4 + qf4;
+                const int acc = s_lu[par] < la ? 1 : 0;  // NaN log alpha never accepts
+                if (log_alpha && rank == 0 && u == update0 + n_updates - 1) log_alpha[B.chain] = la;
+                if (acc) S_cur = S_new;
+                n_acc += acc;
+                s_acc = acc;
+            }
+        }
+        __syncthreads();
+        if (s_acc) {
+            x = xp;
+            g = own ? gp : halo ? HG[par * H.halo() + h] : g;
+        }
+    }
+    if (own && in) {
+        *gx = x;
+        *gg = g;
+    }
+    if (rank == 0 && tid == 0) {
+        Sv[B.chain] = S_cur;
+        if (n_accepted) n_accepted[B.chain] += n_acc;
+    }
+}
+
+// The cluster shape for chains of n elements, s to a slice: as many CTAs per chain (up to 8)
+// as the GPU holds at once; cs = 0 where ho_loop_kernel is the better form (chains of less than
+// kHoClusterMin elements, too many chains, wide slices).
+constexpr int kHoClusterMin = 200;
+HoCluster ho_cluster_shape(int n_chains, int n, int s, int sms)
+{
+    HoCluster h{0, 0, (n + 255) / 256, s};
+    if (n < kHoClusterMin || s > 16) return h;
+    for (int cs = 8; cs >= 2; cs /= 2) {
+        h.cs = cs;
+        h.vw = 8 / cs;
+        if ((long long)cs * n_chains <= sms && h.threads() <= 1024) return h;
+    }
+    h.cs = 0;
+    return h;
+}
+
 }  // namespace
 
 bool ho_update_fusable(int s) { return s <= kHoMaxS; }
@@ -389,6 +569,33 @@ cudaError_t launch_ho_loop(const ElemBlock* blocks, int n_chains, int s, int max
                            cudaStream_t st)
 {
     if (n_chains <= 0 || n_updates <= 0) return cudaSuccess;
+    if constexpr (sizeof(R) == 8) {
+        int dev = 0, sms = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (e != cudaSuccess) return e;
+        const HoCluster h = ho_cluster_shape(n_chains, max_n, s, sms);
+        if (h.cs) {
+            const size_t bytes = sizeof(double) * h.doubles();
+            if (bytes > 48 * 1024) {
+                e = cudaFuncSetAttribute(ho_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+                if (e != cudaSuccess) return e;
+            }
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3((unsigned)(n_chains * h.cs));
+            cfg.blockDim = dim3((unsigned)h.threads());
+            cfg.dynamicSmemBytes = bytes;
+            cfg.stream = st;
+            cudaLaunchAttribute at[1];
+            at[0].id = cudaLaunchAttributeClusterDimension;
+            at[0].val.clusterDim.x = (unsigned)h.cs;
+            at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+            cfg.attrs = at;
+            cfg.numAttrs = 1;
+            return cudaLaunchKernelEx(&cfg, ho_cluster_kernel, blocks, pos, grad, S, md, update0, n_updates, a, ginv,
+                                      S_scale, log_u, n_accepted, log_alpha, err, h);
+        }
+    }
     const size_t arr = (sizeof(R) * ((size_t)max_n + 4) + 15) & ~(size_t)15;
     const size_t smem = HoTrialSmem<R>(max_n, s).bytes + 3 * arr;
     auto k = ho_loop_kernel<R, 0>;
