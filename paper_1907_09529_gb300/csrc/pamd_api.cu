@@ -172,6 +172,7 @@ struct Plan {
     // harmonic systems only: updates run the fused kernels of ho_update.cu, those of chains
     // of one element block (at most ho_max_n elements) in one launch for all updates
     bool ho_fused = false, ho_loop = false;
+    bool ho_direct = false;  // every chain harmonic and one element block: its kernel writes S
     int ho_max_n = 0;
     int* d_overlap = nullptr;
     // host-buffer pipeline: copy streams, the extra compute streams (lanes 1..), events
@@ -522,6 +523,8 @@ int build_plan(const pamd_problem* p, Plan** out)
         P->ho_max_n = (int)std::max<long long>(P->ho_max_n, si.chain_len);
     }
     P->ho_loop = P->ho_fused && P->ho_max_n <= kElemChunk;
+    P->ho_direct = P->ho_max_n <= kElemChunk;
+    for (auto& si : P->sys) P->ho_direct = P->ho_direct && si.kind == PAMD_HARMONIC;
     int slot = (int)P->h_ho.size();
     // LJ: block-size classes, shared-memory budgets, per-system shapes, items.
     std::vector<LJItem> items, grouped;
@@ -855,6 +858,12 @@ int run_action(const pamd_problem* p, Plan* P, const R* pos, R* grad, double* S_
     const bool all = c0 == 0 && c1 == P->n_chains;
     const double a = p->beta * p->D * p->dt, ginv = 1.0 / (2.0 * p->D * p->dt);
     const bool one = (p->flags & PAMD_FLAG_ONE_CHAIN_PER_LAUNCH) != 0;
+    HoDirect direct;
+    if (P->ho_direct && finalize) {
+        direct.S = S_out;
+        direct.scale = 1.0 / (4.0 * p->D * p->dt);
+        direct.err = P->d_err;
+    }
     // harmonic systems: one launch per system (per chain in the plain form)
     for (const auto& si : P->sys) {
         if (si.kind != PAMD_HARMONIC) continue;
@@ -867,10 +876,10 @@ int run_action(const pamd_problem* p, Plan* P, const R* pos, R* grad, double* S_
             if (std::is_same<R, float>::value && sz <= 4)
                 PAMD_CUDA_TRY(launch_ho_action_vec(P->d_ho + b0, nb, sz, (const float*)pos,
                                                    (float*)grad, P->d_part_S, b0, a, ginv, with_grad,
-                                                   lo, hi, st, slab));
+                                                   lo, hi, st, slab, direct));
             else
                 PAMD_CUDA_TRY(launch_ho_action<R>(P->d_ho + b0, nb, P->max_s_ho, pos, grad, P->d_part_S,
-                                                  b0, a, ginv, with_grad, st, slab));
+                                                  b0, a, ginv, with_grad, st, slab, direct));
             return PAMD_OK;
         };
         int rc;
@@ -916,7 +925,7 @@ int run_action(const pamd_problem* p, Plan* P, const R* pos, R* grad, double* S_
             if (n > 0) PAMD_CUDA_TRY(launch(P->d_lj_items_grp + C.grp_off + f, n, std::min(grid, n)));
         }
     }
-    if (finalize)
+    if (finalize && !direct.S)
         PAMD_CUDA_TRY(launch_finalize(P->d_part_S, P->d_S_slots + c0, c1 - c0, 1.0 / (4.0 * p->D * p->dt),
                                       S_out + c0, st, P->d_err));
     if (fault_injected("nonfinite")) PAMD_CUDA_TRY(launch_set_status(P->d_err, PAMD_ERR_NONFINITE, st));

@@ -333,6 +333,13 @@ struct ChainSlots {
 };
 
 // ------------------------------------------------------------------ launchers
+// Where the harmonic kernels write a chain's action when every chain is one block.
+struct HoDirect {
+    double* S = nullptr;  // indexed by global chain; nullptr: partial sums instead
+    double scale = 0.0;
+    int* err = nullptr;
+};
+
 // Harmonic action (+ gradient) over element blocks.  Writes one partial
 // sum of |r|^2 per block into partials[slot0 + block].
 // slab: the blocks belong to a time slab (ElemBlock's owned range and summed
@@ -340,7 +347,7 @@ struct ChainSlots {
 template <typename R>
 cudaError_t launch_ho_action(const ElemBlock* blocks, int n_blocks, int max_s, const R* pos, R* grad,
                              double* partials, int slot0, double a, double ginv, bool with_grad,
-                             cudaStream_t st, bool slab);
+                             cudaStream_t st, bool slab, const HoDirect& direct = HoDirect());
 
 // Single-precision form for slices of s <= 4 elements: aligned float4 loads and
 // stores, neighbours from registers.  The blocks must all belong to one system
@@ -348,7 +355,7 @@ cudaError_t launch_ho_action(const ElemBlock* blocks, int n_blocks, int max_s, c
 cudaError_t launch_ho_action_vec(const ElemBlock* blocks, int n_blocks, int s, const float* pos,
                                  float* grad, double* partials, int slot0, double a, double ginv,
                                  bool with_grad, long long sys_lo, long long sys_hi, cudaStream_t st,
-                                 bool slab);
+                                 bool slab, const HoDirect& direct = HoDirect());
 
 struct LJConst {
     double L, rc, eps, sigma, a, ginv, skin;
