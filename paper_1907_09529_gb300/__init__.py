@@ -132,11 +132,17 @@ def _ptr(t: Optional[torch.Tensor]):
     return None if t is None else ctypes.c_void_p(t.data_ptr())
 
 
+# The current stream's handle of a device: the handle alone where torch offers it (0.1 us;
+# torch.cuda.current_stream builds a Stream object, 2.4 us of a small call).
+_current_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None) or (
+    lambda index: torch.cuda.current_stream(index).cuda_stream)
+
+
 def _stream(t: Optional[torch.Tensor], stream=None):
     if stream is not None:
         return ctypes.c_void_p(stream.cuda_stream if hasattr(stream, "cuda_stream") else stream)
     if t is not None and t.is_cuda:
-        return ctypes.c_void_p(torch.cuda.current_stream(t.device).cuda_stream)
+        return ctypes.c_void_p(_current_stream(t.device.index))
     return ctypes.c_void_p(0)
 
 

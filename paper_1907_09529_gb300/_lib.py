@@ -141,8 +141,9 @@ def check(fn: str, status: int) -> None:
 
 
 def _call(name, *args):
-    st = getattr(load(), name)(*args)
-    check(name, st)
+    st = getattr(_lib or load(), name)(*args)
+    if st != PAMD_OK:
+        check(name, st)
     return st
 
 

@@ -13,7 +13,6 @@
 #include <map>
 #include <memory>
 #include <mutex>
-#include <sstream>
 #include <string>
 #include <vector>
 
@@ -283,28 +282,29 @@ void ho_step_constants(const pamd_problem* p, double k, double* g, double* c)
     }
 }
 
+// The content of a problem and of the settings a plan depends on, as bytes: built at every
+// call, so in raw form (formatting it as text took half of a small call).
 std::string plan_key(const pamd_problem* p)
 {
-    std::ostringstream os;
-    os.precision(17);
-    os << p->precision << '|' << p->flags << '|' << p->D << ',' << p->beta << ',' << p->dt << '|'
-       << p->n_systems << '|' << g_tune_override.tile_steps
-       << ',' << g_tune_override.tpp << ',' << g_tune_override.maxnb << ',' << g_tune_override.skin
-       << ',' << g_tune_override.window << '|';
+    std::string k;
+    k.reserve(160 + 112 * (size_t)p->n_systems);
+    auto put = [&](const auto& v) { k.append(reinterpret_cast<const char*>(&v), sizeof(v)); };
+    put(p->precision), put(p->flags), put(p->D), put(p->beta), put(p->dt), put(p->n_systems);
+    const LJTune& t = g_tune_override;
+    put(t.tile_steps), put(t.tpp), put(t.maxnb), put(t.skin), put(t.window);
     // launch-shape switches read when a plan is built: a change builds a new plan
     for (const char* v : {"PAMD_LJ_ONE_STEP", "PAMD_LJ_NO_PIPE", "PAMD_LJ_ONE_CLASS",
                           "PAMD_LJ_PER_STEP_SHIFT", "PAMD_PIPE_LANES"}) {
         const char* e = std::getenv(v);
-        os << (e ? e : "-") << ',';
+        k += e ? e : "-";
+        k += '\0';
     }
     for (int q = 0; q < p->n_systems; ++q) {
         const pamd_system& s = p->systems[q];
-        os << '|' << s.n_particles << ',' << s.n_steps << ',' << s.dim << ',' << s.n_chains << ','
-           << s.pos_offset << ',' << s.pot.kind << ',' << s.pot.k << ',' << s.pot.eps << ','
-           << s.pot.sigma << ',' << s.pot.rc << ',' << s.pot.box << ',' << s.first_slice << ','
-           << s.halo_lo << ',' << s.halo_hi;
+        put(s.n_particles), put(s.n_steps), put(s.dim), put(s.n_chains), put(s.pos_offset), put(s.pot.kind), put(s.pot.k);
+        put(s.pot.eps), put(s.pot.sigma), put(s.pot.rc), put(s.pot.box), put(s.first_slice), put(s.halo_lo), put(s.halo_hi);
     }
-    return os.str();
+    return k;
 }
 
 int max_dynamic_smem()
