@@ -85,6 +85,21 @@ struct FragGeom {
     __device__ __forceinline__ int b(int f) const { return f == nfrag - 1 ? T : first + (f << l); }
 };
 
+// The fragment of one element, moved forward element by element.
+struct FragWalk {
+    int f, a, b;
+    __device__ __forceinline__ FragWalk(const FragGeom& G, int t) : f(G.of_step(t)), a(G.a(f)), b(G.b(f)) {}
+    // to element t, the one after the last; true when that is another fragment
+    __device__ __forceinline__ bool next(const FragGeom& G, int t)
+    {
+        if (t <= b) return false;
+        ++f;
+        a = b;
+        b = f == G.nfrag - 1 ? G.T : b + (1 << G.l);
+        return true;
+    }
+};
+
 // Metropolis-Hastings test of fragment f with the fragment sums s = sum r'^2 - r^2
 // and s0 = sum dy^2 - dx^2:  log u < log alpha = s0 c0 - s cS, with u given as
 // log u or the 53-bit uniform (mant + 1) 2^-53 of Philox stream 5.  For FP32
@@ -235,17 +250,17 @@ __global__ void __launch_bounds__(kFragMaxThreads)
             const int n_act = min(Lw, t_hi * M - e0);
             const bool act = lane < n_act;
             const int t = D.slice(e);
-            const int f = G.of_step(act ? t : t_lo);
+            const int a = G.a(G.of_step(act ? t : t_lo));
             R v = act ? W[e] : R(0);
 #pragma unroll
             for (int i = 0; (M1 ? 1 : M) << i < 32; ++i) {
                 const int d = M << i;
                 if (d >= Lw) break;
                 const R vu = __shfl_up_sync(0xffffffffu, v, d);
-                if (lane >= d && G.of_step(t - (1 << i)) == f) v += vu;
+                if (lane >= d && t - (1 << i) > a) v += vu;  // slice t - 2^i lies in the same fragment
             }
             const int t0 = D.slice(e0);
-            if (act && f == G.of_step(t0 - 1)) v += carry;  // carry is 0 in the first chunk
+            if (act && t0 - 1 > a) v += carry;  // (first chunk: carry is 0)
             if (act) W[e] = v;
             carry = __shfl_sync(0xffffffffu, v, n_act - M + m_lane);
         }
@@ -303,33 +318,33 @@ __global__ void __launch_bounds__(kFragMaxThreads)
     //    earlier pieces are added below in a fixed order (deterministic sums).
     {
         R carry = R(0), carry0 = R(0);
-        int carry_key = -1;
-        const int e_hi = t_hi * M;
+        const int e_lo = t_lo * M, e_hi = t_hi * M;
         for (int e0 = t_lo * M; e0 < e_hi; e0 += 32) {
             const int e = e0 + lane;
             const bool act = e < e_hi;
             const int t = D.slice(act ? e : e0);
-            const int f = G.of_step(t);
+            const int f = G.of_step(t), a = G.a(f);
+            const int e_first = (a + 1) * M;  // the fragment's first element
             R cs = R(0), cs0 = R(0);
             if (act) {
                 const R x1 = X[e], x0 = X[e - M];
-                const R y1 = W[e], y0 = (t - 1 == G.a(f)) ? x0 : W[e - M];
+                const R y1 = W[e], y0 = (t - 1 == a) ? x0 : W[e - M];
                 const R r = (x1 - x0) + ak * x0, rt = (y1 - y0) + ak * y0;
                 const R dx = x1 - x0, dy = y1 - y0;
                 cs = (rt - r) * (rt + r);
                 cs0 = (dy - dx) * (dy + dx);
             }
+            const int back = min(lane, e - e_first);  // lanes below that hold the same fragment
 #pragma unroll
             for (int d = 1; d < 32; d <<= 1) {
                 const R u1 = __shfl_up_sync(0xffffffffu, cs, d);
                 const R u2 = __shfl_up_sync(0xffffffffu, cs0, d);
-                const int fk = __shfl_up_sync(0xffffffffu, f, d);
-                if (lane >= d && fk == f) {
+                if (d <= back) {
                     cs += u1;
                     cs0 += u2;
                 }
             }
-            if (f == carry_key) {
+            if (e0 > e_lo && e0 > e_first) {  // the chunk before ended in this fragment
                 cs += carry;
                 cs0 += carry0;
             }
@@ -340,7 +355,6 @@ __global__ void __launch_bounds__(kFragMaxThreads)
             const int src = min(31, e_hi - 1 - e0);
             carry = __shfl_sync(0xffffffffu, cs, src);
             carry0 = __shfl_sync(0xffffffffu, cs0, src);
-            carry_key = __shfl_sync(0xffffffffu, f, src);
         }
         if (lane == 0) {
             tS[warp] = (t_lo < t_hi) ? carry : R(0);
@@ -366,16 +380,15 @@ __global__ void __launch_bounds__(kFragMaxThreads)
     }
     __syncthreads();
 
-    // 5. Metropolis-Hastings decision of every fragment with an interior point
+    // 5. Metropolis-Hastings decision of every fragment with an interior point;
+    //    accepted fragments are listed (in any order: their writes are disjoint)
     for (int f = tid; f < G.nfrag; f += nt) {
-        int acc = 0;
         const int fa = G.a(f), fb = G.b(f);
         if (f == G.nfrag - 1 || fb - fa >= 2) {
-            acc = frag_accept<R>(FS[f], FS0[f], cS, cSf, c0, c0f, log_u, fstride, c, f, seed, counter);
             atomicAdd(cnt, 1);
-            if (acc) atomicAdd(cnt + 1, 1);
+            if (frag_accept<R>(FS[f], FS0[f], cS, cSf, c0, c0f, log_u, fstride, c, f, seed, counter))
+                accf[atomicAdd(cnt + 1, 1)] = f;
         }
-        accf[f] = acc;
     }
     __syncthreads();
     if (tid == 0) {
@@ -383,12 +396,12 @@ __global__ void __launch_bounds__(kFragMaxThreads)
         atomicAdd(n_accepted + c, cnt[1]);
     }
 
-    // 6. accepted interiors (and the nose end) back to the path
-#pragma unroll 4
-    for (int e = M + tid; e < E; e += nt) {
-        const int t = D.slice(e);
-        const int f = G.of_step(t);
-        if (accf[f] && (t < G.b(f) || f == G.nfrag - 1)) gX[e] = W[e];
+    // 6. accepted interiors (and the nose end) back to the path, a warp per fragment: its
+    //    elements are contiguous
+    const int n_acc = cnt[1];
+    for (int i = warp; i < n_acc; i += NW) {
+        const int f = accf[i], e1 = (f == G.nfrag - 1 ? T + 1 : G.b(f)) * M;
+        for (int e = (G.a(f) + 1) * M + lane; e < e1; e += 32) gX[e] = W[e];
     }
 }
 
@@ -420,7 +433,9 @@ __host__ __device__ inline size_t frag_line_smem(int T, int nfrag_max, int nwarp
            + up16(sizeof(R) * (size_t)nfrag_max)      // W_b
            + up16(sizeof(R) * (size_t)nwarps * 3)     // piece tails (W, s, s0)
            + up16(sizeof(R) * (size_t)n_shift)        // regeneration normals
-           + up16(sizeof(int) * (2 * (size_t)nfrag_max + 2));  // accepted list and flags, counts
+           // accepted list, counts (two words a fragment: this size also decides which paths
+           // are too long for the kernel, and with that the rounding of their sums)
+           + up16(sizeof(int) * (2 * (size_t)nfrag_max + 2));
 }
 
 template <typename R>
@@ -456,50 +471,52 @@ __device__ __forceinline__ void store_quad(R* p, const R (&v)[4])
     }
 }
 
-// Segmented inclusive scan of one quad per lane in lane order: v[j] (and w[j])
-// of the elements with fragment keys k[j] (non-decreasing along the warp).
-// Adds the earlier lanes' part of each element's segment and the carry from
-// the previous chunk (carry_key), and returns the new carry from lane `src`.
+// Segmented inclusive scan of one quad per lane in lane order, a segment per fragment: lane's
+// elements 4q..4q+3, same[j]: element j lies in the fragment of element j - 1; a0, a3: start
+// points of the fragments of elements 0 and 3 (a fragment holds elements a + 1..b).  Adds the
+// earlier lanes' part of each element's fragment and the carry from the previous chunk (which
+// began at quad q0; `more`: there was one), and returns the new carry from lane `src`.  Which
+// lanes lie in the same fragment follows from the start points, without shuffling keys.
 template <typename R, int NV>
-__device__ __forceinline__ void quad_scan(R (&v)[NV][4], const int (&k)[4], int lane, R (&carry)[NV],
-                                          int& carry_key, int src)
+__device__ __forceinline__ void quad_scan(R (&v)[NV][4], const bool (&same)[4], int a0, int a3, int q, int q0,
+                                          bool more, int lane, R (&carry)[NV], int src)
 {
 #pragma unroll
     for (int j = 1; j < 4; ++j)
-        if (k[j] == k[j - 1])
+        if (same[j])
 #pragma unroll
             for (int n = 0; n < NV; ++n) v[n][j] += v[n][j - 1];
     R agg[NV];
 #pragma unroll
     for (int n = 0; n < NV; ++n) agg[n] = v[n][3];
-    const int akey = k[3];
+    // lane - d ends with element 4 (q - d) + 3, in the fragment of element 3 when beyond a3
+    const int back = min(lane, (4 * q + 2 - a3) >> 2);
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
         R up[NV];
 #pragma unroll
         for (int n = 0; n < NV; ++n) up[n] = __shfl_up_sync(0xffffffffu, agg[n], d);
-        const int uk = __shfl_up_sync(0xffffffffu, akey, d);
-        if (lane >= d && uk == akey)
+        if (d <= back)
 #pragma unroll
             for (int n = 0; n < NV; ++n) agg[n] += up[n];
     }
     R pre[NV];
 #pragma unroll
     for (int n = 0; n < NV; ++n) pre[n] = __shfl_up_sync(0xffffffffu, agg[n], 1);
-    int pkey = __shfl_up_sync(0xffffffffu, akey, 1);
-    if (lane == 0) pkey = -1;
+    const bool in_pre = lane > 0 && 4 * q - 1 > a0, in_carry = more && 4 * q0 - 1 > a0;
     R add[NV];
 #pragma unroll
-    for (int n = 0; n < NV; ++n)
-        add[n] = (pkey == k[0] ? pre[n] : R(0)) + (carry_key == k[0] ? carry[n] : R(0));
+    for (int n = 0; n < NV; ++n) add[n] = (in_pre ? pre[n] : R(0)) + (in_carry ? carry[n] : R(0));
+    bool first = true;  // still the fragment of element 0
 #pragma unroll
-    for (int j = 0; j < 4; ++j)
-        if (k[j] == k[0])
+    for (int j = 0; j < 4; ++j) {
+        if (j) first = first && same[j];
+        if (first)
 #pragma unroll
             for (int n = 0; n < NV; ++n) v[n][j] += add[n];
+    }
 #pragma unroll
     for (int n = 0; n < NV; ++n) carry[n] = __shfl_sync(0xffffffffu, v[n][3], src);
-    carry_key = __shfl_sync(0xffffffffu, k[3], src);
 }
 
 // Optional epilogue of the last MC step of a shifting event (paper Fig. 2): the
@@ -555,8 +572,7 @@ __global__ void __launch_bounds__(kFragMaxThreads)
     PAMD_ARR(R, Zs, (R*)p, sh.out ? sh.n_shift : 0);
     p += up16(sizeof(R) * (size_t)(sh.out ? sh.n_shift : 0));
     PAMD_ARR(int, accf, (int*)p, nfrag_max);
-    PAMD_ARR(int, aflag, (int*)p + nfrag_max, nfrag_max);
-    PAMD_ARR(int, cnt, (int*)p + 2 * nfrag_max, 2);
+    PAMD_ARR(int, cnt, (int*)p + nfrag_max, 2);
 
     PAMD_ARR(R, gX, pos + S.off + (long long)b_chain * E, E);
     PAMD_ARR(const R, gZ, noise ? noise + S.off + (long long)b_chain * E : nullptr, E);
@@ -568,8 +584,7 @@ __global__ void __launch_bounds__(kFragMaxThreads)
     cp_async_commit();
     if (tid < Q * 4 - E) X[E + tid] = R(0);
     if (tid == 0) cnt[0] = cnt[1] = 0;
-    if (sh.out) {
-        for (int f = tid; f < G.nfrag; f += nt) aflag[f] = 0;
+    if (sh.out && sh.sig != 0.0) {
         for (int g = tid; 4 * g < sh.n_shift; g += nt) {
             const float4 z = philox_normals4(seed, sh.counter, kStreamRegenerate, (uint32_t)c, (uint32_t)g);
             const float zq[4] = {z.x, z.y, z.z, z.w};
@@ -590,12 +605,13 @@ __global__ void __launch_bounds__(kFragMaxThreads)
     //    prefix sum over each fragment's slices a+1..b, in place in W
     {
         R carry[1] = {R(0)};
-        int ckey = -1;
         for (int q0 = q_lo; q0 < q_hi; q0 += 32) {
             const int q = q0 + lane;
             const bool qa = q < q_hi;
             R v[1][4];
-            int k[4];
+            bool same[4] = {};
+            FragWalk F(G, min(max(4 * q, 1), T));
+            const int a0 = F.a;
             if (qa && !gZ) {
                 const float4 z = philox_normals4(seed, counter, kStreamFragTrial, (uint32_t)c, (uint32_t)q);
                 v[0][0] = sig * (R)z.x;
@@ -609,9 +625,9 @@ __global__ void __launch_bounds__(kFragMaxThreads)
                 const bool act = qa && e >= 1 && e < E;
                 if (gZ) v[0][j] = act ? sig * gZ[e] : R(0);
                 else if (!act) v[0][j] = R(0);
-                k[j] = G.of_step(min(max(e, 1), T));
+                if (j) same[j] = !F.next(G, min(max(e, 1), T));
             }
-            quad_scan<R, 1>(v, k, lane, carry, ckey, min(31, q_hi - 1 - q0));
+            quad_scan<R, 1>(v, same, a0, F.a, q, q0, q0 > q_lo, lane, carry, min(31, q_hi - 1 - q0));
             if (qa && PAMD_OK_IDX(4 * q + 3, Q * 4)) store_quad((R*)W + 4 * q, v[0]);
         }
         if (lane == 0) tW[warp] = (q_lo < q_hi) ? carry[0] : R(0);
@@ -631,48 +647,60 @@ __global__ void __launch_bounds__(kFragMaxThreads)
     }
     __syncthreads();
 
-    // 3. W_b of every fragment.  The trial point of slice e in fragment f is
-    //    computed where it is needed (the action sums, then the write-back of
-    //    accepted fragments) with explicitly rounded operations, so both uses
-    //    see the same value.
+    // 3. W_b of every fragment.  The trial point of element e in fragment f = (a, b), W_e = w:
     for (int f = tid; f < G.nfrag; f += nt) WB[f] = W[G.b(f)];
     cp_async_wait_all();
     __syncthreads();
-    auto trial = [&](int e, int f, R w) -> R {
-        const int fa = G.a(f), fb = G.b(f);
-        const R xa = X[fa];
+    auto trial = [&](int e, int f, int a, int b, R w, R xe, R xa, R xb, R wb) -> R {
         if (f == G.nfrag - 1) return add_r(xa, w);
-        if (e == fb) return X[e];
-        const R tf = small_int_to_r<R>(e - fa);
-        const R sf = (f == 0) ? div_r(tf, small_int_to_r<R>(fb)) : mul_r(tf, inv_len);
-        return add_r(fma_r(sf, sub_r(X[fb], xa), xa), fma_r(-sf, WB[f], w));
+        if (e == b) return xe;
+        const R tf = small_int_to_r<R>(e - a);
+        const R sf = (f == 0) ? div_r(tf, small_int_to_r<R>(b)) : mul_r(tf, inv_len);
+        return add_r(fma_r(sf, sub_r(xb, xa), xa), fma_r(-sf, wb, w));
     };
+    // slice 4 q_lo - 1, the piece's left neighbour, for lane 0 of the first chunk (before W
+    // becomes the trial)
+    R xl = R(0), yl = R(0);
+    if (lane == 0 && q_lo > 0 && q_lo < q_hi) {
+        const int e = 4 * q_lo - 1;
+        const FragWalk F(G, e);
+        xl = X[e];
+        yl = trial(e, F.f, F.a, F.b, W[e], xl, X[F.a], X[F.b], WB[F.f]);
+    }
+    __syncthreads();
 
-    // 4. per-step terms (r'-r)(r'+r) and (dy-dx)(dy+dx) summed per fragment
+    // 4. the trial, in place of W, and the per-step terms (r'-r)(r'+r) and (dy-dx)(dy+dx)
+    //    summed per fragment
     {
         R carry[2] = {R(0), R(0)};
-        int ckey = -1;
-        // slice 4 q_lo - 1 (the piece's left neighbour) for lane 0 of the first chunk
-        R xl = R(0), yl = R(0);
-        if (lane == 0 && q_lo > 0 && q_lo < q_hi) {
-            const int e = 4 * q_lo - 1, f = G.of_step(e);
-            xl = X[e];
-            yl = trial(e, f, W[e]);
-        }
         for (int q0 = q_lo; q0 < q_hi; q0 += 32) {
             const int q = q0 + lane;
             const bool qa = q < q_hi;
             R v[2][4];
-            int k[4];
+            bool same[4] = {};
             R y[4];
             const bool qok = PAMD_OK_IDX(4 * min(q, Q - 1) + 3, Q * 4);
             const Quad<R> xq = load_quad((R*)X + 4 * (qok ? min(q, Q - 1) : 0));
             const Quad<R> wq = load_quad((R*)W + 4 * (qok ? min(q, Q - 1) : 0));
+            FragWalk F(G, min(max(4 * q, 1), T));
+            const int a0 = F.a;
+            R xa = X[F.a], xb = X[F.b], wb = WB[F.f];
+            int as[4], ends = 0, fs[4];  // start points, fragments, elements that end one
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const int ec = min(max(4 * q + j, 1), T);
-                k[j] = G.of_step(ec);
-                y[j] = trial(ec, k[j], wq.v[j]);
+                if (j && F.next(G, ec)) {
+                    xa = xb;
+                    xb = X[F.b];
+                    wb = WB[F.f];
+                } else if (j) {
+                    same[j] = true;
+                }
+                as[j] = F.a;
+                fs[j] = F.f;
+                if (4 * q + j == F.b) ends |= 1 << j;
+                // (element 0 and the padding beyond T take the trial of elements 1 and T: unused)
+                y[j] = trial(ec, F.f, F.a, F.b, wq.v[j], xq.v[j], xa, xb, wb);
             }
             // slice 4q - 1 from the lane below (lane 0: the previous chunk's lane 31)
             R xp = __shfl_up_sync(0xffffffffu, xq.v[3], 1);
@@ -687,24 +715,23 @@ __global__ void __launch_bounds__(kFragMaxThreads)
             for (int j = 0; j < 4; ++j) {
                 const int e = 4 * q + j;
                 const bool act = qa && e >= 1 && e < E;
-                const int ec = min(max(e, 1), T);
-                const int f = k[j];
                 const R x1 = xq.v[j], x0 = j ? xq.v[j - 1] : xp;
                 const R y1 = y[j];
-                const R y0 = (ec - 1 == G.a(f)) ? x0 : (j ? y[j - 1] : yp);
+                const R y0 = (e - 1 == as[j]) ? x0 : (j ? y[j - 1] : yp);
                 const R r = (x1 - x0) + ak * x0, rt = (y1 - y0) + ak * y0;
                 const R dx = x1 - x0, dy = y1 - y0;
                 v[0][j] = act ? (rt - r) * (rt + r) : R(0);
                 v[1][j] = act ? (dy - dx) * (dy + dx) : R(0);
             }
-            quad_scan<R, 2>(v, k, lane, carry, ckey, min(31, q_hi - 1 - q0));
+            if (qa && PAMD_OK_IDX(4 * q + 3, Q * 4)) store_quad((R*)W + 4 * q, y);
+            quad_scan<R, 2>(v, same, a0, F.a, q, q0, q0 > q_lo, lane, carry, min(31, q_hi - 1 - q0));
+            if (qa && ends) {
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int e = 4 * q + j;
-                if (qa && e >= 1 && e < E && e == G.b(k[j])) {
-                    FS[k[j]] = v[0][j];
-                    FS0[k[j]] = v[1][j];
-                }
+                for (int j = 0; j < 4; ++j)
+                    if ((ends >> j) & 1) {
+                        FS[fs[j]] = v[0][j];
+                        FS0[fs[j]] = v[1][j];
+                    }
             }
         }
         if (lane == 0) {
@@ -739,7 +766,6 @@ __global__ void __launch_bounds__(kFragMaxThreads)
             atomicAdd(cnt, 1);
             if (frag_accept<R>(FS[f], FS0[f], cS, cSf, c0, c0f, log_u, fstride, c, f, seed, counter)) {
                 accf[atomicAdd(cnt + 1, 1)] = f;
-                if (sh.out) aflag[f] = 1;
             }
         }
     }
@@ -749,43 +775,42 @@ __global__ void __launch_bounds__(kFragMaxThreads)
         atomicAdd(n_accepted + c, cnt[1]);
     }
 
-    if (!sh.out) {
-        // 6. accepted interiors (and the nose end) back to the path, a warp per fragment
-        const int n_acc = cnt[1];
-        for (int i = warp; i < n_acc; i += NW) {
-            const int f = accf[i], fa = G.a(f), fb = G.b(f);
-            const int t_end = (f == G.nfrag - 1) ? fb : fb - 1;
-            for (int e = fa + 1 + lane; e <= t_end; e += 32) gX[e] = trial(e, f, W[e]);
+    // 6. accepted interiors (and the nose end) to the path, a warp per fragment; a shifting
+    //    event also needs them in X
+    const int n_acc = cnt[1];
+    for (int i = warp; i < n_acc; i += NW) {
+        const int f = accf[i], fb = G.b(f);
+        const int t_end = (f == G.nfrag - 1) ? fb : fb - 1;
+        for (int e = G.a(f) + 1 + lane; e <= t_end; e += 32) {
+            const R v = W[e];
+            gX[e] = v;
+            if (sh.out) X[e] = v;
         }
-        return;
     }
-    // 6'. final path P: accepted interiors to the path, P shifted to `out`,
-    //     P[1..n_shift] to the trajectory, and the nose regrown
+    if (!sh.out) return;
+    __syncthreads();
+    // 6'. the final path shifted to `out`, its points 1..n_shift to the trajectory, and the
+    //     nose regrown
     const int ns = sh.n_shift;
     PAMD_ARR(R, gO, sh.out + S.off + (long long)b_chain * E, E);
     PAMD_ARR(R, gT, sh.traj + (long long)b_chain * ns, ns);
-    auto final_at = [&](int e) -> R {
-        const int f = G.of_step(e);
-        if (aflag[f] && (e < G.b(f) || f == G.nfrag - 1)) return trial(e, f, W[e]);
-        return X[e];
-    };
-    for (int e = 1 + tid; e < E; e += nt) {
-        const int f = G.of_step(e);
-        R pe = X[e];
-        if (aflag[f] && (e < G.b(f) || f == G.nfrag - 1)) {
-            pe = trial(e, f, W[e]);
-            gX[e] = pe;
+#pragma unroll 4
+    for (int e = tid; e < E - ns; e += nt) gO[e] = X[e + ns];
+    for (int e = tid; e < ns; e += nt) gT[e] = X[e + 1];
+    if (sh.sig == 0.0) {  // the line x_T
+        const R x = X[T];
+        for (int k = 1 + tid; k <= ns; k += nt) gO[T - ns + k] = x;
+    } else if (warp == NW - 1) {
+        if (lane == 31) {
+            R x = X[T];
+            const R sr = (R)sh.sig;
+            for (int k = 0; k < ns; ++k) {
+                x = fma_r(sr, Zs[k], x);
+                Zs[k] = x;
+            }
         }
-        if (e >= ns) gO[e - ns] = pe;
-        if (e <= ns) gT[e - 1] = pe;
-    }
-    if (tid == nt - 1) {
-        R x = final_at(T);
-        const R sr = (R)sh.sig;
-        for (int k = 1; k <= ns; ++k) {
-            x = fma_r(sr, Zs[k - 1], x);
-            gO[T - ns + k] = x;
-        }
+        __syncwarp();
+        for (int k = 1 + lane; k <= ns; k += 32) gO[T - ns + k] = Zs[k - 1];
     }
 }
 
