@@ -370,16 +370,34 @@ struct PairList {
             }
         };
         if (!oovf) {
+            // four words ahead: the words come from L2, and a load may not move above the
+            // stores of the entries before it
             const uint32_t* w = outer + tid;
-            for (int m = 0; m < ocnt; m += 2, w += NT) {
-                const uint32_t v = PAMD_OK_IDX((m >> 1) * NT + tid, (ocap >> 1) * NT) ? *w : 0u;
-                const int o1 = (int)(v & 0xFFFFu);
-                const bool two = m + 1 < ocnt;
-                const int o2 = two ? (int)(v >> 16) : o1;
-                bool in1, in2;
-                test2(P, k, pi, o1, o2, in1, in2);
-                add(in1, o1);
-                add(two && in2, o2);
+            auto word = [&](int m) -> uint32_t {
+                return m < ocnt && PAMD_OK_IDX((m >> 1) * NT + tid, (ocap >> 1) * NT) ? w[(m >> 1) * NT] : 0u;
+            };
+            uint32_t next[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) next[u] = word(2 * u);
+            for (int m0 = 0; m0 < ocnt; m0 += 8) {
+                uint32_t v4[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    v4[u] = next[u];
+                    next[u] = word(m0 + 8 + 2 * u);
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int m = m0 + 2 * u;
+                    if (m >= ocnt) break;
+                    const int o1 = (int)(v4[u] & 0xFFFFu);
+                    const bool two = m + 1 < ocnt;
+                    const int o2 = two ? (int)(v4[u] >> 16) : o1;
+                    bool in1, in2;
+                    test2(P, k, pi, o1, o2, in1, in2);
+                    add(in1, o1);
+                    add(two && in2, o2);
+                }
             }
         } else {
             candidate_pairs([&](int j, int j2) {
