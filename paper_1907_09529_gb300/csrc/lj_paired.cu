@@ -1042,6 +1042,10 @@ __global__ void __launch_bounds__(MAXT, 1)
     __shared__ double red[32];
     __shared__ int s_item;
     __shared__ int s_dmax;  // bits of the largest margin of the window being staged
+    // A second launch of this kernel on other systems (the other block-size class) may start
+    // as SMs become free: the two share nothing but read-only input.  It waits for this one
+    // before it ends, so what follows it on the stream follows both.
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (threadIdx.x == 0) s_dmax = 0;
     for (;;) {
         if (threadIdx.x == 0) s_item = atomicAdd(counter, 1);
@@ -1060,6 +1064,7 @@ __global__ void __launch_bounds__(MAXT, 1)
                                         outer + (long long)blockIdx.x * outer_words, &s_dmax, hs2,
                                         overlap);
     }
+    asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 // The pipelined form is used with the gradient for blocks of up to 512 threads
@@ -1102,18 +1107,28 @@ int lj_paired_blocks_per_sm(int NT, size_t smem, bool with_grad, bool pipe)
 cudaError_t launch_lj_paired(const LJItem* items, int n_items, const void* sys_table,
                              const float* pos, float* grad, double* partials, int* counter, int NT,
                              size_t smem, int grid, bool with_grad, bool pipe, uint32_t* outer,
-                             long long outer_words, cudaStream_t st, const float* hs2, int* overlap)
+                             long long outer_words, cudaStream_t st, bool reset, bool follow, const float* hs2,
+                             int* overlap)
 {
     if (n_items <= 0) return cudaSuccess;
     if (NT > 1024) return cudaErrorInvalidValue;
-    cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(int), st);
+    cudaError_t e = reset ? cudaMemsetAsync(counter, 0, sizeof(int), st) : cudaSuccess;
     if (e != cudaSuccess) return e;
     auto kern = paired_kernel_sel(NT, with_grad, pipe, hs2 != nullptr);
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    kern<<<grid, NT, smem, st>>>(items, n_items, static_cast<const LJSysDev<float>*>(sys_table),
-                                 pos, grad, partials, counter, outer, outer_words, hs2, overlap);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)NT);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = follow ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kern, items, n_items, static_cast<const LJSysDev<float>*>(sys_table), pos, grad,
+                              partials, counter, outer, outer_words, hs2, overlap);
 }
 
 PAMD_DEBUG_FETCHER(lj_paired)

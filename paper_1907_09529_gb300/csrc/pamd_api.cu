@@ -49,13 +49,13 @@ bool fault_injected(const char* what)
 
 struct LJTune {
     int tile_steps = 0, tpp = 0, maxnb = 0;
+    double list = 0.0;  // expected list entries of a particle
     double skin = -1.0;
     int window = 0;     // paired kernel: steps per neighbour-list window
     int outer_cap = 0;  // paired kernel: outer-list entries per thread
 };
 
 LJTune g_tune_override;  // 0 / negative fields mean "automatic"
-constexpr double kItemOverhead = 4.2;   // cost of an item beyond its steps, in steps (paired LJ kernel)
 constexpr int kMaxListPerThread = 1024;  // list entries per thread (uint16 indices)
 std::mutex g_mutex;
 
@@ -84,6 +84,7 @@ struct LJClass {
     bool pipe = false;           // gradient pass pipelined over step pairs
     size_t smem = 0;
     long long outer_words = 0;   // 32-bit words of each CTA's outer-list region
+    long long outer_off = 0;     // its regions in a lane's set
     LJDoubleShape dbl;           // double precision: capacities of lj_double.cu
     int item_off = 0, n_items = 0;  // its items in d_lj_items (cost-sorted)
     int grp_off = 0;             // its items in d_lj_items_grp (grouped by chain)
@@ -155,7 +156,6 @@ struct Plan {
     std::map<GraphKey, cudaGraphExec_t> graphs;
     std::vector<void*> allocs;
     // paired LJ kernel: outer lists, one set per compute lane of one region per CTA
-    // (the classes of a lane run one after another and share its set)
     uint32_t* d_outer = nullptr;
     long long outer_lane_words = 0;  // 32-bit words of one lane's set
     // double precision: one set of pair scratch (a region per CTA) per compute lane, and
@@ -342,9 +342,17 @@ int lj_outer_cap(int N, const pamd_potential& pot, double sig_step, int tile_ste
     return std::max(2, std::min((ow + tpp - 1) / tpp, kMaxListPerThread)) & ~1;
 }
 
-// Relative time of one step: list entries, and a constant for what does not shrink with
-// the system (barriers, staging and the latency of a short list; fitted to N = 108 and 500).
-double lj_step_cost(int N, const LJTune& t) { return (double)N * t.maxnb * t.tpp + 10000.0; }
+// Time of one step in the paired kernel, in us: entries per thread times (latency + issue of
+// the active warps), and a constant.  Fitted to single systems of N = 32..864 in blocks of 512
+// and 864 threads (1.2 us at N = 32, 4.6 at 108, 7.7 at 256, 13.7 at 500, 26.5 at 864).
+double lj_step_cost(int N, const LJTune& t)
+{
+    return 1.0 + t.list / t.tpp * (0.08 + 0.0067 * N * t.tpp / 32.0);
+}
+
+// What an item costs beyond its steps, in us: the pair before it, staging, the outer list
+// (28 us at N = 108, 77 at 500).
+double lj_item_cost(int N) { return 20.0 + 0.11 * N; }
 
 // Per-system LJ launch shape: threads per particle (largest power of two <= 8
 // with N * tpp <= NT), Verlet skin (one-step kernel) or window length (paired
@@ -376,6 +384,7 @@ LJTune choose_lj_tune(const pamd_system& s, int NT, int cap_lane_max, bool paire
     const double L = s.pot.box, rho = N / (L * L * L);
     if (paired) t.outer_cap = lj_outer_cap(N, s.pot, sig_step, t.tile_steps, tpp);
     const double expect = 4.18879020478639 * rl * rl * rl * rho;  // 4/3 pi rl^3 rho
+    t.list = std::min(expect, N - 1.0);
     int want = (int)(1.2 * expect) + 8;
     if (want > N - 1 + tpp) want = N - 1 + tpp;
     if (g_tune_override.maxnb > 0) want = g_tune_override.maxnb;
@@ -615,14 +624,11 @@ int build_plan(const pamd_problem* p, Plan** out)
                         si.tune.tile_steps = (int)std::max(1LL, std::min(32LL, steps / std::max(1LL, 8 * ctas)));
             }
             // Single precision: items of equal cost that fill whole rounds of the persistent grid.
-            // An item costs its steps plus about kItemOverhead step-equivalents (the pair before
-            // it, staging and the outer list: 500 particles, 8 x 16384 steps, take 13.1 ms in
-            // items of 32 steps, 11.6 ms in items of 216), so items are as long as the step
-            // limit allows: the fewest rounds r for which cutting every chain into equal items
-            // of at most `limit` steps needs no more than r times the grid.  (Longer items also
-            // have longer outer lists; past 256 steps that costs more than it saves.)  Unlike
-            // systems get two rounds at least: the cost of a step is only estimated, and the
-            // second round evens it out (12 systems of N = 64..864: 1.90 ms, 1.97 with one).
+            // An item costs its steps plus a constant (lj_item_cost: 500 particles, 8 x 16384
+            // steps, take 13.1 ms in items of 32 steps, 11.6 ms in items of 216), so items are as
+            // long as the step limit allows: the fewest rounds r for which cutting every chain into
+            // equal items of at most `limit` steps needs no more than r times the grid.  (Longer items also
+            // have longer outer lists; past 256 steps that costs more than it saves.)
             if (P->lj_paired && !one) {
                 const int limit = g_tune_override.tile_steps > 0 ? g_tune_override.tile_steps : 256;
                 for (int k = 0; k < (int)P->lj_cls.size(); ++k) {
@@ -634,12 +640,12 @@ int build_plan(const pamd_problem* p, Plan** out)
                         if (si.kind == PAMD_LJ && si.lj_class == k) {
                             in.push_back(&si);
                             cost.push_back(lj_step_cost(si.N, si.tune));
-                            cmax = std::max(cmax, cost.back() * (si.T + kItemOverhead));
+                            cmax = std::max(cmax, cost.back() * si.T + lj_item_cost(si.N));
                         }
                     // steps per item of system q at cost c, and the items all chains then need
                     auto tile = [&](size_t q, double c) {
                         const int own = in[q]->T - in[q]->halo_lo;
-                        const int most = std::max(1, std::min(limit, (int)std::min(2.0e9, c / cost[q] - kItemOverhead)));
+                        const int most = std::max(1, std::min(limit, (int)std::min(2.0e9, (c - lj_item_cost(in[q]->N)) / cost[q])));
                         const int n = (own + most - 1) / most;  // equal parts
                         return (own + n - 1) / n;
                     };
@@ -651,7 +657,20 @@ int build_plan(const pamd_problem* p, Plan** out)
                         }
                         return n;
                     };
-                    const long long rounds = std::max<long long>(in.size() > 1 ? 2 : 1, (items_at(cmax) + G - 1) / G);
+                    long long rounds = (items_at(cmax) + G - 1) / G;
+                    // Unlike systems: a second round evens out what the estimated costs miss, where
+                    // an item stays ten times its constant cost (N = 64..500, 60 steps per CTA:
+                    // 1.01 ms against 1.07; 40 steps: 1.52 against 1.47 ms).  Systems of N > 512
+                    // are even enough (0.75 ms, 0.88 with two rounds).
+                    if (rounds == 1 && in.size() > 1 && P->lj_cls[k].nmax <= 512) {
+                        double work = 0.0, fixed = 0.0;
+                        for (size_t q = 0; q < in.size(); ++q) {
+                            const double w = cost[q] * in[q]->chains * in[q]->T;
+                            work += w;
+                            fixed += w * lj_item_cost(in[q]->N);
+                        }
+                        if (work * work >= 10.0 * (double)G * fixed) rounds = 2;
+                    }
                     double lo = 0.0, hi = cmax;  // smallest item cost that needs no more rounds
                     for (int it = 0; it < 60; ++it) {
                         const double mid = 0.5 * (lo + hi);
@@ -687,7 +706,7 @@ int build_plan(const pamd_problem* p, Plan** out)
                         it.t1 = std::min(si.T, it.t0 + si.tune.tile_steps);
                         it.slot = slot + b * si.n_tiles + tl;
                         sys_items[q].push_back(it);
-                        sys_cost[q].push_back(lj_step_cost(si.N, si.tune) * (it.t1 - it.t0 + 1));
+                        sys_cost[q].push_back(lj_step_cost(si.N, si.tune) * (it.t1 - it.t0) + lj_item_cost(si.N));
                     }
                 }
                 slot += si.chains * si.n_tiles;
@@ -744,8 +763,8 @@ int build_plan(const pamd_problem* p, Plan** out)
                         if (si.kind == PAMD_LJ && &P->lj_cls[si.lj_class] == &C)
                             ocap = std::max(ocap, si.tune.outer_cap);
                     C.outer_words = (long long)(ocap / 2) * C.NT;
-                    P->outer_lane_words = std::max(P->outer_lane_words,
-                                                   (long long)std::max(C.grid_grad, C.grid_nograd) * C.outer_words);
+                    C.outer_off = P->outer_lane_words;  // (the classes of a lane may run at the same time)
+                    P->outer_lane_words += (long long)std::max(C.grid_grad, C.grid_nograd) * C.outer_words;
                 }
                 if ((rc0 = P->alloc(&P->d_outer, sizeof(uint32_t) * P->n_lanes * P->outer_lane_words)))
                     return rc0;
@@ -792,7 +811,7 @@ int build_plan(const pamd_problem* p, Plan** out)
     if ((rc = P->alloc(&P->d_lj_items, sizeof(LJItem) * items.size()))) return rc;
     if ((rc = P->alloc(&P->d_lj_items_grp, sizeof(LJItem) * grouped.size()))) return rc;
     if ((rc = P->alloc(&P->d_lj_sys, P->h_lj_sys.size()))) return rc;
-    if ((rc = P->alloc(&P->d_counter, sizeof(int)))) return rc;
+    if ((rc = P->alloc(&P->d_counter, 2 * sizeof(int)))) return rc;  // one per block-size class
     if ((rc = P->alloc(&P->d_err, sizeof(int)))) return rc;
     PAMD_CUDA_TRY(cudaMemset(P->d_err, 0, sizeof(int)));
     if (!items.empty())
@@ -892,17 +911,25 @@ int run_action(const pamd_problem* p, Plan* P, const R* pos, R* grad, double* S_
             if ((rc = ho(b0, b1 - b0))) return rc;
         }
     }
-    // LJ systems: one persistent launch per block-size class, one after another on st
-    for (int k = 0; k < (int)P->lj_cls.size(); ++k) {
+    // LJ systems: one persistent launch per block-size class.  The second class's CTAs start on
+    // the SMs that the first leaves (lj_paired_kernel), each class with its own counter.
+    const bool classes = !one && P->lj_paired && P->lj_cls.size() > 1;
+    if (classes) PAMD_CUDA_TRY(cudaMemsetAsync(counter, 0, sizeof(int) * P->lj_cls.size(), st));
+    bool launched = false;
+    for (int kk = 0; kk < (int)P->lj_cls.size(); ++kk) {
+        const int k = (int)P->lj_cls.size() - 1 - kk;  // the larger systems first
         const LJClass& C = P->lj_cls[k];
         if (C.n_items <= 0) continue;
         const int grid = with_grad ? C.grid_grad : C.grid_nograd;
         auto launch = [&](const LJItem* items, int n, int g) -> cudaError_t {
-            if (std::is_same<R, float>::value && P->lj_paired)
+            if (std::is_same<R, float>::value && P->lj_paired) {
+                const bool follow = classes && launched;
+                launched = true;
                 return launch_lj_paired(items, n, P->d_lj_sys, (const float*)pos, (float*)grad,
-                                        P->d_part_S, counter, C.NT, C.smem, g, with_grad, C.pipe,
-                                        P->d_outer + (long long)lane * P->outer_lane_words,
-                                        C.outer_words, st, (const float*)hs2, overlap);
+                                        P->d_part_S, counter + (classes ? k : 0), C.NT, C.smem, g, with_grad,
+                                        C.pipe, P->d_outer + lane * P->outer_lane_words + C.outer_off,
+                                        C.outer_words, st, !classes, follow, (const float*)hs2, overlap);
+            }
             if constexpr (std::is_same<R, double>::value)
                 return launch_lj_double(items, n, P->d_lj_sys, C.nmax, C.dbl, pos, grad, P->d_part_S, counter,
                                         g, with_grad, P->d_dbl_scratch + lane * P->dbl_lane_bytes, P->d_dbl_edge,
@@ -1029,7 +1056,7 @@ int path_update_pipelined(const pamd_problem* prob, Plan* P, void* pos, void* gr
         PAMD_CUDA_TRY(cudaStreamCreateWithFlags(&c, cudaStreamNonBlocking));
         P->s_cmp.push_back(c);
     }
-    if (!P->d_chunk_counters && (rc = P->alloc(&P->d_chunk_counters, sizeof(int) * kMaxChunks)))
+    if (!P->d_chunk_counters && (rc = P->alloc(&P->d_chunk_counters, 2 * sizeof(int) * kMaxChunks)))
         return rc;
     // events: per chunk inputs-copied, updated, results-copied; start and end (timed,
     // for the timeline that pamd_pipeline_timeline reports)
@@ -1085,7 +1112,7 @@ int path_update_pipelined(const pamd_problem* prob, Plan* P, void* pos, void* gr
         PAMD_CUDA_TRY(cudaStreamWaitEvent(cs, P->events[3 * k], 0));
         for (int u = 0; u < n_updates; ++u)
             if ((rc = run_one_update<R>(prob, P, (R*)dpos, (R*)dgrad, dS, nullptr, nullptr, dnacc, dla,
-                                        u, cs, c0, c1, P->d_chunk_counters + k, lane)))
+                                        u, cs, c0, c1, P->d_chunk_counters + 2 * k, lane)))
                 return rc;
         PAMD_CUDA_TRY(cudaEventRecord(P->events[3 * k + 1], cs));
         PAMD_CUDA_TRY(cudaStreamWaitEvent(P->s_out, P->events[3 * k + 1], 0));

@@ -470,6 +470,8 @@ cudaError_t launch_hs_fixup(double* S, const int* overlap, int n, cudaStream_t s
 // pipe: the gradient launch uses the pipelined form (blocks of <= 512 threads).
 size_t lj_paired_smem_bytes(int NT, int cap_lane, bool pipe);
 int lj_paired_blocks_per_sm(int NT, size_t smem, bool with_grad, bool pipe);
+// reset: zero the counter first (else the caller has).  follow: the launch before on st is
+// another one of these on other items; start as it leaves SMs free.
 // outer: per-CTA outer lists, outer_words 32-bit words for each of grid CTAs.
 // hs2 (NULL: no bias): squared hard-sphere radii per slice of every LJ system
 // (LJSysDev::hs_off); overlap: per global chain, set to 1 where a pair lies within
@@ -477,8 +479,8 @@ int lj_paired_blocks_per_sm(int NT, size_t smem, bool with_grad, bool pipe);
 cudaError_t launch_lj_paired(const LJItem* items, int n_items, const void* sys_table,
                              const float* pos, float* grad, double* partials, int* counter, int NT,
                              size_t smem, int grid, bool with_grad, bool pipe, uint32_t* outer,
-                             long long outer_words, cudaStream_t st, const float* hs2 = nullptr,
-                             int* overlap = nullptr);
+                             long long outer_words, cudaStream_t st, bool reset, bool follow,
+                             const float* hs2, int* overlap);
 
 // Double-precision action (+ adjoint), lj_double.cu: each unordered pair's coefficients
 // once per slice, in a scratch of `scratch` bytes per CTA (`cap` pairs; more are
