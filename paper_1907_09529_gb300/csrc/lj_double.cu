@@ -19,7 +19,7 @@
 // rc = 2.5, against about 7800 for the former form (Verlet lists of radius rc + 0.3,
 // each ordered pair evaluated in the force and again in the Hessian-vector pass).
 // Action and gradient of 2 x 512 steps of N = 256: 17.24 ms before (32 items of 32
-// steps on 152 SMs, FP64 pipe 86 % busy on those), 1.06 ms now; the FP64 work alone
+// steps on 152 SMs, FP64 pipe 86 % busy on those), 0.95 ms now; the FP64 work alone
 // takes 0.7 ms at 1.25 TFLOP/s.
 //
 // Formulas: the file lj_paired.cu states them; with ir2 = 1/r^2,
@@ -41,7 +41,12 @@ namespace pamd {
 
 namespace {
 
-constexpr int kDblThreads = 256;
+// Threads and CTAs per SM, by what the shared memory of nmax particles allows: the FP64 pipe
+// wants about 16 warps, of small systems more (their rows leave lanes idle); with two or fewer
+// CTAs 128 registers are faster than 64.  Measured per particle-step: N = 256 4.15 ns with
+// (256, 2), 3.6 with (256, 4); N = 500 4.8 with (256, 2), 6.0 with 64 registers; N = 864 9.9
+// with one CTA of 256 threads, 7.2 with one of 512.
+enum { kDblSmall = 0, kDblMedium = 1, kDblLarge = 2 };  // (256, 4), (256, 2), (512, 1)
 
 // One pair's record: vector x_i - x_j (i < j) and fs; nb is kept beside it.
 struct __align__(32) PairRec {
@@ -211,8 +216,8 @@ __device__ __forceinline__ double flip(double v, bool neg)
 }
 
 // HS: the hard-sphere path bias is on (hs2: squared radii, overlap: per global chain).
-template <bool GRAD, bool HS>
-__global__ void __launch_bounds__(kDblThreads, 2)
+template <int NT, int MINB, bool GRAD, bool HS>
+__global__ void __launch_bounds__(NT, MINB)
     lj_double_kernel(const LJItem* __restrict__ items, int n_items,
                      const LJSysDev<double>* __restrict__ systems, int nmax, int cap, int pre_global,
                      const double* __restrict__ pos, double* __restrict__ grad,
@@ -221,10 +226,10 @@ __global__ void __launch_bounds__(kDblThreads, 2)
                      const double* __restrict__ hs2, int* __restrict__ overlap)
 {
     extern __shared__ __align__(32) unsigned char smem_raw[];
-    __shared__ double red[kDblThreads / 32];
-    __shared__ int s_item, s_warp[kDblThreads / 32];
+    constexpr int NWARP = NT / 32;
+    __shared__ double red[NWARP];
+    __shared__ int s_item, s_warp[NWARP];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    constexpr int NT = kDblThreads, NWARP = NT / 32;
     const DblScratch sc(cap, nmax, pre_global != 0);
     const DblSmem sl(nmax, pre_global != 0);
     unsigned char* mine = scratch + (size_t)blockIdx.x * sc.bytes;
@@ -486,10 +491,17 @@ __global__ void lj_double_edge_kernel(const LJItem* __restrict__ items, int n_it
 
 using DoubleKernel = void (*)(const LJItem*, int, const LJSysDev<double>*, int, int, int, const double*,
                               double*, double*, int*, unsigned char*, double*, const double*, int*);
-DoubleKernel double_kernel(bool grad, bool hs)
+template <int NT, int MINB>
+DoubleKernel double_kernel_of(bool grad, bool hs)
 {
-    if (grad) return hs ? lj_double_kernel<true, true> : lj_double_kernel<true, false>;
-    return hs ? lj_double_kernel<false, true> : lj_double_kernel<false, false>;
+    if (grad) return hs ? lj_double_kernel<NT, MINB, true, true> : lj_double_kernel<NT, MINB, true, false>;
+    return hs ? lj_double_kernel<NT, MINB, false, true> : lj_double_kernel<NT, MINB, false, false>;
+}
+DoubleKernel double_kernel(int form, bool grad, bool hs)
+{
+    return form == kDblSmall    ? double_kernel_of<256, 4>(grad, hs)
+           : form == kDblMedium ? double_kernel_of<256, 2>(grad, hs)
+                                : double_kernel_of<512, 1>(grad, hs);
 }
 
 }  // namespace
@@ -503,16 +515,19 @@ LJDoubleShape lj_double_shape(int nmax, double pairs_expected, int max_smem)
     h.smem = DblSmem(nmax, h.pre_global).bytes;
     h.scratch = DblScratch(h.cap, nmax, h.pre_global).bytes;
     h.edge_doubles = 9 * nmax;
+    const size_t each = h.smem + 1536;  // with the static and the reserved part
+    h.form = 4 * each <= (size_t)max_smem ? kDblSmall : 2 * each <= (size_t)max_smem ? kDblMedium : kDblLarge;
+    h.threads = h.form == kDblLarge ? 512 : 256;
     return h;
 }
 
-int lj_double_blocks_per_sm(size_t smem, bool with_grad)
+int lj_double_blocks_per_sm(const LJDoubleShape& h, bool with_grad)
 {
-    auto kern = double_kernel(with_grad, false);
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+    auto kern = double_kernel(h.form, with_grad, false);
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)h.smem) != cudaSuccess)
         return 0;
     int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, kDblThreads, smem) != cudaSuccess) return 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, h.threads, h.smem) != cudaSuccess) return 0;
     return nb;
 }
 
@@ -524,11 +539,11 @@ cudaError_t launch_lj_double(const LJItem* items, int n_items, const void* sys_t
     if (n_items <= 0) return cudaSuccess;
     cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(int), st);
     if (e != cudaSuccess) return e;
-    auto kern = double_kernel(with_grad, hs2 != nullptr);
+    auto kern = double_kernel(h.form, with_grad, hs2 != nullptr);
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)h.smem);
     if (e != cudaSuccess) return e;
     const auto* sys = static_cast<const LJSysDev<double>*>(sys_table);
-    kern<<<grid, kDblThreads, h.smem, st>>>(items, n_items, sys, nmax, h.cap, (int)h.pre_global, pos, grad,
+    kern<<<grid, h.threads, h.smem, st>>>(items, n_items, sys, nmax, h.cap, (int)h.pre_global, pos, grad,
                                             partials, counter, scratch, edge, hs2, overlap);
     e = cudaGetLastError();
     if (e != cudaSuccess || !with_grad) return e;

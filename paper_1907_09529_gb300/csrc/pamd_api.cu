@@ -158,9 +158,9 @@ struct Plan {
     // paired LJ kernel: outer lists, one set per compute lane of one region per CTA
     uint32_t* d_outer = nullptr;
     long long outer_lane_words = 0;  // 32-bit words of one lane's set
-    // double precision: one set of pair scratch (a region per CTA) per compute lane, and
-    // the edge records of every S slot
-    unsigned char* d_dbl_scratch = nullptr;
+    // double precision: one set of pair scratch (a region per CTA) per compute lane (those of
+    // the host-buffer pipeline on its first use), and the edge records of every S slot
+    unsigned char* d_dbl_scratch[4] = {};
     size_t dbl_lane_bytes = 0;
     double* d_dbl_edge = nullptr;
     int n_lanes = 1;            // compute lanes of the host-buffer pipeline
@@ -602,10 +602,10 @@ int build_plan(const pamd_problem* p, Plan** out)
                          : P->fp64    ? C.dbl.smem
                                       : lj_smem_bytes(nmax, NT, cap_used, false);
                 const int bg = P->lj_paired ? lj_paired_blocks_per_sm(NT, C.smem, true, C.pipe)
-                               : P->fp64    ? lj_double_blocks_per_sm(C.smem, true)
+                               : P->fp64    ? lj_double_blocks_per_sm(C.dbl, true)
                                             : lj_blocks_per_sm<float>(NT, C.smem, true);
                 const int bn = P->lj_paired ? lj_paired_blocks_per_sm(NT, C.smem, false, C.pipe)
-                               : P->fp64    ? lj_double_blocks_per_sm(C.smem, false)
+                               : P->fp64    ? lj_double_blocks_per_sm(C.dbl, false)
                                             : lj_blocks_per_sm<float>(NT, C.smem, false);
                 if (bg <= 0 || bn <= 0) return PAMD_ERR_UNSUPPORTED;
                 bg_cls[k] = bg;
@@ -777,7 +777,7 @@ int build_plan(const pamd_problem* p, Plan** out)
                                                  C.dbl.scratch * (size_t)std::max(C.grid_grad, C.grid_nograd));
                     edge = std::max(edge, C.dbl.edge_doubles);
                 }
-                if ((rc0 = P->alloc(&P->d_dbl_scratch, P->n_lanes * P->dbl_lane_bytes))) return rc0;
+                if ((rc0 = P->alloc(&P->d_dbl_scratch[0], P->dbl_lane_bytes))) return rc0;
                 if ((rc0 = P->alloc(&P->d_dbl_edge, sizeof(double) * (size_t)edge * slot))) return rc0;
             }
             if (P->fp64)
@@ -932,7 +932,7 @@ int run_action(const pamd_problem* p, Plan* P, const R* pos, R* grad, double* S_
             }
             if constexpr (std::is_same<R, double>::value)
                 return launch_lj_double(items, n, P->d_lj_sys, C.nmax, C.dbl, pos, grad, P->d_part_S, counter,
-                                        g, with_grad, P->d_dbl_scratch + lane * P->dbl_lane_bytes, P->d_dbl_edge,
+                                        g, with_grad, P->d_dbl_scratch[lane], P->d_dbl_edge,
                                         st, hs2, overlap);
             else
                 return launch_lj_items(items, n, P->d_lj_sys, C.nmax, pos, grad, P->d_part_S, counter, C.NT,
@@ -1056,6 +1056,8 @@ int path_update_pipelined(const pamd_problem* prob, Plan* P, void* pos, void* gr
         PAMD_CUDA_TRY(cudaStreamCreateWithFlags(&c, cudaStreamNonBlocking));
         P->s_cmp.push_back(c);
     }
+    for (int l = 1; P->dbl_lane_bytes && l < P->n_lanes; ++l)
+        if (!P->d_dbl_scratch[l] && (rc = P->alloc(&P->d_dbl_scratch[l], P->dbl_lane_bytes))) return rc;
     if (!P->d_chunk_counters && (rc = P->alloc(&P->d_chunk_counters, 2 * sizeof(int) * kMaxChunks)))
         return rc;
     // events: per chunk inputs-copied, updated, results-copied; start and end (timed,

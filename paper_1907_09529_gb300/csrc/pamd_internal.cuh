@@ -490,9 +490,10 @@ struct LJDoubleShape {
     bool pre_global = false;  // row prefixes in the scratch (shared memory too small)
     size_t smem = 0, scratch = 0;
     int edge_doubles = 0;
+    int form = 0, threads = 0;  // kernel form (threads, CTAs per SM)
 };
 LJDoubleShape lj_double_shape(int nmax, double pairs_expected, int max_smem);
-int lj_double_blocks_per_sm(size_t smem, bool with_grad);
+int lj_double_blocks_per_sm(const LJDoubleShape& h, bool with_grad);
 cudaError_t launch_lj_double(const LJItem* items, int n_items, const void* sys_table, int nmax,
                              const LJDoubleShape& h, const double* pos, double* grad, double* partials,
                              int* counter, int grid, bool with_grad, unsigned char* scratch, double* edge,
