@@ -42,7 +42,7 @@ __global__ void __launch_bounds__(kElemThreads)
 
     const ElemBlock B = blocks[blockIdx.x];
     PAMD_ARR(R, xs, reinterpret_cast<R*>(smem_raw), B.n + 2 * B.s);
-    const R ak = a * (R)B.k;
+    const R ak = a * harmonic_k(B, R(0));
     const R* __restrict__ X = pos + B.chain_base;
     const int s = B.s;
     const int lo = B.e0 - s;  // first staged element (may be negative: zero-filled)
@@ -110,7 +110,7 @@ __global__ void __launch_bounds__(kElemThreads)
 {
     __shared__ double red[kElemThreads];
     const ElemBlock B = blocks[blockIdx.x];
-    const float ak = a * (float)B.k;
+    const float ak = a * B.kf;
     const long long base = B.chain_base;
     const long long glo = base + B.e0, ghi = glo + B.n;
     const long long gal = (glo + 3) & ~3LL, gah = ghi & ~3LL;

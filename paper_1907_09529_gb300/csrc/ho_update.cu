@@ -208,7 +208,7 @@ __global__ void __launch_bounds__(kElemThreads)
     const ElemBlock B = blocks[blockIdx.x];
     R sums[3] = {R(0), R(0), R(0)};
     ho_trial<R, S>(B, pos, grad, prop, nullptr, reinterpret_cast<R*>(smem_raw + L.xp),
-                   reinterpret_cast<float*>(smem_raw + L.zs), (R)md->h, (R)md->s2h, a * (R)B.k, ginv, md->seed,
+                   reinterpret_cast<float*>(smem_raw + L.zs), step_h(*md, R(0)), step_s2h(*md, R(0)), a * harmonic_k(B, R(0)), ginv, md->seed,
                    md->counter + (uint64_t)update_index, sums);
     double tot[3] = {to_double(sums[0]), to_double(sums[1]), to_double(sums[2])};
     block_sums_256<3>(tot, reinterpret_cast<double*>(smem_raw + L.red));
@@ -229,7 +229,7 @@ __global__ void __launch_bounds__(kElemThreads)
     const ElemBlock B = blocks[blockIdx.x];
     if (!accept_flag[B.chain]) return;
     const int s = S ? S : B.s;
-    const R ak = a * (R)B.k;
+    const R ak = a * harmonic_k(B, R(0));
     const R* __restrict__ X = prop + B.chain_base;
     const int rend = B.chain_len - s;
     auto grad_at = [&](int e, R xm, R x0, R xp) -> R {
@@ -304,7 +304,7 @@ __global__ void __launch_bounds__(kElemThreads)
     for (int u = update0; u < update0 + n_updates; ++u) {
         R sums[3] = {R(0), R(0), R(0)};
         const int off = ho_trial<R, S>(B, X, G, (R*)nullptr, GP, XP, reinterpret_cast<float*>(smem_raw + L.zs),
-                                       (R)M.h, (R)M.s2h, a * (R)B.k, ginv, M.seed, M.counter + (uint64_t)u, sums);
+                                       step_h(M, R(0)), step_s2h(M, R(0)), a * harmonic_k(B, R(0)), ginv, M.seed, M.counter + (uint64_t)u, sums);
         double tot[3] = {to_double(sums[0]), to_double(sums[1]), to_double(sums[2])};
         block_sums_256<3>(tot, reinterpret_cast<double*>(smem_raw + L.red));
         if (threadIdx.x == 0) {

@@ -510,6 +510,7 @@ int build_plan(const pamd_problem* p, Plan** out)
                 B.chain = c;
                 B.sys = (int)(&si - &P->sys[0]);
                 B.k = si.pot.k;
+                B.kf = (float)si.pot.k;
                 B.e_glob = si.first_slice * s;
                 B.own_lo = si.halo_lo * s;
                 B.own_hi = (int)si.chain_len - si.halo_hi * s;

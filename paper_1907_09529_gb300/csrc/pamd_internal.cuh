@@ -322,7 +322,11 @@ struct ElemBlock {
     int own_lo, own_hi;    // owned chain-local elements (gradient written, proposed)
     int sum_lo;            // first element whose step counts in S (halo step excluded)
     double k;              // harmonic constant (harmonic systems)
+    float kf;              // the same in single precision: a conversion runs on the FP64 pipe
 };
+__device__ __forceinline__ double harmonic_k(const ElemBlock& B, double) { return B.k; }
+__device__ __forceinline__ float harmonic_k(const ElemBlock& B, float) { return B.kf; }
+
 
 constexpr int kElemThreads = 256;
 constexpr int kElemChunk = 4096;  // elements per ElemBlock
@@ -525,7 +529,12 @@ struct MalaDev {
     uint64_t counter;
     double h;
     double s2h;  // sqrt(2 h), taken once: a double square root in every thread kept the FP64 pipe busy
+    float hf, s2hf;  // both in single precision
 };
+__device__ __forceinline__ double step_h(const MalaDev& m, double) { return m.h; }
+__device__ __forceinline__ float step_h(const MalaDev& m, float) { return m.hf; }
+__device__ __forceinline__ double step_s2h(const MalaDev& m, double) { return m.s2h; }
+__device__ __forceinline__ float step_s2h(const MalaDev& m, float) { return m.s2hf; }
 // slab: some block belongs to a time slab (halo elements copied / skipped, noise
 // indexed from the whole path's slice 0); false for whole paths.
 template <typename R>

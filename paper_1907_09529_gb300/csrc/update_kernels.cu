@@ -58,6 +58,8 @@ __global__ void set_mala_params_kernel(MalaDev* md, uint64_t seed, uint64_t coun
     md->counter = counter;
     md->h = h;
     md->s2h = sqrt(2.0 * h);
+    md->hf = (float)h;
+    md->s2hf = (float)md->s2h;
 }
 
 cudaError_t launch_set_mala_params(MalaDev* md, uint64_t seed, uint64_t counter, double h,
@@ -79,7 +81,7 @@ __global__ void __launch_bounds__(kElemThreads)
 {
     __shared__ double red[kElemThreads];
     const ElemBlock B = blocks[blockIdx.x];
-    const R h = (R)md->h, s2h = (R)md->s2h;
+    const R h = step_h(*md, R(0)), s2h = step_s2h(*md, R(0));
     const uint64_t seed = md->seed, counter = md->counter + (uint64_t)update_index;
     const long long base = B.chain_base;
     R acc = R(0);
@@ -127,7 +129,7 @@ __global__ void __launch_bounds__(kElemThreads)
     __shared__ double red[kElemThreads];
     __shared__ __align__(16) float zs[kElemChunk + 4];
     const ElemBlock B = blocks[blockIdx.x];
-    const R h = (R)md->h, s2h = (R)md->s2h;
+    const R h = step_h(*md, R(0)), s2h = step_s2h(*md, R(0));
     const long long base = B.chain_base;
     if (!noise) {
         const uint64_t seed = md->seed, counter = md->counter + (uint64_t)update_index;
@@ -183,7 +185,7 @@ __global__ void __launch_bounds__(kElemThreads)
 {
     __shared__ double red[kElemThreads];
     const ElemBlock B = blocks[blockIdx.x];
-    const R h = (R)md->h;
+    const R h = step_h(*md, R(0));
     const long long base = B.chain_base;
     R acc = R(0);
     auto term = [&](int e, R x, R xp, R gp) {
