@@ -17,8 +17,9 @@
 //     rc + skin, rebuilt when some particle has moved skin / 2 (a list that overflows scans
 //     all candidates).
 // N = 108, four chains of 1024 steps: 4.89 ms (4.8 us a step) with one CTA of four threads
-// per particle and the normals in the step, 1.69 ms (1.65 us) now; a step of N = 500, eight
-// chains, 17.5 -> 3.8 us, of N = 108 in double precision 101 -> 23 us.
+// per particle and the normals in the step, 1.36 ms (1.33 us) now (1.66 us a step before the
+// lane count and the packed constants of the all-pairs form were known to the compiler); a
+// step of N = 500, eight chains, 17.5 -> 3.6 us, of N = 108 in double precision 101 -> 23 us.
 #include <algorithm>
 #include <cmath>
 #include <type_traits>
@@ -90,7 +91,7 @@ struct EulerPos {
     int n, lg;  // padded particles; log2 of the lanes per particle
     __device__ __forceinline__ R* at(int j, int c) const
     {
-        if (sizeof(R) == 4 && !LIST) {
+        if (sizeof(R) == 4 && !LIST) {  // (LG >= 0)
             const int m = j >> lg, q = j & ((1 << lg) - 1);
             return p + c * n + (((m >> 1) << lg) + q) * 2 + (m & 1);
         }
@@ -98,54 +99,72 @@ struct EulerPos {
     }
 };
 
-// Force on particle i from this lane's candidates, every pair, two per packed operation.
-__device__ __forceinline__ void force_dense(const float* p, int npad, int N, int lg, int q, int i, const float (&xi)[3],
-                                            const LJK<float>& k, float (&f)[3])
-{
-    const float2 nL = pk(-k.L), iL = pk(k.iL), mag = pk(12582912.0f), nmag = pk(-12582912.0f);
-    const float2 c1 = pk(k.c1), c2 = pk(k.c2), m1 = pk(-1.0f), duc = pk(k.duc);
-    const float2 x = pk(xi[0]), y = pk(xi[1]), z = pk(xi[2]);
-    const float inf = __int_as_float(0x7f800000);
-    float2 fx = pk(0.0f), fy = pk(0.0f), fz = pk(0.0f);
-    auto two = [&](int m, bool check) {  // candidates j and j + tpp
-        const float2* a = reinterpret_cast<const float2*>(p) + (m << lg) + q;
-        const int j = q + (m << (lg + 1)), j2 = j + (1 << lg);
-        float2 dx = sub2(x, a[0]), dy = sub2(y, a[npad / 2]), dz = sub2(z, a[npad]);
+// Force on a particle from a lane's candidates, every pair, two per packed operation; the
+// constants are set up once, outside the steps.
+template <int LG>
+struct DenseForce {
+    float2 nL, iL, mag, nmag, c1, c2, m1, duc;
+    float rc2;
+    int N, full, all, i, q, py, pz;
+    __device__ __forceinline__ DenseForce(const LJK<float>& k, int N_, int npad, int i_, int q_)
+        : nL(pk(-k.L)), iL(pk(k.iL)), mag(pk(12582912.0f)), nmag(pk(-12582912.0f)), c1(pk(k.c1)), c2(pk(k.c2)),
+          m1(pk(-1.0f)), duc(pk(k.duc)), rc2(k.rc2), N(N_), full(N_ >> (LG + 1)), all(npad >> (LG + 1)), i(i_), q(q_),
+          py(npad / 2), pz(npad)
+    {
+    }
+    template <bool CHECK>
+    __device__ __forceinline__ void two(const float2* a, int j, float2 x, float2 y, float2 z, float2& fx, float2& fy,
+                                        float2& fz) const
+    {
+        const int j2 = j + (1 << LG);
+        const float inf = __int_as_float(0x7f800000);
+        float2 dx = sub2(x, a[0]), dy = sub2(y, a[py]), dz = sub2(z, a[pz]);
         dx = fma2(nL, add2(fma2(dx, iL, mag), nmag), dx);
         dy = fma2(nL, add2(fma2(dy, iL, mag), nmag), dy);
         dz = fma2(nL, add2(fma2(dz, iL, mag), nmag), dz);
         float2 r2 = fma2(dz, dz, fma2(dy, dy, mul2(dx, dx)));
         // r^2 = +inf: exact zeros (outside the cutoff, itself, padding)
-        r2.x = (r2.x <= k.rc2 && j != i && (!check || j < N)) ? r2.x : inf;
-        r2.y = (r2.y <= k.rc2 && j2 != i && (!check || j2 < N)) ? r2.y : inf;
+        r2.x = (r2.x <= rc2 && j != i && (!CHECK || j < N)) ? r2.x : inf;
+        r2.y = (r2.y <= rc2 && j2 != i && (!CHECK || j2 < N)) ? r2.y : inf;
         const float2 ri = pk(inv_sqrt(r2.x), inv_sqrt(r2.y)), ir2 = mul2(ri, ri);
         const float2 ir6 = mul2(mul2(ir2, ir2), ir2), u = mul2(c1, ir6), t = fma2(c2, ir6, m1);
         const float2 fs = fma2(mul2(u, t), ir2, mul2(duc, ri));
         fx = fma2(fs, dx, fx);
         fy = fma2(fs, dy, fy);
         fz = fma2(fs, dz, fz);
-    };
-    const int full = N >> (lg + 1), all = npad >> (lg + 1);
-#pragma unroll 4
-    for (int m = 0; m < full; ++m) two(m, false);
-    if (full < all) two(full, true);
-    f[0] = fx.x + fx.y;
-    f[1] = fy.x + fy.y;
-    f[2] = fz.x + fz.y;
-}
+    }
+    // p: the slice; lane q's candidates 2m, 2m + 1 are the float2 at m 2^LG + q
+    __device__ __forceinline__ void operator()(const float* p, const float (&xi)[3], float (&f)[3]) const
+    {
+        const float2 x = pk(xi[0]), y = pk(xi[1]), z = pk(xi[2]);
+        float2 fx = pk(0.0f), fy = pk(0.0f), fz = pk(0.0f);
+        const float2* a = reinterpret_cast<const float2*>(p) + q;
+        int j = q;
+#pragma unroll 2
+        for (int m = 0; m < full; ++m, j += 2 << LG, a += 1 << LG) two<false>(a, j, x, y, z, fx, fy, fz);
+        if (full < all) two<true>(a, j, x, y, z, fx, fy, fz);
+        f[0] = fx.x + fx.y;
+        f[1] = fy.x + fy.y;
+        f[2] = fz.x + fz.y;
+    }
+};
+
+__device__ __forceinline__ const LJK<float>& dense_consts(const LJK<float>& k) { return k; }
+__device__ __forceinline__ LJK<float> dense_consts(const LJK<double>&) { return LJK<float>(); }  // (not used)
 
 struct EulerShape {
     int cs, nloc, lg, nt, cap, npad;
     size_t smem;
 };
 
-template <typename R, bool LIST>
-__global__ void __launch_bounds__(1024)
+// LG: log2 of the lanes per particle where it is known (the all-pairs form), else -1.
+template <typename R, bool LIST, int LG, int MAXT>
+__global__ void __launch_bounds__(MAXT)
     lj_euler_kernel(R* __restrict__ pos, const R* __restrict__ noise, const LJSysDev<R> S, const EulerShape H)
 {
     extern __shared__ __align__(32) unsigned char smem_raw[];
     const int N = S.N, T = S.T, s = 3 * N, tid = threadIdx.x, NT = blockDim.x;
-    const int lg = H.lg, tpp = 1 << lg, q = tid & (tpp - 1), cs = H.cs, npad = H.npad;
+    const int lg = LG >= 0 ? LG : H.lg, tpp = 1 << lg, q = tid & (tpp - 1), cs = H.cs, npad = H.npad;
     const unsigned rank = cs > 1 ? cluster_rank() : 0u;
     const int chain = blockIdx.x / cs;
     const int i = (int)rank * H.nloc + (tid >> lg);
@@ -205,6 +224,7 @@ __global__ void __launch_bounds__(1024)
     load_zs(true, z[0]);
     load_zs(T > 1, z[1]);
     step_barrier(cs);  // (also: every lane holds its first normals before slice 1 is written)
+    const DenseForce<LG >= 0 ? LG : 0> dense(dense_consts(k), N, npad, i, q);
     // Step t from buffer PAR to the other; zt: its normals.  The slice that the step before
     // made is stored here: a store directly before the barrier would hold it up (the
     // barrier's release waits for it).
@@ -233,8 +253,8 @@ __global__ void __launch_bounds__(1024)
         if (active) {
 #pragma unroll
             for (int c = 0; c < 3; ++c) xi[c] = A.p[oi + c * npad];
-            if constexpr (sizeof(R) == 4 && !LIST) {
-                force_dense(A.p, npad, N, lg, q, i, xi, k, f);
+            if constexpr (LG >= 0) {
+                dense(A.p, xi, f);
             } else if (LIST && !ovf) {
 #pragma unroll 2
                 for (int m = 0; m < cnt; ++m) {
@@ -246,9 +266,11 @@ __global__ void __launch_bounds__(1024)
                     if (j != i) pair_force<R>(xi[0], xi[1], xi[2], *A.at(j, 0), *A.at(j, 1), *A.at(j, 2), k, f);
             }
         }
-        for (int o = tpp >> 1; o > 0; o >>= 1)
 #pragma unroll
-            for (int c = 0; c < 3; ++c) f[c] += __shfl_xor_sync(0xffffffffu, f[c], o);
+        for (int o = 16; o > 0; o >>= 1)
+            if (o < tpp)
+#pragma unroll
+                for (int c = 0; c < 3; ++c) f[c] += __shfl_xor_sync(0xffffffffu, f[c], o);
         auto move = [&](int c, R x, R fc, R zc) {
             const R xn = x + fma_r(k.a, fc, k.sig_em * zc);
             last[c] = xn;
@@ -287,7 +309,8 @@ __global__ void __launch_bounds__(1024)
 // Cluster size, lanes per particle and block size.
 // A cluster barrier costs about 0.55 us (its release waits for the remote stores), so single
 // precision takes clusters where a step's pairs cost more than that (N = 32: 0.82 us a step
-// with one CTA, 1.38 with two; N = 108: 2.7, 2.1, 1.8 with one, two, four), down to
+// with one CTA, 1.38 with two; N = 108: 2.7, 2.1, 1.8 with one, two, four; all before the
+// lane count was a template argument), down to
 // kEulerMinLocal particles per CTA; double precision, bound by the FP64 pipe, almost always
 // (N = 108: 110, 63, 31 us with one, two, four).  Chains beyond the SMs get no cluster.
 // Lanes per particle: about 512 threads (more lanes add shuffles and overhead: N = 108 on four
@@ -343,7 +366,18 @@ cudaError_t launch_lj_euler(R* pos, const R* noise, const void* sys_entry_host, 
     const double rl2 = (double)S.k.rl2, L = (double)S.k.L;
     const EulerShape h = euler_shape<R>(S.N, n_chains, 4.18879020478639 * rl2 * std::sqrt(rl2) * S.N / (L * L * L), sms,
                                         max_smem - 1024);
-    auto kern = S.N > kEulerDense ? lj_euler_kernel<R, true> : lj_euler_kernel<R, false>;
+    void (*kern)(R*, const R*, LJSysDev<R>, EulerShape);
+    if (S.N > kEulerDense)
+        kern = h.nt <= 512 ? lj_euler_kernel<R, true, -1, 512> : lj_euler_kernel<R, true, -1, 1024>;
+    else if constexpr (sizeof(R) == 8)
+        kern = h.nt <= 512 ? lj_euler_kernel<R, false, -1, 512> : lj_euler_kernel<R, false, -1, 1024>;
+    else  // N <= kEulerDense: at least four lanes
+        kern = h.lg == 5   ? lj_euler_kernel<R, false, 5, 512>
+               : h.lg == 4 ? lj_euler_kernel<R, false, 4, 512>
+               : h.lg == 3 ? lj_euler_kernel<R, false, 3, 512>
+               : h.lg == 2 ? lj_euler_kernel<R, false, 2, 1024>
+                           : nullptr;
+    if (!kern) return cudaErrorInvalidValue;
     if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)h.smem)) != cudaSuccess)
         return e;
     cudaLaunchConfig_t cfg = {};
