@@ -144,20 +144,20 @@ __device__ __forceinline__ R small_int_to_r(int n)
     return (R)small_int_to_float(n);
 }
 
-// Slice index and line of element e of a chain ([T+1][M] layout): M == 1 at
-// compile time, else floor(e / M) = umulhi(e, ceil(2^32 / M)), exact for
-// e < 2^32 / M (a chain in shared memory holds far fewer elements).
-template <bool M1>
+// Slice index of element e of a chain ([T+1][M] layout): M = MC at compile time for up to
+// three lines (a division by a constant, shuffle distances and row strides known), else
+// floor(e / M) = umulhi(e, ceil(2^32 / M)), exact for e < 2^32 / M (a chain in shared memory
+// holds far fewer elements).
+template <int MC>
 struct LineDiv {
     uint32_t inv;
-    int M;
-    __device__ __forceinline__ explicit LineDiv(int M_) : M(M_)
+    __device__ __forceinline__ explicit LineDiv(int M)
     {
-        inv = M1 ? 0u : (uint32_t)((0x100000000ull + (uint64_t)M_ - 1) / (uint64_t)M_);
+        inv = MC ? 0u : (uint32_t)((0x100000000ull + (uint64_t)M - 1) / (uint64_t)M);
     }
     __device__ __forceinline__ int slice(int e) const
     {
-        return M1 ? e : (int)__umulhi((uint32_t)e, inv);
+        return MC ? (int)((unsigned)e / (unsigned)(MC ? MC : 1)) : (int)__umulhi((uint32_t)e, inv);
     }
 };
 
@@ -174,7 +174,7 @@ __host__ __device__ inline size_t frag_block_smem(int T, int M, int nfrag_max, i
            + up16(sizeof(int) * ((size_t)nfrag_max + 2));  // accept flags, counts
 }
 
-template <typename R, bool M1>
+template <typename R, int MC>
 __global__ void __launch_bounds__(kFragMaxThreads)
     fragment_block_kernel(R* __restrict__ pos, const FragSys S, int l_min, int l_max, uint64_t seed,
                           uint64_t counter, const int* __restrict__ levels,
@@ -187,8 +187,9 @@ __global__ void __launch_bounds__(kFragMaxThreads)
     const int tid = threadIdx.x, nt = blockDim.x, NW = nt >> 5, warp = tid >> 5, lane = tid & 31;
     const int b_chain = blockIdx.x;
     const int c = S.chain0 + b_chain;
-    const int T = S.T, M = M1 ? 1 : S.M, E = (T + 1) * M;
-    const LineDiv<M1> D(M);
+    constexpr bool M1 = MC == 1;
+    const int T = S.T, M = MC ? MC : S.M, E = (T + 1) * M;
+    const LineDiv<MC> D(M);
     int l, o;
     frag_cut(seed, counter, (uint32_t)c, l_min, l_max, levels, offsets, c, l, o);
     if (l < l_min || l > l_max || o < 0 || o >= (1 << l)) return;  // invalid cut: chain untouched
@@ -952,7 +953,10 @@ cudaError_t launch_fragment_mc(R* pos, long long off, int T, int M, int n_chains
     }
     const size_t smem = frag_block_smem<R>(T, M, nfrag_max, threads / 32);
     if (M <= 32 && smem <= kFragBlockSmemMax) {
-        auto kern = (M == 1) ? fragment_block_kernel<R, true> : fragment_block_kernel<R, false>;
+        auto kern = M == 1   ? fragment_block_kernel<R, 1>
+                    : M == 2 ? fragment_block_kernel<R, 2>
+                    : M == 3 ? fragment_block_kernel<R, 3>
+                             : fragment_block_kernel<R, 0>;
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
                                              (int)cudaSharedmemCarveoutMaxShared);
         if (e == cudaSuccess && smem > 48 * 1024)
