@@ -345,9 +345,13 @@ __global__ void __launch_bounds__(kElemThreads)
 // warps), forms their terms, adds them per v in increasing k and over each warp, and sends the
 // warp sums to every CTA; each then takes the accept test itself.  The s elements on either
 // side of a run are proposed again here; their gradients come from the CTA that owns them.
-// One cluster barrier per update, during which the next normals and log u are drawn.
-// 100 updates of one path of 1024 steps: 918 us with ho_loop_kernel, 360 us (3.6 us an update,
-// about a third of it the barrier's round trip, the rest FP64 latency).
+// One cluster barrier per update, during which the next normals are drawn; log u of kLuBatch
+// updates at a time, and the accept test without its two divisions where they cannot decide it.
+// 100 updates of one path of 1024 steps: 918 us with ho_loop_kernel, 318 us here (3.2 us an
+// update, about a third of it the barrier's round trip, the rest FP64 latency; 360 us with
+// log u per update and the divisions in every test).
+constexpr int kLuBatch = 64;
+
 struct HoCluster {
     int cs, vw, K, s;  // CTAs, warps of the sum order per CTA, runs per CTA, elements per slice
     __host__ __device__ int run() const { return 32 * vw; }
@@ -375,7 +379,7 @@ __global__ void __launch_bounds__(1024)
 {
     extern __shared__ __align__(16) double smem_d[];
     __shared__ int s_acc;
-    __shared__ double s_lu[2];
+    __shared__ double s_lu[kLuBatch];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, NW = blockDim.x >> 5;
     const int cs = H.cs, s = H.s, RL = H.run(), K = H.K, own_n = H.own(), pitch = RL + 2 * s;
     unsigned rank;
@@ -407,17 +411,21 @@ __global__ void __launch_bounds__(1024)
         const float4 q = philox_normals4(M.seed, M.counter + (uint64_t)u, kStreamMala, (uint32_t)B.chain, (uint32_t)(e >> 2));
         return to_double(pick4(q, e & 3));
     };
-    auto draw_lu = [&](int u) {  // the last warp, one lane
-        if (tid == 32 * (NW - 1))
-            s_lu[u & 1] = log_u ? log_u[B.chain]
-                                : log(philox_uniform53(M.seed, M.counter + (uint64_t)u, kStreamAccept, (uint32_t)B.chain));
+    // log u of updates u .. u + kLuBatch - 1, one per thread: a double logarithm takes longer
+    // than the barrier's round trip
+    auto draw_lu = [&](int u) {
+        for (int q = tid; q < kLuBatch && u + q < update0 + n_updates; q += blockDim.x)
+            s_lu[q] = log_u ? log_u[B.chain]
+                            : log(philox_uniform53(M.seed, M.counter + (uint64_t)(u + q), kStreamAccept,
+                                                   (uint32_t)B.chain));
     };
+    const double h4 = 4.0 * hh, h4_inv = 1.0 / h4;
     double z = normal(update0);
-    draw_lu(update0);
     if (own || halo) XP[xi] = 0.0;
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
     for (int u = update0; u < update0 + n_updates; ++u) {
-        const int par = u & 1;
+        const int par = u & 1, lu_at = (u - update0) % kLuBatch;
+        if (lu_at == 0) draw_lu(u);
         const double xp = moves ? x + fma_r(-hh, g, s2h * z) : x;
         if (in) XP[xi] = xp;
         __syncthreads();
@@ -462,7 +470,6 @@ __global__ void __launch_bounds__(1024)
         asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
         if (u + 1 < update0 + n_updates) {
             z = normal(u + 1);
-            draw_lu(u + 1);
         }
         asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
         if (warp == 0) {
@@ -471,13 +478,19 @@ __global__ void __launch_bounds__(1024)
             v += __shfl_xor_sync(0xffffffffu, v, 4);
             v += __shfl_xor_sync(0xffffffffu, v, 2);
             v += __shfl_xor_sync(0xffffffffu, v, 1);
-            const double S_new = v * S_scale, part = v / (4.0 * hh);  // lanes 0; 8 and 16
-            const double qf4 = __shfl_sync(0xffffffffu, part, 8), qr4 = __shfl_sync(0xffffffffu, part, 16);
+            const double S_new = v * S_scale;  // lane 0; the others below in lanes 8 and 16
+            const double qf = __shfl_sync(0xffffffffu, v, 8), qr = __shfl_sync(0xffffffffu, v, 16);
             if (lane == 0) {
                 if (rank == 0 && !isfinite(v)) atomicExch(err, PAMD_ERR_NONFINITE);
-                const double la = (S_cur - S_new) - qr4 + qf4;
-                const int acc = s_lu[par] < la ? 1 : 0;  // NaN log alpha never accepts
-                if (log_alpha && rank == 0 && u == update0 + n_updates - 1) log_alpha[B.chain] = la;
+                // log alpha with the reciprocal of 4 h: within a few ulp of its largest term, so
+                // the comparison is that of the divided form unless the two sides are that close
+                // (two double divisions are most of this step otherwise)
+                const double lu = s_lu[lu_at], a1 = qr * h4_inv, a2 = qf * h4_inv, dS = S_cur - S_new;
+                double la = dS - a1 + a2;
+                const bool last = u == update0 + n_updates - 1;
+                if ((last && log_alpha) || !(fabs(lu - la) > 1e-12 * (fabs(dS) + a1 + a2))) la = dS - qr / h4 + qf / h4;
+                const int acc = lu < la ? 1 : 0;  // NaN log alpha never accepts
+                if (log_alpha && rank == 0 && last) log_alpha[B.chain] = la;
                 if (acc) S_cur = S_new;
                 n_acc += acc;
                 s_acc = acc;

@@ -58,3 +58,31 @@ def test_update_equals_its_pieces(pamd, shape, precision):
         assert torch.equal(a, b)
     for q in range(len(shape)):
         assert torch.equal(prob.view(g, q), prob.view(g1, q))
+
+
+@pytest.mark.parametrize("n,first", [(64, 1), (65, 64), (130, 63)])
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+def test_updates_of_one_call_equal_those_of_two(pamd, precision, n, first):
+    """Calls longer than one batch of uniforms."""
+    dt = 0.02
+    prob = pamd.Problem([pamd.System("harmonic", 1, 1, 600, 3, k=0.8)], 0.9, 1.1, dt, precision)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(n)
+    pos = prob.empty("cuda")
+    v = prob.view(pos, 0)
+    v.copy_((torch.randn(v.shape, generator=gen, device="cuda") * (2 * 0.9 * dt) ** 0.5).cumsum(1))
+    h = 0.9 * dt * 600 ** (-1.0 / 3.0)
+    S, g = pamd.action_grad(prob, pos)
+    out = []
+    for parts in ([n], [first, n - first]):
+        p1, g1, S1 = pos.clone(), g.clone(), S.clone()
+        nacc = torch.zeros(prob.n_chains, dtype=torch.int32, device="cuda")
+        la = torch.zeros(prob.n_chains, dtype=torch.float64, device="cuda")
+        at = 7
+        for m in parts:
+            pamd.path_update(prob, p1, g1, S1, h, m, seed=5, counter=at, n_accepted=nacc, log_alpha=la)
+            at += m
+        out.append((p1, prob.view(g1, 0).clone(), S1, nacc, la))
+    for a, b in zip(*out):
+        assert torch.equal(a, b)
+    assert 0 < int(out[0][3].min()) and int(out[0][3].max()) < n
