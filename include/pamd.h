@@ -70,8 +70,8 @@ extern "C" {
 #define PAMD_ERR_ARG (-1)          /* invalid argument or shape */
 #define PAMD_ERR_UNSUPPORTED (-2)  /* valid, but outside what the kernels handle */
 #define PAMD_ERR_CUDA (-3)         /* a CUDA runtime call or launch failed */
-#define PAMD_ERR_TIMEOUT (-4)      /* a bounded device wait ran out (reserved: no kernel of
-                                      this library waits on another, so no call returns it) */
+#define PAMD_ERR_TIMEOUT (-4)      /* a bounded device wait ran out: a CTA of a cluster
+                                      waited two seconds for the other CTAs of its chain */
 #define PAMD_ERR_NONFINITE (-5)    /* a non-finite action was produced */
 #define PAMD_ERR_ALLOC (-6)        /* workspace allocation failed */
 
@@ -379,7 +379,7 @@ int pamd_normals(uint64_t seed, uint64_t counter, uint32_t stream_id, uint32_t c
 /* Status left on the device by earlier asynchronous calls: synchronises
  * `stream`, then returns PAMD_ERR_NONFINITE (and clears it) if an action
  * computed since the last check was not finite (overlapping particles, an
- * exploding path), else PAMD_OK. */
+ * exploding path), PAMD_ERR_TIMEOUT if a bounded wait ran out, else PAMD_OK. */
 int pamd_device_status(void* stream);
 
 /* Launch-shape override for the Lennard-Jones kernels (0 or a negative skin

@@ -11,15 +11,16 @@
 //     and Box-Muller on the chain.
 //   * A chain is stepped by a cluster of CTAs (up to 8).  Each CTA holds all positions
 //     and moves N / CS particles, up to 32 lanes to a particle; the new coordinates go to
-//     every CTA's shared memory, and one cluster barrier ends the step.
+//     every CTA's shared memory as asynchronous stores counted by a transaction barrier there.
+//     A step costs one trip between SMs; with plain remote stores and a cluster barrier it
+//     also waited for their acknowledgement (N = 108: 1.33 against 0.96 us a step).
 //   * Small systems (N <= kEulerDense) evaluate every pair: no list, no displacement check,
 //     two candidates per packed f32x2 operation.  Larger ones walk Verlet lists of radius
 //     rc + skin, rebuilt when some particle has moved skin / 2 (a list that overflows scans
 //     all candidates).
 // N = 108, four chains of 1024 steps: 4.89 ms (4.8 us a step) with one CTA of four threads
-// per particle and the normals in the step, 1.36 ms (1.33 us) now (1.66 us a step before the
-// lane count and the packed constants of the all-pairs form were known to the compiler); a
-// step of N = 500, eight chains, 17.5 -> 3.6 us, of N = 108 in double precision 101 -> 23 us.
+// per particle and the normals in the step, 0.98 ms (0.96 us) now; a step of N = 500, eight
+// chains, 17.5 -> 3.5 us, of N = 108 in double precision 101 -> 23 us.
 #include <algorithm>
 #include <cmath>
 #include <type_traits>
@@ -31,6 +32,12 @@ namespace pamd {
 namespace {
 
 constexpr int kEulerDense = 192;   // largest N without lists
+// Up to this size a particle has eight lanes, each adding its candidates in increasing j, and
+// double precision takes the library's 1/sqrt: the arithmetic of the LJ kernels' plain form,
+// bit for bit.  Small boxes are where a start can overlap (33 to 45 particles on a lattice of
+// 108 sites), and such a path turns any other order of the sums into another path.
+constexpr int kEulerOrdered = 64;
+constexpr int kOrderedLg = 3;
 
 __device__ __forceinline__ unsigned cluster_rank()
 {
@@ -42,25 +49,61 @@ __device__ __forceinline__ void cluster_barrier()
 {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-__device__ __forceinline__ void step_barrier(int cs)
+// The new positions travel as asynchronous stores that a transaction barrier of the receiving
+// CTA counts: nobody waits for an acknowledgement, and a CTA goes on as soon as the bytes of
+// its own copy are there.
+struct StepBarriers {
+    uint64_t bar[2];  // of the two slices
+};
+__device__ __forceinline__ unsigned shared_addr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ unsigned remote_addr(unsigned a, unsigned rank)
 {
-    if (cs > 1)
-        cluster_barrier();
-    else
-        __syncthreads();
-}
-// Store to the same shared-memory address in CTA `rank` of the cluster.
-__device__ __forceinline__ void store_remote(float* p, unsigned rank, float v)
-{
-    unsigned a = (unsigned)__cvta_generic_to_shared(p), r;
+    unsigned r;
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
-    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(r), "f"(v) : "memory");
+    return r;
 }
-__device__ __forceinline__ void store_remote(double* p, unsigned rank, double v)
+__device__ __forceinline__ void send_async(unsigned to, float v, unsigned bar)
 {
-    unsigned a = (unsigned)__cvta_generic_to_shared(p), r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
-    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(r), "d"(v) : "memory");
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(to),
+                 "r"(__float_as_uint(v)), "r"(bar)
+                 : "memory");
+}
+__device__ __forceinline__ void send_async(unsigned to, double v, unsigned bar)
+{
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(to),
+                 "l"(__double_as_longlong(v)), "r"(bar)
+                 : "memory");
+}
+// One phase of a barrier: `bytes` of asynchronous stores, and this call.
+__device__ __forceinline__ void expect(unsigned bar, unsigned bytes)
+{
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ bool phase_done(unsigned bar, unsigned parity)
+{
+    unsigned done;
+    asm volatile("{\n\t.reg .pred p;\n\t"
+                 "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+                 "selp.u32 %0, 1, 0, p;\n\t}"
+                 : "=r"(done)
+                 : "r"(bar), "r"(parity)
+                 : "memory");
+    return done != 0;
+}
+__device__ __forceinline__ unsigned long long now_ns()
+{
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    return t;
+}
+// Waits for the phase of the given parity; false when it did not complete within two seconds.
+__device__ __forceinline__ bool wait_phase(unsigned bar, unsigned parity)
+{
+    if (phase_done(bar, parity)) return true;
+    const unsigned long long end = now_ns() + 2000000000ull;
+    while (!phase_done(bar, parity))
+        if (now_ns() > end) return false;
+    return true;
 }
 
 // The normals of every element of slices 1..T of a system's chains, into the path.
@@ -129,9 +172,15 @@ struct DenseForce {
         const float2 ri = pk(inv_sqrt(r2.x), inv_sqrt(r2.y)), ir2 = mul2(ri, ri);
         const float2 ir6 = mul2(mul2(ir2, ir2), ir2), u = mul2(c1, ir6), t = fma2(c2, ir6, m1);
         const float2 fs = fma2(mul2(u, t), ir2, mul2(duc, ri));
-        fx = fma2(fs, dx, fx);
-        fy = fma2(fs, dy, fy);
-        fz = fma2(fs, dz, fz);
+        if (LG == kOrderedLg) {  // one sum, in increasing j
+            fx.x = fma_r(fs.y, dx.y, fma_r(fs.x, dx.x, fx.x));
+            fy.x = fma_r(fs.y, dy.y, fma_r(fs.x, dy.x, fy.x));
+            fz.x = fma_r(fs.y, dz.y, fma_r(fs.x, dz.x, fz.x));
+        } else {
+            fx = fma2(fs, dx, fx);
+            fy = fma2(fs, dy, fy);
+            fz = fma2(fs, dz, fz);
+        }
     }
     // p: the slice; lane q's candidates 2m, 2m + 1 are the float2 at m 2^LG + q
     __device__ __forceinline__ void operator()(const float* p, const float (&xi)[3], float (&f)[3]) const
@@ -160,9 +209,11 @@ struct EulerShape {
 // LG: log2 of the lanes per particle where it is known (the all-pairs form), else -1.
 template <typename R, bool LIST, int LG, int MAXT>
 __global__ void __launch_bounds__(MAXT)
-    lj_euler_kernel(R* __restrict__ pos, const R* __restrict__ noise, const LJSysDev<R> S, const EulerShape H)
+    lj_euler_kernel(R* __restrict__ pos, const R* __restrict__ noise, const LJSysDev<R> S, const EulerShape H,
+                    int* __restrict__ err)
 {
     extern __shared__ __align__(32) unsigned char smem_raw[];
+    __shared__ __align__(8) StepBarriers sync;
     const int N = S.N, T = S.T, s = 3 * N, tid = threadIdx.x, NT = blockDim.x;
     const int lg = LG >= 0 ? LG : H.lg, tpp = 1 << lg, q = tid & (tpp - 1), cs = H.cs, npad = H.npad;
     const unsigned rank = cs > 1 ? cluster_rank() : 0u;
@@ -223,7 +274,28 @@ __global__ void __launch_bounds__(MAXT)
     };
     load_zs(true, z[0]);
     load_zs(T > 1, z[1]);
-    step_barrier(cs);  // (also: every lane holds its first normals before slice 1 is written)
+    // Slice t + 1 goes to the buffer that slice t - 1 was in.  A particle's slice t + 1 is sent
+    // after every slice t has arrived, so after every CTA is done with slice t - 1 (its own
+    // particles' slice t followed from it); the last lanes to read it are those that send.
+    // A barrier is armed for slice t + 2 when slice t has arrived on it.
+    const unsigned bar0 = shared_addr(&sync.bar[0]), bytes = (unsigned)(3 * N * sizeof(R));
+    // A warp without particles does not wait, or it could fall two phases behind (with lists
+    // the displacement check keeps all warps together).
+    const bool waits = LIST || tid < 32 || __any_sync(0xffffffffu, active);
+    bool lost = false;
+    if (cs > 1 && tid == 0) {
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n\tmbarrier.init.shared::cta.b64 [%1], 1;\n\t"
+                     "fence.mbarrier_init.release.cluster;" ::"r"(bar0),
+                     "r"(bar0 + 8)
+                     : "memory");
+        expect(bar0 + 8, bytes);             // slice 1
+        if (T > 1) expect(bar0, bytes);      // slice 2
+    }
+    if (cs > 1)
+        cluster_barrier();
+    else
+        __syncthreads();
+    // (also: every lane holds its first normals before slice 1 is written)
     const DenseForce<LG >= 0 ? LG : 0> dense(dense_consts(k), N, npad, i, q);
     // Step t from buffer PAR to the other; zt: its normals.  The slice that the step before
     // made is stored here: a store directly before the barrier would hold it up (the
@@ -237,6 +309,7 @@ __global__ void __launch_bounds__(MAXT)
                 if (c < nc) xp[c * N] = last[c];
         }
         xp += s;
+        if (cs > 1 && tid == 0 && t > 0 && t + 2 <= T) expect(bar0 + 8 * PAR, bytes);
         load_zs(t + 2 < T, z2);
         if (LIST) {
             bool moved = t == 0;
@@ -253,7 +326,19 @@ __global__ void __launch_bounds__(MAXT)
         if (active) {
 #pragma unroll
             for (int c = 0; c < 3; ++c) xi[c] = A.p[oi + c * npad];
-            if constexpr (LG >= 0) {
+            if constexpr (sizeof(R) == 8 && LG == kOrderedLg) {
+                for (int j = q; j < N; j += tpp)
+                    if (j != i) {
+                        R dx, dy, dz;
+                        const R r2 = pair_r2<R>(xi[0], xi[1], xi[2], *A.at(j, 0), *A.at(j, 1), *A.at(j, 2), k, dx, dy, dz);
+                        if (!(r2 <= k.rc2)) continue;
+                        const R ri = rsqrt(r2), ir2 = ri * ri, ir6 = ir2 * ir2 * ir2, u = k.c1 * ir6;
+                        const R fs = fma_r(u * fma_r(k.c2, ir6, R(-1)), ir2, k.duc * ri);
+                        f[0] = fma_r(fs, dx, f[0]);
+                        f[1] = fma_r(fs, dy, f[1]);
+                        f[2] = fma_r(fs, dz, f[2]);
+                    }
+            } else if constexpr (LG >= 0) {
                 dense(A.p, xi, f);
             } else if (LIST && !ovf) {
 #pragma unroll 2
@@ -278,7 +363,9 @@ __global__ void __launch_bounds__(MAXT)
             if (cs == 1) {
                 if (owner) *w = xn;
             } else {
-                for (int d = first; d < cs; d += stride) store_remote(w, (unsigned)d, xn);
+                const unsigned to = shared_addr(w), bar = bar0 + 8 * (1 - PAR);
+                for (int d = first; d < cs; d += stride)
+                    send_async(remote_addr(to, (unsigned)d), xn, remote_addr(bar, (unsigned)d));
             }
         };
         if (mover) {
@@ -289,7 +376,10 @@ __global__ void __launch_bounds__(MAXT)
                 for (int c = 0; c < 3; ++c) move(c, xi[c], f[c], zt[c]);
             }
         }
-        step_barrier(cs);
+        if (cs == 1)
+            __syncthreads();
+        else if (waits && !lost)
+            lost = !wait_phase(bar0 + 8 * (1 - PAR), (unsigned)(t >> 1) & 1u);
     };
     using P0 = std::integral_constant<int, 0>;
     using P1 = std::integral_constant<int, 1>;
@@ -304,19 +394,23 @@ __global__ void __launch_bounds__(MAXT)
         for (int c = 0; c < NC; ++c)
             if (c < nc) xp[c * N] = last[c];
     }
+    if (cs > 1) {
+        if (lost) atomicExch(err, PAMD_ERR_TIMEOUT);
+        cluster_barrier();  // (no CTA ends while a store to it may be on its way)
+    }
 }
 
 // Cluster size, lanes per particle and block size.
-// A cluster barrier costs about 0.55 us (its release waits for the remote stores), so single
-// precision takes clusters where a step's pairs cost more than that (N = 32: 0.82 us a step
-// with one CTA, 1.38 with two; N = 108: 2.7, 2.1, 1.8 with one, two, four; all before the
-// lane count was a template argument), down to
-// kEulerMinLocal particles per CTA; double precision, bound by the FP64 pipe, almost always
-// (N = 108: 110, 63, 31 us with one, two, four).  Chains beyond the SMs get no cluster.
+// us a step, four chains, with 1, 2, 4, 8 CTAs a chain: N = 32 0.60, 0.70, 0.72, 0.72; N = 48
+// 0.78, 0.83, 0.78, 0.79; N = 56 1.05, 0.92, 0.85, 0.85; N = 108 2.4, 1.6, 1.2, 0.98; N = 500
+// 13, 7.7, 4.7, 3.5.  So single precision takes clusters from kEulerClusterN particles on, of
+// as many CTAs as the chains leave.  Double precision, bound by the FP64 pipe, takes them down
+// to four particles each (N = 32: 10.6, 5.9, 5.4, 5.4; N = 64: 39, 20, 10.5, 9.6; N = 108: 110,
+// 63, 31, 23).  Chains beyond the SMs get no cluster.
 // Lanes per particle: about 512 threads (more lanes add shuffles and overhead: N = 108 on four
-// CTAs 1.92 us with 864 threads, 1.78 with 432), up to 1024 where that keeps four lanes.
-constexpr int kEulerClusterN = 80;
-constexpr int kEulerMinLocal = 13;
+// CTAs took 1.92 us with 864 threads, 1.78 with 432), up to 1024 where that keeps four lanes.
+constexpr int kEulerClusterN = 50;
+constexpr int kEulerMinLocal = 6;
 constexpr int kEulerMinLocalDouble = 4;
 
 template <typename R>
@@ -329,7 +423,10 @@ EulerShape euler_shape(int N, int n_chains, double list_volume, int sms, int max
     while (h.cs < 8 && (!F32 || N >= kEulerClusterN) && N >= 2 * h.cs * local && 2LL * h.cs * n_chains <= sms) h.cs *= 2;
     h.nloc = (N + h.cs - 1) / h.cs;
     h.lg = 0;
-    while (h.lg < 5 && (h.nloc << (h.lg + 1)) <= (h.lg < 2 ? 1024 : 512)) ++h.lg;
+    if (N <= kEulerOrdered)
+        h.lg = kOrderedLg;
+    else
+        while (h.lg < 5 && (h.nloc << (h.lg + 1)) <= (h.lg < 2 ? 1024 : 512)) ++h.lg;
     h.nt = std::max(64, ((h.nloc << h.lg) + 31) / 32 * 32);
     const int tpp = 1 << h.lg;
     const bool list = N > kEulerDense;
@@ -348,7 +445,7 @@ EulerShape euler_shape(int N, int n_chains, double list_volume, int sms, int max
 
 template <typename R>
 cudaError_t launch_lj_euler(R* pos, const R* noise, const void* sys_entry_host, int n_chains, int chain0,
-                            uint64_t seed, uint64_t counter, cudaStream_t st)
+                            uint64_t seed, uint64_t counter, int* err, cudaStream_t st)
 {
     const LJSysDev<R> S = *static_cast<const LJSysDev<R>*>(sys_entry_host);
     if (n_chains <= 0 || S.T <= 0) return cudaSuccess;
@@ -366,11 +463,13 @@ cudaError_t launch_lj_euler(R* pos, const R* noise, const void* sys_entry_host, 
     const double rl2 = (double)S.k.rl2, L = (double)S.k.L;
     const EulerShape h = euler_shape<R>(S.N, n_chains, 4.18879020478639 * rl2 * std::sqrt(rl2) * S.N / (L * L * L), sms,
                                         max_smem - 1024);
-    void (*kern)(R*, const R*, LJSysDev<R>, EulerShape);
+    void (*kern)(R*, const R*, LJSysDev<R>, EulerShape, int*);
     if (S.N > kEulerDense)
         kern = h.nt <= 512 ? lj_euler_kernel<R, true, -1, 512> : lj_euler_kernel<R, true, -1, 1024>;
     else if constexpr (sizeof(R) == 8)
-        kern = h.nt <= 512 ? lj_euler_kernel<R, false, -1, 512> : lj_euler_kernel<R, false, -1, 1024>;
+        kern = h.lg == kOrderedLg && S.N <= kEulerOrdered ? lj_euler_kernel<R, false, kOrderedLg, 512>
+               : h.nt <= 512                                  ? lj_euler_kernel<R, false, -1, 512>
+                                                              : lj_euler_kernel<R, false, -1, 1024>;
     else  // N <= kEulerDense: at least four lanes
         kern = h.lg == 5   ? lj_euler_kernel<R, false, 5, 512>
                : h.lg == 4 ? lj_euler_kernel<R, false, 4, 512>
@@ -391,12 +490,12 @@ cudaError_t launch_lj_euler(R* pos, const R* noise, const void* sys_entry_host, 
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = h.cs > 1 ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kern, pos, noise, S, h);
+    return cudaLaunchKernelEx(&cfg, kern, pos, noise, S, h, err);
 }
 
-template cudaError_t launch_lj_euler<float>(float*, const float*, const void*, int, int, uint64_t, uint64_t,
+template cudaError_t launch_lj_euler<float>(float*, const float*, const void*, int, int, uint64_t, uint64_t, int*,
                                             cudaStream_t);
-template cudaError_t launch_lj_euler<double>(double*, const double*, const void*, int, int, uint64_t, uint64_t,
+template cudaError_t launch_lj_euler<double>(double*, const double*, const void*, int, int, uint64_t, uint64_t, int*,
                                              cudaStream_t);
 
 PAMD_DEBUG_FETCHER(lj_euler)

@@ -1647,10 +1647,10 @@ int pamd_euler_reference(const pamd_problem* prob, void* pos, uint64_t seed, uin
             const void* row = &P->h_lj_sys[P->lj_sys_stride * si.lj_index];
             if (P->fp64)
                 PAMD_CUDA_TRY(launch_lj_euler<double>((double*)dpos, (const double*)dnoise, row, si.chains,
-                                                      si.chain0, seed, counter, st));
+                                                      si.chain0, seed, counter, P->d_err, st));
             else
                 PAMD_CUDA_TRY(launch_lj_euler<float>((float*)dpos, (const float*)dnoise, row, si.chains, si.chain0,
-                                                     seed, counter, st));
+                                                     seed, counter, P->d_err, st));
         }
     }
     if (host) {

@@ -513,7 +513,7 @@ cudaError_t launch_ho_euler(R* pos, const R* noise, int s, int T, int n_chains, 
                             uint64_t counter, cudaStream_t st);
 template <typename R>
 cudaError_t launch_lj_euler(R* pos, const R* noise, const void* sys_entry_host, int n_chains, int chain0,
-                            uint64_t seed, uint64_t counter, cudaStream_t st);
+                            uint64_t seed, uint64_t counter, int* err, cudaStream_t st);
 
 // Deterministic per-chain sums of partials: out[c] = scale * sum(partials[slots[c]]);
 // a non-finite sum sets *err (if given) to PAMD_ERR_NONFINITE.

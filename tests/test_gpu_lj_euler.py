@@ -25,7 +25,9 @@ def pamd():
 @pytest.mark.parametrize("precision", ["fp32", "fp64"])
 @pytest.mark.parametrize("N,B,L,T", [(2, 1, 6.0, 12), (3, 200, 6.0, 3), (31, 3, 0, 12), (33, 1, 0, 12), (65, 160, 0, 3),
                                      (108, 4, 0, 12), (129, 2, 0, 12), (192, 1, 0, 12), (193, 1, 0, 12),
-                                     (257, 80, 0, 3), (500, 2, 0, 12), (1024, 1, 0, 6), (250, 1, 40.0, 6)])
+                                     (257, 80, 0, 3), (500, 2, 0, 12), (1024, 1, 0, 6), (250, 1, 40.0, 6),
+                                     (40, 3, 0, 12), (49, 1, 0, 12), (50, 1, 0, 12), (57, 1, 0, 12),
+                                     (64, 40, 0, 6)])
 def test_paths_match_the_oracle(pamd, precision, N, B, L, T):
     D, beta, dt = 0.9, 1.1, 1e-4
     # the box of the whole FCC lattice that the particles occupy at density 0.85 (a partly
@@ -68,3 +70,18 @@ def test_drawn_normals_equal_given_ones(pamd, N):
     pamd.euler_reference(prob, b, noise=nbuf)
     torch.cuda.synchronize()
     assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("N", [57, 108, 200])
+def test_long_paths_repeat(pamd, N):
+    """Thousands of barrier phases, a cluster with an empty CTA among them: the same path
+    in two calls, and no wait that ran out."""
+    T, B, L = 3000, 5, inputs.box_side(256, 0.85)
+    prob = pamd.Problem([pamd.System("lj", N, 3, T, B, box=L, rc=2.5)], 1.0, 1.0, 1e-4)
+    a = prob.empty("cuda")
+    prob.view(a, 0)[:, 0].copy_(torch.from_numpy(inputs.fcc_lattice(256, L)[:, :N].copy()))
+    b = a.clone()
+    pamd.euler_reference(prob, a, seed=1, counter=2)
+    pamd.euler_reference(prob, b, seed=1, counter=2)
+    pamd.device_status()
+    assert torch.equal(a, b) and bool(torch.isfinite(prob.view(a, 0)).all())
