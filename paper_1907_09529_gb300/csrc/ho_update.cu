@@ -19,6 +19,7 @@
 // normals are most of its instructions), ho_commit_kernel memory; ho_loop_kernel the
 // latency of one update's chain of proposal, residuals, block sums and accept test, and in
 // double precision the FP64 pipe of one SM (14 instructions per element at 16 clocks a warp).
+#include "cluster.cuh"
 #include "elem.cuh"
 
 namespace pamd {
@@ -345,11 +346,13 @@ __global__ void __launch_bounds__(kElemThreads)
 // warps), forms their terms, adds them per v in increasing k and over each warp, and sends the
 // warp sums to every CTA; each then takes the accept test itself.  The s elements on either
 // side of a run are proposed again here; their gradients come from the CTA that owns them.
-// One cluster barrier per update, during which the next normals are drawn; log u of kLuBatch
+// One exchange per update, during which the next normals are drawn; log u of kLuBatch
 // updates at a time, and the accept test without its two divisions where they cannot decide it.
-// 100 updates of one path of 1024 steps: 918 us with ho_loop_kernel, 318 us here (3.2 us an
-// update, about a third of it the barrier's round trip, the rest FP64 latency; 360 us with
-// log u per update and the divisions in every test).
+// 100 updates of one path of 1024 steps: 918 us with ho_loop_kernel, 308 us here (360 us with
+// log u per update, the divisions in every test, and a cluster barrier).  Of an update's 5900
+// cycles about 700 go to the trial positions, 1300 to gradients and terms, 1650 to the warp sums
+// (five dependent FP64 additions), 1100 to the exchange (the normals within it), 1500 to the
+// eight-warp sums and the test: FP64 latency throughout.
 constexpr int kLuBatch = 64;
 
 struct HoCluster {
@@ -364,13 +367,6 @@ struct HoCluster {
     }
 };
 
-__device__ __forceinline__ void send(double* p, unsigned rank, double v)
-{
-    unsigned a = (unsigned)__cvta_generic_to_shared(p), r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
-    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(r), "d"(v) : "memory");
-}
-
 __global__ void __launch_bounds__(1024)
     ho_cluster_kernel(const ElemBlock* __restrict__ blocks, double* __restrict__ pos, double* __restrict__ grad,
                       double* __restrict__ Sv, const MalaDev* __restrict__ md, int update0, int n_updates, double a,
@@ -380,10 +376,10 @@ __global__ void __launch_bounds__(1024)
     extern __shared__ __align__(16) double smem_d[];
     __shared__ int s_acc;
     __shared__ double s_lu[kLuBatch];
+    __shared__ __align__(8) uint64_t s_bar[2];  // of even and odd updates
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, NW = blockDim.x >> 5;
     const int cs = H.cs, s = H.s, RL = H.run(), K = H.K, own_n = H.own(), pitch = RL + 2 * s;
-    unsigned rank;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+    const unsigned rank = cluster_rank();
     const ElemBlock B = blocks[blockIdx.x / cs];
     const MalaDev M = *md;
     PAMD_ARR(double, XP, smem_d, K * pitch);
@@ -422,9 +418,25 @@ __global__ void __launch_bounds__(1024)
     const double h4 = 4.0 * hh, h4_inv = 1.0 / h4;
     double z = normal(update0);
     if (own || halo) XP[xi] = 0.0;
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    // Received per update: 24 warp sums and the gradients of this CTA's halo elements.  Those of
+    // update n + 2 replace those of update n: they are sent after the sums of update n + 1 have
+    // come from every CTA, so after every thread of every CTA is done with update n.
+    const unsigned bar0 = shared_addr(s_bar), bytes = 8u * (24u + (unsigned)__syncthreads_count(halo && in));
+    bool lost = false;
+    if (tid == 0) {
+        barrier_init(bar0);
+        barrier_init(bar0 + 8);
+        barrier_init_done();
+        expect(bar0, bytes);
+        if (n_updates > 1) expect(bar0 + 8, bytes);
+    }
+    cluster_barrier();
     for (int u = update0; u < update0 + n_updates; ++u) {
-        const int par = u & 1, lu_at = (u - update0) % kLuBatch;
+        const int n = u - update0, par = n & 1, lu_at = n % kLuBatch;
+        const unsigned bar = bar0 + 8 * par;
+        auto send = [&](double* p, unsigned to, double v) {
+            send_async(remote_addr(shared_addr(p), to), v, remote_addr(bar, to));
+        };
         if (lu_at == 0) draw_lu(u);
         const double xp = moves ? x + fma_r(-hh, g, s2h * z) : x;
         if (in) XP[xi] = xp;
@@ -467,11 +479,10 @@ __global__ void __launch_bounds__(1024)
             acc = warp_sum(acc);
             if (lane < cs) send(VS + 24 * par + 8 * t + (int)rank * H.vw + w, (unsigned)lane, acc);
         }
-        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-        if (u + 1 < update0 + n_updates) {
-            z = normal(u + 1);
-        }
-        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        if (n + 1 < n_updates) z = normal(u + 1);
+        asm volatile("" : "+d"(z));  // (here, not after the wait)
+        if (!lost) lost = !wait_phase(bar, (unsigned)(n >> 1) & 1u);
+        if (tid == 32 * (NW - 1) && n + 2 < n_updates) expect(bar, bytes);  // (not by the accept test's warp: 1.3 us an update)
         if (warp == 0) {
             // lanes 8 t + w: sum t of warp w
             double v = lane < 24 ? VS[24 * par + lane] : 0.0;
@@ -510,6 +521,8 @@ __global__ void __launch_bounds__(1024)
         Sv[B.chain] = S_cur;
         if (n_accepted) n_accepted[B.chain] += n_acc;
     }
+    if (lost) atomicExch(err, PAMD_ERR_TIMEOUT);
+    cluster_barrier();  // (no CTA ends while a store to it may be on its way)
 }
 
 // The cluster shape for chains of n elements, s to a slice: as many CTAs per chain (up to 8)

@@ -25,6 +25,7 @@
 #include <cmath>
 #include <type_traits>
 
+#include "cluster.cuh"
 #include "lj_math.cuh"
 
 namespace pamd {
@@ -38,73 +39,6 @@ constexpr int kEulerDense = 192;   // largest N without lists
 // 108 sites), and such a path turns any other order of the sums into another path.
 constexpr int kEulerOrdered = 64;
 constexpr int kOrderedLg = 3;
-
-__device__ __forceinline__ unsigned cluster_rank()
-{
-    unsigned r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ void cluster_barrier()
-{
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-// The new positions travel as asynchronous stores that a transaction barrier of the receiving
-// CTA counts: nobody waits for an acknowledgement, and a CTA goes on as soon as the bytes of
-// its own copy are there.
-struct StepBarriers {
-    uint64_t bar[2];  // of the two slices
-};
-__device__ __forceinline__ unsigned shared_addr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ unsigned remote_addr(unsigned a, unsigned rank)
-{
-    unsigned r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
-    return r;
-}
-__device__ __forceinline__ void send_async(unsigned to, float v, unsigned bar)
-{
-    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(to),
-                 "r"(__float_as_uint(v)), "r"(bar)
-                 : "memory");
-}
-__device__ __forceinline__ void send_async(unsigned to, double v, unsigned bar)
-{
-    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(to),
-                 "l"(__double_as_longlong(v)), "r"(bar)
-                 : "memory");
-}
-// One phase of a barrier: `bytes` of asynchronous stores, and this call.
-__device__ __forceinline__ void expect(unsigned bar, unsigned bytes)
-{
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ bool phase_done(unsigned bar, unsigned parity)
-{
-    unsigned done;
-    asm volatile("{\n\t.reg .pred p;\n\t"
-                 "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-                 "selp.u32 %0, 1, 0, p;\n\t}"
-                 : "=r"(done)
-                 : "r"(bar), "r"(parity)
-                 : "memory");
-    return done != 0;
-}
-__device__ __forceinline__ unsigned long long now_ns()
-{
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-// Waits for the phase of the given parity; false when it did not complete within two seconds.
-__device__ __forceinline__ bool wait_phase(unsigned bar, unsigned parity)
-{
-    if (phase_done(bar, parity)) return true;
-    const unsigned long long end = now_ns() + 2000000000ull;
-    while (!phase_done(bar, parity))
-        if (now_ns() > end) return false;
-    return true;
-}
 
 // The normals of every element of slices 1..T of a system's chains, into the path.
 template <typename R>
@@ -213,7 +147,7 @@ __global__ void __launch_bounds__(MAXT)
                     int* __restrict__ err)
 {
     extern __shared__ __align__(32) unsigned char smem_raw[];
-    __shared__ __align__(8) StepBarriers sync;
+    __shared__ __align__(8) uint64_t s_bar[2];  // of the two slices
     const int N = S.N, T = S.T, s = 3 * N, tid = threadIdx.x, NT = blockDim.x;
     const int lg = LG >= 0 ? LG : H.lg, tpp = 1 << lg, q = tid & (tpp - 1), cs = H.cs, npad = H.npad;
     const unsigned rank = cs > 1 ? cluster_rank() : 0u;
@@ -278,16 +212,15 @@ __global__ void __launch_bounds__(MAXT)
     // after every slice t has arrived, so after every CTA is done with slice t - 1 (its own
     // particles' slice t followed from it); the last lanes to read it are those that send.
     // A barrier is armed for slice t + 2 when slice t has arrived on it.
-    const unsigned bar0 = shared_addr(&sync.bar[0]), bytes = (unsigned)(3 * N * sizeof(R));
+    const unsigned bar0 = shared_addr(s_bar), bytes = (unsigned)(3 * N * sizeof(R));
     // A warp without particles does not wait, or it could fall two phases behind (with lists
     // the displacement check keeps all warps together).
     const bool waits = LIST || tid < 32 || __any_sync(0xffffffffu, active);
     bool lost = false;
     if (cs > 1 && tid == 0) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n\tmbarrier.init.shared::cta.b64 [%1], 1;\n\t"
-                     "fence.mbarrier_init.release.cluster;" ::"r"(bar0),
-                     "r"(bar0 + 8)
-                     : "memory");
+        barrier_init(bar0);
+        barrier_init(bar0 + 8);
+        barrier_init_done();
         expect(bar0 + 8, bytes);             // slice 1
         if (T > 1) expect(bar0, bytes);      // slice 2
     }
