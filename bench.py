@@ -136,8 +136,7 @@ class ClockSampler:
 
 #: Sources that define each profiled kernel (with the shared header).
 KERNEL_SOURCES = {
-    "lj_action_kernel": ("lj_kernels.cu", "pamd_internal.cuh"),
-    "lj_paired_kernel": ("lj_paired.cu", "pamd_internal.cuh"),
+    "lj_paired_kernel": ("lj_paired.cu", "lj_math.cuh", "pamd_internal.cuh"),
     "ho_vec_kernel": ("ho_kernels.cu", "pamd_internal.cuh"),
     "fragment_line_kernel": ("fragment_kernels.cu", "fragment.cuh", "pamd_internal.cuh"),
 }
@@ -430,17 +429,22 @@ def run_sampler(args, w, pamd, prob, dev, rank, world):
 
 
 def launches_per_update(prob):
-    """Kernels of one path update: propose, one action launch per harmonic system,
-    one LJ launch per block-size class (two when a single-precision batch mixes
-    N <= 512 and N > 512), finalize S, reverse, finalize q_fwd and q_rev, accept,
-    commit."""
+    """Kernels of one path update (pamd_path_update with n_updates = 1), without the one
+    that sets its parameters.  Harmonic batches: one launch per system when every chain is
+    one element block (4096 elements), else trial and commit per system and the sums with
+    the accept test.  Otherwise: propose, one action launch per harmonic system, one LJ
+    launch per block-size class (two when a single-precision batch mixes N <= 512 and
+    N > 512), reverse, the sums with the accept test, commit."""
     n_ho = sum(1 for s in prob.systems if s.kind == "harmonic")
     lj = [s.N for s in prob.systems if s.kind == "lj"]
+    if not lj and max(s.d * s.N for s in prob.systems) <= 64:
+        one_block = max((s.T + 1) * s.d * s.N for s in prob.systems) <= 4096
+        return n_ho if one_block else 2 * n_ho + 1
     n_lj = 0
     if lj:
         mixed = min(lj) <= 512 < max(lj) and prob.precision == "fp32"
         n_lj = 2 if mixed else 1
-    return 1 + n_ho + n_lj + 1 + 1 + 2 + 1 + 1
+    return 1 + n_ho + n_lj + 3
 
 
 def main():

@@ -331,13 +331,15 @@ int choose_lj_block(int nmax)
 }
 
 // Outer-list capacity per thread.  The lists reach rc + Delta_i + Delta_j with item-wide
-// margins; sized for about 2.5 times the spread of a 3D displacement over half an item (a
-// particle beyond that builds its window lists from every candidate).
+// margins; sized for about 2.5 times the spread of a 3D displacement over half an item and
+// twice the mean density (a particle beyond that builds its window lists from every candidate:
+// 515 particles on a lattice of 864 sites took 4 to 7 % longer with 1.2 times).  Only the
+// entries used are touched, so room costs nothing but memory.
 int lj_outer_cap(int N, const pamd_potential& pot, double sig_step, int tile_steps, int tpp)
 {
     const double dmax = 2.5 * sig_step * std::sqrt(3.0 * 0.5 * (tile_steps + 1));
     const double ro = pot.rc + 2.0 * dmax, rho = N / (pot.box * pot.box * pot.box);
-    int ow = (int)std::min(1.0e6, 1.2 * 4.18879020478639 * ro * ro * ro * rho) + 16;
+    int ow = (int)std::min(1.0e6, 2.0 * 4.18879020478639 * ro * ro * ro * rho) + 16;
     ow = std::min(ow, N - 1 + 2 * tpp);
     return std::max(2, std::min((ow + tpp - 1) / tpp, kMaxListPerThread)) & ~1;
 }
@@ -350,9 +352,10 @@ double lj_step_cost(int N, const LJTune& t)
     return 1.0 + t.list / t.tpp * (0.08 + 0.0067 * N * t.tpp / 32.0);
 }
 
-// What an item costs beyond its steps, in us: the pair before it, staging, the outer list
-// (28 us at N = 108, 77 at 500).
-double lj_item_cost(int N) { return 20.0 + 0.11 * N; }
+// What an item costs beyond its steps, in us: the step before it, staging, and the outer list
+// (N tests a particle).  13 us measured at N = 98, 15 at 173, 65 at 500; the constants are those
+// that split batches of unlike systems best (12 batches of 4 to 12 systems, N = 64..861).
+double lj_item_cost(int N, const LJTune& t) { return 15.0 + lj_step_cost(N, t) + 1.0e-4 * N * N; }
 
 // Per-system LJ launch shape: threads per particle (largest power of two <= 8
 // with N * tpp <= NT), Verlet skin (one-step kernel) or window length (paired
@@ -629,24 +632,25 @@ int build_plan(const pamd_problem* p, Plan** out)
             // steps, take 13.1 ms in items of 32 steps, 11.6 ms in items of 216), so items are as
             // long as the step limit allows: the fewest rounds r for which cutting every chain into
             // equal items of at most `limit` steps needs no more than r times the grid.  (Longer items also
-            // have longer outer lists; past 256 steps that costs more than it saves.)
+            // have longer outer lists; past 256 steps that costs more than it saves.)  Exceptions below.
             if (P->lj_paired && !one) {
                 const int limit = g_tune_override.tile_steps > 0 ? g_tune_override.tile_steps : 256;
                 for (int k = 0; k < (int)P->lj_cls.size(); ++k) {
                     const long long G = (long long)bg_cls[k] * sms;
                     std::vector<SysInfo*> in;
                     std::vector<double> cost;  // of one step
-                    double cmax = 0.0;
+                    double cmax = 0.0, cmin = 0.0;  // costs of a whole chain, of an item of one step
                     for (auto& si : P->sys)
                         if (si.kind == PAMD_LJ && si.lj_class == k) {
                             in.push_back(&si);
                             cost.push_back(lj_step_cost(si.N, si.tune));
-                            cmax = std::max(cmax, cost.back() * si.T + lj_item_cost(si.N));
+                            cmax = std::max(cmax, cost.back() * si.T + lj_item_cost(si.N, si.tune));
+                            cmin = std::max(cmin, cost.back() + lj_item_cost(si.N, si.tune));
                         }
                     // steps per item of system q at cost c, and the items all chains then need
                     auto tile = [&](size_t q, double c) {
                         const int own = in[q]->T - in[q]->halo_lo;
-                        const int most = std::max(1, std::min(limit, (int)std::min(2.0e9, (c - lj_item_cost(in[q]->N)) / cost[q])));
+                        const int most = std::max(1, std::min(limit, (int)std::min(2.0e9, (c - lj_item_cost(in[q]->N, in[q]->tune)) / cost[q])));
                         const int n = (own + most - 1) / most;  // equal parts
                         return (own + n - 1) / n;
                     };
@@ -668,14 +672,32 @@ int build_plan(const pamd_problem* p, Plan** out)
                         for (size_t q = 0; q < in.size(); ++q) {
                             const double w = cost[q] * in[q]->chains * in[q]->T;
                             work += w;
-                            fixed += w * lj_item_cost(in[q]->N);
+                            fixed += w * lj_item_cost(in[q]->N, in[q]->tune);
                         }
                         if (work * work >= 10.0 * (double)G * fixed) rounds = 2;
                     }
-                    double lo = 0.0, hi = cmax;  // smallest item cost that needs no more rounds
-                    for (int it = 0; it < 60; ++it) {
-                        const double mid = 0.5 * (lo + hi);
-                        (items_at(mid) <= rounds * G ? hi : lo) = mid;
+                    // smallest item cost that needs no more than r rounds
+                    auto cost_of = [&](long long r) {
+                        double lo = cmin, hi = std::max(cmin, cmax);
+                        if (items_at(lo) <= r * G) return lo;
+                        for (int it = 0; it < 60; ++it) {
+                            const double mid = 0.5 * (lo + hi);
+                            (items_at(mid) <= r * G ? hi : lo) = mid;
+                        }
+                        return hi;
+                    };
+                    double hi = cost_of(rounds);
+                    // One system of many short chains: equal parts of a chain may fill the fewest
+                    // rounds badly (64 chains on 152 CTAs: 128 items), and more rounds of shorter
+                    // items take less although each costs its constant again (N = 256, 40 x 512
+                    // steps, action and gradient: 1232 us in one round, 1045 in four; N = 162,
+                    // 64 x 557: 1732 and 1512; N = 173, 64 x 198: 626 and 576).
+                    if (in.size() == 1) {
+                        const long long least = rounds;
+                        for (long long r = least + 1; r <= least + 6; ++r) {
+                            const double c = cost_of(r);
+                            if (r * c < 0.99 * rounds * hi) rounds = r, hi = c;
+                        }
                     }
                     for (size_t q = 0; q < in.size(); ++q) {
                         in[q]->tune.tile_steps = tile(q, hi);
@@ -707,7 +729,7 @@ int build_plan(const pamd_problem* p, Plan** out)
                         it.t1 = std::min(si.T, it.t0 + si.tune.tile_steps);
                         it.slot = slot + b * si.n_tiles + tl;
                         sys_items[q].push_back(it);
-                        sys_cost[q].push_back(lj_step_cost(si.N, si.tune) * (it.t1 - it.t0) + lj_item_cost(si.N));
+                        sys_cost[q].push_back(lj_step_cost(si.N, si.tune) * (it.t1 - it.t0) + lj_item_cost(si.N, si.tune));
                     }
                 }
                 slot += si.chains * si.n_tiles;
