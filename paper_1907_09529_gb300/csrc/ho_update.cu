@@ -8,7 +8,7 @@
 // (mala_propose_kernel, ho_vec_kernel / ho_action_kernel, mala_reverse_kernel), so the
 // results are bitwise the same.
 //
-//   ho_trial_kernel + mala_sums_accept_kernel + ho_commit_kernel: any chain length.
+//   ho_trial_kernel + mala_sums_accept_kernel + ho_commit_kernel: single precision, any length.
 //     Memory traffic per coordinate 8 B read + 4 B written, then 4 + 8 B for accepted
 //     chains: the gradient of the proposal is never stored, the commit pass forms it
 //     again from the proposal.  The separate kernels move 48 B.
@@ -641,11 +641,11 @@ cudaError_t launch_ho_loop(const ElemBlock* blocks, int n_chains, int s, int max
     return cudaGetLastError();
 }
 
+template cudaError_t launch_ho_trial<float>(const ElemBlock*, int, int, const float*, const float*, float*, double*,
+                                            double*, double*, const MalaDev*, int, double, double, cudaStream_t);
+template cudaError_t launch_ho_commit<float>(const ElemBlock*, int, int, float*, float*, const float*, const int*,
+                                             double*, const double*, double, double, cudaStream_t);
 #define PAMD_INST(R)                                                                                             \
-    template cudaError_t launch_ho_trial<R>(const ElemBlock*, int, int, const R*, const R*, R*, double*,    \
-                                            double*, double*, const MalaDev*, int, double, double, cudaStream_t); \
-    template cudaError_t launch_ho_commit<R>(const ElemBlock*, int, int, R*, R*, const R*, const int*, double*,  \
-                                             const double*, double, double, cudaStream_t);                       \
     template cudaError_t launch_ho_loop<R>(const ElemBlock*, int, int, int, R*, R*, double*, const MalaDev*, \
                                            int, int, double, double, double, const double*, int*, double*, int*, \
                                            cudaStream_t);

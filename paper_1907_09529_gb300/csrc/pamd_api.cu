@@ -536,6 +536,10 @@ int build_plan(const pamd_problem* p, Plan** out)
         P->ho_max_n = (int)std::max<long long>(P->ho_max_n, si.chain_len);
     }
     P->ho_loop = P->ho_fused && P->ho_max_n <= kElemChunk;
+    // Longer chains in three passes, in single precision: what they save is traffic.  In double
+    // precision forming the proposal's gradient twice costs more FP64 work than that (an update
+    // of 1.9e7 elements: 860 us in three passes, 759 in five; 110 and 168 in single).
+    P->ho_fused = P->ho_loop || (P->ho_fused && !P->fp64);
     P->ho_direct = P->ho_max_n <= kElemChunk;
     for (auto& si : P->sys) P->ho_direct = P->ho_direct && si.kind == PAMD_HARMONIC;
     int slot = (int)P->h_ho.size();
@@ -998,6 +1002,8 @@ int run_ho_updates(const pamd_problem* p, Plan* P, R* pos, R* grad, double* S, c
             if (P->ho_loop)
                 PAMD_CUDA_TRY(launch_ho_loop<R>(P->d_all + b0, nb, s, (int)si.chain_len, pos, grad, S, P->d_md, u, n,
                                                 a, ginv, scale, log_u, n_acc, la, P->d_err, st));
+            else if constexpr (std::is_same<R, double>::value)
+                return PAMD_ERR_UNSUPPORTED;  // (not reached: Plan::ho_fused)
             else if (pass == 0)
                 PAMD_CUDA_TRY(launch_ho_trial<R>(P->d_all + b0, nb, s, pos, grad, prop, P->d_part_S + b0,
                                                  P->d_part_qf + b0, P->d_part_qr + b0, P->d_md, u, a, ginv, st));
