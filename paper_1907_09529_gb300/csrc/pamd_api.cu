@@ -388,7 +388,11 @@ LJTune choose_lj_tune(const pamd_system& s, int NT, int cap_lane_max, bool paire
     if (paired) t.outer_cap = lj_outer_cap(N, s.pot, sig_step, t.tile_steps, tpp);
     const double expect = 4.18879020478639 * rl * rl * rl * rho;  // 4/3 pi rl^3 rho
     t.list = std::min(expect, N - 1.0);
-    int want = (int)(1.2 * expect) + 8;
+    // Room for one and a half times the mean density (partly filled boxes, droplets), where the
+    // shared memory has it: a list that overflows scans all candidates at every step (a batch
+    // with 502 particles on a lattice of 864 sites: 3725 us with 1.2 times, 1779 with 1.5; the
+    // shared memory it takes from L1 costs N = 500 0.1 %, N = 600 1 %).
+    int want = (int)((paired ? 1.5 : 1.2) * expect) + 8;
     if (want > N - 1 + tpp) want = N - 1 + tpp;
     if (g_tune_override.maxnb > 0) want = g_tune_override.maxnb;
     int lane = (want + tpp - 1) / tpp;
