@@ -26,6 +26,14 @@
 // written back with coalesced stores.  HBM traffic: the path is read once and
 // accepted interiors written once.
 //
+// What bounds both: instruction issue (ncu: 78 to 84 % active, DRAM 4 to 11 %).  8192 one-line
+// paths of 4096 steps, one event: 277 us, of it 38 % normals and walk scan, 37 % trial, terms
+// and their scan, 11 % staging, 5 % the shifted output, the rest carries, decisions and
+// copies (324 us with fragment keys shuffled along the scans and the trial formed twice); 4096
+// three-line paths of 1024 steps, one step: 142 us (186 us with the line count at run time,
+// and the same two things).  The normals' Philox rounds are 32-bit products and their high
+// halves: as 64-bit products they took 3 % longer here and 10 % in the path updates.
+//
 // fragment_thread_kernel: the fallback for chains too large for shared memory,
 // one thread per fragment walking it three times (W_b; trial and action
 // differences; write-back on acceptance).
