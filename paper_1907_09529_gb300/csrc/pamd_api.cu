@@ -391,7 +391,7 @@ LJTune choose_lj_tune(const pamd_system& s, int NT, int cap_lane_max, bool paire
     // Room for one and a half times the mean density (partly filled boxes, droplets), where the
     // shared memory has it: a list that overflows scans all candidates at every step (a batch
     // with 502 particles on a lattice of 864 sites: 3725 us with 1.2 times, 1779 with 1.5; the
-    // shared memory it takes from L1 costs N = 500 0.1 %, N = 600 1 %).
+    // shared memory it takes from L1 costs N = 500 0.1 to 0.3 %, N = 600 1 %).
     int want = (int)((paired ? 1.5 : 1.2) * expect) + 8;
     if (want > N - 1 + tpp) want = N - 1 + tpp;
     if (g_tune_override.maxnb > 0) want = g_tune_override.maxnb;
@@ -655,10 +655,17 @@ int build_plan(const pamd_problem* p, Plan** out)
                             cmax = std::max(cmax, cost.back() * si.T + lj_item_cost(si.N, si.tune));
                             cmin = std::max(cmin, cost.back() + lj_item_cost(si.N, si.tune));
                         }
+                    // Unlike systems with N > 512: their lists have no room beyond the mean density
+                    // (shared memory), and a system that is denser than its mean scans all
+                    // candidates and takes several times its estimate.  Short items spread that (a
+                    // batch with 513 and 532 particles on lattices of 864 sites: 8851 us with the
+                    // longest items, 5331 with at most 32 steps; one with 514 and 531: 8873, 3932;
+                    // batches without such systems 0 to 10 % more, two of twelve).
+                    const int lim = in.size() > 1 && P->lj_cls[k].nmax > 512 ? std::min(limit, 32) : limit;
                     // steps per item of system q at cost c, and the items all chains then need
                     auto tile = [&](size_t q, double c) {
                         const int own = in[q]->T - in[q]->halo_lo;
-                        const int most = std::max(1, std::min(limit, (int)std::min(2.0e9, (c - lj_item_cost(in[q]->N, in[q]->tune)) / cost[q])));
+                        const int most = std::max(1, std::min(lim, (int)std::min(2.0e9, (c - lj_item_cost(in[q]->N, in[q]->tune)) / cost[q])));
                         const int n = (own + most - 1) / most;  // equal parts
                         return (own + n - 1) / n;
                     };
