@@ -98,7 +98,7 @@ __device__ __forceinline__ double widen_int(int k)
 struct DblCtx {
     int N, NW;
     LJK<double> k;
-    float Lf, iLf, lim2, hbf;  // single-precision box, widened squared cutoff, image guard
+    float Lf, iLf, lim2, hbf;  // single-precision box, widened squared cutoff, image guard (negative: far slice)
     float4* W;
     double *X, *R;
     int *K, *base;
@@ -265,7 +265,6 @@ __global__ void __launch_bounds__(NT, MINB)
         // 5e-7 L per component: r^2 within 2e-6 rc L + 3e-7 rc^2, ten times less than this
         const float rcf = sqrtf((float)C.k.rc2);
         C.lim2 = rcf * rcf + 2e-5f * rcf * (rcf + C.Lf);
-        C.hbf = 0.4999f * C.Lf;
         int lg = 0;  // threads per particle of the gathers: a power of two up to 8
         while (lg < 3 && (N << (lg + 1)) <= NT) ++lg;
         const int q = tid & ((1 << lg) - 1), per = NT >> lg;
@@ -280,17 +279,21 @@ __global__ void __launch_bounds__(NT, MINB)
         bool ov = false;
         for (int t = ts; t < I.t1; ++t) {
             const double* Xt = Xg + (long long)t * s;
-            // positions: double as stored, wrapped to [-L/2, L/2] in single precision
+            // positions: double as stored, wrapped to [-L/2, L/2] in single precision.  Box
+            // indices are kept in 32 bits: a slice with one of 2^30 or more (an exploding path)
+            // takes its candidates and images in double
+            bool far = false;
             for (int e = tid; e < s; e += NT) {
                 if (!PAMD_OK_IDX((long long)t * s + e, (long long)(T + 1) * s)) continue;
                 const int c = e / N, n = e - c * N;
                 const double x = __ldg(Xt + e);
                 const double m = __fma_rn(x, C.k.iL, 6755399441055744.0);
+                far |= !(fabs(__dsub_rn(m, 6755399441055744.0)) < 1073741824.0);
                 C.X[3 * n + c] = x;
                 C.K[3 * n + c] = __double2loint(m);
                 reinterpret_cast<float*>(C.W + n)[c] = (float)__fma_rn(-C.k.L, __dsub_rn(m, 6755399441055744.0), x);
             }
-            __syncthreads();
+            C.hbf = __syncthreads_or(far) ? -1.0f : 0.4999f * C.Lf;
             // adjacency rows: a warp per particle, 32 candidates per step
             for (int i = warp; i < N; i += NWARP) {
                 const float4 wi = C.W[i];
@@ -305,6 +308,11 @@ __global__ void __launch_bounds__(NT, MINB)
                         dy = fmaf(-C.Lf, C.image(dy), dy);
                         dz = fmaf(-C.Lf, C.image(dz), dz);
                         in = fmaf(dz, dz, fmaf(dy, dy, dx * dx)) <= C.lim2 && j != i;
+                        if (C.hbf < 0.0f) {
+                            double ex, ey, ez;
+                            in = j != i && pair_r2<double>(C.X[3 * i], C.X[3 * i + 1], C.X[3 * i + 2], C.X[3 * j],
+                                                           C.X[3 * j + 1], C.X[3 * j + 2], C.k, ex, ey, ez) <= C.k.rc2;
+                        }
                     }
                     const uint32_t m = __ballot_sync(0xffffffffu, in);
                     if (lane == 0) {

@@ -78,3 +78,36 @@ def test_clustered_pairs_exceed_the_capacity(pamd):
     N = 256
     x0 = inputs.fcc_lattice(N, inputs.box_side(N, 0.85))
     _check(pamd, N, 4, 2, 60.0, 2.5, x0, seed=6)
+
+
+@pytest.mark.parametrize("boxes", [2 ** 20, 2 ** 30 - 1, 2 ** 30, 2 ** 31 + 5, 2 ** 33 - 2, 2 ** 40, 2 ** 43])
+@pytest.mark.parametrize("tile", [0, 2])
+def test_images_far_away(pamd, boxes, tile):
+    """Every third particle stored some 2^20 to 2^43 box lengths away, as exploding paths
+    are: box indices beyond 32 bits.  With a box of 8 every coordinate, difference and
+    image is exact (multiples of 2^-5 below 2^48), so the tolerance is that of the parity tests."""
+    N, L, T = 100, 8.0, 5
+    x0 = inputs.fcc_lattice(N, L * 0.75)
+    walk = 0.02 * inputs.rng(boxes % 1000).standard_normal((1, T + 1, 3, N)).cumsum(1)
+    paths = np.round((x0 + walk) * 32.0) / 32.0
+    paths[..., ::3] += boxes * L
+    paths[:, :, 1, 1::3] -= boxes * L
+    D, beta, dt = 0.9, 1.1, 1e-4
+    prob = pamd.Problem([pamd.System("lj", N, 3, T, 1, box=L, rc=2.5)], D, beta, dt, "fp64")
+    buf = prob.empty("cuda")
+    prob.view(buf, 0).copy_(torch.from_numpy(paths))
+    try:
+        pamd.tune(tile)
+        S, g = pamd.action_grad(prob, buf)
+        S1 = pamd.action(prob, buf)
+        torch.cuda.synchronize()
+    finally:
+        pamd.tune()
+    So, go = oracle.action_grad(oracle.lennard_jones(L, 2.5), paths[0], D, beta, dt, nthreads=8)
+    near = paths[0].copy()
+    near[..., ::3] -= boxes * L
+    near[:, 1, 1::3] += boxes * L
+    Sn, gn = oracle.action_grad(oracle.lennard_jones(L, 2.5), near, D, beta, dt, nthreads=8)
+    assert abs(So - Sn) <= 1e-12 * Sn and rel(go, gn) <= 1e-12  # (the oracle's images are exact too)
+    assert torch.equal(S, S1) and abs(S[0].item() - So) <= 1e-12 * So
+    assert rel(prob.view(g, 0)[0].cpu().numpy(), go) <= 1e-12
