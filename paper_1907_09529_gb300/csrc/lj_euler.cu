@@ -26,19 +26,12 @@
 #include <type_traits>
 
 #include "cluster.cuh"
+#include "euler_shape.cuh"
 #include "lj_math.cuh"
 
 namespace pamd {
 
 namespace {
-
-constexpr int kEulerDense = 192;   // largest N without lists
-// Up to this size a particle has eight lanes, each adding its candidates in increasing j, and
-// double precision takes the library's 1/sqrt: the arithmetic of the LJ kernels' plain form,
-// bit for bit.  Small boxes are where a start can overlap (33 to 45 particles on a lattice of
-// 108 sites), and such a path turns any other order of the sums into another path.
-constexpr int kEulerOrdered = 64;
-constexpr int kOrderedLg = 3;
 
 // The normals of every element of slices 1..T of a system's chains, into the path.
 template <typename R>
@@ -135,11 +128,6 @@ struct DenseForce {
 __device__ __forceinline__ const LJK<float>& dense_consts(const LJK<float>& k) { return k; }
 __device__ __forceinline__ LJK<float> dense_consts(const LJK<double>&) { return LJK<float>(); }  // (not used)
 
-struct EulerShape {
-    int cs, nloc, lg, nt, cap, npad;
-    size_t smem;
-};
-
 // LG: log2 of the lanes per particle where it is known (the all-pairs form), else -1.
 template <typename R, bool LIST, int LG, int MAXT>
 __global__ void __launch_bounds__(MAXT)
@@ -152,8 +140,9 @@ __global__ void __launch_bounds__(MAXT)
     const int lg = LG >= 0 ? LG : H.lg, tpp = 1 << lg, q = tid & (tpp - 1), cs = H.cs, npad = H.npad;
     const unsigned rank = cs > 1 ? cluster_rank() : 0u;
     const int chain = blockIdx.x / cs;
-    const int i = (int)rank * H.nloc + (tid >> lg);
-    const bool active = (tid >> lg) < H.nloc && i < N;
+    const int first_i = euler_first(N, cs, (int)rank), mine = euler_first(N, cs, (int)rank + 1) - first_i;
+    const int i = first_i + (tid >> lg);
+    const bool active = (tid >> lg) < mine;
     const LJK<R>& k = S.k;
     R* X = pos + S.off + (long long)chain * S.chain_len;
     const R* Z = noise ? noise + S.off + (long long)chain * S.chain_len : X;
@@ -211,11 +200,12 @@ __global__ void __launch_bounds__(MAXT)
     // Slice t + 1 goes to the buffer that slice t - 1 was in.  A particle's slice t + 1 is sent
     // after every slice t has arrived, so after every CTA is done with slice t - 1 (its own
     // particles' slice t followed from it); the last lanes to read it are those that send.
-    // A barrier is armed for slice t + 2 when slice t has arrived on it.
+    // A barrier is armed for slice t + 2 when slice t has arrived on it.  All of this needs a
+    // particle in every CTA (euler_first): nothing would order the others behind one without.
     const unsigned bar0 = shared_addr(s_bar), bytes = (unsigned)(3 * N * sizeof(R));
     // A warp without particles does not wait, or it could fall two phases behind (with lists
     // the displacement check keeps all warps together).
-    const bool waits = LIST || tid < 32 || __any_sync(0xffffffffu, active);
+    const bool waits = LIST || __any_sync(0xffffffffu, active);
     bool lost = false;
     if (cs > 1 && tid == 0) {
         barrier_init(bar0);
@@ -331,47 +321,6 @@ __global__ void __launch_bounds__(MAXT)
         if (lost) atomicExch(err, PAMD_ERR_TIMEOUT);
         cluster_barrier();  // (no CTA ends while a store to it may be on its way)
     }
-}
-
-// Cluster size, lanes per particle and block size.
-// us a step, four chains, with 1, 2, 4, 8 CTAs a chain: N = 32 0.60, 0.70, 0.72, 0.72; N = 48
-// 0.78, 0.83, 0.78, 0.79; N = 56 1.05, 0.92, 0.85, 0.85; N = 108 2.4, 1.6, 1.2, 0.98; N = 500
-// 13, 7.7, 4.7, 3.5.  So single precision takes clusters from kEulerClusterN particles on, of
-// as many CTAs as the chains leave.  Double precision, bound by the FP64 pipe, takes them down
-// to four particles each (N = 32: 10.6, 5.9, 5.4, 5.4; N = 64: 39, 20, 10.5, 9.6; N = 108: 110,
-// 63, 31, 23).  Chains beyond the SMs get no cluster.
-// Lanes per particle: about 512 threads (more lanes add shuffles and overhead: N = 108 on four
-// CTAs took 1.92 us with 864 threads, 1.78 with 432), up to 1024 where that keeps four lanes.
-constexpr int kEulerClusterN = 50;
-constexpr int kEulerMinLocal = 6;
-constexpr int kEulerMinLocalDouble = 4;
-
-template <typename R>
-EulerShape euler_shape(int N, int n_chains, double list_volume, int sms, int max_smem)
-{
-    constexpr bool F32 = sizeof(R) == 4;
-    const int local = F32 ? kEulerMinLocal : kEulerMinLocalDouble;
-    EulerShape h;
-    h.cs = 1;
-    while (h.cs < 8 && (!F32 || N >= kEulerClusterN) && N >= 2 * h.cs * local && 2LL * h.cs * n_chains <= sms) h.cs *= 2;
-    h.nloc = (N + h.cs - 1) / h.cs;
-    h.lg = 0;
-    if (N <= kEulerOrdered)
-        h.lg = kOrderedLg;
-    else
-        while (h.lg < 5 && (h.nloc << (h.lg + 1)) <= (h.lg < 2 ? 1024 : 512)) ++h.lg;
-    h.nt = std::max(64, ((h.nloc << h.lg) + 31) / 32 * 32);
-    const int tpp = 1 << h.lg;
-    const bool list = N > kEulerDense;
-    h.npad = (N + 2 * tpp - 1) / (2 * tpp) * (2 * tpp);
-    h.smem = sizeof(R) * (size_t)(list ? 9 : 6) * h.npad;
-    h.cap = 0;
-    if (list) {  // expected list length plus a margin, every candidate at most, what fits
-        const int fit = (int)((max_smem - (long long)h.smem) / (2 * h.nt));
-        h.cap = std::max(1, std::min(std::min((N + tpp - 1) / tpp, fit), (int)(1.5 * list_volume / tpp) + 12));
-    }
-    h.smem += sizeof(uint16_t) * (size_t)h.cap * h.nt;
-    return h;
 }
 
 }  // namespace

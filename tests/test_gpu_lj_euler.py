@@ -85,3 +85,19 @@ def test_long_paths_repeat(pamd, N):
     pamd.euler_reference(prob, b, seed=1, counter=2)
     pamd.device_status()
     assert torch.equal(a, b) and bool(torch.isfinite(prob.view(a, 0)).all())
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+@pytest.mark.parametrize("N,B", [(33, 1), (34, 19), (42, 2), (49, 3), (57, 1), (65, 9)])
+def test_uneven_shares_repeat(pamd, precision, N, B):
+    """Particle counts that eight CTAs cannot share equally, over thousands of barrier
+    phases: the same path in two calls, and no wait that ran out."""
+    T, L = 3000, inputs.box_side(256, 0.85)
+    prob = pamd.Problem([pamd.System("lj", N, 3, T, B, box=L, rc=2.5)], 1.0, 1.0, 1e-4, precision)
+    a = prob.empty("cuda")
+    prob.view(a, 0)[:, 0].copy_(torch.from_numpy(inputs.fcc_lattice(256, L)[:, :N].copy()))
+    b = a.clone()
+    pamd.euler_reference(prob, a, seed=1, counter=2)
+    pamd.euler_reference(prob, b, seed=1, counter=2)
+    pamd.device_status()
+    assert torch.equal(a, b) and bool(torch.isfinite(prob.view(a, 0)).all())
