@@ -68,14 +68,83 @@ __device__ __forceinline__ unsigned long long now_ns()
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
     return t;
 }
-// Waits for the phase of the given parity; false when it did not complete within two seconds.
-__device__ __forceinline__ bool wait_phase(unsigned bar, unsigned parity)
+// The limit of a launch's waits: `ns` of time, twice, so that a wait does not run out because the
+// process was stopped for a while.  Tests make waits run out: the odd CTAs of a cluster leave
+// after `rounds` rounds.
+struct WaitLimit {
+    unsigned ns = 2000000000u;
+    int rounds = 0x7fffffff;
+};
+
+// Waits for the phase of the given parity; false when the wait ran out.
+__device__ __forceinline__ bool poll_phase(unsigned bar, unsigned parity, unsigned ns)
 {
-    if (phase_done(bar, parity)) return true;
-    const unsigned long long end = now_ns() + 2000000000ull;
+    const unsigned long long end = now_ns() + ns;
     while (!phase_done(bar, parity))
         if (now_ns() > end) return false;
     return true;
+}
+__device__ __forceinline__ bool wait_phase(unsigned bar, unsigned parity, const WaitLimit& w)
+{
+    return poll_phase(bar, parity, w.ns) || poll_phase(bar, parity, w.ns);
+}
+
+// How the CTAs of a cluster part: in shared memory, cleared before the first cluster barrier.
+struct ClusterEnd {
+    unsigned lost;       // some wait of the cluster ran out
+    unsigned out[8][2];  // bytes this CTA sent to the barriers of every CTA
+    unsigned in[8][2];   // bytes every CTA sent to this one's
+};
+
+__device__ __forceinline__ void put_remote(unsigned* p, unsigned rank, unsigned v)
+{
+    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(remote_addr(shared_addr(p), rank)), "r"(v) : "memory");
+}
+// Takes `bytes` off what a barrier's phase waits for, as if they had arrived.
+__device__ __forceinline__ void complete_bytes(unsigned bar, unsigned bytes)
+{
+    asm volatile("mbarrier.complete_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
+
+// Called by every thread of a cluster after its last round, with `lost` where a wait ran out
+// (that thread has sent and armed nothing since).  False: nothing was lost, and since every phase
+// was waited for, no store is under way.  True, for every thread of the cluster: some wait ran
+// out, and cluster_drain has to follow.
+__device__ __forceinline__ bool cluster_lost(ClusterEnd* E, bool lost, int cs)
+{
+    if (__syncthreads_or(lost) && threadIdx.x < cs) put_remote(&E->lost, threadIdx.x, 1u);
+    cluster_barrier();  // (no CTA sends any more)
+    return *reinterpret_cast<volatile unsigned*>(&E->lost) != 0u;
+}
+
+// After a lost wait stores may still be under way to CTAs that wait for nothing any more, and a
+// CTA must not end before they have landed.  `count` adds up in E->out what this CTA has sent
+// (called by every thread); phases(b) of `bytes` each were armed on barrier b.  With what every
+// CTA has sent known, each barrier is made to wait for just that.
+template <typename Phases, typename Count>
+__device__ __forceinline__ void cluster_drain(ClusterEnd* E, unsigned bar0, unsigned bytes, int cs, Phases&& phases,
+                                              Count&& count)
+{
+    const int tid = threadIdx.x;
+    const unsigned rank = cluster_rank();
+    count();
+    __syncthreads();
+    if (tid < 2 * cs) put_remote(&E->in[rank][tid & 1], (unsigned)tid >> 1, E->out[tid >> 1][tid & 1]);
+    cluster_barrier();
+    if (tid < 2) {
+        const unsigned bar = bar0 + 8u * (unsigned)tid, n = phases(tid);
+        unsigned sent = 0;
+        for (int r = 0; r < cs; ++r) sent += E->in[r][tid];
+        const int missing = (int)(n * bytes - sent);  // (below 2^20 in size: differences of the last phases)
+        if (missing > 0) complete_bytes(bar, (unsigned)missing);
+        bool there = n == 0 || wait_phase(bar, (n - 1) & 1u, WaitLimit());
+        if (missing < 0 && there) {  // bytes of a phase that was not armed
+            expect(bar, (unsigned)-missing);
+            wait_phase(bar, n & 1u, WaitLimit());
+        }
+    }
+    __syncthreads();
+    cluster_barrier();
 }
 
 }  // namespace pamd

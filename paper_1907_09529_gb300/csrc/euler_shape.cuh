@@ -69,7 +69,7 @@ EulerShape euler_shape(int N, int n_chains, double list_volume, int sms, int max
         const int fit = (int)((max_smem - (long long)h.smem) / (2 * h.nt));
         h.cap = std::max(1, std::min(std::min((N + tpp - 1) / tpp, fit), (int)(1.5 * list_volume / tpp) + 12));
     }
-    h.smem += sizeof(uint16_t) * (size_t)h.cap * h.nt;
+    h.smem = (h.smem + sizeof(uint16_t) * (size_t)h.cap * h.nt + 15) & ~(size_t)15;
     return h;
 }
 

@@ -364,22 +364,50 @@ struct HoCluster {
     __host__ __device__ int own() const { return 32 * vw * K; }
     __host__ __device__ int halo() const { return 2 * s * K; }
     __host__ __device__ int threads() const { return own() + (halo() + 31) / 32 * 32; }
+    // whether the run before (after) has a copy of the gradient at place p of run k, and its CTA
+    __device__ bool to_prev(unsigned rank, int k, int p) const { return p < s && (rank > 0 || k > 0); }
+    __device__ bool to_next(unsigned rank, int k, int p) const { return p >= run() - s && ((int)rank < cs - 1 || k < K - 1); }
+    __device__ unsigned prev(unsigned rank) const { return rank > 0 ? rank - 1 : cs - 1; }
+    __device__ unsigned next(unsigned rank) const { return (int)rank < cs - 1 ? rank + 1 : 0u; }
     __host__ __device__ size_t doubles() const  // x', terms, halo gradients (2), warp sums (2)
     {
         return (size_t)K * (run() + 2 * s) + 3 * (size_t)own() + 2 * (size_t)halo() + 2 * 24;
     }
 };
 
+// After a lost wait of a cluster.  A thread has sent its part of `sent[tid]` updates; mine: its
+// element is one of the CTA's, at place p of run k.
+__device__ __noinline__ void ho_cluster_drain(ClusterEnd* E, const int* sent, const int* armed, unsigned bar0,
+                                              unsigned bytes, bool mine, int k, int p, const HoCluster& H)
+{
+    const int tid = threadIdx.x, lane = tid & 31;
+    const unsigned rank = cluster_rank();
+    auto count = [&] {
+        for (int b = 0; b < 2; ++b) {
+            const unsigned n8 = 8u * (unsigned)((sent[tid] + 1 - b) / 2);  // of even, odd updates
+            if (mine && H.to_prev(rank, k, p)) atomicAdd(&E->out[H.prev(rank)][b], n8);
+            if (mine && H.to_next(rank, k, p)) atomicAdd(&E->out[H.next(rank)][b], n8);
+            for (int q = tid >> 5; q < 3 * H.vw; q += blockDim.x >> 5)
+                if (lane < H.cs) atomicAdd(&E->out[lane][b], n8);
+        }
+    };
+    cluster_drain(E, bar0, bytes, H.cs, [&](int b) { return (unsigned)((*armed + 1 - b) / 2); }, count);
+}
+
 __global__ void __launch_bounds__(1024)
     ho_cluster_kernel(const ElemBlock* __restrict__ blocks, double* __restrict__ pos, double* __restrict__ grad,
                       double* __restrict__ Sv, const MalaDev* __restrict__ md, int update0, int n_updates, double a,
                       double ginv, double S_scale, const double* __restrict__ log_u, int* __restrict__ n_accepted,
-                      double* __restrict__ log_alpha, int* __restrict__ err, const HoCluster H)
+                      double* __restrict__ log_alpha, int* __restrict__ err, const HoCluster H, const WaitLimit limit)
 {
     extern __shared__ __align__(16) double smem_d[];
     __shared__ int s_acc;
     __shared__ double s_lu[kLuBatch];
     __shared__ __align__(8) uint64_t s_bar[2];  // of even and odd updates
+    __shared__ ClusterEnd s_end;
+    __shared__ int s_sent[1024];  // updates a thread sends
+    __shared__ int s_armed;
+    __shared__ double s_la;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, NW = blockDim.x >> 5;
     const int cs = H.cs, s = H.s, RL = H.run(), K = H.K, own_n = H.own(), pitch = RL + 2 * s;
     const unsigned rank = cluster_rank();
@@ -421,11 +449,14 @@ __global__ void __launch_bounds__(1024)
     const double h4 = 4.0 * hh, h4_inv = 1.0 / h4;
     double z = normal(update0);
     if (own || halo) XP[xi] = 0.0;
+    for (int j = tid; j < (int)(sizeof(ClusterEnd) / sizeof(unsigned)); j += blockDim.x) reinterpret_cast<unsigned*>(&s_end)[j] = 0u;
     // Received per update: 24 warp sums and the gradients of this CTA's halo elements.  Those of
     // update n + 2 replace those of update n: they are sent after the sums of update n + 1 have
     // come from every CTA, so after every thread of every CTA is done with update n.
     const unsigned bar0 = shared_addr(s_bar), bytes = 8u * (24u + (unsigned)__syncthreads_count(halo && in));
     bool lost = false;
+    const int rounds = (rank & 1u) ? min(n_updates, limit.rounds) : n_updates;
+    s_sent[tid] = rounds;
     if (tid == 0) {
         barrier_init(bar0);
         barrier_init(bar0 + 8);
@@ -434,7 +465,7 @@ __global__ void __launch_bounds__(1024)
         if (n_updates > 1) expect(bar0 + 8, bytes);
     }
     cluster_barrier();
-    for (int u = update0; u < update0 + n_updates; ++u) {
+    for (int u = update0; u < update0 + rounds; ++u) {
         const int n = u - update0, par = n & 1, lu_at = n % kLuBatch;
         const unsigned bar = bar0 + 8 * par;
         auto send = [&](double* p, unsigned to, double v) {
@@ -457,15 +488,10 @@ __global__ void __launch_bounds__(1024)
                     f = fma_r(hh, g, d);
                     b = fma_r(hh, gp, -d);
                 }
-                // the neighbours' copies of this gradient
-                if (p < s && (rank > 0 || k > 0)) {
-                    const int kk = rank > 0 ? k : k - 1;
-                    send(HG + par * H.halo() + kk * 2 * s + s + p, rank > 0 ? rank - 1 : cs - 1, gp);
-                }
-                if (p >= RL - s && ((int)rank < cs - 1 || k < K - 1)) {
-                    const int kk = (int)rank < cs - 1 ? k : k + 1;
-                    send(HG + par * H.halo() + kk * 2 * s + p - (RL - s), (int)rank < cs - 1 ? rank + 1 : 0u, gp);
-                }
+                if (H.to_prev(rank, k, p) && !lost)
+                    send(HG + par * H.halo() + (rank > 0 ? k : k - 1) * 2 * s + s + p, H.prev(rank), gp);
+                if (H.to_next(rank, k, p) && !lost)
+                    send(HG + par * H.halo() + ((int)rank < cs - 1 ? k : k + 1) * 2 * s + p - (RL - s), H.next(rank), gp);
             }
             V[tid] = r;
             V[own_n + tid] = f;
@@ -480,12 +506,14 @@ __global__ void __launch_bounds__(1024)
                 acc = fma_r(v, v, acc);
             }
             acc = warp_sum(acc);
-            if (lane < cs) send(VS + 24 * par + 8 * t + (int)rank * H.vw + w, (unsigned)lane, acc);
+            if (lane < cs && !lost) send(VS + 24 * par + 8 * t + (int)rank * H.vw + w, (unsigned)lane, acc);
         }
         if (n + 1 < n_updates) z = normal(u + 1);
         asm volatile("" : "+d"(z));  // (here, not after the wait)
-        if (!lost) lost = !wait_phase(bar, (unsigned)(n >> 1) & 1u);
-        if (tid == 32 * (NW - 1) && n + 2 < n_updates) expect(bar, bytes);  // (not by the accept test's warp: 1.3 us an update)
+        // (lost: nothing is sent or armed any more, and nothing will be committed)
+        if (!lost && !phase_done(bar, (unsigned)(n >> 1) & 1u) && !wait_phase(bar, (unsigned)(n >> 1) & 1u, limit))
+            lost = true, s_sent[tid] = n + 1;
+        if (tid == 32 * (NW - 1) && n + 2 < n_updates && !lost) expect(bar, bytes);  // (not by the accept test's warp: 1.3 us an update)
         if (warp == 0) {
             // lanes 8 t + w: sum t of warp w
             double v = lane < 24 ? VS[24 * par + lane] : 0.0;
@@ -504,7 +532,7 @@ __global__ void __launch_bounds__(1024)
                 const bool last = u == update0 + n_updates - 1;
                 if ((last && log_alpha) || !(fabs(lu - la) > 1e-12 * (fabs(dS) + a1 + a2))) la = dS - qr / h4 + qf / h4;
                 const int acc = lu < la ? 1 : 0;  // NaN log alpha never accepts
-                if (log_alpha && rank == 0 && last) log_alpha[B.chain] = la;
+                if (last) s_la = la;
                 if (acc) S_cur = S_new;
                 n_acc += acc;
                 s_acc = acc;
@@ -516,6 +544,13 @@ __global__ void __launch_bounds__(1024)
             g = own ? gp : halo ? HG[par * H.halo() + h] : g;
         }
     }
+    // updates armed: the first two, and n + 2 when the sums of update n had come
+    if (tid == 32 * (NW - 1)) s_armed = min(n_updates, s_sent[tid] + (lost ? 1 : 2));
+    if (cluster_lost(&s_end, lost || rounds < n_updates, cs)) {
+        ho_cluster_drain(&s_end, s_sent, &s_armed, bar0, bytes, own && in, k, p, H);
+        if (tid == 0) atomicExch(err, PAMD_ERR_TIMEOUT);  // the chain stays as it was
+        return;
+    }
     if (own && in) {
         *gx = x;
         *gg = g;
@@ -523,9 +558,8 @@ __global__ void __launch_bounds__(1024)
     if (rank == 0 && tid == 0) {
         Sv[B.chain] = S_cur;
         if (n_accepted) n_accepted[B.chain] += n_acc;
+        if (log_alpha) log_alpha[B.chain] = s_la;
     }
-    if (lost) atomicExch(err, PAMD_ERR_TIMEOUT);
-    cluster_barrier();  // (no CTA ends while a store to it may be on its way)
 }
 
 // The cluster shape for chains of n elements, s to a slice: as many CTAs per chain (up to 8)
@@ -595,7 +629,7 @@ template <typename R>
 cudaError_t launch_ho_loop(const ElemBlock* blocks, int n_chains, int s, int max_n, R* pos, R* grad,
                            double* S, const MalaDev* md, int update0, int n_updates, double a, double ginv,
                            double S_scale, const double* log_u, int* n_accepted, double* log_alpha, int* err,
-                           cudaStream_t st)
+                           const WaitLimit& limit, cudaStream_t st)
 {
     if (n_chains <= 0 || n_updates <= 0) return cudaSuccess;
     if constexpr (sizeof(R) == 8) {
@@ -622,7 +656,7 @@ cudaError_t launch_ho_loop(const ElemBlock* blocks, int n_chains, int s, int max
             cfg.attrs = at;
             cfg.numAttrs = 1;
             return cudaLaunchKernelEx(&cfg, ho_cluster_kernel, blocks, pos, grad, S, md, update0, n_updates, a, ginv,
-                                      S_scale, log_u, n_accepted, log_alpha, err, h);
+                                      S_scale, log_u, n_accepted, log_alpha, err, h, limit);
         }
     }
     const size_t arr = (sizeof(R) * ((size_t)max_n + 4) + 15) & ~(size_t)15;
@@ -651,7 +685,7 @@ template cudaError_t launch_ho_commit<float>(const ElemBlock*, int, int, float*,
 #define PAMD_INST(R)                                                                                             \
     template cudaError_t launch_ho_loop<R>(const ElemBlock*, int, int, int, R*, R*, double*, const MalaDev*, \
                                            int, int, double, double, double, const double*, int*, double*, int*, \
-                                           cudaStream_t);
+                                           const WaitLimit&, cudaStream_t);
 PAMD_INST(float)
 PAMD_INST(double)
 #undef PAMD_INST

@@ -128,14 +128,55 @@ struct DenseForce {
 __device__ __forceinline__ const LJK<float>& dense_consts(const LJK<float>& k) { return k; }
 __device__ __forceinline__ LJK<float> dense_consts(const LJK<double>&) { return LJK<float>(); }  // (not used)
 
+// Lanes 0..2 of a particle (one lane when it has fewer) take its components x, y, z; lane
+// q writes component q mod 3 of the new position to CTAs q / 3, q / 3 + tpp / 3, ...
+struct EulerLane {
+    int comp, first, stride, nc;  // nc: components of a mover lane
+    bool mover, owner;            // of a lane of a particle
+    __device__ __forceinline__ EulerLane(int q, int tpp, bool active)
+    {
+        const int lanes3 = tpp / 3;
+        comp = tpp >= 3 ? q % 3 : 0, first = tpp >= 3 ? q / 3 : 0, stride = tpp >= 3 ? lanes3 : 1, nc = tpp >= 3 ? 1 : 3;
+        mover = active && (tpp >= 3 ? q < 3 * lanes3 : q == 0), owner = mover && q < 3;
+    }
+};
+
+// After a lost wait of a cluster; a thread has sent slices 1..sent[tid].  The chain is left as
+// NaN after slice 0: what it holds by then, normals among it, looks like positions.  (Not inlined:
+// what it needs would be kept in registers throughout the steps.)
+template <typename R>
+__device__ __noinline__ void euler_drain(ClusterEnd* E, const int* sent, unsigned bar0, int N, int T, int cs, int lg,
+                                         R* X)
+{
+    const int rank = (int)cluster_rank(), tid = threadIdx.x;
+    auto count = [&] {
+        const int mine = euler_first(N, cs, rank + 1) - euler_first(N, cs, rank);
+        const EulerLane l(tid & ((1 << lg) - 1), 1 << lg, (tid >> lg) < mine);
+        for (int d = l.first; l.mover && d < cs; d += l.stride) {
+            atomicAdd(&E->out[d][0], (unsigned)(sent[tid] / 2) * (unsigned)(l.nc * sizeof(R)));
+            atomicAdd(&E->out[d][1], (unsigned)((sent[tid] + 1) / 2) * (unsigned)(l.nc * sizeof(R)));
+        }
+    };
+    // slices 1..armed: 1 and 2 to begin with, t + 2 in step t
+    auto phases = [&](int b) { return (unsigned)((min(T, max(sent[0] + 1, 2)) + b) / 2); };
+    cluster_drain(E, bar0, (unsigned)(3 * N * sizeof(R)), cs, phases, count);
+    const long long s = 3 * N, n = (long long)(T + 1) * s;
+    for (long long e = s + (long long)rank * blockDim.x + tid; e < n; e += (long long)cs * blockDim.x)
+        if (PAMD_OK_IDX(e, n)) X[e] = (R)__int_as_float(0x7fffffff);
+}
+
 // LG: log2 of the lanes per particle where it is known (the all-pairs form), else -1.
 template <typename R, bool LIST, int LG, int MAXT>
 __global__ void __launch_bounds__(MAXT)
     lj_euler_kernel(R* __restrict__ pos, const R* __restrict__ noise, const LJSysDev<R> S, const EulerShape H,
-                    int* __restrict__ err)
+                    int* __restrict__ err, const WaitLimit limit)
 {
     extern __shared__ __align__(32) unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t s_bar[2];  // of the two slices
+    // Behind the arrays of the steps: as static shared memory, in front of them, these two made a
+    // step of N = 108 take 8 to 10 % longer (1.05 against 0.96 us; where the slices lie matters)
+    ClusterEnd& s_end = *reinterpret_cast<ClusterEnd*>(smem_raw + H.smem);
+    int* s_sent = reinterpret_cast<int*>(&s_end + 1);
     const int N = S.N, T = S.T, s = 3 * N, tid = threadIdx.x, NT = blockDim.x;
     const int lg = LG >= 0 ? LG : H.lg, tpp = 1 << lg, q = tid & (tpp - 1), cs = H.cs, npad = H.npad;
     const unsigned rank = cs > 1 ? cluster_rank() : 0u;
@@ -177,18 +218,16 @@ __global__ void __launch_bounds__(MAXT)
         }
         ovf = cnt > H.cap;
     };
-    // Lanes 0..2 of a particle (one lane when it has fewer) take its components x, y, z; lane
-    // q writes component q mod 3 of the new position to CTAs q / 3, q / 3 + tpp / 3, ...
-    const int comp = tpp >= 3 ? q % 3 : 0, lanes3 = tpp / 3, first = tpp >= 3 ? q / 3 : 0, stride = tpp >= 3 ? lanes3 : 1;
-    const bool mover = active && (tpp >= 3 ? q < 3 * lanes3 : q == 0), owner = mover && q < 3;
     constexpr int NC = 3;
-    const int nc = tpp >= 3 ? 1 : NC;  // components of a mover lane
+    const EulerLane lane(q, tpp, active);
+    const int comp = lane.comp, first = lane.first, stride = lane.stride, nc = lane.nc;
+    const bool mover = lane.mover, owner = lane.owner;
     const int oi = (int)(P.at(active ? i : 0, 0) - buf);
     R* const W = buf + oi + comp * npad;                       // own component, buffer 0
     const R* zp = Z + (long long)s + comp * N + (active ? i : 0);  // its normal of the step to load next
     R* xp = X + (long long)comp * N + (active ? i : 0);            // its place in slice t
-    // (a ring indexed by the unrolled step: copying a register would wait for its load)
-    R z[4][NC], last[NC] = {R(0), R(0), R(0)};
+    // (indexed by the unrolled step: copying a register would wait for its load)
+    R z[2][NC], last[NC] = {R(0), R(0), R(0)};
     auto load_zs = [&](bool in, R (&v)[NC]) {
 #pragma unroll
         for (int c = 0; c < NC; ++c)
@@ -206,7 +245,11 @@ __global__ void __launch_bounds__(MAXT)
     // A warp without particles does not wait, or it could fall two phases behind (with lists
     // the displacement check keeps all warps together).
     const bool waits = LIST || __any_sync(0xffffffffu, active);
-    bool lost = false;
+    bool lost = false;  // a wait ran out: nothing is sent or armed any more, the steps count for nothing
+    const int steps = (rank & 1u) ? min(T, max(1, limit.rounds)) : T;
+    s_sent[tid] = steps;  // slices 1..steps are sent
+    if (cs > 1)
+        for (int j = tid; j < (int)(sizeof(ClusterEnd) / sizeof(unsigned)); j += NT) reinterpret_cast<unsigned*>(&s_end)[j] = 0u;
     if (cs > 1 && tid == 0) {
         barrier_init(bar0);
         barrier_init(bar0 + 8);
@@ -220,10 +263,10 @@ __global__ void __launch_bounds__(MAXT)
         __syncthreads();
     // (also: every lane holds its first normals before slice 1 is written)
     const DenseForce<LG >= 0 ? LG : 0> dense(dense_consts(k), N, npad, i, q);
-    // Step t from buffer PAR to the other; zt: its normals.  The slice that the step before
+    // Step t from buffer PAR to the other; zt: its normals, then those of step t + 2.  The slice that the step before
     // made is stored here: a store directly before the barrier would hold it up (the
     // barrier's release waits for it).
-    auto step = [&](int t, auto par, const R (&zt)[NC], R (&z2)[NC]) {
+    auto step = [&](int t, auto par, R (&zt)[NC]) {
         constexpr int PAR = decltype(par)::value;
         const EulerPos<R, LIST> A{buf + PAR * 3 * npad, npad, lg};
         if (t > 0 && owner) {
@@ -232,8 +275,7 @@ __global__ void __launch_bounds__(MAXT)
                 if (c < nc) xp[c * N] = last[c];
         }
         xp += s;
-        if (cs > 1 && tid == 0 && t > 0 && t + 2 <= T) expect(bar0 + 8 * PAR, bytes);
-        load_zs(t + 2 < T, z2);
+        if (cs > 1 && tid == 0 && t > 0 && t + 2 <= T && !lost) expect(bar0 + 8 * PAR, bytes);
         if (LIST) {
             bool moved = t == 0;
             for (int j = tid; j < N; j += NT) {
@@ -285,7 +327,7 @@ __global__ void __launch_bounds__(MAXT)
             R* w = W + (1 - PAR) * 3 * npad + c * npad;
             if (cs == 1) {
                 if (owner) *w = xn;
-            } else {
+            } else if (!lost) {
                 const unsigned to = shared_addr(w), bar = bar0 + 8 * (1 - PAR);
                 for (int d = first; d < cs; d += stride)
                     send_async(remote_addr(to, (unsigned)d), xn, remote_addr(bar, (unsigned)d));
@@ -299,18 +341,17 @@ __global__ void __launch_bounds__(MAXT)
                 for (int c = 0; c < 3; ++c) move(c, xi[c], f[c], zt[c]);
             }
         }
+        load_zs(t + 2 < T, zt);
         if (cs == 1)
             __syncthreads();
-        else if (waits && !lost)
-            lost = !wait_phase(bar0 + 8 * (1 - PAR), (unsigned)(t >> 1) & 1u);
+        else if (waits && !lost && !wait_phase(bar0 + 8 * (1 - PAR), (unsigned)(t >> 1) & 1u, limit))
+            lost = true, s_sent[tid] = t + 1;
     };
     using P0 = std::integral_constant<int, 0>;
     using P1 = std::integral_constant<int, 1>;
-    for (int t = 0; t < T; t += 4) {
-        step(t, P0{}, z[0], z[2]);
-        if (t + 1 < T) step(t + 1, P1{}, z[1], z[3]);
-        if (t + 2 < T) step(t + 2, P0{}, z[2], z[0]);
-        if (t + 3 < T) step(t + 3, P1{}, z[3], z[1]);
+    for (int t = 0; t < steps; t += 2) {
+        step(t, P0{}, z[0]);
+        if (t + 1 < steps) step(t + 1, P1{}, z[1]);
     }
     if (owner) {
 #pragma unroll
@@ -318,8 +359,10 @@ __global__ void __launch_bounds__(MAXT)
             if (c < nc) xp[c * N] = last[c];
     }
     if (cs > 1) {
-        if (lost) atomicExch(err, PAMD_ERR_TIMEOUT);
-        cluster_barrier();  // (no CTA ends while a store to it may be on its way)
+        if (cluster_lost(&s_end, lost || steps < T, cs)) {
+            euler_drain<R>(&s_end, s_sent, shared_addr(s_bar), S.N, S.T, H.cs, H.lg, X);
+            if (tid == 0) atomicExch(err, PAMD_ERR_TIMEOUT);
+        }
     }
 }
 
@@ -327,7 +370,7 @@ __global__ void __launch_bounds__(MAXT)
 
 template <typename R>
 cudaError_t launch_lj_euler(R* pos, const R* noise, const void* sys_entry_host, int n_chains, int chain0,
-                            uint64_t seed, uint64_t counter, int* err, cudaStream_t st)
+                            uint64_t seed, uint64_t counter, int* err, const WaitLimit& limit, cudaStream_t st)
 {
     const LJSysDev<R> S = *static_cast<const LJSysDev<R>*>(sys_entry_host);
     if (n_chains <= 0 || S.T <= 0) return cudaSuccess;
@@ -344,8 +387,8 @@ cudaError_t launch_lj_euler(R* pos, const R* noise, const void* sys_entry_host, 
     }
     const double rl2 = (double)S.k.rl2, L = (double)S.k.L;
     const EulerShape h = euler_shape<R>(S.N, n_chains, 4.18879020478639 * rl2 * std::sqrt(rl2) * S.N / (L * L * L), sms,
-                                        max_smem - 1024);
-    void (*kern)(R*, const R*, LJSysDev<R>, EulerShape, int*);
+                                        max_smem - 6 * 1024);
+    void (*kern)(R*, const R*, LJSysDev<R>, EulerShape, int*, WaitLimit);
     if (S.N > kEulerDense)
         kern = h.nt <= 512 ? lj_euler_kernel<R, true, -1, 512> : lj_euler_kernel<R, true, -1, 1024>;
     else if constexpr (sizeof(R) == 8)
@@ -359,12 +402,13 @@ cudaError_t launch_lj_euler(R* pos, const R* noise, const void* sys_entry_host, 
                : h.lg == 2 ? lj_euler_kernel<R, false, 2, 1024>
                            : nullptr;
     if (!kern) return cudaErrorInvalidValue;
-    if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)h.smem)) != cudaSuccess)
+    const size_t smem = h.smem + sizeof(ClusterEnd) + sizeof(int) * (size_t)h.nt;
+    if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
         return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(n_chains * h.cs));
     cfg.blockDim = dim3((unsigned)h.nt);
-    cfg.dynamicSmemBytes = h.smem;
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
@@ -372,13 +416,13 @@ cudaError_t launch_lj_euler(R* pos, const R* noise, const void* sys_entry_host, 
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = h.cs > 1 ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kern, pos, noise, S, h, err);
+    return cudaLaunchKernelEx(&cfg, kern, pos, noise, S, h, err, limit);
 }
 
 template cudaError_t launch_lj_euler<float>(float*, const float*, const void*, int, int, uint64_t, uint64_t, int*,
-                                            cudaStream_t);
+                                            const WaitLimit&, cudaStream_t);
 template cudaError_t launch_lj_euler<double>(double*, const double*, const void*, int, int, uint64_t, uint64_t, int*,
-                                             cudaStream_t);
+                                             const WaitLimit&, cudaStream_t);
 
 PAMD_DEBUG_FETCHER(lj_euler)
 

@@ -18,6 +18,7 @@
 
 #include <nvtx3/nvToolsExt.h>
 
+#include "cluster.cuh"
 #include "pamd_internal.cuh"
 #include "fragment.cuh"
 
@@ -34,11 +35,24 @@ struct NvtxRange {
 // Host-side fault injection, for tests of the error paths (nothing faults on the
 // device): PAMD_FAULT_INJECT=alloc makes every workspace allocation fail,
 // =launch makes every CUDA call the library checks report failure, =nonfinite
-// flags every action computed as non-finite.
+// flags every action computed as non-finite, =wait:N makes waits run out (wait_limit).
 bool fault_injected(const char* what)
 {
     const char* e = std::getenv("PAMD_FAULT_INJECT");
     return e && std::strcmp(e, what) == 0;
+}
+
+// The limit of waits between the CTAs of a cluster.  PAMD_FAULT_INJECT=wait:N makes them run out
+// after two milliseconds: the odd CTAs leave after N rounds (steps or updates).
+WaitLimit wait_limit()
+{
+    WaitLimit w;
+    const char* e = std::getenv("PAMD_FAULT_INJECT");
+    if (e && std::strncmp(e, "wait:", 5) == 0) {
+        w.rounds = std::atoi(e + 5);
+        w.ns = 1000000u;
+    }
+    return w;
 }
 
 #define PAMD_CUDA_TRY(expr)                                                    \
@@ -1012,7 +1026,7 @@ int run_ho_updates(const pamd_problem* p, Plan* P, R* pos, R* grad, double* S, c
             const int b0 = P->h_E_slots[lo].begin, nb = P->h_E_slots[hi - 1].end - b0, s = si.d * si.N;
             if (P->ho_loop)
                 PAMD_CUDA_TRY(launch_ho_loop<R>(P->d_all + b0, nb, s, (int)si.chain_len, pos, grad, S, P->d_md, u, n,
-                                                a, ginv, scale, log_u, n_acc, la, P->d_err, st));
+                                                a, ginv, scale, log_u, n_acc, la, P->d_err, wait_limit(), st));
             else if constexpr (std::is_same<R, double>::value)
                 return PAMD_ERR_UNSUPPORTED;  // (not reached: Plan::ho_fused)
             else if (pass == 0)
@@ -1686,10 +1700,10 @@ int pamd_euler_reference(const pamd_problem* prob, void* pos, uint64_t seed, uin
             const void* row = &P->h_lj_sys[P->lj_sys_stride * si.lj_index];
             if (P->fp64)
                 PAMD_CUDA_TRY(launch_lj_euler<double>((double*)dpos, (const double*)dnoise, row, si.chains,
-                                                      si.chain0, seed, counter, P->d_err, st));
+                                                      si.chain0, seed, counter, P->d_err, wait_limit(), st));
             else
                 PAMD_CUDA_TRY(launch_lj_euler<float>((float*)dpos, (const float*)dnoise, row, si.chains, si.chain0,
-                                                     seed, counter, P->d_err, st));
+                                                     seed, counter, P->d_err, wait_limit(), st));
         }
     }
     if (host) {

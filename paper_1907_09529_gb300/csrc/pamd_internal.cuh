@@ -337,6 +337,7 @@ struct ChainSlots {
 };
 
 // ------------------------------------------------------------------ launchers
+struct WaitLimit;  // cluster.cuh: the limits of waits between the CTAs of a cluster
 // Where the harmonic kernels write a chain's action when every chain is one block.
 struct HoDirect {
     double* S = nullptr;  // indexed by global chain; nullptr: partial sums instead
@@ -513,7 +514,7 @@ cudaError_t launch_ho_euler(R* pos, const R* noise, int s, int T, int n_chains, 
                             uint64_t counter, cudaStream_t st);
 template <typename R>
 cudaError_t launch_lj_euler(R* pos, const R* noise, const void* sys_entry_host, int n_chains, int chain0,
-                            uint64_t seed, uint64_t counter, int* err, cudaStream_t st);
+                            uint64_t seed, uint64_t counter, int* err, const WaitLimit& limit, cudaStream_t st);
 
 // Deterministic per-chain sums of partials: out[c] = scale * sum(partials[slots[c]]);
 // a non-finite sum sets *err (if given) to PAMD_ERR_NONFINITE.
@@ -580,7 +581,8 @@ cudaError_t launch_ho_commit(const ElemBlock* blocks, int n_blocks, int s, R* po
 template <typename R>
 cudaError_t launch_ho_loop(const ElemBlock* blocks, int n_chains, int s, int max_n, R* pos, R* grad, double* S,
                            const MalaDev* md, int update0, int n_updates, double a, double ginv, double S_scale,
-                           const double* log_u, int* n_accepted, double* log_alpha, int* err, cudaStream_t st);
+                           const double* log_u, int* n_accepted, double* log_alpha, int* err,
+                           const WaitLimit& limit, cudaStream_t st);
 cudaError_t launch_set_mala_params(MalaDev* md, uint64_t seed, uint64_t counter, double h,
                                    cudaStream_t st);
 

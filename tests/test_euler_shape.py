@@ -28,7 +28,7 @@ int check(int N, int chains, int sms)
             ok = ok && n >= 1 && n <= h.nloc;
         }
         ok = ok && (h.nloc << h.lg) <= h.nt && h.nt % 32 == 0 && h.nt >= 64 && h.nt <= 1024 && h.lg <= 5;
-        ok = ok && h.npad >= N && h.npad % (2 << h.lg) == 0 && h.smem <= 227 * 1024 - 1024;
+        ok = ok && h.npad >= N && h.npad % (2 << h.lg) == 0 && h.smem <= 227 * 1024 - 1024 && h.smem % 16 == 0;
         ok = ok && (N <= kEulerDense ? h.cap == 0 && h.lg >= 2 : h.cap >= 1);
         if (!ok) {
             std::printf("N %d chains %d sms %d double %d: cs %d nloc %d lg %d nt %d cap %d npad %d smem %zu\n", N, chains,
