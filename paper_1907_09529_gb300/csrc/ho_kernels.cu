@@ -23,7 +23,7 @@ __device__ __forceinline__ void put_sum(double tot, const ElemBlock& B, double* 
     if (threadIdx.x != 0) return;
     if (D.S) {
         D.S[B.chain] = tot * D.scale;
-        if (!isfinite(tot)) atomicExch(D.err, PAMD_ERR_NONFINITE);
+        if (!isfinite(tot)) flag_nonfinite(D.err);
     } else {
         *partial = tot;
     }

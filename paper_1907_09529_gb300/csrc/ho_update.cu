@@ -312,7 +312,7 @@ __global__ void __launch_bounds__(kElemThreads)
         double tot[3] = {to_double(sums[0]), to_double(sums[1]), to_double(sums[2])};
         block_sums_256<3>(tot, reinterpret_cast<double*>(smem_raw + L.red));
         if (threadIdx.x == 0) {
-            if (!isfinite(tot[0])) atomicExch(err, PAMD_ERR_NONFINITE);
+            if (!isfinite(tot[0])) flag_nonfinite(err);
             const double S_new = tot[0] * S_scale;
             const int acc = mala_decide(c, S_cur, S_new, tot[1], tot[2], log_u, M, u,
                                         u == update0 + n_updates - 1 ? log_alpha : nullptr);
@@ -523,7 +523,7 @@ __global__ void __launch_bounds__(1024)
             const double S_new = v * S_scale;  // lane 0; the others below in lanes 8 and 16
             const double qf = __shfl_sync(0xffffffffu, v, 8), qr = __shfl_sync(0xffffffffu, v, 16);
             if (lane == 0) {
-                if (rank == 0 && !isfinite(v)) atomicExch(err, PAMD_ERR_NONFINITE);
+                if (rank == 0 && !isfinite(v)) flag_nonfinite(err);
                 // log alpha with the reciprocal of 4 h: within a few ulp of its largest term, so
                 // the comparison is that of the divided form unless the two sides are that close
                 // (two double divisions are most of this step otherwise)

@@ -1290,7 +1290,7 @@ int pamd_device_status(void* stream)
         if (cudaMemcpy(&v, kv.second->d_err, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess)
             return PAMD_ERR_CUDA;
         if (v != PAMD_OK) {
-            worst = v;
+            if (worst != PAMD_ERR_TIMEOUT) worst = v;
             cudaMemset(kv.second->d_err, 0, sizeof(int));
         }
     }

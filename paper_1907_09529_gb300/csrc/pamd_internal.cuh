@@ -286,6 +286,10 @@ __device__ __forceinline__ double to_double(float v)
     return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7FFFFFFFu) >> 3) + 0x38000000u)), (int)(b << 29));
 }
 
+// A non-finite action: the status word keeps what it holds (a wait that ran out, which may be
+// why the action is not finite, is reported first).
+__device__ __forceinline__ void flag_nonfinite(int* err) { atomicCAS(err, PAMD_OK, PAMD_ERR_NONFINITE); }
+
 // A device buffer whose address is not 16-byte aligned: the element kernels read
 // and write whole 16-byte units, so such a buffer is refused (PAMD_ERR_ARG) before
 // anything is launched.  Host buffers are staged into the library's own aligned
@@ -521,7 +525,7 @@ cudaError_t launch_lj_euler(R* pos, const R* noise, const void* sys_entry_host, 
 cudaError_t launch_finalize(const double* partials, const ChainSlots* slots, int n_chains,
                             double scale, double* out, cudaStream_t st, int* err = nullptr);
 
-// Sets a device status word (host-side fault injection of non-finite actions).
+// Sets a device status word that holds none yet (host-side fault injection of non-finite actions).
 cudaError_t launch_set_status(int* err, int v, cudaStream_t st);
 
 // MALA update pieces (element-wise over all systems' blocks).

@@ -29,7 +29,7 @@ __global__ void finalize_kernel(const double* __restrict__ partials, const Chain
     s = warp_sum(s);
     if (lane == 0) {
         out[warp] = s * scale;
-        if (err && !isfinite(s)) atomicExch(err, PAMD_ERR_NONFINITE);
+        if (err && !isfinite(s)) flag_nonfinite(err);
     }
 }
 
@@ -43,7 +43,7 @@ cudaError_t launch_finalize(const double* partials, const ChainSlots* slots, int
     return cudaGetLastError();
 }
 
-__global__ void set_status_kernel(int* err, int v) { *err = v; }
+__global__ void set_status_kernel(int* err, int v) { atomicCAS(err, PAMD_OK, v); }
 
 cudaError_t launch_set_status(int* err, int v, cudaStream_t st)
 {
@@ -256,7 +256,7 @@ __global__ void __launch_bounds__(96)
     s = warp_sum(s);
     if (lane == 0) {
         sums[w] = w == 0 ? s * S_scale : s;
-        if (w == 0 && !isfinite(s)) atomicExch(err, PAMD_ERR_NONFINITE);
+        if (w == 0 && !isfinite(s)) flag_nonfinite(err);
     }
     __syncthreads();
     if (threadIdx.x != 0) return;

@@ -113,3 +113,23 @@ def test_updates(pamd, fault, d, T, B):
     update(s)
     pamd.device_status()
     same(s, want)
+
+
+def test_a_later_status_does_not_replace_it(pamd, fault):
+    prob = pamd.Problem([pamd.System("harmonic", 1, 1, 500, 1, k=0.8)], 0.9, 1.1, 0.02, "fp64")
+    pos = prob.empty("cuda")
+    prob.view(pos, 0).zero_()
+    S, g = pamd.action_grad(prob, pos)
+    pamd.device_status()
+    fault("wait:0")
+    pamd.path_update(prob, pos, g, S, 1e-6, 4, seed=1)
+    fault(None)
+    prob.view(pos, 0)[0, 3] = float("nan")
+    pamd.action_grad(prob, pos)  # a non-finite action
+    with pytest.raises(pamd.PamdError) as ei:
+        pamd.device_status()
+    assert ei.value.status == TIMEOUT
+    pamd.action_grad(prob, pos)
+    with pytest.raises(pamd.PamdError) as ei:
+        pamd.device_status()
+    assert ei.value.status == -5  # PAMD_ERR_NONFINITE
