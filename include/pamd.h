@@ -71,7 +71,11 @@ extern "C" {
 #define PAMD_ERR_UNSUPPORTED (-2)  /* valid, but outside what the kernels handle */
 #define PAMD_ERR_CUDA (-3)         /* a CUDA runtime call or launch failed */
 #define PAMD_ERR_TIMEOUT (-4)      /* a bounded device wait ran out: a CTA of a cluster
-                                      waited two seconds for the other CTAs of its chain */
+                                      waited four seconds for the other CTAs of its chain
+                                      (pamd_euler_reference: the chain is NaN after slice 0;
+                                      pamd_path_update: it keeps its last complete state).
+                                      Returned by the call itself with host buffers, else by
+                                      pamd_device_status */
 #define PAMD_ERR_NONFINITE (-5)    /* a non-finite action was produced */
 #define PAMD_ERR_ALLOC (-6)        /* workspace allocation failed */
 

@@ -1073,6 +1073,18 @@ int run_one_update(const pamd_problem* p, Plan* P, R* pos, R* grad, double* S, c
     return PAMD_OK;
 }
 
+// After a call with host buffers whose kernels wait for one another: PAMD_ERR_TIMEOUT (cleared)
+// if a wait ran out, since the buffers that the caller gets then are not the call's results.  Any
+// other status stays for pamd_device_status.  The stream has been synchronised.
+int waits_status(Plan* P)
+{
+    int v = 0;
+    PAMD_CUDA_TRY(cudaMemcpy(&v, P->d_err, sizeof(int), cudaMemcpyDeviceToHost));
+    if (v != PAMD_ERR_TIMEOUT) return PAMD_OK;
+    PAMD_CUDA_TRY(cudaMemset(P->d_err, 0, sizeof(int)));
+    return PAMD_ERR_TIMEOUT;
+}
+
 // Path updates with host buffers (no explicit noise or uniforms), pipelined over
 // chunks of chains: chunk k's inputs are copied in on one stream while earlier
 // chunks are updated and copied back on others.  Updates alternate between the
@@ -1197,7 +1209,7 @@ int path_update_pipelined(const pamd_problem* prob, Plan* P, void* pos, void* gr
             PAMD_CUDA_TRY(cudaEventElapsedTime(&tl[1 + 3 * k + q], ev_start, P->events[3 * k + q]));
     }
     g_last_timeline.swap(tl);
-    return PAMD_OK;
+    return P->ho_loop && P->fp64 ? waits_status(P) : PAMD_OK;
 }
 
 }  // namespace
@@ -1545,6 +1557,7 @@ int pamd_path_update(const pamd_problem* prob, void* pos, void* grad, double* S,
         if (dla != log_alpha)
             PAMD_CUDA_TRY(cudaMemcpyAsync(log_alpha, dla, sizeof(double) * nc, cudaMemcpyDeviceToHost, st));
         PAMD_CUDA_TRY(cudaStreamSynchronize(st));
+        if (P->ho_loop && P->fp64) return waits_status(P);
     }
     return PAMD_OK;
 }
@@ -1709,6 +1722,7 @@ int pamd_euler_reference(const pamd_problem* prob, void* pos, uint64_t seed, uin
     if (host) {
         if (dpos != pos) PAMD_CUDA_TRY(cudaMemcpyAsync(pos, dpos, bytes, cudaMemcpyDeviceToHost, st));
         PAMD_CUDA_TRY(cudaStreamSynchronize(st));
+        if (!P->lj_cls.empty()) return waits_status(P);
     }
     return PAMD_OK;
 }

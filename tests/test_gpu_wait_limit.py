@@ -115,6 +115,39 @@ def test_updates(pamd, fault, d, T, B):
     same(s, want)
 
 
+def test_host_buffers_get_the_status(pamd, fault):
+    """Calls with host buffers return it themselves, and it is cleared."""
+    N, T, B, L = 108, 20, 2, inputs.box_side(108, 0.85)
+    prob = pamd.Problem([pamd.System("lj", N, 3, T, B, box=L, rc=2.3)], 1.0, 1.0, 1e-4, "fp64")
+    buf = prob.empty("cpu")
+    prob.view(buf, 0)[:, 0].copy_(torch.from_numpy(inputs.fcc_lattice(N, L)))
+    fault("wait:3")
+    with pytest.raises(pamd.PamdError) as ei:
+        pamd.euler_reference(prob, buf, seed=3, counter=1)
+    assert ei.value.status == TIMEOUT
+    fault(None)
+    pamd.device_status()
+    pamd.euler_reference(prob, buf, seed=3, counter=1)
+    assert bool(torch.isfinite(prob.view(buf, 0)).all())
+    for chains in (1, 3):  # one stream, and the pipeline over chunks
+        ho = pamd.Problem([pamd.System("harmonic", 1, 1, 500, chains, k=0.8)], 0.9, 1.1, 0.02, "fp64")
+        pos = 0.1 * torch.randn(ho.span, dtype=torch.float64)
+        S, g = torch.zeros(chains, dtype=torch.float64), torch.zeros(ho.span, dtype=torch.float64)
+        pamd.action_grad(ho, pos, S, g)
+        before = [t.clone() for t in (pos, g, S)]
+        nacc = torch.zeros(chains, dtype=torch.int32)
+        fault("wait:0")
+        with pytest.raises(pamd.PamdError) as ei:
+            pamd.path_update(ho, pos, g, S, 1e-6, 4, seed=1, n_accepted=nacc)
+        assert ei.value.status == TIMEOUT
+        fault(None)
+        pamd.device_status()
+        assert all(torch.equal(a, b) for a, b in zip((pos, g, S), before))
+        pamd.path_update(ho, pos, g, S, 1e-6, 4, seed=1, n_accepted=nacc)
+        pamd.device_status()
+        assert int(nacc.min()) > 0
+
+
 def test_a_later_status_does_not_replace_it(pamd, fault):
     prob = pamd.Problem([pamd.System("harmonic", 1, 1, 500, 1, k=0.8)], 0.9, 1.1, 0.02, "fp64")
     pos = prob.empty("cuda")
