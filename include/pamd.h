@@ -54,7 +54,8 @@
  * not cached); "launch": every CUDA call the library checks reports failure
  * (PAMD_ERR_CUDA; a graph whose capture failed is not cached); "nonfinite":
  * every action computed is flagged non-finite (pamd_device_status then returns
- * PAMD_ERR_NONFINITE).  The variable is read at each call.
+ * PAMD_ERR_NONFINITE); "wait:N": waits between the CTAs of a cluster run out
+ * after N rounds (PAMD_ERR_TIMEOUT).  The variable is read at each call.
  */
 #ifndef PAMD_H
 #define PAMD_H
@@ -273,6 +274,8 @@ int pamd_mala_commit(const pamd_problem* prob, void* pos, void* grad, double* S,
 /* Forward Euler-Maruyama paths (Eq. (2)), sequential in time:
  *     x_{t+1} = x_t + beta D dt F(x_t) + sqrt(2 D dt) xi_t,
  * each new slice stored in the precision's element type and used as stored.
+ * A chain's path follows from x_0, the parameters and its normals alone, bit for
+ * bit: neither the other chains of the call nor the GPU's size play a part.
  *   pos   : in/out; slice 0 of every chain holds x_0 on entry, slices 1..T
  *           are written.
  *   noise : NULL (normals from Philox, stream 0, seed/counter) or standard

@@ -22,8 +22,10 @@ constexpr int kEulerDense = 192;  // largest N without lists
 constexpr int kEulerOrdered = 64;
 constexpr int kOrderedLg = 3;
 
+// lg: log2 of the partial sums of a particle's force; a thread forms 2^vr of them (the particle
+// has 2^(lg - vr) lanes), one after the other, and adds them as the lanes' shuffles would.
 struct EulerShape {
-    int cs, nloc, lg, nt, cap, npad;
+    int cs, nloc, lg, vr, nt, cap, npad;
     size_t smem;
 };
 
@@ -39,11 +41,25 @@ PAMD_HD inline int euler_first(int N, int cs, int rank) { return rank * N / cs; 
 // as many CTAs as the chains leave.  Double precision, bound by the FP64 pipe, takes them down
 // to four particles each (N = 32: 10.6, 5.9, 5.4, 5.4; N = 64: 39, 20, 10.5, 9.6; N = 108: 110,
 // 63, 31, 23).  Chains beyond the SMs get no cluster.
-// Lanes per particle: about 512 threads (more lanes add shuffles and overhead: N = 108 on four
-// CTAs took 1.92 us with 864 threads, 1.78 with 432), up to 1024 where that keeps four lanes.
+// Partial sums per particle: they set the order of the sums, so they follow from N alone, and a
+// chain's path does not depend on the chains beside it or on the GPU: as many as a particle has
+// lanes in clusters of eight with about 512 threads (more lanes add shuffles and overhead: N =
+// 108 on four CTAs took 1.92 us with 864 threads, 1.78 with 432).  With fewer CTAs a chain a lane
+// takes two or four of them, rather than more than 1024 threads, or 512 of more than eight lanes.
+// (Lanes by the cluster size instead were up to 1.5 times as fast for 50 chains and more, 96 steps
+// of N = 256: 382 us for 50 chains, 529 here, 811 with one CTA of four threads a particle.)
 constexpr int kEulerClusterN = 50;
 constexpr int kEulerMinLocal = 6;
 constexpr int kEulerMinLocalDouble = 4;
+
+inline int euler_lg(int N)
+{
+    if (N <= kEulerOrdered) return kOrderedLg;
+    const int n8 = (N + 7) / 8;
+    int lg = 0;
+    while (lg < 5 && (n8 << (lg + 1)) <= 512) ++lg;
+    return lg;
+}
 
 template <typename R>
 EulerShape euler_shape(int N, int n_chains, double list_volume, int sms, int max_smem)
@@ -54,15 +70,13 @@ EulerShape euler_shape(int N, int n_chains, double list_volume, int sms, int max
     h.cs = 1;
     while (h.cs < 8 && (!F32 || N >= kEulerClusterN) && N >= 2 * h.cs * local && 2LL * h.cs * n_chains <= sms) h.cs *= 2;
     h.nloc = (N + h.cs - 1) / h.cs;
-    h.lg = 0;
-    if (N <= kEulerOrdered)
-        h.lg = kOrderedLg;
-    else
-        while (h.lg < 5 && (h.nloc << (h.lg + 1)) <= (h.lg < 2 ? 1024 : 512)) ++h.lg;
-    h.nt = std::max(64, ((h.nloc << h.lg) + 31) / 32 * 32);
-    const int tpp = 1 << h.lg;
+    h.lg = euler_lg(N);
+    h.vr = 0;
+    while (h.vr < 2 && h.vr < h.lg && (h.nloc << (h.lg - h.vr)) > (h.lg - h.vr <= 3 ? 1024 : 512)) ++h.vr;
+    const int tpp = 1 << (h.lg - h.vr), sums2 = 2 << h.lg;
+    h.nt = std::max(64, (h.nloc * tpp + 31) / 32 * 32);
     const bool list = N > kEulerDense;
-    h.npad = (N + 2 * tpp - 1) / (2 * tpp) * (2 * tpp);
+    h.npad = (N + sums2 - 1) / sums2 * sums2;
     h.smem = sizeof(R) * (size_t)(list ? 9 : 6) * h.npad;
     h.cap = 0;
     if (list) {  // expected list length plus a margin, every candidate at most, what fits

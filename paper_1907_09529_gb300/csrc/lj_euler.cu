@@ -10,7 +10,8 @@
 //     loads its own two steps ahead.  Drawing them inside the step put ten Philox rounds
 //     and Box-Muller on the chain.
 //   * A chain is stepped by a cluster of CTAs (up to 8).  Each CTA holds all positions
-//     and moves N / CS particles, up to 32 lanes to a particle; the new coordinates go to
+//     and moves N / CS particles, up to 32 lanes to a particle (how many partial sums a force
+//     has, and so every bit of a path, follows from N alone: euler_shape.cuh); the new coordinates go to
 //     every CTA's shared memory as asynchronous stores counted by a transaction barrier there.
 //     A step costs one trip between SMs; with plain remote stores and a cluster barrier it
 //     also waited for their acknowledgement (N = 108: 1.33 against 0.96 us a step).
@@ -58,7 +59,7 @@ __global__ void euler_normals_kernel(R* __restrict__ pos, long long off, long lo
 template <typename R, bool LIST>
 struct EulerPos {
     R* p;
-    int n, lg;  // padded particles; log2 of the lanes per particle
+    int n, lg;  // padded particles; log2 of the partial sums per particle
     __device__ __forceinline__ R* at(int j, int c) const
     {
         if (sizeof(R) == 4 && !LIST) {  // (LG >= 0)
@@ -75,10 +76,10 @@ template <int LG>
 struct DenseForce {
     float2 nL, iL, mag, nmag, c1, c2, m1, duc;
     float rc2;
-    int N, full, all, i, q, py, pz;
-    __device__ __forceinline__ DenseForce(const LJK<float>& k, int N_, int npad, int i_, int q_)
+    int N, full, all, i, py, pz;
+    __device__ __forceinline__ DenseForce(const LJK<float>& k, int N_, int npad, int i_)
         : nL(pk(-k.L)), iL(pk(k.iL)), mag(pk(12582912.0f)), nmag(pk(-12582912.0f)), c1(pk(k.c1)), c2(pk(k.c2)),
-          m1(pk(-1.0f)), duc(pk(k.duc)), rc2(k.rc2), N(N_), full(N_ >> (LG + 1)), all(npad >> (LG + 1)), i(i_), q(q_),
+          m1(pk(-1.0f)), duc(pk(k.duc)), rc2(k.rc2), N(N_), full(N_ >> (LG + 1)), all(npad >> (LG + 1)), i(i_),
           py(npad / 2), pz(npad)
     {
     }
@@ -109,8 +110,8 @@ struct DenseForce {
             fz = fma2(fs, dz, fz);
         }
     }
-    // p: the slice; lane q's candidates 2m, 2m + 1 are the float2 at m 2^LG + q
-    __device__ __forceinline__ void operator()(const float* p, const float (&xi)[3], float (&f)[3]) const
+    // p: the slice; candidates 2m, 2m + 1 of sum q are the float2 at m 2^LG + q
+    __device__ __forceinline__ void operator()(const float* p, const float (&xi)[3], int q, float (&f)[3]) const
     {
         const float2 x = pk(xi[0]), y = pk(xi[1]), z = pk(xi[2]);
         float2 fx = pk(0.0f), fy = pk(0.0f), fz = pk(0.0f);
@@ -145,13 +146,13 @@ struct EulerLane {
 // NaN after slice 0: what it holds by then, normals among it, looks like positions.  (Not inlined:
 // what it needs would be kept in registers throughout the steps.)
 template <typename R>
-__device__ __noinline__ void euler_drain(ClusterEnd* E, const int* sent, unsigned bar0, int N, int T, int cs, int lg,
+__device__ __noinline__ void euler_drain(ClusterEnd* E, const int* sent, unsigned bar0, int N, int T, int cs, int lanes,
                                          R* X)
 {
     const int rank = (int)cluster_rank(), tid = threadIdx.x;
     auto count = [&] {
         const int mine = euler_first(N, cs, rank + 1) - euler_first(N, cs, rank);
-        const EulerLane l(tid & ((1 << lg) - 1), 1 << lg, (tid >> lg) < mine);
+        const EulerLane l(tid & ((1 << lanes) - 1), 1 << lanes, (tid >> lanes) < mine);
         for (int d = l.first; l.mover && d < cs; d += l.stride) {
             atomicAdd(&E->out[d][0], (unsigned)(sent[tid] / 2) * (unsigned)(l.nc * sizeof(R)));
             atomicAdd(&E->out[d][1], (unsigned)((sent[tid] + 1) / 2) * (unsigned)(l.nc * sizeof(R)));
@@ -165,8 +166,25 @@ __device__ __noinline__ void euler_drain(ClusterEnd* E, const int* sent, unsigne
         if (PAMD_OK_IDX(e, n)) X[e] = (R)__int_as_float(0x7fffffff);
 }
 
-// LG: log2 of the lanes per particle where it is known (the all-pairs form), else -1.
-template <typename R, bool LIST, int LG, int MAXT>
+// f = the sum over s = V, V + W, ... of the partial sums `leaf(s, f)` (S of them in all), as the
+// shuffles of lanes s would add them: first s and s + S/2, then s and s + S/4, ...
+template <typename R, int V, int W, int S, typename F>
+__device__ __forceinline__ void sum_tree(R (&f)[3], F&& leaf)
+{
+    if constexpr (W == S) {
+        leaf(std::integral_constant<int, V>{}, f);
+    } else {
+        R g[3];
+        sum_tree<R, V, 2 * W, S>(f, leaf);
+        sum_tree<R, V + W, 2 * W, S>(g, leaf);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) f[c] += g[c];
+    }
+}
+
+// LG: log2 of the partial sums per particle where it is known (the all-pairs form), else -1; a
+// lane takes 2^VR of them.
+template <typename R, bool LIST, int LG, int VR, int MAXT>
 __global__ void __launch_bounds__(MAXT)
     lj_euler_kernel(R* __restrict__ pos, const R* __restrict__ noise, const LJSysDev<R> S, const EulerShape H,
                     int* __restrict__ err, const WaitLimit limit)
@@ -178,12 +196,13 @@ __global__ void __launch_bounds__(MAXT)
     ClusterEnd& s_end = *reinterpret_cast<ClusterEnd*>(smem_raw + H.smem);
     int* s_sent = reinterpret_cast<int*>(&s_end + 1);
     const int N = S.N, T = S.T, s = 3 * N, tid = threadIdx.x, NT = blockDim.x;
-    const int lg = LG >= 0 ? LG : H.lg, tpp = 1 << lg, q = tid & (tpp - 1), cs = H.cs, npad = H.npad;
+    constexpr int NV = 1 << VR;
+    const int lg = LG >= 0 ? LG : H.lg, lanes = lg - VR, tpp = 1 << lanes, q = tid & (tpp - 1), cs = H.cs, npad = H.npad;
     const unsigned rank = cs > 1 ? cluster_rank() : 0u;
     const int chain = blockIdx.x / cs;
     const int first_i = euler_first(N, cs, (int)rank), mine = euler_first(N, cs, (int)rank + 1) - first_i;
-    const int i = first_i + (tid >> lg);
-    const bool active = (tid >> lg) < mine;
+    const int i = first_i + (tid >> lanes);
+    const bool active = (tid >> lanes) < mine;
     const LJK<R>& k = S.k;
     R* X = pos + S.off + (long long)chain * S.chain_len;
     const R* Z = noise ? noise + S.off + (long long)chain * S.chain_len : X;
@@ -197,26 +216,30 @@ __global__ void __launch_bounds__(MAXT)
             *P.at(j, c) = j < N ? X[c * N + j] : R(0);
             P.at(j, c)[3 * npad] = R(0);  // (padding of the other buffer)
         }
-    int cnt = 0;
+    int cnt[NV];  // list entries up to the end of each of this lane's sums (of four in the order
+                  // in which they are added up: 0, 2, 1, 3)
     bool ovf = false;
-    // candidates of this lane
+    // candidates of this lane, sum by sum
     auto build = [&](const EulerPos<R, LIST>& A) {
         for (int j = tid; j < N; j += NT)
 #pragma unroll
             for (int c = 0; c < 3; ++c) ref[c * npad + j] = *A.at(j, c);
-        cnt = 0;
-        if (active) {
-            const R xi = *A.at(i, 0), yi = *A.at(i, 1), zi = *A.at(i, 2);
-            for (int j = q; j < N; j += tpp) {
+        int n = 0;
+        const R xi = active ? *A.at(i, 0) : R(0), yi = active ? *A.at(i, 1) : R(0), zi = active ? *A.at(i, 2) : R(0);
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+            const int sum = NV == 4 ? (v & 1) * 2 + (v >> 1) : v;
+            for (int j = active ? q + sum * tpp : N; j < N; j += 1 << lg) {
                 R dx, dy, dz;
                 const R r2 = pair_r2<R>(xi, yi, zi, *A.at(j, 0), *A.at(j, 1), *A.at(j, 2), k, dx, dy, dz);
                 if (r2 <= k.rl2 && j != i) {
-                    if (cnt < H.cap && PAMD_OK_IDX(cnt * NT + tid, H.cap * NT)) nbr[cnt * NT + tid] = (uint16_t)j;
-                    ++cnt;
+                    if (n < H.cap && PAMD_OK_IDX(n * NT + tid, H.cap * NT)) nbr[n * NT + tid] = (uint16_t)j;
+                    ++n;
                 }
             }
+            cnt[v] = n;
         }
-        ovf = cnt > H.cap;
+        ovf = n > H.cap;
     };
     constexpr int NC = 3;
     const EulerLane lane(q, tpp, active);
@@ -262,7 +285,7 @@ __global__ void __launch_bounds__(MAXT)
     else
         __syncthreads();
     // (also: every lane holds its first normals before slice 1 is written)
-    const DenseForce<LG >= 0 ? LG : 0> dense(dense_consts(k), N, npad, i, q);
+    const DenseForce<LG >= 0 ? LG : 0> dense(dense_consts(k), N, npad, i);
     // Step t from buffer PAR to the other; zt: its normals, then those of step t + 2.  The slice that the step before
     // made is stored here: a store directly before the barrier would hold it up (the
     // barrier's release waits for it).
@@ -291,29 +314,53 @@ __global__ void __launch_bounds__(MAXT)
         if (active) {
 #pragma unroll
             for (int c = 0; c < 3; ++c) xi[c] = A.p[oi + c * npad];
-            if constexpr (sizeof(R) == 8 && LG == kOrderedLg) {
-                for (int j = q; j < N; j += tpp)
-                    if (j != i) {
-                        R dx, dy, dz;
-                        const R r2 = pair_r2<R>(xi[0], xi[1], xi[2], *A.at(j, 0), *A.at(j, 1), *A.at(j, 2), k, dx, dy, dz);
-                        if (!(r2 <= k.rc2)) continue;
-                        const R ri = rsqrt(r2), ir2 = ri * ri, ir6 = ir2 * ir2 * ir2, u = k.c1 * ir6;
-                        const R fs = fma_r(u * fma_r(k.c2, ir6, R(-1)), ir2, k.duc * ri);
-                        f[0] = fma_r(fs, dx, f[0]);
-                        f[1] = fma_r(fs, dy, f[1]);
-                        f[2] = fma_r(fs, dz, f[2]);
+            if (LIST && !ovf) {
+                // one loop over the entries of all sums (a loop for each would take the longest
+                // lane's entries in every one of them: up to 1.5 times as long in double)
+                R g[3] = {R(0), R(0), R(0)}, g1[3] = {R(0), R(0), R(0)};
+                auto turn = [&](int m) {  // entry m is the first of another sum
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) {
+                        if (m == cnt[0]) g[c] = f[c], f[c] = R(0);
+                        if (NV == 4 && m == cnt[1 % NV]) g[c] += f[c], f[c] = R(0);
+                        if (NV == 4 && m == cnt[2 % NV]) g1[c] = f[c], f[c] = R(0);
                     }
-            } else if constexpr (LG >= 0) {
-                dense(A.p, xi, f);
-            } else if (LIST && !ovf) {
+                };
 #pragma unroll 2
-                for (int m = 0; m < cnt; ++m) {
+                for (int m = 0; m < cnt[NV - 1]; ++m) {
+                    if (NV > 1) turn(m);
                     const int j = nbr[m * NT + tid];
                     pair_force<R>(xi[0], xi[1], xi[2], *A.at(j, 0), *A.at(j, 1), *A.at(j, 2), k, f);
                 }
+                if (NV > 1) {
+                    turn(cnt[NV - 1]);
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) f[c] = NV == 4 ? g[c] + (g1[c] + f[c]) : g[c] + f[c];
+                }
             } else {
-                for (int j = q; j < N; j += tpp)
-                    if (j != i) pair_force<R>(xi[0], xi[1], xi[2], *A.at(j, 0), *A.at(j, 1), *A.at(j, 2), k, f);
+                sum_tree<R, 0, 1, NV>(f, [&](auto sum, R (&f)[3]) {
+                    constexpr int v = decltype(sum)::value;
+                    const int j0 = q + v * tpp, dj = 1 << lg;  // candidates j0, j0 + dj, ...
+                    f[0] = f[1] = f[2] = R(0);
+                    if constexpr (sizeof(R) == 8 && LG == kOrderedLg) {
+                        for (int j = j0; j < N; j += dj)
+                            if (j != i) {
+                                R dx, dy, dz;
+                                const R r2 = pair_r2<R>(xi[0], xi[1], xi[2], *A.at(j, 0), *A.at(j, 1), *A.at(j, 2), k, dx, dy, dz);
+                                if (!(r2 <= k.rc2)) continue;
+                                const R ri = rsqrt(r2), ir2 = ri * ri, ir6 = ir2 * ir2 * ir2, u = k.c1 * ir6;
+                                const R fs = fma_r(u * fma_r(k.c2, ir6, R(-1)), ir2, k.duc * ri);
+                                f[0] = fma_r(fs, dx, f[0]);
+                                f[1] = fma_r(fs, dy, f[1]);
+                                f[2] = fma_r(fs, dz, f[2]);
+                            }
+                    } else if constexpr (LG >= 0) {
+                        dense(A.p, xi, j0, f);
+                    } else {
+                        for (int j = j0; j < N; j += dj)
+                            if (j != i) pair_force<R>(xi[0], xi[1], xi[2], *A.at(j, 0), *A.at(j, 1), *A.at(j, 2), k, f);
+                    }
+                });
             }
         }
 #pragma unroll
@@ -360,10 +407,34 @@ __global__ void __launch_bounds__(MAXT)
     }
     if (cs > 1) {
         if (cluster_lost(&s_end, lost || steps < T, cs)) {
-            euler_drain<R>(&s_end, s_sent, shared_addr(s_bar), S.N, S.T, H.cs, H.lg, X);
+            euler_drain<R>(&s_end, s_sent, shared_addr(s_bar), S.N, S.T, H.cs, lanes, X);
             if (tid == 0) atomicExch(err, PAMD_ERR_TIMEOUT);
         }
     }
+}
+
+template <typename R>
+using EulerKernel = void (*)(R*, const R*, LJSysDev<R>, EulerShape, int*, WaitLimit);
+template <typename R, bool LIST, int LG>
+EulerKernel<R> euler_kernel_vr(const EulerShape& h)
+{
+    if (h.nt <= 512)
+        return h.vr == 0   ? lj_euler_kernel<R, LIST, LG, 0, 512>
+               : h.vr == 1 ? lj_euler_kernel<R, LIST, LG, 1, 512>
+                           : lj_euler_kernel<R, LIST, LG, 2, 512>;
+    return h.vr == 0   ? lj_euler_kernel<R, LIST, LG, 0, 1024>
+           : h.vr == 1 ? lj_euler_kernel<R, LIST, LG, 1, 1024>
+                       : lj_euler_kernel<R, LIST, LG, 2, 1024>;
+}
+template <typename R>
+EulerKernel<R> euler_kernel(int N, const EulerShape& h)
+{
+    if (N > kEulerDense) return euler_kernel_vr<R, true, -1>(h);
+    if (h.lg == kOrderedLg) return lj_euler_kernel<R, false, kOrderedLg, 0, 512>;  // (N <= kEulerOrdered)
+    if constexpr (sizeof(R) == 8)
+        return euler_kernel_vr<R, false, -1>(h);
+    else
+        return h.lg == 5 ? euler_kernel_vr<R, false, 5>(h) : h.lg == 4 ? euler_kernel_vr<R, false, 4>(h) : nullptr;
 }
 
 }  // namespace
@@ -388,19 +459,7 @@ cudaError_t launch_lj_euler(R* pos, const R* noise, const void* sys_entry_host, 
     const double rl2 = (double)S.k.rl2, L = (double)S.k.L;
     const EulerShape h = euler_shape<R>(S.N, n_chains, 4.18879020478639 * rl2 * std::sqrt(rl2) * S.N / (L * L * L), sms,
                                         max_smem - 6 * 1024);
-    void (*kern)(R*, const R*, LJSysDev<R>, EulerShape, int*, WaitLimit);
-    if (S.N > kEulerDense)
-        kern = h.nt <= 512 ? lj_euler_kernel<R, true, -1, 512> : lj_euler_kernel<R, true, -1, 1024>;
-    else if constexpr (sizeof(R) == 8)
-        kern = h.lg == kOrderedLg && S.N <= kEulerOrdered ? lj_euler_kernel<R, false, kOrderedLg, 512>
-               : h.nt <= 512                                  ? lj_euler_kernel<R, false, -1, 512>
-                                                              : lj_euler_kernel<R, false, -1, 1024>;
-    else  // N <= kEulerDense: at least four lanes
-        kern = h.lg == 5   ? lj_euler_kernel<R, false, 5, 512>
-               : h.lg == 4 ? lj_euler_kernel<R, false, 4, 512>
-               : h.lg == 3 ? lj_euler_kernel<R, false, 3, 512>
-               : h.lg == 2 ? lj_euler_kernel<R, false, 2, 1024>
-                           : nullptr;
+    const EulerKernel<R> kern = euler_kernel<R>(S.N, h);
     if (!kern) return cudaErrorInvalidValue;
     const size_t smem = h.smem + sizeof(ClusterEnd) + sizeof(int) * (size_t)h.nt;
     if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)

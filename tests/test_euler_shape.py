@@ -1,7 +1,8 @@
 """Launch shapes of the Euler-Maruyama kernel (csrc/euler_shape.cuh), compiled for the host:
 over all particle counts, every CTA of a cluster owns particles (a CTA without any would be
 ordered behind nobody while the others fill its barriers), the shares cover the particles
-once and fit the block, and the block fits the kernel's limits."""
+once and fit the block, the block fits the kernel's limits, and the order of the force sums
+depends on the particle count alone."""
 import os
 import shutil
 import subprocess
@@ -27,9 +28,11 @@ int check(int N, int chains, int sms)
             const int n = euler_first(N, h.cs, r + 1) - euler_first(N, h.cs, r);
             ok = ok && n >= 1 && n <= h.nloc;
         }
-        ok = ok && (h.nloc << h.lg) <= h.nt && h.nt % 32 == 0 && h.nt >= 64 && h.nt <= 1024 && h.lg <= 5;
+        ok = ok && h.lg == euler_shape<R>(N, 1, v, 152, 227 * 1024 - 1024).lg;  // by N alone
+        ok = ok && h.vr >= 0 && h.vr <= 2 && h.vr <= h.lg;
+        ok = ok && (h.nloc << (h.lg - h.vr)) <= h.nt && h.nt % 32 == 0 && h.nt >= 64 && h.nt <= 1024 && h.lg <= 5;
         ok = ok && h.npad >= N && h.npad % (2 << h.lg) == 0 && h.smem <= 227 * 1024 - 1024 && h.smem % 16 == 0;
-        ok = ok && (N <= kEulerDense ? h.cap == 0 && h.lg >= 2 : h.cap >= 1);
+        ok = ok && (N <= kEulerDense ? h.cap == 0 && h.lg == (N <= kEulerOrdered ? 3 : N <= 128 ? 5 : 4) && (N > kEulerOrdered || h.vr == 0) : h.cap >= 1);
         if (!ok) {
             std::printf("N %d chains %d sms %d double %d: cs %d nloc %d lg %d nt %d cap %d npad %d smem %zu\n", N, chains,
                         sms, (int)(sizeof(R) == 8), h.cs, h.nloc, h.lg, h.nt, h.cap, h.npad, h.smem);

@@ -101,3 +101,23 @@ def test_uneven_shares_repeat(pamd, precision, N, B):
     pamd.euler_reference(prob, b, seed=1, counter=2)
     pamd.device_status()
     assert torch.equal(a, b) and bool(torch.isfinite(prob.view(a, 0)).all())
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+@pytest.mark.parametrize("N", [50, 64, 65, 108, 128, 129, 192, 193, 256, 300, 512, 513, 864, 1024])
+def test_paths_do_not_depend_on_the_chains_beside_them(pamd, precision, N):
+    """A chain's path is the same in calls of few chains (clusters of eight CTAs) and many
+    (fewer CTAs a chain, one to four partial sums a lane), bit for bit."""
+    T, L = 6, inputs.box_side(1372, 0.85)
+    x0 = torch.from_numpy(inputs.fcc_lattice(1372, L)[:, :N].copy())
+    paths = []
+    for B in (1, 16, 30, 60, 100):
+        prob = pamd.Problem([pamd.System("lj", N, 3, T, B, box=L, rc=2.5)], 1.0, 1.0, 1e-4, precision)
+        buf = prob.empty("cuda")
+        prob.view(buf, 0)[:, 0].copy_(x0)
+        pamd.euler_reference(prob, buf, seed=1, counter=2)
+        paths.append(prob.view(buf, 0)[:min(B, 16)].clone())
+    pamd.device_status()
+    for p in paths[2:]:
+        assert torch.equal(p, paths[1])
+    assert torch.equal(paths[0], paths[1][:1])
