@@ -33,13 +33,19 @@ struct NvtxRange {
 };
 
 // Host-side fault injection, for tests of the error paths (nothing faults on the
-// device): PAMD_FAULT_INJECT=alloc makes every workspace allocation fail,
-// =launch makes every CUDA call the library checks report failure, =nonfinite
+// device): PAMD_FAULT_INJECT=alloc makes every workspace allocation fail, =alloc:N those of more
+// than N bytes, =launch makes every CUDA call the library checks report failure, =nonfinite
 // flags every action computed as non-finite, =wait:N makes waits run out (wait_limit).
 bool fault_injected(const char* what)
 {
     const char* e = std::getenv("PAMD_FAULT_INJECT");
     return e && std::strcmp(e, what) == 0;
+}
+bool alloc_fault(size_t bytes)
+{
+    const char* e = std::getenv("PAMD_FAULT_INJECT");
+    return e && (std::strcmp(e, "alloc") == 0 ||
+                 (std::strncmp(e, "alloc:", 6) == 0 && bytes > std::strtoull(e + 6, nullptr, 10)));
 }
 
 // The limit of waits between the CTAs of a cluster.  PAMD_FAULT_INJECT=wait:N makes them run out
@@ -100,6 +106,7 @@ struct LJClass {
     long long outer_words = 0;   // 32-bit words of each CTA's outer-list region
     long long outer_off = 0;     // its regions in a lane's set
     LJDoubleShape dbl;           // double precision: capacities of lj_double.cu
+    double dbl_pairs = 0.0;      // pairs a slice it has records for
     int item_off = 0, n_items = 0;  // its items in d_lj_items (cost-sorted)
     int grp_off = 0;             // its items in d_lj_items_grp (grouped by chain)
     std::vector<int> grp_first;  // per global chain c: [grp_first[c], grp_first[c + 1]), relative
@@ -169,11 +176,11 @@ struct Plan {
     int* d_stage_int = nullptr;
     std::map<GraphKey, cudaGraphExec_t> graphs;
     std::vector<void*> allocs;
-    // paired LJ kernel: outer lists, one set per compute lane of one region per CTA
-    uint32_t* d_outer = nullptr;
+    // One set of scratch (a region per CTA) per compute lane: lane 0's with the plan, those of
+    // the host-buffer pipeline on its first use.  Paired LJ kernel: outer lists.
+    uint32_t* d_outer[4] = {};
     long long outer_lane_words = 0;  // 32-bit words of one lane's set
-    // double precision: one set of pair scratch (a region per CTA) per compute lane (those of
-    // the host-buffer pipeline on its first use), and the edge records of every S slot
+    // double precision: pair records, and the edge records of every S slot
     unsigned char* d_dbl_scratch[4] = {};
     size_t dbl_lane_bytes = 0;
     double* d_dbl_edge = nullptr;
@@ -209,7 +216,11 @@ struct Plan {
     {
         void* q = nullptr;
         if (bytes == 0) bytes = 16;
-        if (fault_injected("alloc") || cudaMalloc(&q, bytes) != cudaSuccess) return PAMD_ERR_ALLOC;
+        if (alloc_fault(bytes)) return PAMD_ERR_ALLOC;
+        if (cudaMalloc(&q, bytes) != cudaSuccess) {
+            cudaGetLastError();  // (a later launch would report it)
+            return PAMD_ERR_ALLOC;
+        }
         allocs.push_back(q);
         *p = reinterpret_cast<T*>(q);
         return PAMD_OK;
@@ -622,6 +633,7 @@ int build_plan(const pamd_problem* p, Plan** out)
                         const double L = si.pot.box, f = 4.18879020478639 * si.pot.rc * si.pot.rc * si.pot.rc / (L * L * L);
                         pairs = std::max(pairs, 0.5 * si.N * si.N * f);
                     }
+                    C.dbl_pairs = pairs;
                     C.dbl = lj_double_shape(nmax, pairs, max_dynamic_smem() - 1024);
                 }
                 C.smem = P->lj_paired ? lj_paired_smem_bytes(NT, cap_used, C.pipe)
@@ -809,27 +821,46 @@ int build_plan(const pamd_problem* p, Plan** out)
             }
             if (P->lj_paired) {
                 P->n_lanes = pipeline_lanes();
-                for (auto& C : P->lj_cls) {
-                    int ocap = 2;
+                // (on a nearly full device shorter lists: an overflowing one costs time only)
+                for (bool shorter = true; shorter;) {
+                    P->outer_lane_words = 0;
+                    shorter = false;
+                    for (auto& C : P->lj_cls) {
+                        int ocap = 2;
+                        for (auto& si : P->sys)
+                            if (si.kind == PAMD_LJ && &P->lj_cls[si.lj_class] == &C)
+                                ocap = std::max(ocap, si.tune.outer_cap);
+                        shorter = shorter || ocap > 2;
+                        C.outer_words = (long long)(ocap / 2) * C.NT;
+                        C.outer_off = P->outer_lane_words;  // (the classes of a lane may run at the same time)
+                        P->outer_lane_words += (long long)std::max(C.grid_grad, C.grid_nograd) * C.outer_words;
+                    }
+                    if (!(rc0 = P->alloc(&P->d_outer[0], sizeof(uint32_t) * P->outer_lane_words))) break;
                     for (auto& si : P->sys)
-                        if (si.kind == PAMD_LJ && &P->lj_cls[si.lj_class] == &C)
-                            ocap = std::max(ocap, si.tune.outer_cap);
-                    C.outer_words = (long long)(ocap / 2) * C.NT;
-                    C.outer_off = P->outer_lane_words;  // (the classes of a lane may run at the same time)
-                    P->outer_lane_words += (long long)std::max(C.grid_grad, C.grid_nograd) * C.outer_words;
+                        if (si.kind == PAMD_LJ) si.tune.outer_cap = std::max(2, (si.tune.outer_cap / 2) & ~1);
                 }
-                if ((rc0 = P->alloc(&P->d_outer, sizeof(uint32_t) * P->n_lanes * P->outer_lane_words)))
-                    return rc0;
+                if (rc0) return rc0;
             }
             if (P->fp64) {
                 P->n_lanes = pipeline_lanes();
                 int edge = 0;
-                for (auto& C : P->lj_cls) {
-                    P->dbl_lane_bytes = std::max(P->dbl_lane_bytes,
-                                                 C.dbl.scratch * (size_t)std::max(C.grid_grad, C.grid_nograd));
-                    edge = std::max(edge, C.dbl.edge_doubles);
+                // (on a nearly full device room for fewer records: the other pairs are evaluated again)
+                for (bool fewer = true; fewer;) {
+                    P->dbl_lane_bytes = 0;
+                    fewer = false;
+                    for (auto& C : P->lj_cls) {
+                        P->dbl_lane_bytes = std::max(P->dbl_lane_bytes,
+                                                     C.dbl.scratch * (size_t)std::max(C.grid_grad, C.grid_nograd));
+                        edge = std::max(edge, C.dbl.edge_doubles);
+                        fewer = fewer || C.dbl_pairs >= 1.0;
+                    }
+                    if (!(rc0 = P->alloc(&P->d_dbl_scratch[0], P->dbl_lane_bytes))) break;
+                    for (auto& C : P->lj_cls) {
+                        C.dbl_pairs *= 0.5;
+                        C.dbl = lj_double_shape(C.nmax, C.dbl_pairs, max_dynamic_smem() - 1024);
+                    }
                 }
-                if ((rc0 = P->alloc(&P->d_dbl_scratch[0], P->dbl_lane_bytes))) return rc0;
+                if (rc0) return rc0;
                 if ((rc0 = P->alloc(&P->d_dbl_edge, sizeof(double) * (size_t)edge * slot))) return rc0;
             }
             if (P->fp64)
@@ -979,7 +1010,7 @@ int run_action(const pamd_problem* p, Plan* P, const R* pos, R* grad, double* S_
                 launched = true;
                 return launch_lj_paired(items, n, P->d_lj_sys, (const float*)pos, (float*)grad,
                                         P->d_part_S, counter + (classes ? k : 0), C.NT, C.smem, g, with_grad,
-                                        C.pipe, P->d_outer + lane * P->outer_lane_words + C.outer_off,
+                                        C.pipe, P->d_outer[lane] + C.outer_off,
                                         C.outer_words, st, !classes, follow, (const float*)hs2, overlap);
             }
             if constexpr (std::is_same<R, double>::value)
@@ -1122,8 +1153,14 @@ int path_update_pipelined(const pamd_problem* prob, Plan* P, void* pos, void* gr
         PAMD_CUDA_TRY(cudaStreamCreateWithFlags(&c, cudaStreamNonBlocking));
         P->s_cmp.push_back(c);
     }
-    for (int l = 1; P->dbl_lane_bytes && l < P->n_lanes; ++l)
-        if (!P->d_dbl_scratch[l] && (rc = P->alloc(&P->d_dbl_scratch[l], P->dbl_lane_bytes))) return rc;
+    // the scratch of lanes 1..; without it (a nearly full device) the lanes there are
+    int lanes = 1;
+    for (; lanes < P->n_lanes; ++lanes) {
+        if (P->dbl_lane_bytes && !P->d_dbl_scratch[lanes] && P->alloc(&P->d_dbl_scratch[lanes], P->dbl_lane_bytes)) break;
+        if (P->outer_lane_words && !P->d_outer[lanes] &&
+            P->alloc(&P->d_outer[lanes], sizeof(uint32_t) * P->outer_lane_words))
+            break;
+    }
     if (!P->d_chunk_counters && (rc = P->alloc(&P->d_chunk_counters, 2 * sizeof(int) * kMaxChunks)))
         return rc;
     // events: per chunk inputs-copied, updated, results-copied; start and end (timed,
@@ -1143,7 +1180,7 @@ int path_update_pipelined(const pamd_problem* prob, Plan* P, void* pos, void* gr
     int K = std::min(nc, kMaxChunks);
     for (const auto& C : P->lj_cls)
         if (P->lj_paired)
-            K = std::max(1, std::min(K, (int)((long long)P->n_lanes * C.n_items / std::max(1, C.grid_grad))));
+            K = std::max(1, std::min(K, (int)((long long)lanes * C.n_items / std::max(1, C.grid_grad))));
     long long total = 0;
     for (int c = 0; c < nc; ++c) total += e_end(c) - e_begin(c);
     std::vector<int> cut(K + 1, nc);
@@ -1174,7 +1211,7 @@ int path_update_pipelined(const pamd_problem* prob, Plan* P, void* pos, void* gr
         if (hn)
             PAMD_CUDA_TRY(cudaMemcpyAsync(dnacc + c0, n_accepted + c0, sizeof(int) * (c1 - c0),
                                           cudaMemcpyHostToDevice, P->s_in));
-        const int lane = k % P->n_lanes;
+        const int lane = k % lanes;
         cudaStream_t cs = lane ? P->s_cmp[lane - 1] : st;
         PAMD_CUDA_TRY(cudaEventRecord(P->events[3 * k], P->s_in));
         PAMD_CUDA_TRY(cudaStreamWaitEvent(cs, P->events[3 * k], 0));

@@ -92,3 +92,73 @@ def test_nonfinite_flag_is_reported_once(pamd, fault):
     pamd.device_status()  # cleared
     pamd.action_grad(prob, buf)
     pamd.device_status()  # a clean call reports nothing
+
+
+@pytest.mark.parametrize("precision,limit", [("fp32", 1 << 21), ("fp32", 1 << 19), ("fp64", 1 << 26), ("fp64", 1 << 24)])
+def test_less_scratch_gives_the_same_results(pamd, fault, precision, limit):
+    """Neighbour lists and pair records that do not fit the device become shorter, and the
+    host-buffer pipeline runs with the lanes it has scratch for; the results stay."""
+    N, T, B, L = 200, 160, 4, inputs.box_side(256, 0.85)
+    prob = pamd.Problem([pamd.System("lj", N, 3, T, B, box=L, rc=2.5)], 1.0, 1.0, 1e-4, precision)
+    buf = prob.empty("cuda")
+    prob.view(buf, 0)[:, 0].copy_(torch.from_numpy(inputs.fcc_lattice(256, L)[:, :N].copy()))
+    pamd.euler_reference(prob, buf, seed=4)
+
+    def update():
+        host = [t.cpu() for t in (buf, g, S)]
+        pamd.path_update(prob, *host, 1e-7, 2, seed=3)
+        return host
+
+    pamd.release_cache()
+    S, g = pamd.action_grad(prob, buf)
+    want = update()
+    pamd.release_cache()
+    fault("alloc:%d" % limit)
+    S1, g1 = pamd.action_grad(prob, buf)
+    torch.cuda.synchronize()
+    assert torch.equal(S, S1) and torch.equal(prob.view(g, 0), prob.view(g1, 0))
+    fault(None)  # the plan has its short lists; the staging buffers fit, two more lanes do not
+    pamd.action_grad(prob, buf.cpu())
+    got = update()
+    assert all(torch.equal(a, b) for a, b in zip(got, want))
+    pamd.release_cache()
+
+
+def test_pipeline_without_scratch_for_its_lanes(pamd, fault):
+    N, T, B, L = 200, 160, 4, inputs.box_side(256, 0.85)
+    prob = pamd.Problem([pamd.System("lj", N, 3, T, B, box=L, rc=2.5)], 1.0, 1.0, 1e-4, "fp64")
+    buf = prob.empty("cuda")
+    prob.view(buf, 0)[:, 0].copy_(torch.from_numpy(inputs.fcc_lattice(256, L)[:, :N].copy()))
+    pamd.euler_reference(prob, buf, seed=4)
+    out = []
+    for limit in (None, "alloc:%d" % (1 << 24)):  # (the path takes 3.1 MB, a lane's scratch 110 MB)
+        pamd.release_cache()
+        S, g = pamd.action_grad(prob, buf)  # lane 0's scratch
+        host = [t.cpu() for t in (buf, g, S)]
+        fault(limit)
+        pamd.path_update(prob, *host, 1e-7, 2, seed=3)
+        fault(None)
+        out.append(host)
+    assert all(torch.equal(a, b) for a, b in zip(*out))
+    pamd.release_cache()
+
+
+def test_device_memory_of_a_plan(pamd):
+    """A plan that the host-buffer pipeline has not used holds one lane's lists: about 70 MB
+    for 500 particles on 152 SMs, not three times that."""
+    L = inputs.box_side(500, 0.85)
+    small = pamd.Problem([pamd.System("lj", 500, 3, 16, 1, box=L, rc=2.5)], 1.0, 1.0, 1e-4)
+    prob = pamd.Problem([pamd.System("lj", 500, 3, 4096, 8, box=L, rc=2.5)], 1.0, 1.0, 1e-4)
+    buf, sbuf = torch.zeros(prob.span, device="cuda"), torch.zeros(small.span, device="cuda")
+    for p, b in ((small, sbuf), (prob, buf)):
+        p.view(b, 0)[:] = torch.from_numpy(inputs.fcc_lattice(500, L)).float()[None, None].cuda()
+    pamd.release_cache()
+    pamd.action(small, sbuf)
+    S = torch.empty(8, dtype=torch.float64, device="cuda")
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    pamd.action(prob, buf, S)
+    torch.cuda.synchronize()
+    used = free - torch.cuda.mem_get_info()[0]
+    pamd.release_cache()
+    assert used < 100 << 20
