@@ -657,9 +657,43 @@ __device__ __forceinline__ bool window_shared_shift(const LJSysDev<float>& S, co
     return S.shared_shift && k.rcm + 4.0f * __int_as_float(*dmax_bits) <= k.hb;
 }
 
+// The |r|^2 sums of an item's parts.  `add` takes the terms of steps a, a + 1 (one thread per
+// particle), `flush` (every thread) writes the parts that end with these steps.
+struct PartSums {
+    const LJItem* item;            // (in global memory: registers are short)
+    double acc = 0.0, next = 0.0;  // of the part of step a, and of a part that begins with a + 1
+    int bound;                     // first step of the next part
+    __device__ __forceinline__ explicit PartSums(const LJItem* I) : item(I), bound(I->t0 + I->sub) {}
+    __device__ __forceinline__ void add(int a, bool real_a, bool hasb, float ta, float tb)
+    {
+        next = 0.0;
+        if (real_a) acc += (double)ta;
+        if (hasb) {
+            if (a + 1 == bound)
+                next = (double)tb;
+            else
+                acc += (double)tb;
+        }
+    }
+    __device__ __forceinline__ void put(double* partials, double* red)
+    {
+        const double tot = block_sum(acc, red);
+        if (threadIdx.x == 0) partials[item->slot + (bound - item->t0) / item->sub - 1] = tot;
+    }
+    __device__ __forceinline__ void flush(int a, int t1, double* partials, double* red)
+    {
+        while (bound <= a + 2 && bound < t1) {
+            put(partials, red);
+            acc = next;
+            next = 0.0;
+            bound += item->sub;
+        }
+    }
+};
+
 // One work item: steps [t0, t1) of one chain.
 template <bool GRAD, int NMAX, bool HS>
-__device__ __forceinline__ void paired_item(const LJItem& I, const LJSysDev<float>& S,
+__device__ __forceinline__ void paired_item(const LJItem* Ip, const LJItem& I, const LJSysDev<float>& S,
                                             unsigned char* smem, const float* __restrict__ pos,
                                             float* __restrict__ grad, double* __restrict__ partials,
                                             double* red, uint32_t* outer, int* dmax_bits,
@@ -703,7 +737,7 @@ __device__ __forceinline__ void paired_item(const LJItem& I, const LJSysDev<floa
     __syncthreads();
 
     float rpx = 0.0f, rpy = 0.0f, rpz = 0.0f;  // r_{a-1}
-    double acc = 0.0;
+    PartSums sums(Ip);
     const int W = max(2, S.window);
     int win_end = ts;  // slices [.., win_end) are covered by the current list
     bool sk = false;   // the current window allows one image shift per entry
@@ -766,10 +800,10 @@ __device__ __forceinline__ void paired_item(const LJItem& I, const LJSysDev<floa
                     P.rxy(8 * i) = make_float4(rx.x, rx.y, ry.x, ry.y);
                     P.rz(8 * i) = rz;
                 }
-                if (real_a) acc += (double)sq3(rx.x, ry.x, rz.x);
-                if (hasb) acc += (double)sq3(rx.y, ry.y, rz.y);
+                sums.add(a, real_a, hasb, sq3(rx.x, ry.x, rz.x), sq3(rx.y, ry.y, rz.y));
             }
         }
+        sums.flush(a, t1, partials, red);
         if (GRAD) {
             __syncthreads();
             float2 hx, hy, hz;
@@ -816,8 +850,7 @@ __device__ __forceinline__ void paired_item(const LJItem& I, const LJSysDev<floa
         }
     }
     if (HS && __syncthreads_or(ov) && threadIdx.x == 0) atomicOr(overlap + S.chain0 + I.chain, 1);
-    const double tot = block_sum(acc, red);
-    if (threadIdx.x == 0) partials[I.slot] = tot;
+    sums.put(partials, red);
 }
 
 // One work item, action and gradient, pipelined over step pairs: the list walk of
@@ -827,7 +860,7 @@ __device__ __forceinline__ void paired_item(const LJItem& I, const LJSysDev<floa
 // windows are at least 4 steps long and overlap by one pair.  Every sum is the
 // same as in paired_item.
 template <int NMAX, bool HS>
-__device__ __forceinline__ void paired_item_pipe(const LJItem& I, const LJSysDev<float>& S,
+__device__ __forceinline__ void paired_item_pipe(const LJItem* Ip, const LJItem& I, const LJSysDev<float>& S,
                                                  unsigned char* smem, const float* __restrict__ pos,
                                                  float* __restrict__ grad,
                                                  double* __restrict__ partials, double* red,
@@ -904,13 +937,14 @@ __device__ __forceinline__ void paired_item_pipe(const LJItem& I, const LJSysDev
         rz = fma2(na, fz, sub2(pk(pz.y, zn), pz));
         if (!hb) rx.y = ry.y = rz.y = 0.0f;
     };
-    double acc = 0.0;
+    PartSums sums(Ip);
     auto account = [&](int a, float2 rx, float2 ry, float2 rz) {
-        if (!lead) return;
-        P.rxy(8 * i) = make_float4(rx.x, rx.y, ry.x, ry.y);
-        P.rz(8 * i) = rz;
-        if (a >= t0) acc += (double)sq3(rx.x, ry.x, rz.x);
-        if (a + 1 < t1) acc += (double)sq3(rx.y, ry.y, rz.y);
+        if (lead) {
+            P.rxy(8 * i) = make_float4(rx.x, rx.y, ry.x, ry.y);
+            P.rz(8 * i) = rz;
+            sums.add(a, a >= t0, a + 1 < t1, sq3(rx.x, ry.x, rz.x), sq3(rx.y, ry.y, rz.y));
+        }
+        sums.flush(a, t1, partials, red);
     };
 
     // Item-wide outer list.
@@ -1028,8 +1062,7 @@ __device__ __forceinline__ void paired_item_pipe(const LJItem& I, const LJSysDev
         }
     }
     if (HS && __syncthreads_or(ov) && threadIdx.x == 0) atomicOr(overlap + S.chain0 + I.chain, 1);
-    const double tot = block_sum(acc, red);
-    if (threadIdx.x == 0) partials[I.slot] = tot;
+    sums.put(partials, red);
 }
 
 // Persistent grid: each CTA takes items from *counter until none is left.
@@ -1062,11 +1095,11 @@ __global__ void __launch_bounds__(MAXT, 1)
         const LJItem I = items[it];
         const LJSysDev<float> S = systems[I.sys];
         if (GRAD && PIPE)
-            paired_item_pipe<MAXT, HS>(I, S, smem_raw, pos, grad, partials, red,
+            paired_item_pipe<MAXT, HS>(items + it, I, S, smem_raw, pos, grad, partials, red,
                                        outer + (long long)blockIdx.x * outer_words, &s_dmax, hs2,
                                        overlap);
         else
-            paired_item<GRAD, MAXT, HS>(I, S, smem_raw, pos, grad, partials, red,
+            paired_item<GRAD, MAXT, HS>(items + it, I, S, smem_raw, pos, grad, partials, red,
                                         outer + (long long)blockIdx.x * outer_words, &s_dmax, hs2,
                                         overlap);
     }

@@ -69,6 +69,7 @@ WaitLimit wait_limit()
 
 struct LJTune {
     int tile_steps = 0, tpp = 0, maxnb = 0;
+    int parts = 1;      // parts of an item with an S slot each
     double list = 0.0;  // expected list entries of a particle
     double skin = -1.0;
     int window = 0;     // paired kernel: steps per neighbour-list window
@@ -101,6 +102,7 @@ struct SysInfo {
 // leaving most of a 1024-thread block idle.
 struct LJClass {
     int NT = 0, nmax = 0, grid_grad = 0, grid_nograd = 0;
+    int grid_full = 0;           // CTAs that fit the GPU (gradient)
     bool pipe = false;           // gradient pass pipelined over step pairs
     size_t smem = 0;
     long long outer_words = 0;   // 32-bit words of each CTA's outer-list region
@@ -647,7 +649,7 @@ int build_plan(const pamd_problem* p, Plan** out)
                                             : lj_blocks_per_sm<float>(NT, C.smem, false);
                 if (bg <= 0 || bn <= 0) return PAMD_ERR_UNSUPPORTED;
                 bg_cls[k] = bg;
-                C.grid_grad = bg * sms;  // trimmed to the item count below
+                C.grid_grad = C.grid_full = bg * sms;  // trimmed to the item count below
                 C.grid_nograd = bn * sms;
             }
             // Double precision: a step costs tens of microseconds and an item nothing more
@@ -740,8 +742,19 @@ int build_plan(const pamd_problem* p, Plan** out)
                             if (r * c < 0.99 * rounds * hi) rounds = r, hi = c;
                         }
                     }
+                    // The host-buffer pipeline updates chunks of chains, which need enough items
+                    // for the GPU: where these long ones do not make six chunks (one for every
+                    // chain) it takes parts of about 32 steps, each with a sum of its own (at most
+                    // 3 % more in an item).  N = 500, 8 x 4096 steps with host buffers: 5.8 ms in
+                    // three chunks of long items, 9.3 in eight, 4.3 in eight of parts; 8 x 16384:
+                    // 15.9 in eight of long items, 17.0 of parts.  (Unlike systems keep the long items:
+                    // 12 systems of N = 64..864 take 2.7 ms, in parts 3.0.)
+                    const bool in_parts = in.size() == 1 && chain > 1 && pipeline_lanes() * rounds < std::min(chain, 6);
                     for (size_t q = 0; q < in.size(); ++q) {
-                        in[q]->tune.tile_steps = tile(q, hi);
+                        LJTune& t = in[q]->tune;
+                        t.tile_steps = tile(q, hi);
+                        t.parts = in_parts ? std::max(1, (t.tile_steps + 16) / 32) : 1;
+                        t.tile_steps = (t.tile_steps + t.parts - 1) / t.parts * t.parts;
                         const SysInfo& si = *in[q];
                         in[q]->tune.outer_cap = lj_outer_cap(si.N, si.pot, std::sqrt(2.0 * p->D * p->dt),
                                                              si.tune.tile_steps, si.tune.tpp);
@@ -749,65 +762,81 @@ int build_plan(const pamd_problem* p, Plan** out)
                 }
             }
             // Items of every system (S slots in system order), with their cost.
-            std::vector<std::vector<LJItem>> sys_items(P->sys.size());
-            std::vector<std::vector<double>> sys_cost(P->sys.size());
+            struct SysItems {
+                std::vector<LJItem> items;
+                std::vector<double> cost;
+            };
+            std::vector<SysItems> sys_items(P->sys.size()), sys_parts(P->sys.size());
             for (int q = 0; q < (int)P->sys.size(); ++q) {
                 SysInfo& si = P->sys[q];
                 if (si.kind != PAMD_LJ) continue;
-                si.n_tiles = (si.T - si.halo_lo + si.tune.tile_steps - 1) / si.tune.tile_steps;
+                const int own = si.T - si.halo_lo, sub = si.tune.tile_steps / si.tune.parts;
+                const int n_sub = (own + sub - 1) / sub;
+                si.n_tiles = (own + si.tune.tile_steps - 1) / si.tune.tile_steps;
                 si.slot0 = slot;
                 for (int b = 0; b < si.chains; ++b) {
-                    const int c = si.chain0 + b;
-                    Sslots[c].begin = slot + b * si.n_tiles;
-                    Sslots[c].end = slot + (b + 1) * si.n_tiles;
+                    const int c = si.chain0 + b, slot_c = slot + b * n_sub;
+                    Sslots[c].begin = slot_c;
+                    Sslots[c].end = slot_c + n_sub;
                     P->lj_chain_count[c] = si.n_tiles;
                     P->lj_chain_class[c] = si.lj_class;
-                    for (int tl = 0; tl < si.n_tiles; ++tl) {
-                        LJItem it;
-                        it.sys = si.lj_index;
-                        it.chain = b;
-                        it.t0 = si.halo_lo + tl * si.tune.tile_steps;  // owned steps only
-                        it.t1 = std::min(si.T, it.t0 + si.tune.tile_steps);
-                        it.slot = slot + b * si.n_tiles + tl;
-                        sys_items[q].push_back(it);
-                        sys_cost[q].push_back(lj_step_cost(si.N, si.tune) * (it.t1 - it.t0) + lj_item_cost(si.N, si.tune));
+                    // items of `parts` parts, and every part as an item
+                    for (int n : {si.tune.parts, 1}) {
+                        SysItems& out = n == si.tune.parts ? sys_items[q] : sys_parts[q];
+                        for (int tl = 0; tl * n < n_sub; ++tl) {
+                            LJItem it;
+                            it.sys = si.lj_index;
+                            it.chain = b;
+                            it.t0 = si.halo_lo + tl * n * sub;  // owned steps only
+                            it.t1 = std::min(si.T, it.t0 + n * sub);
+                            it.slot = slot_c + tl * n;
+                            it.sub = sub;
+                            out.items.push_back(it);
+                            out.cost.push_back(lj_step_cost(si.N, si.tune) * (it.t1 - it.t0) + lj_item_cost(si.N, si.tune));
+                        }
+                        if (si.tune.parts == 1) break;  // (the same)
                     }
                 }
-                slot += si.chains * si.n_tiles;
+                slot += si.chains * n_sub;
             }
-            // Per class: its items (largest first unless one chain per launch) and a
-            // copy grouped by chain (chains in order, each chain's items largest first)
-            // for launches over a range of chains.
+            // Per class: its items (largest first unless one chain per launch) and, for launches
+            // over a range of chains, the parts grouped by chain (chains in order, each chain's
+            // items largest first).
             for (int k = 0; k < (int)P->lj_cls.size(); ++k) {
                 LJClass& C = P->lj_cls[k];
-                std::vector<LJItem> ci;
-                std::vector<double> cc;
-                std::vector<int> cchain;
-                for (int q = 0; q < (int)P->sys.size(); ++q) {
-                    const SysInfo& si = P->sys[q];
-                    if (si.kind != PAMD_LJ || si.lj_class != k) continue;
-                    for (size_t m = 0; m < sys_items[q].size(); ++m) {
-                        const int c = si.chain0 + sys_items[q][m].chain;
-                        if (P->lj_chain_first[c] < 0) P->lj_chain_first[c] = (int)(items.size() + ci.size());
-                        ci.push_back(sys_items[q][m]);
-                        cc.push_back(sys_cost[q][m]);
-                        cchain.push_back(c);
+                auto gather = [&](bool parts, std::vector<LJItem>& ci, std::vector<double>& cc, std::vector<int>& cchain) {
+                    for (int q = 0; q < (int)P->sys.size(); ++q) {
+                        const SysInfo& si = P->sys[q];
+                        if (si.kind != PAMD_LJ || si.lj_class != k) continue;
+                        const SysItems& from = parts && si.tune.parts > 1 ? sys_parts[q] : sys_items[q];
+                        for (size_t m = 0; m < from.items.size(); ++m) {
+                            const int c = si.chain0 + from.items[m].chain;
+                            if (!parts && P->lj_chain_first[c] < 0) P->lj_chain_first[c] = (int)(items.size() + ci.size());
+                            ci.push_back(from.items[m]);
+                            cc.push_back(from.cost[m]);
+                            cchain.push_back(c);
+                        }
                     }
-                }
-                std::vector<int> ord(ci.size());
-                for (size_t q = 0; q < ord.size(); ++q) ord[q] = (int)q;
+                    std::vector<int> ord(ci.size());
+                    for (size_t q = 0; q < ord.size(); ++q) ord[q] = (int)q;
+                    return ord;
+                };
+                std::vector<LJItem> ci, pi;
+                std::vector<double> cc, pc;
+                std::vector<int> cchain, pchain;
+                std::vector<int> ord = gather(true, pi, pc, pchain);
                 std::stable_sort(ord.begin(), ord.end(), [&](int x, int y) {
-                    return cchain[x] != cchain[y] ? cchain[x] < cchain[y] : cc[x] > cc[y];
+                    return pchain[x] != pchain[y] ? pchain[x] < pchain[y] : pc[x] > pc[y];
                 });
                 C.grp_off = (int)grouped.size();
                 C.grp_first.assign(chain + 1, 0);
                 for (int q : ord) {
-                    grouped.push_back(ci[q]);
-                    ++C.grp_first[cchain[q] + 1];
+                    grouped.push_back(pi[q]);
+                    ++C.grp_first[pchain[q] + 1];
                 }
                 for (int c = 0; c < chain; ++c) C.grp_first[c + 1] += C.grp_first[c];
+                ord = gather(false, ci, cc, cchain);
                 if (!one) {  // largest items first
-                    for (size_t q = 0; q < ord.size(); ++q) ord[q] = (int)q;
                     std::stable_sort(ord.begin(), ord.end(), [&](int x, int y) { return cc[x] > cc[y]; });
                     std::vector<LJItem> sorted;
                     for (int q : ord) sorted.push_back(ci[q]);
@@ -1180,7 +1209,7 @@ int path_update_pipelined(const pamd_problem* prob, Plan* P, void* pos, void* gr
     int K = std::min(nc, kMaxChunks);
     for (const auto& C : P->lj_cls)
         if (P->lj_paired)
-            K = std::max(1, std::min(K, (int)((long long)lanes * C.n_items / std::max(1, C.grid_grad))));
+            K = std::max(1, std::min(K, (int)((long long)lanes * C.grp_first.back() / std::max(1, std::min(C.grp_first.back(), C.grid_full)))));
     long long total = 0;
     for (int c = 0; c < nc; ++c) total += e_end(c) - e_begin(c);
     std::vector<int> cut(K + 1, nc);

@@ -443,10 +443,11 @@ struct LJSysDev {
     LJK<R> k;
 };
 
-// A work item: steps [t0, t1) of one chain of one system; its |r|^2 sum goes
-// to partials[slot].
+// A work item: steps [t0, t1) of one chain of one system.  The |r|^2 sums of its parts of `sub`
+// steps go to partials[slot], partials[slot + 1], ... (paired kernel; one part elsewhere), so
+// an action does not depend on how many parts an item has.
 struct LJItem {
-    int sys, chain, t0, t1, slot;
+    int sys, chain, t0, t1, slot, sub;
 };
 
 // Shared memory of the LJ action kernel: three slices of nmax particles and a

@@ -50,3 +50,32 @@ def test_automatic_items_equal_items_of_32_steps(pamd, shape):
     # sums of at most 300 items a chain in FP64
     for a in (S, S1):
         assert float(((a - S32).abs() / S32.abs()).max()) < 1e-13
+
+
+@pytest.mark.parametrize("shapes", [[(64, 2001, 8)], [(600, 2503, 4)], [(96, 1777, 5), (560, 1333, 6)]])
+def test_parts_of_long_items(pamd, shapes):
+    """Items of several parts (device buffers) and the parts as items of their own (chunks of
+    chains in the host-buffer pipeline): the same action, update and acceptance, bit for bit."""
+    systems = []
+    for N, T, B in shapes:
+        L = inputs.box_side(max(N, 108), 0.85)
+        systems.append(pamd.System("lj", N, 3, T, B, box=L, rc=2.3))
+    prob = pamd.Problem(systems, 1.0, 1.0, 1e-4)
+    buf = prob.empty("cuda")
+    for q, s in enumerate(systems):
+        prob.view(buf, q)[:, 0].copy_(torch.from_numpy(inputs.fcc_lattice(s.N, s.box)))
+    pamd.euler_reference(prob, buf, seed=6)
+    S, g = pamd.action_grad(prob, buf)
+    assert torch.equal(S, pamd.action(prob, buf))
+    host = [t.cpu() for t in (buf, g, S)]
+    nacc = [torch.zeros(prob.n_chains, dtype=torch.int32, device=d) for d in ("cuda", "cpu")]
+    la = [torch.zeros(prob.n_chains, dtype=torch.float64, device=d) for d in ("cuda", "cpu")]
+    h = 2e-7
+    pamd.path_update(prob, buf, g, S, h, 2, seed=3, n_accepted=nacc[0], log_alpha=la[0])
+    pamd.path_update(prob, *host, h, 2, seed=3, n_accepted=nacc[1], log_alpha=la[1])
+    torch.cuda.synchronize()
+    assert torch.equal(nacc[0].cpu(), nacc[1]) and torch.equal(la[0].cpu(), la[1])
+    assert torch.equal(S.cpu(), host[2])
+    for q in range(len(systems)):
+        assert torch.equal(prob.view(buf, q).cpu(), prob.view(host[0], q))
+        assert torch.equal(prob.view(g, q).cpu(), prob.view(host[1], q))
