@@ -658,41 +658,48 @@ __device__ __forceinline__ bool window_shared_shift(const LJSysDev<float>& S, co
 }
 
 // The |r|^2 sums of an item's parts.  `add` takes the terms of steps a, a + 1 (one thread per
-// particle), `flush` (every thread) writes the parts that end with these steps.
+// particle), `flush` (every thread) writes the parts that end with these steps.  PARTS: some item
+// has several (looking for their ends takes 1 to 4 % of the action of small systems).
+template <bool PARTS>
 struct PartSums {
     const LJItem* item;            // (in global memory: registers are short)
     double acc = 0.0, next = 0.0;  // of the part of step a, and of a part that begins with a + 1
-    int bound;                     // first step of the next part
-    __device__ __forceinline__ explicit PartSums(const LJItem* I) : item(I), bound(I->t0 + I->sub) {}
-    __device__ __forceinline__ void add(int a, bool real_a, bool hasb, float ta, float tb)
+    int bound;                     // end of the part of step a
+    __device__ __forceinline__ explicit PartSums(const LJItem* I) : item(I), bound(min(I->t0 + I->sub, I->t1)) {}
+    // (the squares are formed where they are added: before the tests they cost the action of small
+    // systems 2 to 4 %)
+    __device__ __forceinline__ void add(int a, bool real_a, bool hasb, float2 rx, float2 ry, float2 rz)
     {
         next = 0.0;
-        if (real_a) acc += (double)ta;
-        if (hasb) {
-            if (a + 1 == bound)
-                next = (double)tb;
-            else
-                acc += (double)tb;
-        }
+        if (real_a) acc += (double)sq3(rx.x, ry.x, rz.x);
+        if (PARTS && hasb && a + 1 == bound)
+            next = (double)sq3(rx.y, ry.y, rz.y);
+        else if (hasb)
+            acc += (double)sq3(rx.y, ry.y, rz.y);
     }
     __device__ __forceinline__ void put(double* partials, double* red)
     {
         const double tot = block_sum(acc, red);
-        if (threadIdx.x == 0) partials[item->slot + (bound - item->t0) / item->sub - 1] = tot;
+        if (threadIdx.x == 0) partials[item->slot + (PARTS ? (bound - item->t0 - 1) / item->sub : 0)] = tot;
     }
-    __device__ __forceinline__ void flush(int a, int t1, double* partials, double* red)
+    __device__ __forceinline__ void flush(int a, double* partials, double* red)
     {
-        while (bound <= a + 2 && bound < t1) {
+        while (PARTS && bound <= a + 2) {
             put(partials, red);
             acc = next;
             next = 0.0;
-            bound += item->sub;
+            bound = bound == item->t1 ? 0x7fffffff : min(bound + item->sub, item->t1);
         }
+    }
+    // (the last part of several has been written by flush)
+    __device__ __forceinline__ void finish(double* partials, double* red)
+    {
+        if (!PARTS) put(partials, red);
     }
 };
 
 // One work item: steps [t0, t1) of one chain.
-template <bool GRAD, int NMAX, bool HS>
+template <bool GRAD, int NMAX, bool HS, bool PARTS>
 __device__ __forceinline__ void paired_item(const LJItem* Ip, const LJItem& I, const LJSysDev<float>& S,
                                             unsigned char* smem, const float* __restrict__ pos,
                                             float* __restrict__ grad, double* __restrict__ partials,
@@ -737,7 +744,7 @@ __device__ __forceinline__ void paired_item(const LJItem* Ip, const LJItem& I, c
     __syncthreads();
 
     float rpx = 0.0f, rpy = 0.0f, rpz = 0.0f;  // r_{a-1}
-    PartSums sums(Ip);
+    PartSums<PARTS> sums(Ip);
     const int W = max(2, S.window);
     int win_end = ts;  // slices [.., win_end) are covered by the current list
     bool sk = false;   // the current window allows one image shift per entry
@@ -800,10 +807,10 @@ __device__ __forceinline__ void paired_item(const LJItem* Ip, const LJItem& I, c
                     P.rxy(8 * i) = make_float4(rx.x, rx.y, ry.x, ry.y);
                     P.rz(8 * i) = rz;
                 }
-                sums.add(a, real_a, hasb, sq3(rx.x, ry.x, rz.x), sq3(rx.y, ry.y, rz.y));
+                sums.add(a, real_a, hasb, rx, ry, rz);
             }
         }
-        sums.flush(a, t1, partials, red);
+        sums.flush(a, partials, red);
         if (GRAD) {
             __syncthreads();
             float2 hx, hy, hz;
@@ -850,7 +857,7 @@ __device__ __forceinline__ void paired_item(const LJItem* Ip, const LJItem& I, c
         }
     }
     if (HS && __syncthreads_or(ov) && threadIdx.x == 0) atomicOr(overlap + S.chain0 + I.chain, 1);
-    sums.put(partials, red);
+    sums.finish(partials, red);
 }
 
 // One work item, action and gradient, pipelined over step pairs: the list walk of
@@ -859,7 +866,7 @@ __device__ __forceinline__ void paired_item(const LJItem* Ip, const LJItem& I, c
 // positions of two pairs are resident.  Window lists cover two consecutive pairs;
 // windows are at least 4 steps long and overlap by one pair.  Every sum is the
 // same as in paired_item.
-template <int NMAX, bool HS>
+template <int NMAX, bool HS, bool PARTS>
 __device__ __forceinline__ void paired_item_pipe(const LJItem* Ip, const LJItem& I, const LJSysDev<float>& S,
                                                  unsigned char* smem, const float* __restrict__ pos,
                                                  float* __restrict__ grad,
@@ -937,14 +944,14 @@ __device__ __forceinline__ void paired_item_pipe(const LJItem* Ip, const LJItem&
         rz = fma2(na, fz, sub2(pk(pz.y, zn), pz));
         if (!hb) rx.y = ry.y = rz.y = 0.0f;
     };
-    PartSums sums(Ip);
+    PartSums<PARTS> sums(Ip);
     auto account = [&](int a, float2 rx, float2 ry, float2 rz) {
         if (lead) {
             P.rxy(8 * i) = make_float4(rx.x, rx.y, ry.x, ry.y);
             P.rz(8 * i) = rz;
-            sums.add(a, a >= t0, a + 1 < t1, sq3(rx.x, ry.x, rz.x), sq3(rx.y, ry.y, rz.y));
+            sums.add(a, a >= t0, a + 1 < t1, rx, ry, rz);
         }
-        sums.flush(a, t1, partials, red);
+        sums.flush(a, partials, red);
     };
 
     // Item-wide outer list.
@@ -1062,14 +1069,15 @@ __device__ __forceinline__ void paired_item_pipe(const LJItem* Ip, const LJItem&
         }
     }
     if (HS && __syncthreads_or(ov) && threadIdx.x == 0) atomicOr(overlap + S.chain0 + I.chain, 1);
-    sums.put(partials, red);
+    sums.finish(partials, red);
 }
 
 // Persistent grid: each CTA takes items from *counter until none is left.
 // Systems must have N <= MAXT (the block size is at most MAXT).
 // HS: the hard-sphere path bias is on (hs2: squared radii per slice of every LJ
 // system, at LJSysDev::hs_off; overlap: a flag per global chain).
-template <bool GRAD, int MAXT, bool PIPE, bool HS>
+// PARTS: some item has several parts.
+template <bool GRAD, int MAXT, bool PIPE, bool HS, bool PARTS>
 __global__ void __launch_bounds__(MAXT, 1)
     lj_paired_kernel(const LJItem* __restrict__ items, int n_items,
                      const LJSysDev<float>* __restrict__ systems, const float* __restrict__ pos,
@@ -1095,32 +1103,38 @@ __global__ void __launch_bounds__(MAXT, 1)
         const LJItem I = items[it];
         const LJSysDev<float> S = systems[I.sys];
         if (GRAD && PIPE)
-            paired_item_pipe<MAXT, HS>(items + it, I, S, smem_raw, pos, grad, partials, red,
-                                       outer + (long long)blockIdx.x * outer_words, &s_dmax, hs2,
-                                       overlap);
+            paired_item_pipe<MAXT, HS, PARTS>(items + it, I, S, smem_raw, pos, grad, partials, red,
+                                              outer + (long long)blockIdx.x * outer_words, &s_dmax, hs2,
+                                              overlap);
         else
-            paired_item<GRAD, MAXT, HS>(items + it, I, S, smem_raw, pos, grad, partials, red,
-                                        outer + (long long)blockIdx.x * outer_words, &s_dmax, hs2,
-                                        overlap);
+            paired_item<GRAD, MAXT, HS, PARTS>(items + it, I, S, smem_raw, pos, grad, partials, red,
+                                               outer + (long long)blockIdx.x * outer_words, &s_dmax, hs2,
+                                               overlap);
     }
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 // The pipelined form is used with the gradient for blocks of up to 512 threads
 // (its two position buffers and staging area take 88 bytes per particle slot).
-template <bool GRAD, bool HS>
-auto paired_kernel_ptr(int NT, bool pipe)
-{
-    if (GRAD && pipe && NT <= 512) return lj_paired_kernel<GRAD, 512, true, HS>;
-    return NT <= 512 ? lj_paired_kernel<GRAD, 512, false, HS> : lj_paired_kernel<GRAD, 1024, false, HS>;
-}
-
 using PairedKernel = void (*)(const LJItem*, int, const LJSysDev<float>*, const float*, float*,
                               double*, int*, uint32_t*, long long, const float*, int*);
-PairedKernel paired_kernel_sel(int NT, bool with_grad, bool pipe, bool hs)
+template <bool GRAD, bool HS, bool PARTS>
+PairedKernel paired_kernel_ptr(int NT, bool pipe)
 {
-    if (with_grad) return hs ? paired_kernel_ptr<true, true>(NT, pipe) : paired_kernel_ptr<true, false>(NT, pipe);
-    return hs ? paired_kernel_ptr<false, true>(NT, pipe) : paired_kernel_ptr<false, false>(NT, pipe);
+    if constexpr (GRAD)
+        if (pipe && NT <= 512) return lj_paired_kernel<GRAD, 512, true, HS, PARTS>;
+    return NT <= 512 ? lj_paired_kernel<GRAD, 512, false, HS, PARTS> : lj_paired_kernel<GRAD, 1024, false, HS, PARTS>;
+}
+template <bool GRAD>
+PairedKernel paired_kernel_of(int NT, bool pipe, bool hs, bool parts)
+{
+    return hs      ? paired_kernel_ptr<GRAD, true, true>(NT, pipe)
+           : parts ? paired_kernel_ptr<GRAD, false, true>(NT, pipe)
+                   : paired_kernel_ptr<GRAD, false, false>(NT, pipe);
+}
+PairedKernel paired_kernel_sel(int NT, bool with_grad, bool pipe, bool hs, bool parts)
+{
+    return with_grad ? paired_kernel_of<true>(NT, pipe, hs, parts) : paired_kernel_of<false>(NT, pipe, hs, parts);
 }
 
 }  // namespace
@@ -1134,7 +1148,7 @@ size_t lj_paired_smem_bytes(int NT, int cap_lane, bool pipe)
 
 int lj_paired_blocks_per_sm(int NT, size_t smem, bool with_grad, bool pipe)
 {
-    auto kern = paired_kernel_sel(NT, with_grad, pipe, false);
+    auto kern = paired_kernel_sel(NT, with_grad, pipe, false, false);
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
         cudaSuccess)
         return 0;
@@ -1146,14 +1160,14 @@ int lj_paired_blocks_per_sm(int NT, size_t smem, bool with_grad, bool pipe)
 cudaError_t launch_lj_paired(const LJItem* items, int n_items, const void* sys_table,
                              const float* pos, float* grad, double* partials, int* counter, int NT,
                              size_t smem, int grid, bool with_grad, bool pipe, uint32_t* outer,
-                             long long outer_words, cudaStream_t st, bool reset, bool follow, const float* hs2,
+                             long long outer_words, cudaStream_t st, bool reset, bool follow, bool parts, const float* hs2,
                              int* overlap)
 {
     if (n_items <= 0) return cudaSuccess;
     if (NT > 1024) return cudaErrorInvalidValue;
     cudaError_t e = reset ? cudaMemsetAsync(counter, 0, sizeof(int), st) : cudaSuccess;
     if (e != cudaSuccess) return e;
-    auto kern = paired_kernel_sel(NT, with_grad, pipe, hs2 != nullptr);
+    auto kern = paired_kernel_sel(NT, with_grad, pipe, hs2 != nullptr, parts);
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};

@@ -109,6 +109,7 @@ struct LJClass {
     long long outer_off = 0;     // its regions in a lane's set
     LJDoubleShape dbl;           // double precision: capacities of lj_double.cu
     double dbl_pairs = 0.0;      // pairs a slice it has records for
+    bool parts = false;          // some of its items have several parts
     int item_off = 0, n_items = 0;  // its items in d_lj_items (cost-sorted)
     int grp_off = 0;             // its items in d_lj_items_grp (grouped by chain)
     std::vector<int> grp_first;  // per global chain c: [grp_first[c], grp_first[c + 1]), relative
@@ -744,17 +745,17 @@ int build_plan(const pamd_problem* p, Plan** out)
                     }
                     // The host-buffer pipeline updates chunks of chains, which need enough items
                     // for the GPU: where these long ones do not make six chunks (one for every
-                    // chain) it takes parts of about 32 steps, each with a sum of its own (at most
-                    // 3 % more in an item).  N = 500, 8 x 4096 steps with host buffers: 5.8 ms in
-                    // three chunks of long items, 9.3 in eight, 4.3 in eight of parts; 8 x 16384:
-                    // 15.9 in eight of long items, 17.0 of parts.  (Unlike systems keep the long items:
-                    // 12 systems of N = 64..864 take 2.7 ms, in parts 3.0.)
+                    // chain) it takes parts of about 32 steps and no less than 250 us, each with a sum
+                    // of its own (a sum takes an item 2 to 4 us).  N = 500, 8 x 4096 steps with host
+                    // buffers: 5.8 ms in three chunks of long items, 9.3 in eight, 4.3 in eight of
+                    // parts; 8 x 16384: 15.9 in eight of long items, 17.0 of parts.  (Unlike systems
+                    // keep the long items: 12 systems of N = 64..864 take 2.7 ms, in parts 3.0.)
                     const bool in_parts = in.size() == 1 && chain > 1 && pipeline_lanes() * rounds < std::min(chain, 6);
                     for (size_t q = 0; q < in.size(); ++q) {
                         LJTune& t = in[q]->tune;
                         t.tile_steps = tile(q, hi);
-                        t.parts = in_parts ? std::max(1, (t.tile_steps + 16) / 32) : 1;
-                        t.tile_steps = (t.tile_steps + t.parts - 1) / t.parts * t.parts;
+                        t.parts = in_parts ? std::max(1, std::min((t.tile_steps + 16) / 32, (int)(t.tile_steps * cost[q] / 250.0))) : 1;
+                        P->lj_cls[k].parts = P->lj_cls[k].parts || t.parts > 1;
                         const SysInfo& si = *in[q];
                         in[q]->tune.outer_cap = lj_outer_cap(si.N, si.pot, std::sqrt(2.0 * p->D * p->dt),
                                                              si.tune.tile_steps, si.tune.tpp);
@@ -770,9 +771,10 @@ int build_plan(const pamd_problem* p, Plan** out)
             for (int q = 0; q < (int)P->sys.size(); ++q) {
                 SysInfo& si = P->sys[q];
                 if (si.kind != PAMD_LJ) continue;
-                const int own = si.T - si.halo_lo, sub = si.tune.tile_steps / si.tune.parts;
-                const int n_sub = (own + sub - 1) / sub;
-                si.n_tiles = (own + si.tune.tile_steps - 1) / si.tune.tile_steps;
+                const int own = si.T - si.halo_lo, tile = si.tune.tile_steps;
+                const int sub = (tile + si.tune.parts - 1) / si.tune.parts, per = (tile + sub - 1) / sub;
+                si.n_tiles = (own + tile - 1) / tile;
+                const int n_sub = (si.n_tiles - 1) * per + (own - (si.n_tiles - 1) * tile + sub - 1) / sub;
                 si.slot0 = slot;
                 for (int b = 0; b < si.chains; ++b) {
                     const int c = si.chain0 + b, slot_c = slot + b * n_sub;
@@ -780,21 +782,15 @@ int build_plan(const pamd_problem* p, Plan** out)
                     Sslots[c].end = slot_c + n_sub;
                     P->lj_chain_count[c] = si.n_tiles;
                     P->lj_chain_class[c] = si.lj_class;
-                    // items of `parts` parts, and every part as an item
-                    for (int n : {si.tune.parts, 1}) {
-                        SysItems& out = n == si.tune.parts ? sys_items[q] : sys_parts[q];
-                        for (int tl = 0; tl * n < n_sub; ++tl) {
-                            LJItem it;
-                            it.sys = si.lj_index;
-                            it.chain = b;
-                            it.t0 = si.halo_lo + tl * n * sub;  // owned steps only
-                            it.t1 = std::min(si.T, it.t0 + n * sub);
-                            it.slot = slot_c + tl * n;
-                            it.sub = sub;
-                            out.items.push_back(it);
-                            out.cost.push_back(lj_step_cost(si.N, si.tune) * (it.t1 - it.t0) + lj_item_cost(si.N, si.tune));
-                        }
-                        if (si.tune.parts == 1) break;  // (the same)
+                    auto add = [&](SysItems& out, int t0, int t1, int at) {
+                        out.items.push_back(LJItem{si.lj_index, b, t0, t1, at, sub});
+                        out.cost.push_back(lj_step_cost(si.N, si.tune) * (t1 - t0) + lj_item_cost(si.N, si.tune));
+                    };
+                    for (int tl = 0; tl < si.n_tiles; ++tl) {
+                        const int t0 = si.halo_lo + tl * tile, t1 = std::min(si.T, t0 + tile);  // owned steps only
+                        add(sys_items[q], t0, t1, slot_c + tl * per);
+                        for (int p = 0; per > 1 && t0 + p * sub < t1; ++p)  // every part as an item
+                            add(sys_parts[q], t0 + p * sub, std::min(t1, t0 + (p + 1) * sub), slot_c + tl * per + p);
                     }
                 }
                 slot += si.chains * n_sub;
@@ -808,7 +804,7 @@ int build_plan(const pamd_problem* p, Plan** out)
                     for (int q = 0; q < (int)P->sys.size(); ++q) {
                         const SysInfo& si = P->sys[q];
                         if (si.kind != PAMD_LJ || si.lj_class != k) continue;
-                        const SysItems& from = parts && si.tune.parts > 1 ? sys_parts[q] : sys_items[q];
+                        const SysItems& from = parts && !sys_parts[q].items.empty() ? sys_parts[q] : sys_items[q];
                         for (size_t m = 0; m < from.items.size(); ++m) {
                             const int c = si.chain0 + from.items[m].chain;
                             if (!parts && P->lj_chain_first[c] < 0) P->lj_chain_first[c] = (int)(items.size() + ci.size());
@@ -1033,14 +1029,14 @@ int run_action(const pamd_problem* p, Plan* P, const R* pos, R* grad, double* S_
         const LJClass& C = P->lj_cls[k];
         if (C.n_items <= 0) continue;
         const int grid = with_grad ? C.grid_grad : C.grid_nograd;
-        auto launch = [&](const LJItem* items, int n, int g) -> cudaError_t {
+        auto launch = [&](const LJItem* items, int n, int g, bool parts = false) -> cudaError_t {
             if (std::is_same<R, float>::value && P->lj_paired) {
                 const bool follow = classes && launched;
                 launched = true;
                 return launch_lj_paired(items, n, P->d_lj_sys, (const float*)pos, (float*)grad,
                                         P->d_part_S, counter + (classes ? k : 0), C.NT, C.smem, g, with_grad,
                                         C.pipe, P->d_outer[lane] + C.outer_off,
-                                        C.outer_words, st, !classes, follow, (const float*)hs2, overlap);
+                                        C.outer_words, st, !classes, follow, parts, (const float*)hs2, overlap);
             }
             if constexpr (std::is_same<R, double>::value)
                 return launch_lj_double(items, n, P->d_lj_sys, C.nmax, C.dbl, pos, grad, P->d_part_S, counter,
@@ -1058,7 +1054,7 @@ int run_action(const pamd_problem* p, Plan* P, const R* pos, R* grad, double* S_
                 PAMD_CUDA_TRY(launch(P->d_lj_items + f, n, std::min(grid, n)));
             }
         } else if (all) {
-            PAMD_CUDA_TRY(launch(P->d_lj_items + C.item_off, C.n_items, grid));
+            PAMD_CUDA_TRY(launch(P->d_lj_items + C.item_off, C.n_items, grid, C.parts));
         } else {
             const int f = C.grp_first[c0], n = C.grp_first[c1] - f;
             if (n > 0) PAMD_CUDA_TRY(launch(P->d_lj_items_grp + C.grp_off + f, n, std::min(grid, n)));

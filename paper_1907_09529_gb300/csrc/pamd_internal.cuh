@@ -481,7 +481,8 @@ cudaError_t launch_hs_fixup(double* S, const int* overlap, int n, cudaStream_t s
 size_t lj_paired_smem_bytes(int NT, int cap_lane, bool pipe);
 int lj_paired_blocks_per_sm(int NT, size_t smem, bool with_grad, bool pipe);
 // reset: zero the counter first (else the caller has).  follow: the launch before on st is
-// another one of these on other items; start as it leaves SMs free.
+// another one of these on other items; start as it leaves SMs free.  parts: some item has
+// several parts.
 // outer: per-CTA outer lists, outer_words 32-bit words for each of grid CTAs.
 // hs2 (NULL: no bias): squared hard-sphere radii per slice of every LJ system
 // (LJSysDev::hs_off); overlap: per global chain, set to 1 where a pair lies within
@@ -489,7 +490,7 @@ int lj_paired_blocks_per_sm(int NT, size_t smem, bool with_grad, bool pipe);
 cudaError_t launch_lj_paired(const LJItem* items, int n_items, const void* sys_table,
                              const float* pos, float* grad, double* partials, int* counter, int NT,
                              size_t smem, int grid, bool with_grad, bool pipe, uint32_t* outer,
-                             long long outer_words, cudaStream_t st, bool reset, bool follow,
+                             long long outer_words, cudaStream_t st, bool reset, bool follow, bool parts,
                              const float* hs2, int* overlap);
 
 // Double-precision action (+ adjoint), lj_double.cu: each unordered pair's coefficients
