@@ -735,12 +735,20 @@ int build_plan(const pamd_problem* p, Plan** out)
                     // rounds badly (64 chains on 152 CTAs: 128 items), and more rounds of shorter
                     // items take less although each costs its constant again (N = 256, 40 x 512
                     // steps, action and gradient: 1232 us in one round, 1045 in four; N = 162,
-                    // 64 x 557: 1732 and 1512; N = 173, 64 x 198: 626 and 576).
+                    // 64 x 557: 1732 and 1512; N = 53, 64 x 216: 253 in one, 231 in three).  Steps
+                    // come in pairs, the step before the item among them; what an item costs beyond
+                    // them was fitted to sweeps of 1 to 9 rounds of 15 shapes, N = 33..256 (5 us at
+                    // N = 60, 10 at 108, 22 at 256).
                     if (in.size() == 1) {
+                        const SysInfo& si = *in[0];
+                        const double fixed = std::min(3.0 + 6.0e-4 * si.N * si.N, 15.0 + 1.0e-4 * si.N * si.N);
+                        auto time = [&](long long r, double c) {
+                            return r * (fixed + cost[0] * (2 * ((tile(0, c) + 2) / 2)));
+                        };
                         const long long least = rounds;
                         for (long long r = least + 1; r <= least + 6; ++r) {
                             const double c = cost_of(r);
-                            if (r * c < 0.99 * rounds * hi) rounds = r, hi = c;
+                            if (time(r, c) < 0.99 * time(rounds, hi)) rounds = r, hi = c;
                         }
                     }
                     // The host-buffer pipeline updates chunks of chains, which need enough items
