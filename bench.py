@@ -431,19 +431,21 @@ def run_sampler(args, w, pamd, prob, dev, rank, world):
 def launches_per_update(prob):
     """Kernels of one path update (pamd_path_update with n_updates = 1), without the one
     that sets its parameters.  Harmonic batches: one launch per system when every chain is
-    one element block (4096 elements), else trial and commit per system and the sums with
-    the accept test.  Otherwise: propose, one action launch per harmonic system, one LJ
-    launch per block-size class (two when a single-precision batch mixes N <= 512 and
-    N > 512), reverse, the sums with the accept test, commit."""
+    one element block (4096 elements), else in single precision trial and commit per system
+    and the sums with the accept test.  Otherwise: propose, one action launch per harmonic
+    system, one LJ launch per block-size class (two when a single-precision batch mixes
+    N <= 512 and N > 512; in double precision one, and one for the edges of its items),
+    reverse, the sums with the accept test, commit."""
     n_ho = sum(1 for s in prob.systems if s.kind == "harmonic")
     lj = [s.N for s in prob.systems if s.kind == "lj"]
     if not lj and max(s.d * s.N for s in prob.systems) <= 64:
         one_block = max((s.T + 1) * s.d * s.N for s in prob.systems) <= 4096
-        return n_ho if one_block else 2 * n_ho + 1
+        if one_block or prob.precision == "fp32":
+            return n_ho if one_block else 2 * n_ho + 1
     n_lj = 0
     if lj:
         mixed = min(lj) <= 512 < max(lj) and prob.precision == "fp32"
-        n_lj = 2 if mixed else 1
+        n_lj = 2 if mixed or prob.precision == "fp64" else 1
     return 1 + n_ho + n_lj + 3
 
 

@@ -64,3 +64,24 @@ def test_reference_arm_prints_one_json_line():
     assert d["impl"] == "reference" and d["value"] > 0 and d["unit"] == "particle-timeslices/s"
     assert d["cpu_baseline"]["kind"] == "oracle" and d["cpu_baseline"]["cores"] >= 1
     assert d["e2e"]["h2d_bytes_per_step"] == 0
+
+
+def test_launches_of_an_update():
+    """The kernels that an update launches, by precision and shape (pamd_api.cu: run_ho_updates
+    for harmonic batches in one pass, run_one_update otherwise)."""
+    from types import SimpleNamespace as NS
+    b = _bench()
+
+    def count(precision, *systems):
+        return b.launches_per_update(NS(precision=precision, systems=[
+            NS(kind=kind, N=N, d=d, T=T) for kind, N, d, T in systems]))
+
+    short, long, wide = ("harmonic", 1, 1, 4095), ("harmonic", 1, 1, 4096), ("harmonic", 65, 1, 10)
+    for p in ("fp32", "fp64"):
+        assert count(p, short) == 1 and count(p, short, short) == 2
+        assert count(p, wide) == 5  # propose, action, reverse, sums and test, commit
+    assert count("fp32", long) == 3 and count("fp32", long, short) == 5
+    assert count("fp64", long) == 5 and count("fp64", long, short) == 6
+    small, large = ("lj", 108, 3, 100), ("lj", 600, 3, 100)
+    assert count("fp32", small) == 5 and count("fp32", small, large) == 6 and count("fp32", small, short) == 6
+    assert count("fp64", small) == 6 and count("fp64", small, large) == 6
