@@ -79,3 +79,28 @@ def test_parts_of_long_items(pamd, shapes):
     for q in range(len(systems)):
         assert torch.equal(prob.view(buf, q).cpu(), prob.view(host[0], q))
         assert torch.equal(prob.view(g, q).cpu(), prob.view(host[1], q))
+
+
+@pytest.mark.parametrize("N,B", [(520, 1), (560, 3), (700, 2), (300, 2), (90, 3), (33, 4)])
+def test_overflowing_lists_give_the_same_results(pamd, N, B):
+    """Window lists that overflow (all of them, with room for a few entries) take their
+    candidates from the outer lists, or from all particles where these are not much shorter:
+    bit for bit the results of lists with room, for long and short items."""
+    T, L = 70, inputs.box_side(864, 0.85)
+    prob = pamd.Problem([pamd.System("lj", N, 3, T, B, box=L, rc=2.5)], 1.0, 1.0, 1e-4)
+    pos = prob.empty("cuda")
+    prob.view(pos, 0)[:, 0].copy_(torch.from_numpy(inputs.fcc_lattice(864, L)[:, :N].copy()))
+    pamd.euler_reference(prob, pos, seed=2)
+    out = []
+    try:
+        for tile, cap in ((0, 0), (0, 24), (7, 24), (0, 1)):
+            pamd.tune(tile, 0, cap)
+            S, g = pamd.action_grad(prob, pos)
+            assert torch.equal(S, pamd.action(prob, pos))
+            out.append((S.clone(), prob.view(g, 0).clone()))
+    finally:
+        pamd.tune()
+    torch.cuda.synchronize()
+    for S, g in out[1:]:
+        assert torch.equal(g, out[0][1])
+        assert float(((S - out[0][0]).abs() / S.abs()).max()) < 1e-13  # FP64 sums of the items
