@@ -111,3 +111,54 @@ def test_images_far_away(pamd, boxes, tile):
     assert abs(So - Sn) <= 1e-12 * Sn and rel(go, gn) <= 1e-12  # (the oracle's images are exact too)
     assert torch.equal(S, S1) and abs(S[0].item() - So) <= 1e-12 * So
     assert rel(prob.view(g, 0)[0].cpu().numpy(), go) <= 1e-12
+
+
+@pytest.mark.parametrize("k", [-58, -57, -56, -55, -54, -1, 1, 46, 47, 48, 49, 50])
+def test_units_of_any_size(pamd, k):
+    """Lengths in units of 2^k (energies of 4^k): every term scales by a power of two, but for
+    1/r, which has a form of its own where r^2 lies in 2^-111..2^97 and the library's elsewhere.
+    A few ulp of 1/r (2e-16 each) to the power 14 and sums of 60 terms: 1e-12 covers them."""
+    N, T, B, D, beta, dt = 60, 4, 2, 0.9, 1.1, 1e-4
+    L = inputs.box_side(N, 0.85)
+    walk = np.cumsum(0.01 * inputs.rng(3).standard_normal((B, T + 1, 3, N)), axis=1)
+    paths = inputs.fcc_lattice(N, L)[None, None] + walk
+    out = []
+    for s in (1.0, 2.0 ** k):
+        prob = pamd.Problem([pamd.System("lj", N, 3, T, B, box=L * s, rc=L / 2 * s, eps=s * s, sigma=s)], D, beta, dt,
+                            "fp64")
+        buf = prob.empty("cuda")
+        prob.view(buf, 0).copy_(torch.from_numpy(paths * s))
+        S, g = pamd.action_grad(prob, buf)
+        torch.cuda.synchronize()
+        out.append((S.cpu().numpy() / (s * s), prob.view(g, 0).cpu().numpy() / s))
+    (S0, g0), (S1, g1) = out
+    assert np.isfinite(g1).all() and np.abs(S1 - S0).max() <= 1e-12 * S0.max()
+    assert np.abs(g1 - g0).max() <= 1e-12 * np.abs(g0).max()
+
+
+@pytest.mark.parametrize("L", [16.0, 1024.0, 16384.0])
+def test_pairs_at_the_cutoff(pamd, L):
+    """Pairs a relative 1e-10 to 1e-6 inside and outside the cutoff, in boxes much larger than
+    it and across their faces: the single-precision search may miss none, and the decision is
+    that of the stored coordinates (their spacing moves a distance by 1e-11 at most).  A
+    wrong decision would change the gradient by the pair's curvature, 1e-6 of it."""
+    N, T, rc, D, beta, dt = 64, 6, 2.5, 0.9, 1.1, 1e-3
+    rng = inputs.rng(int(L))
+    grid = np.array([(x, y, z) for x in range(4) for y in range(4) for z in range(2)], float) * (L / 4)
+    u = rng.standard_normal((32, 3))
+    u /= np.linalg.norm(u, axis=1)[:, None]
+    paths = np.empty((1, T + 1, 3, N))
+    for t in range(T + 1):
+        off = rng.choice([-1, 1], 32) * 10.0 ** rng.uniform(-9.5 if L > 100 else -10, -6, 32)
+        c = grid + 0.01 * rng.standard_normal((32, 3))
+        paths[0, t, :, :32] = (c - 0.5 * rc * (1 + off)[:, None] * u).T
+        paths[0, t, :, 32:] = (c + 0.5 * rc * (1 + off)[:, None] * u).T
+    paths[0, :, :, ::5] += L * 3
+    prob = pamd.Problem([pamd.System("lj", N, 3, T, 1, box=L, rc=rc)], D, beta, dt, "fp64")
+    buf = prob.empty("cuda")
+    prob.view(buf, 0).copy_(torch.from_numpy(paths))
+    S, g = pamd.action_grad(prob, buf)
+    torch.cuda.synchronize()
+    So, go = oracle.action_grad(oracle.lennard_jones(L, rc), paths[0], D, beta, dt, nthreads=8)
+    assert abs(S[0].item() - So) <= 1e-12 * So
+    assert np.abs(prob.view(g, 0)[0].cpu().numpy() - go).max() <= 1e-12 * np.abs(go).max()
