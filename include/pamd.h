@@ -390,10 +390,12 @@ int pamd_normals(uint64_t seed, uint64_t counter, uint32_t stream_id, uint32_t c
 int pamd_device_status(void* stream);
 
 /* Launch-shape override for the Lennard-Jones kernels (0 or a negative skin
- * keeps the automatic choice): steps per CTA tile, threads per particle
- * (1, 2 or 4), neighbour-list capacity per particle, Verlet skin (sigma
- * units; Euler-Maruyama paths and the one-step form), steps per neighbour-list window (single
- * precision; >= 2).  Affects plans built afterwards.  Results do not depend
+ * keeps the automatic choice).  Action, gradient and updates: steps per CTA
+ * tile (single precision: the most that an item takes); in single precision also
+ * threads per particle (1, 2 or 4), neighbour-list capacity per particle and
+ * steps per neighbour-list window (>= 2), which double precision has no use for.
+ * Verlet skin (sigma units): Euler-Maruyama paths above 192 particles and the
+ * one-step form.  Affects plans built afterwards.  Results do not depend
  * on the tile, capacity, skin or window (candidate order is fixed); the
  * number of threads per particle changes how a particle's force and
  * Hessian sums are split, so results differ by rounding only.  PAMD_ERR_ARG

@@ -318,10 +318,9 @@ __global__ void __launch_bounds__(MAXT, (MAXT <= 512 ? 2 : 1))
     }
 }
 
-size_t lj_smem_bytes(int nmax, int NT, int cap_lane, bool fp64)
+size_t lj_smem_bytes(int nmax, int NT, int cap_lane)
 {
-    const size_t v4 = fp64 ? sizeof(double4a) : sizeof(float4);
-    return 3 * (size_t)nmax * v4 + (size_t)cap_lane * NT * sizeof(uint16_t);
+    return 3 * (size_t)nmax * sizeof(float4) + (size_t)cap_lane * NT * sizeof(uint16_t);
 }
 
 template <typename R, bool GRAD>

@@ -388,7 +388,8 @@ double lj_item_cost(int N, const LJTune& t) { return 15.0 + lj_step_cost(N, t) +
 // Per-system LJ launch shape: threads per particle (largest power of two <= 8
 // with N * tpp <= NT), Verlet skin (one-step kernel) or window length (paired
 // kernel), list capacity per thread, tile length.  sig_step = sqrt(2 D dt), the
-// per-component spread of one Brownian step.
+// per-component spread of one Brownian step.  (Double precision takes the tile length alone,
+// and Euler-Maruyama paths the skin.)
 LJTune choose_lj_tune(const pamd_system& s, int NT, int cap_lane_max, bool paired, double sig_step)
 {
     LJTune t;
@@ -616,10 +617,7 @@ int build_plan(const pamd_problem* p, Plan** out)
                 const int budget = (NT <= 512 && !P->fp64 && !P->lj_paired && g_tune_override.maxnb <= 0)
                                        ? 113 * 1024
                                        : max_dynamic_smem() - 1024;
-                // (the one-step Euler kernel shares the capacity: its slices must fit too)
-                const long long slices_euler = 3 * (long long)nmax * v4;
-                const int cap_lane_max = std::max(
-                    1, (int)((budget - std::max(slices, slices_euler)) / (2 * (long long)NT)));
+                const int cap_lane_max = std::max(1, (int)((budget - slices) / (2 * (long long)NT)));
                 int cap_used = 1;
                 for (int q = 0; q < (int)P->sys.size(); ++q) {
                     SysInfo& si = P->sys[q];
@@ -641,7 +639,7 @@ int build_plan(const pamd_problem* p, Plan** out)
                 }
                 C.smem = P->lj_paired ? lj_paired_smem_bytes(NT, cap_used, C.pipe)
                          : P->fp64    ? C.dbl.smem
-                                      : lj_smem_bytes(nmax, NT, cap_used, false);
+                                      : lj_smem_bytes(nmax, NT, cap_used);
                 const int bg = P->lj_paired ? lj_paired_blocks_per_sm(NT, C.smem, true, C.pipe)
                                : P->fp64    ? lj_double_blocks_per_sm(C.dbl, true)
                                             : lj_blocks_per_sm<float>(NT, C.smem, true);

@@ -452,7 +452,7 @@ struct LJItem {
 
 // Shared memory of the LJ action kernel: three slices of nmax particles and a
 // list of cap_lane entries for each of NT threads.
-size_t lj_smem_bytes(int nmax, int NT, int cap_lane, bool fp64);
+size_t lj_smem_bytes(int nmax, int NT, int cap_lane);
 
 template <typename R>
 int lj_blocks_per_sm(int NT, size_t smem, bool with_grad);
