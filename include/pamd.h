@@ -51,8 +51,9 @@
  * Fault injection (tests of the error paths; nothing faults on the device).
  * With the environment variable PAMD_FAULT_INJECT set to "alloc", every
  * workspace allocation fails (PAMD_ERR_ALLOC; a plan that could not be built is
- * not cached), "alloc:N" those of more than N bytes; "launch": every CUDA call the library checks reports failure
- * (PAMD_ERR_CUDA; a graph whose capture failed is not cached); "nonfinite":
+ * not cached), "alloc:N" those of more than N bytes; "launch": every CUDA call
+ * the library checks reports failure (PAMD_ERR_CUDA; a graph whose capture
+ * failed is not cached); "nonfinite":
  * every action computed is flagged non-finite (pamd_device_status then returns
  * PAMD_ERR_NONFINITE); "wait:N": waits between the CTAs of a cluster run out
  * after N rounds (PAMD_ERR_TIMEOUT).  The variable is read at each call.

@@ -15,10 +15,11 @@
 namespace pamd {
 
 constexpr int kEulerDense = 192;  // largest N without lists
-// Up to this size a particle has eight lanes, each adding its candidates in increasing j, and
-// double precision takes the library's 1/sqrt: the arithmetic of the LJ kernels' plain form,
-// bit for bit.  Small boxes are where a start can overlap (33 to 45 particles on a lattice of
-// 108 sites), and such a path turns any other order of the sums into another path.
+// Up to this size a particle has eight sums, each over its candidates in increasing j one after
+// the other, and double precision takes the library's 1/sqrt; above it two candidates are added
+// at a time (single precision), and 1/sqrt is inv_sqrt of lj_math.cuh.  Both are accurate to the
+// rounding of the sums (1e-7, 1e-16).  The older order stays where it is as fast, so that small
+// paths keep their bits from version to version.
 constexpr int kEulerOrdered = 64;
 constexpr int kOrderedLg = 3;
 

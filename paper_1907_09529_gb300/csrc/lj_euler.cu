@@ -11,17 +11,18 @@
 //     and Box-Muller on the chain.
 //   * A chain is stepped by a cluster of CTAs (up to 8).  Each CTA holds all positions
 //     and moves N / CS particles, up to 32 lanes to a particle (how many partial sums a force
-//     has, and so every bit of a path, follows from N alone: euler_shape.cuh); the new coordinates go to
-//     every CTA's shared memory as asynchronous stores counted by a transaction barrier there.
-//     A step costs one trip between SMs; with plain remote stores and a cluster barrier it
-//     also waited for their acknowledgement (N = 108: 1.33 against 0.96 us a step).
+//     has, and so every bit of a path, follows from N alone: euler_shape.cuh); the new
+//     coordinates go to every CTA's shared memory as asynchronous stores counted by a
+//     transaction barrier there.  A step costs one trip between SMs; with plain remote stores
+//     and a cluster barrier it also waited for their acknowledgement (N = 108: 1.33 against
+//     0.96 us a step).  Waits are bounded; what follows one that runs out is in cluster.cuh.
 //   * Small systems (N <= kEulerDense) evaluate every pair: no list, no displacement check,
 //     two candidates per packed f32x2 operation.  Larger ones walk Verlet lists of radius
 //     rc + skin, rebuilt when some particle has moved skin / 2 (a list that overflows scans
 //     all candidates).
 // N = 108, four chains of 1024 steps: 4.89 ms (4.8 us a step) with one CTA of four threads
-// per particle and the normals in the step, 0.98 ms (0.96 us) now; a step of N = 500, eight
-// chains, 17.5 -> 3.5 us, of N = 108 in double precision 101 -> 23 us.
+// per particle and the normals in the step, 0.96 ms (0.94 us) now; a step of N = 500, eight
+// chains, 17.5 -> 3.4 us, of N = 108 in double precision 101 -> 23 us.
 #include <algorithm>
 #include <cmath>
 #include <type_traits>

@@ -19,7 +19,7 @@
 //   r_t   = x_{t+1} - x_t - a F(x_t),               a = beta D dt
 //   (Hv)_i = sum_j [ -fs v_ij + Bc (r_ij . v_ij) r_ij ],   v_ij = v_i - v_j
 //   g_t   = [r_{t-1} - r_t + a H(x_t) r_t] / (2 D dt),  r_{-1} = r_T = 0
-//   S     = sum_t |r_t|^2 / (4 D dt)   (per-item partial sums in FP64)
+//   S     = sum_t |r_t|^2 / (4 D dt)   (partial sums in FP64 per item, or per part of one)
 // A pair outside the cutoff gets r^2 = +inf, which makes every coefficient an
 // exact zero (rsqrt(+inf) = +0).
 //
@@ -27,7 +27,7 @@
 // 118 registers).  500 particles, 8 chains of 4096 steps, action and gradient: 3176 us before
 // the two entries of a list word were interleaved, the window build loaded its words ahead and
 // the items were cut by estimated cost, 2810 us now.  More warps with fewer registers lose
-// (two CTAs of 64 registers an SM: 3100 us two-pass; the action alone 408 against 388).
+// (two CTAs of 64 registers an SM: 3100 us two-pass; the action alone 408 against 389).
 //
 // Work decomposition: a persistent grid pulls (system, chain, tile of steps)
 // items from an atomic queue.  Within an item the steps are walked in pairs
@@ -44,9 +44,10 @@
 // pairs suffices.  The window lists are built from an outer list made once per
 // item by the same rule with item-wide margins (reference at the item's middle
 // slice), which holds every pair that any of the item's windows can need; it
-// sits in global memory (one region per CTA, L2-resident).  A particle whose
-// outer list overflows builds its window lists from all candidates; one whose
-// window list overflows scans all candidates.  Candidates are visited in one
+// sits in global memory (one region per CTA; what is used of them stays in L2).
+// A particle whose outer list overflows builds its window lists from all
+// candidates; one whose window list overflows scans all candidates, in blocks of
+// 1024 threads those of its outer list.  Candidates are visited in one
 // fixed order in every case -- by class (j - tid) mod 8, then by increasing j --
 // so each force and Hessian sum runs over the in-cutoff pairs in one order
 // whatever the tiling, window or list capacity, and the results are bitwise

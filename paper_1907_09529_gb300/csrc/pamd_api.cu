@@ -420,7 +420,8 @@ LJTune choose_lj_tune(const pamd_system& s, int NT, int cap_lane_max, bool paire
     // Room for one and a half times the mean density (partly filled boxes, droplets), where the
     // shared memory has it: a list that overflows scans all candidates at every step (a batch
     // with 502 particles on a lattice of 864 sites: 3725 us with 1.2 times, 1779 with 1.5; the
-    // shared memory it takes from L1 costs N = 500 0.1 to 0.3 %, N = 600 1 %).
+    // shared memory it takes from L1 costs the action and gradient of N = 500 0.1 to 0.3 %, of
+    // N = 600 1 %).
     int want = (int)((paired ? 1.5 : 1.2) * expect) + 8;
     if (want > N - 1 + tpp) want = N - 1 + tpp;
     if (g_tune_override.maxnb > 0) want = g_tune_override.maxnb;
@@ -683,11 +684,11 @@ int build_plan(const pamd_problem* p, Plan** out)
                             cmin = std::max(cmin, cost.back() + lj_item_cost(si.N, si.tune));
                         }
                     // Unlike systems with N > 512: their lists have no room beyond the mean density
-                    // (shared memory), and a system that is denser than its mean scans all
-                    // candidates and takes several times its estimate.  Short items spread that (a
-                    // batch with 513 and 532 particles on lattices of 864 sites: 8851 us with the
-                    // longest items, 5331 with at most 32 steps; one with 514 and 531: 8873, 3932;
-                    // batches without such systems 0 to 10 % more, two of twelve).
+                    // (shared memory), and a system that is denser than its mean takes more than its
+                    // estimate.  Short items spread that (when overflowing lists scanned all
+                    // candidates, a batch with 513 and 532 particles on lattices of 864 sites took
+                    // 8851 us with the longest items, 5331 with at most 32 steps; longer items have
+                    // not been tried since such lists walk the outer list).
                     const int lim = in.size() > 1 && P->lj_cls[k].nmax > 512 ? std::min(limit, 32) : limit;
                     // steps per item of system q at cost c, and the items all chains then need
                     auto tile = [&](size_t q, double c) {
@@ -1149,10 +1150,11 @@ int waits_status(Plan* P)
 
 // Path updates with host buffers (no explicit noise or uniforms), pipelined over
 // chunks of chains: chunk k's inputs are copied in on one stream while earlier
-// chunks are updated and copied back on others.  Updates alternate between the
-// caller's stream and a second compute stream, each chunk with its own LJ work
-// counter, so that the last items of one chunk overlap the next chunk.  Chains
-// are independent, so the results equal those of one update over all.
+// chunks are updated and copied back on others.  Updates rotate over the compute
+// lanes (the caller's stream and others), each chunk with its own LJ work
+// counters, so that the last items of one chunk overlap the next chunk.  Chains
+// are independent, and items of chunks are the parts of the whole batch's items,
+// so the results equal those of one update over all.
 template <typename R>
 int path_update_pipelined(const pamd_problem* prob, Plan* P, void* pos, void* grad, double* S,
                           int n_updates, int* n_accepted, double* log_alpha, cudaStream_t st)
