@@ -111,8 +111,11 @@ struct DenseForce {
             fz = fma2(fs, dz, fz);
         }
     }
-    // p: the slice; candidates 2m, 2m + 1 of sum q are the float2 at m 2^LG + q
-    __device__ __forceinline__ void operator()(const float* p, const float (&xi)[3], int q, float (&f)[3]) const
+    // p: the slice; candidates 2m, 2m + 1 of sum q are the float2 at m 2^LG + q.  SKIP: nothing
+    // is done for a last pair of padding (exact zeros): for lanes with several sums, where it
+    // is worth the test (200 chains of N = 65: 3.5 against 4.4 us a step)
+    template <bool SKIP>
+    __device__ __forceinline__ void sum(const float* p, const float (&xi)[3], int q, float (&f)[3]) const
     {
         const float2 x = pk(xi[0]), y = pk(xi[1]), z = pk(xi[2]);
         float2 fx = pk(0.0f), fy = pk(0.0f), fz = pk(0.0f);
@@ -120,7 +123,7 @@ struct DenseForce {
         int j = q;
 #pragma unroll 2
         for (int m = 0; m < full; ++m, j += 2 << LG, a += 1 << LG) two<false>(a, j, x, y, z, fx, fy, fz);
-        if (full < all) two<true>(a, j, x, y, z, fx, fy, fz);
+        if (full < all && (!SKIP || j < N)) two<true>(a, j, x, y, z, fx, fy, fz);
         f[0] = fx.x + fx.y;
         f[1] = fy.x + fy.y;
         f[2] = fz.x + fz.y;
@@ -356,7 +359,7 @@ __global__ void __launch_bounds__(MAXT)
                                 f[2] = fma_r(fs, dz, f[2]);
                             }
                     } else if constexpr (LG >= 0) {
-                        dense(A.p, xi, j0, f);
+                        dense.template sum<(VR > 0)>(A.p, xi, j0, f);
                     } else {
                         for (int j = j0; j < N; j += dj)
                             if (j != i) pair_force<R>(xi[0], xi[1], xi[2], *A.at(j, 0), *A.at(j, 1), *A.at(j, 2), k, f);
