@@ -35,6 +35,7 @@
 // length nor on the scratch capacity (a pair beyond the capacity is evaluated again
 // where it is needed, by the same instructions).
 #include <algorithm>
+#include <type_traits>
 
 #include "lj_math.cuh"
 
@@ -289,40 +290,47 @@ __global__ void __launch_bounds__(NT, MINB)
                 const int c = e / N, n = e - c * N;
                 const double x = __ldg(Xt + e);
                 const double m = __fma_rn(x, C.k.iL, 6755399441055744.0);
-                far |= !(fabs(__dsub_rn(m, 6755399441055744.0)) < 1073741824.0);
+                // m = 1.5 2^52 + k, k the box index: |k| < 2^30 told from the words of m
+                const int k = __double2loint(m);
+                far |= (__double2hiint(m) != 0x43380000 + (k >> 31)) | ((unsigned)k + 0x40000000u >= 0x80000000u);
                 C.X[3 * n + c] = x;
-                C.K[3 * n + c] = __double2loint(m);
+                C.K[3 * n + c] = k;
                 reinterpret_cast<float*>(C.W + n)[c] = (float)__fma_rn(-C.k.L, __dsub_rn(m, 6755399441055744.0), x);
             }
             C.hbf = __syncthreads_or(far) ? -1.0f : 0.4999f * C.Lf;
             // adjacency rows: a warp per particle, 32 candidates per step
-            for (int i = warp; i < N; i += NWARP) {
-                const float4 wi = C.W[i];
-                int cnt = 0;
-                for (int w = 0; w < C.NW; ++w) {
-                    const int j = 32 * w + lane;
-                    bool in = false;
-                    if (j < N) {
-                        const float4 wj = C.W[j];
-                        float dx = wi.x - wj.x, dy = wi.y - wj.y, dz = wi.z - wj.z;
-                        dx = fmaf(-C.Lf, C.image(dx), dx);
-                        dy = fmaf(-C.Lf, C.image(dy), dy);
-                        dz = fmaf(-C.Lf, C.image(dz), dz);
-                        in = fmaf(dz, dz, fmaf(dy, dy, dx * dx)) <= C.lim2 && j != i;
-                        if (C.hbf < 0.0f) {
+            auto search = [&](auto far_c) {
+                for (int i = warp; i < N; i += NWARP) {
+                    const float4 wi = C.W[i];
+                    int cnt = 0;
+                    for (int w = 0; w < C.NW; ++w) {
+                        const int j = 32 * w + lane;
+                        bool in = false;
+                        if (j < N && !decltype(far_c)::value) {
+                            const float4 wj = C.W[j];
+                            float dx = wi.x - wj.x, dy = wi.y - wj.y, dz = wi.z - wj.z;
+                            dx = fmaf(-C.Lf, C.image(dx), dx);
+                            dy = fmaf(-C.Lf, C.image(dy), dy);
+                            dz = fmaf(-C.Lf, C.image(dz), dz);
+                            in = fmaf(dz, dz, fmaf(dy, dy, dx * dx)) <= C.lim2 && j != i;
+                        } else if (decltype(far_c)::value && j < N && j != i) {
                             double ex, ey, ez;
-                            in = j != i && pair_r2<double>(C.X[3 * i], C.X[3 * i + 1], C.X[3 * i + 2], C.X[3 * j],
-                                                           C.X[3 * j + 1], C.X[3 * j + 2], C.k, ex, ey, ez) <= C.k.rc2;
+                            in = pair_r2<double>(C.X[3 * i], C.X[3 * i + 1], C.X[3 * i + 2], C.X[3 * j], C.X[3 * j + 1],
+                                                 C.X[3 * j + 2], C.k, ex, ey, ez) <= C.k.rc2;
                         }
+                        const uint32_t m = __ballot_sync(0xffffffffu, in);
+                        if (lane == 0) {
+                            C.bits[i * C.NW + w] = m;
+                            C.pre[i * C.NW + w] = (uint16_t)cnt;
+                        }
+                        cnt += __popc(m);
                     }
-                    const uint32_t m = __ballot_sync(0xffffffffu, in);
-                    if (lane == 0) {
-                        C.bits[i * C.NW + w] = m;
-                        C.pre[i * C.NW + w] = (uint16_t)cnt;
-                    }
-                    cnt += __popc(m);
                 }
-            }
+            };
+            if (C.hbf < 0.0f)
+                search(std::true_type{});
+            else
+                search(std::false_type{});
             __syncthreads();
             // pairs j > i are numbered row by row: pair (i, j) has slot
             // base[i] + (neighbours of i below j); base[i] = pairs of earlier rows - neighbours below i
